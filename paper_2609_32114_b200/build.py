@@ -28,6 +28,8 @@ INCLUDE = os.path.join(ROOT, "include")
 UNITS = [("api", "api.cu", []), ("plan", "plan.cu", []), ("tc", "tc.cu", []), ("tc_prep", "tc_prep.cu", []), ("tc_chain", "tc_chain.cu", []), ("tc_seg", "tc_seg.cu", []),
          ("noalloc", "noalloc.cu", []), ("decode", "decode.cu", [])] + [
     (f"simt{u}", "simt.cu", [f"-DHA_LA_SIMT_UNIT={u}"]) for u in range(5)
+] + [
+    (f"fp32_{u}", "fp32.cu", [f"-DHA_LA_FP32_UNIT={u}"]) for u in range(5)
 ]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 

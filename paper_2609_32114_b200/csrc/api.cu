@@ -74,7 +74,7 @@ int ha_la_prefill_workspace_bytes(const ha_la_prefill_args* args, size_t* out_by
   const int rc = make_problem(args, &p);
   if (rc != HA_LA_OK) return rc;
   size_t bytes = plan_bytes(p);
-  if (tc_supported(p)) bytes += tc_workspace_bytes(p);
+  bytes += use_tc(p) ? tc_workspace_bytes(p) : fp32_workspace_bytes(p);
   *out_bytes = align_up(bytes, 256);
   return HA_LA_OK;
 }
@@ -85,16 +85,13 @@ const char* ha_la_prefill_path(const ha_la_prefill_args* args) {
   return use_tc(p) ? "tc" : "simt";
 }
 
-// The chunk table is only needed for packed batches and by the CUDA-core kernel; the tensor-core
-// kernels index equal-length rows arithmetically.
-static bool needs_plan(const ha_la_prefill_args* a, const Problem& p) {
-  return a->num_seqs > 0 || a->cu_seqlens != nullptr || !use_tc(p);
-}
+// The chunk table is only needed for packed batches; equal-length rows are indexed arithmetically.
+static bool needs_plan(const ha_la_prefill_args* a) { return a->num_seqs > 0 || a->cu_seqlens != nullptr; }
 
 int ha_la_prefill_num_launches(const ha_la_prefill_args* args) {
   Problem p;
   if (make_problem(args, &p) != HA_LA_OK) return 0;
-  return (needs_plan(args, p) ? 1 : 0) + (use_tc(p) ? tc_num_launches(p) : 1);
+  return (needs_plan(args) ? 1 : 0) + (use_tc(p) ? tc_num_launches(p) : 2);
 }
 
 int ha_la_prefill_num_segments(const ha_la_prefill_args* args) {
@@ -135,7 +132,7 @@ int ha_la_prefill(const ha_la_prefill_args* a, void* cuda_stream) {
 
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   PlanView plan = plan_view(a->workspace, p);
-  if (needs_plan(a, p)) {
+  if (needs_plan(a)) {
     if (launch_plan(p, a->cu_seqlens, plan, a->status_word, stream) != cudaSuccess) return HA_LA_ERR_CUDA;
   } else {
     plan = PlanView{};                                   // null table: equal-length rows, indexed arithmetically
@@ -143,12 +140,8 @@ int ha_la_prefill(const ha_la_prefill_args* a, void* cuda_stream) {
   if (p.T_total == 0 && !a->hT) return HA_LA_OK;
 
   cudaError_t e;
-  if (use_tc(p)) {
-    void* tc_ws = reinterpret_cast<char*>(a->workspace) + plan_bytes(p);
-    e = launch_tc(p, *a, plan, tc_ws, stream);
-  } else {
-    e = launch_simt(p, *a, plan, stream);
-  }
+  void* ws = reinterpret_cast<char*>(a->workspace) + plan_bytes(p);
+  e = use_tc(p) ? launch_tc(p, *a, plan, ws, stream) : launch_fp32(p, *a, plan, ws, stream);
   return e == cudaSuccess ? HA_LA_OK : HA_LA_ERR_CUDA;
 }
 

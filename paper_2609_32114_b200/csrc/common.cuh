@@ -65,6 +65,10 @@ cudaError_t launch_plan(const Problem& p, const int32_t* cu_seqlens, PlanView pl
 cudaError_t launch_simt(const Problem& p, const ha_la_prefill_args& a, PlanView plan, cudaStream_t stream);
 bool simt_supported(const Problem& p);
 
+// fp32 CUDA-core path in two kernels (chunk-local part, sequential part) with a workspace.
+size_t fp32_workspace_bytes(const Problem& p);
+cudaError_t launch_fp32(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* ws, cudaStream_t stream);
+
 // Tensor-core (tcgen05) path: bf16, d_k = d_v = 128.
 bool tc_supported(const Problem& p);
 size_t tc_workspace_bytes(const Problem& p);

@@ -1,0 +1,642 @@
+// fp32 chunkwise delta-rule prefill (GDN and KDA) on the CUDA cores, in two kernels: fp32 inputs (where the 1e-4 tolerance
+// rules out 16-bit tensor-core operands) and head dimension 64.  All arithmetic is fp32.
+//
+//   fp32_prep_kernel   one CTA per (chunk, V-head): operators #1-#4 of the paper's pipeline (Section 2.1, "Chunkwise
+//                      Map-Reduce-Map Execution").  Chunks are independent here, so a single short sequence already
+//                      keeps several SMs busy instead of one.
+//   fp32_walk_kernel   one CTA per (sequence, V-head, 8 or 16 value channels) walks the chunks in order: operator #5 with #6 in
+//                      the paper's chunk-first order.  Value channels are independent ("Computation Splitting"), so the
+//                      sequential part of a head is spread over several SMs.
+//
+// Per chunk the prep kernel leaves, as fp32 rows padded for conflict-free 16-byte shared-memory reads:
+//   W = T diag(beta) (K e^G)   QG = Q e^G   KD = K e^{G_L-G}   P = decay-masked Q K^T   U = T diag(beta) V   e^{G_L}
+// and the walk does    U~ = U - W h;   o = scale (QG h + P U~);   h <- e^{G_L} h + KD^T U~.
+//
+// What bounds it: shared-memory reads (a 16-byte read costs four cycles of the SM's 128 bytes whatever is shared between
+// lanes; the thread tiles here do 16 multiply-adds for five of them: 4.2 k cycles per chunk of the d = 64 walk, 76 % of its
+// time), and for short sequences the walk's chain of chunks.  One call with T = 256, one head, d = 64: one CTA for
+// everything took 237 us, split like this 21.6 us; d = 64, 8 heads, T = 1000: 924 us -> 53.7 us.
+#include "common.cuh"
+#include "tc_ptx.cuh"
+
+#include <atomic>
+
+namespace ha_la {
+
+using namespace ptx;
+
+namespace {
+
+template <typename T> __device__ __forceinline__ float to_f32(T x);
+template <> __device__ __forceinline__ float to_f32<float>(float x) { return x; }
+template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
+template <typename T> __device__ __forceinline__ T from_f32(float x);
+template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
+template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
+
+constexpr int C = kChunk;
+constexpr int kNV = 16;                                  // value channels per slice of U in a record
+constexpr int LDP = C + 4;                               // row strides in floats: rows 16 bytes apart in the banks
+
+// record of one (chunk slot, V-head), in floats
+template <int D> struct Rec {
+  static constexpr int LD = D + 4;
+  static constexpr int W = 0;                            // [C][LD]
+  static constexpr int QG = W + C * LD;                  // [C][LD]
+  static constexpr int KD = QG + C * LD;                 // [C][LD]
+  static constexpr int P = KD + C * LD;                  // [C][LDP]
+  static constexpr int GAM = P + C * LDP;                // [D]  e^{G_L} per key channel
+  static constexpr int U = GAM + D;                      // [D / kNV][C][kNV]
+  static constexpr int size = U + C * D;
+};
+
+struct Fp32Params {
+  const void* q; const void* k; const void* v;
+  const float* g; const float* beta; const float* h0;
+  void* o; float* hT;
+  float* rec;
+  const int32_t* chunk_tok0;   // chunk table of the plan kernel, or NULL for equal-length rows:
+  const int32_t* chunk_len;    //   slot s is chunk s % cps of row s / cps, T_row tokens per row
+  const int32_t* seq_tok0; const int32_t* seq_len; const int32_t* seq_chunk0; const int32_t* seq_order;
+  int T_row, cps;
+  int HK, HV;
+  float scale;
+  int32_t* status;
+};
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+template <typename In> __device__ __forceinline__ float4 load4(const In* p);   // four consecutive inputs
+template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return ld4(p); }
+template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
+  const uint2 w = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float c) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+}
+
+// ------------------------------------------------------------------------------------------------ chunk-local part
+template <int D, bool KDA> struct PrepSmem {
+  static constexpr int LD = D + 4;
+  static constexpr int K = 0;                            // [C][LD]
+  static constexpr int Q = K + C * LD;                   // [C][LD]
+  static constexpr int A = Q + C * LD;                   // [C][LDP]
+  static constexpr int G = A + C * LDP;                  // GDN [C]; KDA [C][LD]: cumulative log-gate
+  static constexpr int B = G + (KDA ? C * LD : C);       // [C] beta
+  static constexpr int RHS = B + C;                      // [C][2 D]: (W |) U columns of the substitution
+  static constexpr int KM = KDA && D == 128 ? RHS : RHS + C * 2 * D;   // KDA: K e^{R_I-G}, block rows I = 1, 2, 3 (16, 32, 48
+                                                         // rows); d = 128: over the columns, which are filled later
+  static constexpr int size = KDA && D == 64 ? KM + 96 * LD : RHS + C * 2 * D;
+};
+
+template <typename In, int D, bool KDA>
+__global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
+  using S = PrepSmem<D, KDA>;
+  using R = Rec<D>;
+  constexpr int LD = D + 4;
+  extern __shared__ __align__(16) float sf[];
+  float* sK = sf + S::K;
+  float* sQ = sf + S::Q;
+  float* sA = sf + S::A;
+  float* sG = sf + S::G;
+  float* sB = sf + S::B;
+  const int tid = threadIdx.x;
+  const int slot = blockIdx.x / p.HV, j = blockIdx.x % p.HV, jq = j / (p.HV / p.HK);
+  // (this call's kernels are launched as programmatic dependents; nothing has been read so far)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int L, t0;
+  if (p.chunk_len) {
+    L = p.chunk_len[slot];
+    t0 = p.chunk_tok0[slot];
+  } else {
+    const int cc = slot % p.cps;
+    t0 = (slot / p.cps) * p.T_row + cc * C;
+    L = min(C, p.T_row - cc * C);
+  }
+  if (L <= 0) return;                                    // a slot that a packed batch does not use
+  const In* gq = reinterpret_cast<const In*>(p.q);
+  const In* gk = reinterpret_cast<const In*>(p.k);
+  const In* gv = reinterpret_cast<const In*>(p.v);
+  float* rec = p.rec + (size_t)blockIdx.x * R::size;
+
+  constexpr bool kLateV = KDA && D == 128;               // (its room holds the rescaled K rows first)
+  auto v_row = [&](int i, int c) {
+    return i < L ? load4<In>(gv + ((size_t)(t0 + i) * p.HV + j) * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  // ---- load the chunk; rows >= L are no-op tokens (k = q = v = 0, beta = 0, g = 0)
+#pragma unroll
+  for (int idx = tid; idx < C * (D / 4); idx += 256) {
+    const int i = idx / (D / 4), c = (idx % (D / 4)) * 4;
+    float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f), k4 = q4, g4 = q4;
+    if (i < L) {
+      const size_t off = ((size_t)(t0 + i) * p.HK + jq) * D + c;
+      q4 = load4<In>(gq + off);
+      k4 = load4<In>(gk + off);
+      if (KDA) g4 = ld4(p.g + ((size_t)(t0 + i) * p.HV + j) * D + c);
+    }
+    *reinterpret_cast<float4*>(sQ + i * LD + c) = q4;
+    *reinterpret_cast<float4*>(sK + i * LD + c) = k4;
+    if (!kLateV) *reinterpret_cast<float4*>(sf + S::RHS + i * 2 * D + D + c) = v_row(i, c);
+    if (KDA) *reinterpret_cast<float4*>(sG + i * LD + c) = g4;
+  }
+  if (tid < C) {
+    sB[tid] = tid < L ? p.beta[(size_t)(t0 + tid) * p.HV + j] : 0.f;
+    if (!KDA) sG[tid] = tid < L ? p.g[(size_t)(t0 + tid) * p.HV + j] : 0.f;
+  }
+  __syncthreads();
+
+  // ---- op #1 Gate: chunk-local inclusive cumulative sum of the log-gate
+  if (KDA) {
+    if (tid < D) {
+      float acc = 0.f;
+      for (int i = 0; i < C; ++i) { acc += sG[i * LD + tid]; sG[i * LD + tid] = acc; }
+    }
+  } else if (tid < 32) {
+    float x0 = sG[tid], x1 = sG[tid + 32];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
+      if (tid >= o) { x0 += y0; x1 += y1; }
+    }
+    x1 += __shfl_sync(0xffffffffu, x0, 31);
+    sG[tid] = x0;
+    sG[tid + 32] = x1;
+  }
+  __syncthreads();
+
+  // ---- op #2: A (strictly lower, beta-scaled, negated: what the substitution adds) and P (lower incl. diagonal), in
+  // 16 x 16 blocks; thread (tr, tc) owns one entry of every block.
+  const int tr = tid >> 4, tc = tid & 15;
+  float kk[4][4], qk[4][4];                              // [block row][block column <= block row]
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) kk[a][b] = qk[a][b] = 0.f;
+  if constexpr (!KDA) {
+#pragma unroll 2
+    for (int c = 0; c < D; c += 4) {
+      float4 kj[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) kj[b] = ld4(sK + (16 * b + tc) * LD + c);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const float4 ki = ld4(sK + (16 * a + tr) * LD + c), qi = ld4(sQ + (16 * a + tr) * LD + c);
+#pragma unroll
+        for (int b = 0; b <= a; ++b) {
+          kk[a][b] = dot4(ki, kj[b], kk[a][b]);
+          qk[a][b] = dot4(qi, kj[b], qk[a][b]);
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b <= a; ++b) {
+        const float e = 16 * b + tc <= 16 * a + tr ? expf(sG[16 * a + tr] - sG[16 * b + tc]) : 0.f;
+        kk[a][b] *= e;
+        qk[a][b] *= e;
+      }
+  } else {
+    // The decay sits inside the contraction.  For i in block row I and j in an EARLIER block it factors through the gate
+    // R_I of the block row's first token, e^{G_i-R_I} e^{R_I-G_j}, both exponents <= 0: a plain contraction of rescaled
+    // rows.  Inside the diagonal block the second exponent would be >= 0 without bound, so it is evaluated entry by entry.
+    float* sM = sf + S::KM;
+    for (int idx = tid; idx < 96 * (D / 4); idx += 256) {
+      const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
+      const int I = r < 16 ? 1 : (r < 48 ? 2 : 3), jj = r - (I == 1 ? 0 : (I == 2 ? 16 : 48));
+      const float4 k4 = ld4(sK + jj * LD + c), g4 = ld4(sG + jj * LD + c), r4 = ld4(sG + 16 * I * LD + c);
+      *reinterpret_cast<float4*>(sM + r * LD + c) = make_float4(k4.x * expf(r4.x - g4.x), k4.y * expf(r4.y - g4.y),
+                                                                k4.z * expf(r4.z - g4.z), k4.w * expf(r4.w - g4.w));
+    }
+#pragma unroll 1
+    for (int a = 0; a < 4; ++a) {
+      if (tc > tr) continue;
+      float s0 = 0.f, s1 = 0.f;
+      const int i = 16 * a + tr, jj = 16 * a + tc;
+#pragma unroll 2
+      for (int c = 0; c < D; c += 4) {
+        const float4 ki = ld4(sK + i * LD + c), qi = ld4(sQ + i * LD + c), kj = ld4(sK + jj * LD + c);
+        const float4 gi = ld4(sG + i * LD + c), gj = ld4(sG + jj * LD + c);
+        const float4 x = make_float4(kj.x * expf(gi.x - gj.x), kj.y * expf(gi.y - gj.y), kj.z * expf(gi.z - gj.z),
+                                     kj.w * expf(gi.w - gj.w));
+        s0 = dot4(ki, x, s0);
+        s1 = dot4(qi, x, s1);
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (b == a) { kk[b][b] = s0; qk[b][b] = s1; }
+    }
+    __syncthreads();
+    // images for the walk from the raw rows, then the rows rescaled in place: k, q <- k, q e^{G-R_I}
+    for (int idx = tid; idx < C * (D / 4); idx += 256) {
+      const int i = idx / (D / 4), c = (idx % (D / 4)) * 4;
+      float4 k4 = ld4(sK + i * LD + c), q4 = ld4(sQ + i * LD + c);
+      const float4 g4 = ld4(sG + i * LD + c), r4 = ld4(sG + (i & 48) * LD + c), l4 = ld4(sG + 63 * LD + c);
+      *reinterpret_cast<float4*>(rec + R::KD + i * LD + c) = make_float4(
+          k4.x * expf(l4.x - g4.x), k4.y * expf(l4.y - g4.y), k4.z * expf(l4.z - g4.z), k4.w * expf(l4.w - g4.w));
+      *reinterpret_cast<float4*>(rec + R::QG + i * LD + c) =
+          make_float4(q4.x * expf(g4.x), q4.y * expf(g4.y), q4.z * expf(g4.z), q4.w * expf(g4.w));
+      const float4 e = make_float4(expf(g4.x - r4.x), expf(g4.y - r4.y), expf(g4.z - r4.z), expf(g4.w - r4.w));
+      *reinterpret_cast<float4*>(sK + i * LD + c) = make_float4(k4.x * e.x, k4.y * e.y, k4.z * e.z, k4.w * e.w);
+      *reinterpret_cast<float4*>(sQ + i * LD + c) = make_float4(q4.x * e.x, q4.y * e.y, q4.z * e.z, q4.w * e.w);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int c = 0; c < D; c += 4) {
+#pragma unroll
+      for (int a = 1; a < 4; ++a) {
+        const float4 ki = ld4(sK + (16 * a + tr) * LD + c), qi = ld4(sQ + (16 * a + tr) * LD + c);
+        const float* m = sM + (a == 1 ? 0 : (a == 2 ? 16 : 48)) * LD + c;
+#pragma unroll
+        for (int b = 0; b < a; ++b) {
+          const float4 kj = ld4(m + (16 * b + tc) * LD);
+          kk[a][b] = dot4(ki, kj, kk[a][b]);
+          qk[a][b] = dot4(qi, kj, qk[a][b]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int i = 16 * a + tr, jj = 16 * b + tc;
+      if (b <= a) sA[jj * LDP + i] = jj < i ? -sB[i] * kk[a][b] : 0.f;   // transposed
+      rec[R::P + i * LDP + jj] = jj <= i ? qk[a][b] : 0.f;
+    }
+  if (kLateV) {
+    __syncthreads();
+#pragma unroll 4
+    for (int idx = tid; idx < C * (D / 4); idx += 256)
+      *reinterpret_cast<float4*>(sf + S::RHS + (idx / (D / 4)) * 2 * D + D + (idx % (D / 4)) * 4) = v_row(idx / (D / 4), (idx % (D / 4)) * 4);
+  }
+  __syncthreads();
+
+  // ---- op #3 Solve + op #4 W/U: forward substitution of (I + A) [W | U] = diag(beta) [K e^G | V], one thread per column,
+  // in blocks of 16 rows held in registers.  The coefficients are broadcast reads of A^T.  (Unrolled over all 64 rows the
+  // code was 40 KiB run once per launch: 13 us of instruction fetches.)
+  if (tid < 2 * D) {
+    const int c = tid % D;
+    float* col = sf + S::RHS + tid;                      // [C][2 D]: this thread's column
+    float* dst = tid < D ? rec + R::W + c : rec + R::U + (c / kNV) * (C * kNV) + c % kNV;
+    const int ld = tid < D ? LD : kNV;
+#pragma unroll 1
+    for (int I = 0; I < 4; ++I) {
+      float y[16];
+      if (tid < D) {
+        const float eI = KDA ? expf(sG[16 * I * LD + c]) : 1.f;            // (KDA: the rows are scaled up to R_I already)
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          y[i] = sB[16 * I + i] * sK[(16 * I + i) * LD + c] * (KDA ? eI : expf(sG[KDA ? 0 : 16 * I + i]));
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) y[i] = sB[16 * I + i] * col[(16 * I + i) * 2 * D];
+      }
+      const float* at = sA + 16 * I;                     // A^T[m][16 I ..]
+#pragma unroll 4
+      for (int m = 0; m < 16 * I; ++m) {
+        const float v = col[m * 2 * D];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 a = ld4(at + m * LDP + 4 * q);
+          y[4 * q] = fmaf(a.x, v, y[4 * q]);
+          y[4 * q + 1] = fmaf(a.y, v, y[4 * q + 1]);
+          y[4 * q + 2] = fmaf(a.z, v, y[4 * q + 2]);
+          y[4 * q + 3] = fmaf(a.w, v, y[4 * q + 3]);
+        }
+      }
+      at += 16 * I * LDP;
+#pragma unroll
+      for (int m = 0; m < 15; ++m)
+#pragma unroll
+        for (int q = (m + 1) / 4; q < 4; ++q) {
+          const float4 a = ld4(at + m * LDP + 4 * q);
+          if (4 * q > m) y[4 * q] = fmaf(a.x, y[m], y[4 * q]);
+          if (4 * q + 1 > m) y[4 * q + 1] = fmaf(a.y, y[m], y[4 * q + 1]);
+          if (4 * q + 2 > m) y[4 * q + 2] = fmaf(a.z, y[m], y[4 * q + 2]);
+          if (4 * q + 3 > m) y[4 * q + 3] = fmaf(a.w, y[m], y[4 * q + 3]);
+        }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        col[(16 * I + i) * 2 * D] = y[i];
+        dst[(16 * I + i) * ld] = y[i];
+      }
+    }
+  }
+  if (D == 128 || tid >= 2 * D) {                        // the walk's other images (d = 64: by the idle half of the CTA)
+    const int t = D == 128 ? tid : tid - 2 * D;
+    constexpr int NT = D == 128 ? 256 : 256 - 2 * D;
+    if (!KDA) {
+      const float gl = sG[C - 1];
+      for (int idx = t; idx < C * (D / 4); idx += NT) {
+        const int i = idx / (D / 4), c = (idx % (D / 4)) * 4;
+        const float4 k4 = ld4(sK + i * LD + c), q4 = ld4(sQ + i * LD + c);
+        const float ek = expf(gl - sG[i]), eq = expf(sG[i]);
+        *reinterpret_cast<float4*>(rec + R::KD + i * LD + c) = make_float4(k4.x * ek, k4.y * ek, k4.z * ek, k4.w * ek);
+        *reinterpret_cast<float4*>(rec + R::QG + i * LD + c) = make_float4(q4.x * eq, q4.y * eq, q4.z * eq, q4.w * eq);
+      }
+    }
+    for (int c = t; c < D; c += NT) rec[R::GAM + c] = expf(KDA ? sG[(C - 1) * LD + c] : sG[C - 1]);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ sequential part
+template <int D> struct WalkSmem {
+  static constexpr int LD = D + 4;
+  static constexpr int kStages = D == 64 ? 2 : 1;        // chunks whose operands fit (a load takes about as long as a half step)
+  static constexpr int WQ = 0;                           // W, QG of the chunk
+  static constexpr int KP = WQ + 2 * C * LD;             // KD, P, e^{G_L}
+  static constexpr int U = KP + C * LD + C * LDP + D;    // U slice [C][kNV]
+  static constexpr int kStage = U + C * kNV;
+  static constexpr int HT = kStages * kStage;            // state [kNV][LD]
+  static constexpr int UT = HT + kNV * LD;               // U~ [kNV][LDP]
+  static constexpr int Y = UT + kNV * LDP;               // QG h [C][kNV + 1]
+  static constexpr int BAR = (Y + C * (kNV + 1) + 3) / 4 * 4;
+  static constexpr size_t bytes = (size_t)BAR * 4 + 32;
+};
+// Threads: the first kUpd<D> update the state (four keys of NV / 8 channels, over half of the tokens each), then 256 for the
+// outputs (four rows, over half of the tokens); the first 512 compute W h and QG h (two tokens, over half of the keys).
+// Neighbouring lanes hold the two halves of a sum: enough warps to cover the shared-memory latency of a CTA that has an
+// SM to itself.
+template <int D> constexpr int kUpd = D * 4;
+template <int D> constexpr int kWalkThreads = kUpd<D> + 256;
+__device__ __forceinline__ float pair_sum(float x) { return x + __shfl_xor_sync(0xffffffffu, x, 1); }
+
+template <typename In, int D, int NV>
+__global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Params p) {
+  using S = WalkSmem<D>;
+  using R = Rec<D>;
+  constexpr int LD = D + 4, NSL = D / NV, E = NV / 8;     // E channels per thread: cg, cg + 8
+  extern __shared__ __align__(16) float sf[];
+  constexpr int ST = S::kStages;
+  float* sH = sf + S::HT;
+  float* sT = sf + S::UT;
+  float* sY = sf + S::Y;
+  uint64_t* bar1 = reinterpret_cast<uint64_t*>(sf + S::BAR);   // [stages] W, QG, U
+  uint64_t* bar3 = bar1 + 2;                                   // [stages] KD, P, e^{G_L}
+  const int tid = threadIdx.x, half = tid & 1, cg = (tid >> 1) & 7;
+  const int slice = blockIdx.x % NSL, nj = blockIdx.x / NSL, j = nj % p.HV;
+  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;
+  const int tok0 = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
+  const int len = p.seq_tok0 ? p.seq_len[n] : p.T_row;
+  const int slot0 = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
+  const int nch = (len + C - 1) / C;
+  if (tid == 0) {
+    for (int i = 0; i < ST; ++i) { mbar_init(&bar1[i], 1); mbar_init(&bar3[i], 1); }
+    mbar_fence_init();
+  }
+  // state: thread -> four keys, its channels of the slice (held by both lanes of a pair)
+  const int kg = tid >> 4;
+  const bool upd = tid < kUpd<D>;
+  const size_t hbase = (((size_t)n * p.HV + j) * D + 4 * kg) * D + slice * NV + cg;
+  const int uc = (NV == kNV ? 0 : (slice & 1) * NV) + cg;      // first channel within the record's U slice
+  float h[E][4];
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) h[e][x] = 0.f;
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (upd) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) h[e][x] = p.h0 ? p.h0[hbase + (size_t)x * D + 8 * e] : 0.f;
+      *reinterpret_cast<float4*>(sH + (cg + 8 * e) * LD + 4 * kg) = make_float4(h[e][0], h[e][1], h[e][2], h[e][3]);
+    }
+  }
+  auto load1 = [&](int c) {
+    const float* rec = p.rec + ((size_t)(slot0 + c) * p.HV + j) * R::size;
+    float* st = sf + (c % ST) * S::kStage;
+    mbar_expect_tx(&bar1[c % ST], (2 * C * LD + C * kNV) * 4);
+    bulk_load(st + S::WQ, rec + R::W, 2 * C * LD * 4, &bar1[c % ST]);
+    bulk_load(st + S::U, rec + R::U + (slice * NV / kNV) * (C * kNV), C * kNV * 4, &bar1[c % ST]);
+  };
+  auto load3 = [&](int c) {
+    const float* rec = p.rec + ((size_t)(slot0 + c) * p.HV + j) * R::size;
+    constexpr uint32_t bytes = (C * LD + C * LDP + D) * 4;
+    mbar_expect_tx(&bar3[c % ST], bytes);
+    bulk_load(sf + (c % ST) * S::kStage + S::KP, rec + R::KD, bytes, &bar3[c % ST]);
+  };
+  if (tid == 0) {
+    fence_proxy_async_all();
+    for (int c = 0; c < ST && c < nch; ++c) { load1(c); load3(c); }
+  }
+  int gave_up = 0;
+  volatile int* abort_flag = &gave_up;                   // (every wait is bounded)
+  __syncthreads();
+
+  for (int c = 0; c < nch; ++c) {
+    const float* sW = sf + (c % ST) * S::kStage + S::WQ;
+    const float* sQ = sW + C * LD;
+    const float* sK = sf + (c % ST) * S::kStage + S::KP;
+    const float* sP = sK + C * LD;
+    const float* sGam = sP + C * LDP;
+    const float* sU = sf + (c % ST) * S::kStage + S::U;
+    // ---- W h and QG h: 64 tokens x NV channels each; token rows rg, rg + 32
+    if (tid < 512) {
+      if (!mbar_test_wait(&bar1[c % ST], (c / ST) & 1)) mbar_wait(&bar1[c % ST], (c / ST) & 1, abort_flag);
+      const int rg = tid >> 4;
+      float x[2][E] = {}, y[2][E] = {};
+#pragma unroll 4
+      for (int k = 4 * half; k < D; k += 8) {
+        float4 hv[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) hv[e] = ld4(sH + (cg + 8 * e) * LD + k);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const float4 w = ld4(sW + (rg + 32 * r) * LD + k), q = ld4(sQ + (rg + 32 * r) * LD + k);
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            x[r][e] = dot4(w, hv[e], x[r][e]);
+            y[r][e] = dot4(q, hv[e], y[r][e]);
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int t = rg + 32 * r, ch = cg + 8 * e;
+          const float xs = pair_sum(x[r][e]), ys = pair_sum(y[r][e]);
+          if (half == 0) sT[ch * LDP + t] = sU[t * kNV + uc + 8 * e] - xs;
+          else sY[t * (kNV + 1) + ch] = ys;
+        }
+    }
+    __syncthreads();                                     // U~ and QG h are complete; W, QG, U and the old state are free
+    if (tid == 0 && c + ST < nch) load1(c + ST);
+    if (!mbar_test_wait(&bar3[c % ST], (c / ST) & 1)) mbar_wait(&bar3[c % ST], (c / ST) & 1, abort_flag);
+    if (upd) {
+      // ---- h <- e^{G_L} h + KD^T U~
+      float d[E][4] = {};
+#pragma unroll 4
+      for (int t = 4 * half; t < C; t += 8) {
+        float uu[E][4];
+#pragma unroll
+        for (int e = 0; e < E; ++e) *reinterpret_cast<float4*>(uu[e]) = ld4(sT + (cg + 8 * e) * LDP + t);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const float4 k4 = ld4(sK + (t + s) * LD + 4 * kg);
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            d[e][0] = fmaf(k4.x, uu[e][s], d[e][0]);
+            d[e][1] = fmaf(k4.y, uu[e][s], d[e][1]);
+            d[e][2] = fmaf(k4.z, uu[e][s], d[e][2]);
+            d[e][3] = fmaf(k4.w, uu[e][s], d[e][3]);
+          }
+        }
+      }
+      const float4 gm = ld4(sGam + 4 * kg);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        h[e][0] = fmaf(gm.x, h[e][0], pair_sum(d[e][0]));
+        h[e][1] = fmaf(gm.y, h[e][1], pair_sum(d[e][1]));
+        h[e][2] = fmaf(gm.z, h[e][2], pair_sum(d[e][2]));
+        h[e][3] = fmaf(gm.w, h[e][3], pair_sum(d[e][3]));
+        if (half == 0)
+          *reinterpret_cast<float4*>(sH + (cg + 8 * e) * LD + 4 * kg) = make_float4(h[e][0], h[e][1], h[e][2], h[e][3]);
+      }
+    } else {
+      // ---- o = scale (QG h + P U~): rows rg, rg + 16, ..; P is lower triangular
+      const int rg = (tid - kUpd<D>) >> 4;
+      float s[4][E] = {};
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int t = 16 * b; t < 16 * b + 16; t += 8) {
+          float4 u[E];
+#pragma unroll
+          for (int e = 0; e < E; ++e) u[e] = ld4(sT + (cg + 8 * e) * LDP + t + 4 * half);
+#pragma unroll
+          for (int r = b; r < 4; ++r) {
+            const float4 q = ld4(sP + (rg + 16 * r) * LDP + t + 4 * half);
+#pragma unroll
+            for (int e = 0; e < E; ++e) s[r][e] = dot4(q, u[e], s[r][e]);
+          }
+        }
+      In* go = reinterpret_cast<In*>(p.o) + ((size_t)(tok0 + c * C) * p.HV + j) * D + slice * NV + cg;
+      const int left = len - c * C;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int t = rg + 16 * r;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const float o = sY[t * (kNV + 1) + cg + 8 * e] + pair_sum(s[r][e]);
+          if (t < left && half == 0) go[(size_t)t * p.HV * D + 8 * e] = from_f32<In>(p.scale * o);
+        }
+      }
+    }
+    __syncthreads();                                     // the new state is complete; KD, P, U~ and QG h are free
+    if (tid == 0 && c + ST < nch) load3(c + ST);
+  }
+  if (gave_up) report_status(p.status, HA_LA_ERR_TIMEOUT);
+  if (p.hT && upd && half == 0) {
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) p.hT[hbase + (size_t)x * D + 8 * e] = h[e][x];
+  }
+}
+
+// Launch attribute of both kernels: each is set up under the tail of the kernel before it and waits on the device.
+template <auto kern>
+cudaError_t launch(unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, const Fp32Params& fp) {
+  static std::atomic<uint64_t> configured{0};            // (of this kernel: a bit per device)
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  if (dev >= 64 || !(configured.load() >> dev & 1)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) configured.fetch_or(1ull << dev);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = g_timer ? 0 : 1;                        // (per-kernel timing wants one kernel at a time)
+  return cudaLaunchKernelEx(&cfg, kern, fp);
+}
+
+template <typename In, int D, bool KDA>
+cudaError_t run(const Problem& p, const Fp32Params& fp, cudaStream_t stream) {
+  static_assert(PrepSmem<D, KDA>::size * 4 <= 227 * 1024 && WalkSmem<D>::bytes <= 227 * 1024, "shared memory budget");
+  if (p.max_chunks * p.HV > 0) {
+    timer_mark(stream, "simt_prep");
+    const cudaError_t e = launch<fp32_prep_kernel<In, D, KDA>>((unsigned)(p.max_chunks * p.HV), 256u, PrepSmem<D, KDA>::size * 4,
+                                                               stream, fp);
+    if (e != cudaSuccess) return e;
+  }
+  timer_mark(stream, "simt_prefill");
+  // Slices of 8 channels while that leaves every CTA an SM (a chunk then takes about 0.6 of the time), else of 16 (fewer
+  // reads of the shared operands per channel).
+  const long long heads = (long long)p.N * p.HV;
+  if (heads * (D / 8) <= 148)
+    return launch<fp32_walk_kernel<In, D, 8>>((unsigned)(heads * (D / 8)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
+  return launch<fp32_walk_kernel<In, D, 16>>((unsigned)(heads * (D / 16)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
+}
+
+template <typename In, bool KDA>
+cudaError_t run_dims(const Problem& p, const Fp32Params& fp, cudaStream_t stream) {
+  return p.dk == 128 ? run<In, 128, KDA>(p, fp, stream) : run<In, 64, KDA>(p, fp, stream);
+}
+
+Fp32Params make_params(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* ws) {
+  Fp32Params fp;
+  fp.q = a.q; fp.k = a.k; fp.v = a.v; fp.g = a.g; fp.beta = a.beta; fp.h0 = a.h0;
+  fp.o = a.o; fp.hT = a.hT; fp.rec = reinterpret_cast<float*>(ws);
+  fp.chunk_tok0 = plan.chunk_tok0; fp.chunk_len = plan.chunk_len;
+  fp.seq_tok0 = plan.seq_tok0; fp.seq_len = plan.seq_len; fp.seq_chunk0 = plan.seq_chunk0;
+  fp.seq_order = plan.seq_tok0 ? plan.seq_order : nullptr;
+  fp.T_row = p.T_row; fp.cps = p.max_seq_chunks > 0 ? p.max_seq_chunks : 1;
+  fp.HK = p.HK; fp.HV = p.HV; fp.scale = p.scale; fp.status = a.status_word;
+  return fp;
+}
+
+}  // namespace
+
+// The instantiations are spread over translation units (HA_LA_FP32_UNIT = 0..3, one per dtype x variant) so that they
+// compile in parallel; unit 4 holds the dispatcher.
+#ifndef HA_LA_FP32_UNIT
+#error "compile with -DHA_LA_FP32_UNIT=0..4"
+#endif
+
+#define HA_LA_FP32_DEFINE(NAME, IN, KDA)                                                                         \
+  cudaError_t NAME(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* ws, cudaStream_t stream) { \
+    return run_dims<IN, KDA>(p, make_params(p, a, plan, ws), stream);                                             \
+  }
+
+#if HA_LA_FP32_UNIT == 0
+HA_LA_FP32_DEFINE(fp32_bf16_gdn, __nv_bfloat16, false)
+#elif HA_LA_FP32_UNIT == 1
+HA_LA_FP32_DEFINE(fp32_bf16_kda, __nv_bfloat16, true)
+#elif HA_LA_FP32_UNIT == 2
+HA_LA_FP32_DEFINE(fp32_f32_gdn, float, false)
+#elif HA_LA_FP32_UNIT == 3
+HA_LA_FP32_DEFINE(fp32_f32_kda, float, true)
+#else
+cudaError_t fp32_bf16_gdn(const Problem&, const ha_la_prefill_args&, PlanView, void*, cudaStream_t);
+cudaError_t fp32_bf16_kda(const Problem&, const ha_la_prefill_args&, PlanView, void*, cudaStream_t);
+cudaError_t fp32_f32_gdn(const Problem&, const ha_la_prefill_args&, PlanView, void*, cudaStream_t);
+cudaError_t fp32_f32_kda(const Problem&, const ha_la_prefill_args&, PlanView, void*, cudaStream_t);
+
+size_t fp32_workspace_bytes(const Problem& p) {
+  const size_t rec = p.dk == 128 ? Rec<128>::size : Rec<64>::size;
+  return align_up((size_t)p.max_chunks * p.HV * rec * sizeof(float), 1024);
+}
+
+cudaError_t launch_fp32(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* ws, cudaStream_t stream) {
+  if (p.N * p.HV == 0) return cudaSuccess;
+  const bool kda = p.variant == HA_LA_KDA;
+  if (p.dtype == HA_LA_BF16) return kda ? fp32_bf16_kda(p, a, plan, ws, stream) : fp32_bf16_gdn(p, a, plan, ws, stream);
+  return kda ? fp32_f32_kda(p, a, plan, ws, stream) : fp32_f32_gdn(p, a, plan, ws, stream);
+}
+#endif
+
+}  // namespace ha_la

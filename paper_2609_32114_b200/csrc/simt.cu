@@ -10,8 +10,8 @@
 // 5 (the paper's "chunk-first" order, Section "Lifetime-Aware Operator Reordering"), so the state
 // is updated in place.
 //
-// This path serves fp32 inputs (where the 1e-4 tolerance rules out 16-bit tensor-core operands)
-// and head dimensions / variants the tensor-core path does not cover.  All arithmetic is fp32.
+// This kernel serves ha_la_prefill_noalloc, which has no workspace to hand anything from one kernel to another
+// (ha_la_prefill runs fp32.cu where the tensor-core path does not apply).  All arithmetic is fp32.
 #include "common.cuh"
 
 namespace ha_la {

@@ -1,0 +1,28 @@
+"""The two-kernel fp32 path against the fp64 oracle, where its indexing can go wrong: lengths around a chunk, empty and
+one-token sequences, packed and equal-length rows, both slice widths of the sequential kernel (few and many heads)."""
+import pytest
+
+from paper_2609_32114_b200 import synth
+from tests import helpers
+
+pytestmark = pytest.mark.gpu
+W = synth.WORKLOADS
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("dtype,d", [("fp32", 64), ("fp32", 128), ("bf16", 64)])
+@pytest.mark.parametrize("lens,packed,hk,hv", [([1], False, 1, 1), ([63, 63], False, 1, 2), ([129], False, 2, 2),
+                                               ([64, 0, 65, 1, 130], True, 2, 4), ([70] * 7, True, 4, 8)])
+def test_fp32_path(variant, dtype, d, lens, packed, hk, hv):
+    base = W["gdn_varlen"] if variant == "gdn" else W["kda_8k"]
+    w = synth.shrink(base, seq_lens=lens, hk=hk, hv=hv, dtype=dtype, dk=d, dv=d, gate_shift=-1.0, h0_std=0.05, varlen=packed)
+    helpers.check_parity(synth.make_inputs(w, seed=211 + len(lens)), scale=0.5)
+
+
+def test_fp32_kda_strong_decay_inside_a_block():
+    """Log-gates of -90 in a few channels: the decay inside a 16-token block leaves the range of a factored product."""
+    w = synth.shrink(W["kda_8k"], seq_lens=[150], hk=1, hv=2, dtype="fp32")
+    inp = synth.make_inputs(w, seed=223)
+    for tok in (5, 37, 70, 71):
+        inp["g"][tok, :, ::7] = -90.0
+    helpers.check_parity(inp)
