@@ -97,6 +97,8 @@ class HaLaError(RuntimeError):
 
 
 _lib = None
+_call = None          # the native half of ha_la_prefill / ha_la_decode (csrc/torch_call.cpp), once loaded
+_call_lib = None      # ... and the library it is bound to
 
 
 def load_library(path: Optional[str] = None):
@@ -141,6 +143,29 @@ def load_library(path: Optional[str] = None):
     if path is None:
         _lib = lib
     return lib
+
+
+def _torch_call():
+    """Load ha_la_torch_call.so and bind it to the library's entry points.  Raises if it is missing."""
+    global _call, _call_lib
+    lib = load_library()
+    if _call is None:
+        import importlib.util
+
+        import torch  # noqa: F401  (its libraries first: the extension links against them)
+
+        path = os.path.join(_PKG, "ha_la_torch_call.so")
+        if not os.path.exists(path):
+            raise FileNotFoundError(f"{path} not found: build it with `python -m paper_2609_32114_b200.build`")
+        spec = importlib.util.spec_from_file_location("ha_la_torch_call", path)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _call = mod
+    if _call_lib is not lib:
+        _call.bind(*(ctypes.cast(f, ctypes.c_void_p).value
+                     for f in (lib.ha_la_prefill, lib.ha_la_prefill_workspace_bytes, lib.ha_la_decode)))
+        _call_lib = lib
+    return _call
 
 
 def status_string(status: int) -> str:
@@ -271,6 +296,16 @@ def prepare_args(q, k, v, g, beta, *, variant="gdn", h0=None, cu_seqlens=None, m
     return args, keep
 
 
+_KDA = {"gdn": False, "kda": True}
+
+
+def _prefill_call(q, k, v, g, beta, stream, *, variant="gdn", h0=None, cu_seqlens=None, max_seqlen=0, scale=1.0, o=None,
+                  hT=None, want_hT=True, workspace=None, status_word=None):
+    """The arguments of the native call (prepare_args' keywords and defaults, in order)."""
+    return (q, k, v, g, beta, h0, cu_seqlens, max_seqlen, stream, _KDA.get(variant), scale, o, hT, want_hT, workspace,
+            status_word)
+
+
 def ha_la_prefill(q, k, v, g, beta, *, stream=None, **kw):
     """Prefill on torch CUDA tensors: prepare_args + the C call on torch's current stream.
 
@@ -279,6 +314,12 @@ def ha_la_prefill(q, k, v, g, beta, *, stream=None, **kw):
     h0   : fp32 [N, HV, dk, dv] or None      cu_seqlens : int32 [N+1] device tensor or None (packed, B = 1)
     Returns (o, hT, status_word, workspace); nothing is synchronised.
     """
+    r = (_call if _call_lib is not None else _torch_call()).prefill(*_prefill_call(q, k, v, g, beta, stream, **kw))
+    if r.__class__ is tuple:
+        return r
+    if r is not None:
+        raise HaLaError(r, "ha_la_prefill")
+    # not an entirely ordinary call: marshalled here
     import torch
 
     squeeze = q.dim() == 3
@@ -316,10 +357,19 @@ def ha_la_decode_raw(args: ha_la_decode_args, stream: int = 0) -> int:
     return load_library().ha_la_decode(ctypes.byref(args), ctypes.c_void_p(stream))
 
 
-def ha_la_decode(q, k, v, g, beta, state, *, stream=None, **kw):
+def ha_la_decode(q, k, v, g, beta, state, *, stream=None, variant="gdn", scale=1.0, o=None, state_out=None):
     """One decoding step on torch CUDA tensors (see prepare_decode_args).  Returns (o, new_state); nothing is
     synchronised."""
+    r = (_call if _call_lib is not None else _torch_call()).decode(q, k, v, g, beta, state, stream, variant != "gdn", scale,
+                                                                   o, state_out)
+    if r.__class__ is tuple:
+        return r
+    if r is not None:
+        raise HaLaError(r, "ha_la_decode")
+    # not an entirely ordinary call: marshalled here
     import torch
+
+    kw = dict(variant=variant, scale=scale, o=o, state_out=state_out)
 
     args, keep = prepare_decode_args(q, k, v, g, beta, state, **kw)
     if stream is None:

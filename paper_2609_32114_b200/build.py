@@ -22,6 +22,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "build")
 LIB = os.path.join(PKG, "libha_la.so")
+TORCH_CALL = os.path.join(PKG, "ha_la_torch_call.so")   # binding.py's native half (csrc/torch_call.cpp)
 INCLUDE = os.path.join(ROOT, "include")
 
 # (object name, source, extra flags)
@@ -59,6 +60,32 @@ def _compile(unit, verbose: bool, obj_dir: str = OBJ, more=()):
     return name, r.returncode, r.stdout + r.stderr
 
 
+def build_torch_call(force: bool = False) -> str:
+    """The CPython extension that binding.py calls with torch tensors (host code only, compiled against torch)."""
+    src = os.path.join(CSRC, "torch_call.cpp")
+    newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(INCLUDE, "ha_la.h")))
+    if not force and os.path.exists(TORCH_CALL) and os.path.getmtime(TORCH_CALL) >= newest:
+        return TORCH_CALL
+    import sysconfig
+
+    import torch
+
+    base = os.path.join(os.path.dirname(torch.__file__))
+    inc = os.path.join(base, "include")
+    libs = os.path.join(base, "lib")
+    tmp = TORCH_CALL + f".tmp{os.getpid()}"
+    r = subprocess.run(
+        ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+         "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", sysconfig.get_paths()["include"],
+         "-I", os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), "-I", INCLUDE, src, "-o", tmp,
+         "-L", libs, "-ltorch", "-ltorch_cpu", "-ltorch_python", "-lc10", "-lc10_cuda"],
+        capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed on torch_call.cpp\n" + r.stderr[-4000:])
+    os.replace(tmp, TORCH_CALL)
+    return TORCH_CALL
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=(), lib_path: str = LIB, obj_dir: str = OBJ) -> str:
     """Compile what is stale and link.  `extra_flags`, `lib_path`, `obj_dir` serve developer builds."""
     os.makedirs(obj_dir, exist_ok=True)
@@ -81,6 +108,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), lib_path: 
         tmp = lib_path + f".tmp{os.getpid()}"
         subprocess.check_call([_nvcc(), *ARCH, "-shared", "-o", tmp, *objs])
         os.replace(tmp, lib_path)
+    build_torch_call(force)
     return lib_path
 
 
