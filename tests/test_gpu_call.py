@@ -52,3 +52,33 @@ def test_decode_and_errors():
         ha.ha_la_prefill(t[0].transpose(1, 2), *t[1:])
     with pytest.raises(ValueError):
         ha.ha_la_prefill(*(x.cpu() for x in _inputs()))
+
+
+@pytest.mark.parametrize("variant,dtype,d,n,hk,hv", [("gdn", "bf16", 128, 1, 1, 1), ("kda", "fp32", 64, 3, 1, 3),
+                                                     ("kda", "bf16", 128, 149, 2, 2)])
+def test_decode_steps_queued_in_place(variant, dtype, d, n, hk, hv):
+    """Eight steps on one state, in place and queued directly behind each other (each step is launched under the tail of
+    the one before it), against the oracle's run over the same eight tokens."""
+    import numpy as np
+    import torch
+    import paper_2609_32114_b200 as ha
+    from paper_2609_32114_b200 import synth
+    from tests import helpers
+
+    steps = 8
+    base = synth.WORKLOADS["gdn_varlen" if variant == "gdn" else "kda_8k"]
+    w = synth.shrink(base, seq_lens=[steps] * n, hk=hk, hv=hv, dtype=dtype, dk=d, dv=d, h0_std=0.5, gate_shift=-2.0, varlen=True)
+    inp = synth.make_inputs(w, seed=231)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    per_step = lambda a, t: [torch.from_numpy(np.ascontiguousarray(a.reshape(n, steps, *a.shape[1:])[:, i])).cuda().to(t)
+                             for i in range(steps)]
+    q, k, v = (per_step(inp[x], dt) for x in "qkv")
+    g, beta = (per_step(inp[x], torch.float32) for x in ("g", "beta"))
+    state = torch.from_numpy(inp["h0"]).cuda()
+    torch.cuda.synchronize()
+    outs = [ha.ha_la_decode(q[i], k[i], v[i], g[i], beta[i], state, variant=variant)[0] for i in range(steps)]
+    torch.cuda.synchronize()
+    o_ref, h_ref = helpers.run_oracle(inp)
+    o = torch.stack(outs, 1).float().cpu().numpy().reshape(o_ref.shape)
+    assert helpers.rel_max_err(o, o_ref) <= helpers.TOL[dtype]
+    assert helpers.rel_max_err(state.cpu().numpy().astype(np.float64), h_ref) <= 1e-5
