@@ -13,6 +13,14 @@ namespace {
 
 bool dim_ok(int d) { return d == 64 || d == 128; }
 
+bool use_tc(const Problem& p) {
+  static const bool forced_off = [] {
+    const char* e = getenv("HA_LA_FORCE_SIMT");
+    return e && e[0] == '1';
+  }();
+  return !forced_off && tc_supported(p);
+}
+
 // Shape-only validation (no pointer checks).  Fills `p` on success.
 int make_problem(const ha_la_prefill_args* a, Problem* p) {
   if (!a) return HA_LA_ERR_INVALID_ARG;
@@ -44,24 +52,17 @@ int make_problem(const ha_la_prefill_args* a, Problem* p) {
   p->dv = a->d_v;
   p->scale = a->scale;
   p->varlen = varlen ? 1 : 0;
+  p->step = use_tc(*p) && p->variant == HA_LA_GDN ? 128 : kChunk;
   if (varlen) {
     p->max_len = (a->max_seqlen > 0 && a->max_seqlen < a->seqlen) ? a->max_seqlen : a->seqlen;
-    p->max_chunks = (int)(((long long)p->T_total + 63LL * p->N) / kChunk);
+    p->max_chunks = (int)(((long long)p->T_total + (p->step - 1LL) * p->N) / p->step);
   } else {
     p->max_len = a->seqlen;
-    p->max_chunks = a->batch * ((a->seqlen + kChunk - 1) / kChunk);
+    p->max_chunks = a->batch * ((a->seqlen + p->step - 1) / p->step);
   }
-  p->max_seq_chunks = (p->max_len + kChunk - 1) / kChunk;
+  p->max_seq_chunks = (p->max_len + p->step - 1) / p->step;
   if (!tc_supported(*p) && !simt_supported(*p)) return HA_LA_ERR_UNSUPPORTED;
   return HA_LA_OK;
-}
-
-bool use_tc(const Problem& p) {
-  static const bool forced_off = [] {
-    const char* e = getenv("HA_LA_FORCE_SIMT");
-    return e && e[0] == '1';
-  }();
-  return !forced_off && tc_supported(p);
 }
 
 }  // namespace

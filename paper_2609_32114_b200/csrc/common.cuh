@@ -32,6 +32,7 @@ struct Problem {
   int T_row;        // tokens per batch row when cu_seqlens == NULL
   int HK, HV, dk, dv;
   int max_len;      // bound on one sequence's length
+  int step;         // tokens per chunk slot (64; 128 on the tensor-core path)
   int max_chunks;   // bound on chunk slots (MC)
   int max_seq_chunks;
   float scale;

@@ -10,7 +10,7 @@ namespace ha_la {
 namespace {
 
 struct PlanParams {
-  int N, T_total, T_row, max_len, max_chunks;
+  int N, T_total, T_row, max_len, max_chunks, step;
 };
 
 __global__ void __launch_bounds__(256) plan_kernel(PlanParams p, const int32_t* __restrict__ cu, PlanView v,
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p, const int32_t* 
   // 2. exclusive prefix sum of chunk counts over sequences, 256 at a time
   for (int base = 0; base < p.N; base += blockDim.x) {
     const int n = base + tid;
-    const int cnt = n < p.N ? (v.seq_len[n] + kChunk - 1) / kChunk : 0;
+    const int cnt = n < p.N ? (v.seq_len[n] + p.step - 1) / p.step : 0;
     int x = cnt;
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p, const int32_t* 
     const int c = s - v.seq_chunk0[lo];
     const int L = v.seq_len[lo];
     v.chunk_seq[s] = lo;
-    v.chunk_tok0[s] = v.seq_tok0[lo] + c * kChunk;
-    v.chunk_len[s] = min(kChunk, L - c * kChunk);
+    v.chunk_tok0[s] = v.seq_tok0[lo] + c * p.step;
+    v.chunk_len[s] = min(p.step, L - c * p.step);
   }
 }
 
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) plan_kernel(PlanParams p, const int32_t* 
 
 cudaError_t launch_plan(const Problem& p, const int32_t* cu_seqlens, PlanView plan, int32_t* status,
                         cudaStream_t stream) {
-  PlanParams pp{p.N, p.T_total, p.T_row, p.max_len, p.max_chunks};
+  PlanParams pp{p.N, p.T_total, p.T_row, p.max_len, p.max_chunks, p.step};
   timer_mark(stream, "plan");
   plan_kernel<<<1, 256, 0, stream>>>(pp, cu_seqlens, plan, status);
   return cudaGetLastError();

@@ -29,6 +29,16 @@ cudaError_t launch_tc_chain(const Problem& p, const ha_la_prefill_args& a, PlanV
 cudaError_t launch_tc_seg_fix(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const SegBuffers& sg,
                               cudaStream_t stream);
 
+cudaError_t launch_tc_tp(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
+                         const CUtensorMap& mq, const CUtensorMap& mk, int64_t epoch, int ctas, cudaStream_t stream);
+cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
+                           const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, int64_t epoch,
+                           bool dependent, uint32_t spin_limit, const SpanBuffers& sb, bool states_only,
+                           cudaStream_t stream);
+cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& sb, int32_t* status, cudaStream_t stream);
+cudaError_t configure_span_fix();
+cudaError_t configure_tc_tp();
+cudaError_t configure_tc_walk(const Problem& p);
 cudaError_t configure_tc_prep(const Problem& p);
 cudaError_t configure_tc_chain(const Problem& p, int nv);
 
@@ -59,6 +69,20 @@ bool make_map(CUtensorMap* m, const void* base, int T, int H) {
   const cuuint32_t box[3] = {64, 1, 64};
   const cuuint32_t es[3] = {1, 1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The same tensor in tiles of 128 features x 1 head x 128 tokens, as two 64-feature halves of 128-byte rows one after the
+// other ([kb][128 tok][64 feat], 128-byte swizzle): the feature halves are the outermost dimension of the map.
+bool make_map_tile(CUtensorMap* m, const void* base, int T, int H) {
+  EncodeTiledFn enc = encode_fn();
+  if (!enc) return false;
+  const cuuint64_t dims[4] = {64, (cuuint64_t)H, (cuuint64_t)(T > 0 ? T : 1), 2};
+  const cuuint64_t strides[3] = {128 * 2, (cuuint64_t)H * 128 * 2, 64 * 2};
+  const cuuint32_t box[4] = {64, 1, (cuuint32_t)kStep, 2};
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -118,11 +142,47 @@ int64_t next_epoch() {
 // Only bounds are known on the host: max_len for the longest sequence, max_chunks for the total.
 struct TcPlan { int nv; bool concurrent; int nseg; };
 
+// HA_LA_TC_SEGMENTS, or 0
+int forced_segments() {
+  const char* e = getenv("HA_LA_TC_SEGMENTS");
+  const int v = e ? atoi(e) : 0;
+  return v == 1 || v == 2 || v == 4 || v == 8 ? v : 0;
+}
+
+// Spans per sequence of the step path (tc_walk.cu): with few (sequence, head) pairs a sequence is cut into S runs that
+// are walked at the same time, in two launches, 2 S - 3 state-only runs and then S runs with outputs, with S - 2
+// products of 128^3 between them.  Costs measured on B200: 2.0 us per state-only step, 2.45 per step with outputs, 1.25
+// per product and about 8 for the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack
+// (the longest first) to within some 15 %.
+int plan_spans(const Problem& p) {
+  const long long chains = (long long)p.N * p.HV;
+  const int sms = sm_count(), longest = (p.max_len + kStep - 1) / kStep;
+  const double avg_len = p.N > 0 ? (double)p.T_total / p.N : 0.0;
+  const bool even = p.max_len < 1.5 * avg_len;
+  const double total = (double)p.max_chunks * p.HV;
+  auto launch_us = [&](int runs, int spans, double step_us) {
+    const int cps = (longest + spans - 1) / spans;
+    const long long ctas = chains * runs;
+    if (ctas <= sms) return cps * step_us;
+    if (even) return cps * step_us * (double)((ctas + sms - 1) / sms);
+    const double spread = 1.15 * total * runs / spans / sms;
+    return (spread > cps ? spread : cps) * step_us;
+  };
+  int best_s = 1;
+  double best = launch_us(1, 1, 2.45);
+  for (int S = 2; S <= 32 && S <= longest; ++S) {
+    const double t = launch_us(2 * S - 3, S, 2.0) + launch_us(S, S, 2.45) + 1.25 * (S - 2) + 8.0;
+    if (t < best) { best = t; best_s = S; }
+  }
+  return best_s;
+}
+
 TcPlan plan_tc(const Problem& p) {
   const int sms = sm_count();
   const long long chains = (long long)p.N * p.HV;
   const double longest = (double)((p.max_len + kChunk - 1) / kChunk);
-  const double items = (double)p.max_chunks * p.HV;
+  const long long chunks = p.varlen ? ((long long)p.T_total + (kChunk - 1LL) * p.N) / kChunk : (long long)p.N * ((p.max_len + kChunk - 1) / kChunk);
+  const double items = (double)chunks * p.HV;
   const int widths[3] = {32, 64, 128};
   const double per_chunk_us[3] = {0.90, 1.23, 1.50};
   const bool kda = p.variant == HA_LA_KDA;
@@ -137,7 +197,7 @@ TcPlan plan_tc(const Problem& p) {
   // cannot be packed any better than in rounds of one CTA per SM
   const double avg_len = p.N > 0 ? (double)p.T_total / p.N : 0.0;
   const bool even = avg_len <= 0.0 || p.max_len < 1.5 * avg_len;
-  bool may_overlap = p.max_chunks > 1;
+  bool may_overlap = chunks > 1;
   bool force_overlap = false;                            // "2": side by side whenever that is legal (tests)
   if (const char* e = getenv("HA_LA_TC_OVERLAP")) {
     may_overlap = may_overlap && e[0] != '0';
@@ -177,11 +237,7 @@ TcPlan plan_tc(const Problem& p) {
   // SM each, i.e. for few heads and long sequences.  Costs measured on B200: the chain's per-chunk times above,
   // 7 us + 3.1 us per further segment for the start states (S - 1 products of 128^3 in turn) and 9 us + 15 ns per
   // corrected chunk-head for the outputs.
-  int forced_seg = 0;
-  if (const char* e = getenv("HA_LA_TC_SEGMENTS")) {
-    const int v = atoi(e);
-    if (v == 1 || v == 2 || v == 4 || v == 8) forced_seg = v;
-  }
+  const int forced_seg = forced_segments();
   if ((!p.varlen || forced_seg > 1) && forced_seg != 1 && longest >= 2) {
     for (int w = 0; w < 2; ++w) {                          // 32- and 64-channel slices
       if (forced_nv && widths[w] != forced_nv) continue;
@@ -207,15 +263,35 @@ bool tc_supported(const Problem& p) {
   return p.dtype == HA_LA_BF16 && p.dk == 128 && p.dv == 128;
 }
 
-// Images plus, when the planner cuts the sequences into segments, the segment scratch for that many.  (The call
+// Images or step records, the scratch of the planned spans (GDN), and, when the planner cuts the sequences into segments,
+// the segment scratch for that many.  (The call
 // checks the caller's size against this same function, so an environment switch that is changed between sizing and
 // calling ends in HA_LA_ERR_WORKSPACE, not in an overrun.)
-size_t tc_workspace_bytes(const Problem& p) {
-  const size_t img = tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA);
-  return img + tc_seg_bytes((size_t)p.N * p.HV, plan_tc(p).nseg, (size_t)p.T_total, p.HV);
+static size_t tc_base_bytes(const Problem& p) {
+  const bool kda = p.variant == HA_LA_KDA;
+  return tc_ws_bytes_for((size_t)p.max_chunks * p.HV, kda) + (kda ? 0 : tc_span_bytes((size_t)p.N * p.HV, plan_spans(p)));
 }
 
-int tc_num_launches(const Problem& p) { return plan_tc(p).nseg > 1 ? 4 : 2; }
+size_t tc_workspace_bytes(const Problem& p) {
+  return tc_base_bytes(p) + tc_seg_bytes((size_t)p.N * p.HV, plan_tc(p).nseg, (size_t)p.T_total, p.HV);
+}
+
+// HA_LA_TC_SEGMENTS forces the spans too (1: none); their scratch is then the segment scratch, which is larger.
+static SpanBuffers gdn_spans(const Problem& p, const TcPlan& tp, void* tc_ws) {
+  uint8_t* b = reinterpret_cast<uint8_t*>(tc_ws);
+  const size_t nj = (size_t)p.N * p.HV;
+  const int forced = forced_segments();
+  if (forced == 1) return tc_span_view(nullptr, nj, 1);
+  if (forced > 1 && tp.nseg > 1) return tc_span_view(b + tc_base_bytes(p), nj, tp.nseg);
+  return tc_span_view(b + tc_ws_bytes_for((size_t)p.max_chunks * p.HV, false), nj, plan_spans(p));
+}
+
+int tc_num_launches(const Problem& p) {
+  const int nseg = plan_tc(p).nseg;
+  if (p.variant == HA_LA_KDA) return nseg > 1 ? 4 : 2;
+  const int forced = forced_segments();
+  return (forced == 1 ? 1 : forced > 1 && nseg > 1 ? nseg : plan_spans(p)) > 1 ? 4 : 2;
+}
 
 int tc_num_segments(const Problem& p) { return plan_tc(p).nseg; }
 
@@ -225,8 +301,41 @@ void tc_launch_plan(const Problem& p, int* slice_width, int* concurrent) {
   *concurrent = tp.concurrent ? 1 : 0;
 }
 
+static cudaError_t launch_tc_gdn(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
+                                 const SpanBuffers& sb, cudaStream_t stream) {
+  CUtensorMap mq, mk, mv;
+  if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk, a.k, p.T_total, p.HK) ||
+      !make_map_tile(&mv, a.v, p.T_total, p.HV))
+    return cudaErrorInvalidValue;
+  static std::atomic<uint32_t> configured[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  const uint32_t bit = 1u << (p.variant == HA_LA_KDA ? 1 : 0);
+  if (dev < 0 || dev >= kMaxDevices || !(configured[dev].load() & bit)) {
+    cudaError_t ce = configure_tc_tp();
+    if (ce != cudaSuccess) return ce;
+    ce = configure_tc_walk(p);
+    if (ce != cudaSuccess) return ce;
+    ce = configure_span_fix();
+    if (ce != cudaSuccess) return ce;
+    if (dev >= 0 && dev < kMaxDevices) configured[dev].fetch_or(bit);
+  }
+  const bool dependent = g_timer == nullptr;
+  cudaError_t e = launch_tc_tp(p, a, plan, ws, mq, mk, 0, sm_count(), stream);
+  if (e != cudaSuccess) return e;
+  if (sb.nspan > 1) {
+    e = launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, true, stream);
+    if (e != cudaSuccess) return e;
+    e = launch_span_fix(p, plan, sb, a.status_word, stream);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, false, stream);
+}
+
 cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* tc_ws, cudaStream_t stream) {
   const TcPlan tp = plan_tc(p);
+  if (p.variant != HA_LA_KDA)
+    return launch_tc_gdn(p, a, plan, tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, false), gdn_spans(p, tp, tc_ws), stream);
   const int nv = tp.nv;
   CUtensorMap mq, mk, mv, mo;
   if (!make_map(&mq, a.q, p.T_total, p.HK) || !make_map(&mk, a.k, p.T_total, p.HK) ||
@@ -284,6 +393,17 @@ cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView pl
 cudaError_t launch_tc_chain_unpublished(const Problem& p, const ha_la_prefill_args& a, void* tc_ws, uint32_t spin_limit,
                                         cudaStream_t stream) {
   const int nv = 32;
+  if (p.variant != HA_LA_KDA) {
+    CUtensorMap mq, mk2, mv;
+    if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk2, a.k, p.T_total, p.HK) ||
+        !make_map_tile(&mv, a.v, p.T_total, p.HV))
+      return cudaErrorInvalidValue;
+    const TcWorkspace w = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, false);
+    cudaError_t ce2 = configure_tc_walk(p);
+    if (ce2 != cudaSuccess) return ce2;
+    return launch_tc_walk(p, a, PlanView{}, w, mk2, mq, mv, next_epoch(), false, spin_limit,
+                          SpanBuffers{1, nullptr, nullptr}, false, stream);
+  }
   CUtensorMap mk, mo;
   if (!make_map(&mk, a.k, p.T_total, p.HK) || !make_map_o(&mo, a.o, p.T_total, p.HV, nv)) return cudaErrorInvalidValue;
   const TcWorkspace ws = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA);

@@ -23,6 +23,24 @@ namespace ha_la {
 constexpr size_t kImgBytes = 128 * 64 * 2;     // 16 KiB
 constexpr int kScFloats = 192;
 
+// The path works in steps of 128 tokens.  Record of one (step slot, V-head): T diag(beta) and P as bf16 MMA operands, then
+// the gate factors (GDN: e^{G_t}[128], e^{G_L-G_t}[128]; KDA: e^{G_L}[128 keys]).
+// Triangular operand (128 x 128, lower): eight slabs of 16 columns one after the other, slab J with the rows 16 J .. 127
+// only, rows of 32 bytes with the 32-byte swizzle; a product takes slab J as an operand of 128 - 16 J rows.  The 16
+// columns of a row are stored in the order 0 1 8 9 2 3 10 11 .. (step_pos), which is the order a lane of a warp-level
+// fragment holds them in: eight bytes per lane and row.  The other operand of the product has its K index in that order.
+constexpr int kStep = 128;
+constexpr uint32_t kTriB = 18432, kStepScB = 1024;
+constexpr uint32_t kStepT = 0, kStepP = kTriB, kStepSc = 2 * kTriB, kStepRecB = 2 * kTriB + kStepScB;
+constexpr uint32_t kTileBytes = 32768;        // a 128-token, 128-feature bf16 tile, [kb][128 tok][64 feat], 128-byte swizzle
+constexpr __host__ __device__ int tri_block(int I, int J) { return I * (I + 1) / 2 + J; }
+constexpr __host__ __device__ uint32_t tri_slab(int J) { return 32u * (128 * J - 8 * J * (J - 1)); }   // byte offset of slab J
+constexpr __host__ __device__ uint32_t tri_row(int row, int J) { return tri_slab(J) + (row - 16 * J) * 32; }
+static_assert(tri_slab(8) == kTriB, "eight slabs");
+constexpr __host__ __device__ int step_pos(int t) {                // stored position of row / column t
+  return (t & ~15) | ((t & 6) << 1) | ((t & 8) >> 2) | (t & 1);
+}
+
 // A chunk's ready flag holds the call's epoch (low byte zero) when the prep kernel has published it; the chain
 // kernel's slices then count themselves off in the low byte as they finish with the chunk.
 constexpr long long kFlagCountMask = 0xff;
@@ -34,16 +52,24 @@ struct TcWorkspace {
   uint8_t* kd;      // KDA only
   int64_t* flags;
   float* sc;
+  uint8_t* rec;     // new layout
+  uint8_t* img;
 };
 
 inline __host__ size_t tc_ws_bytes_for(size_t ncj, bool kda) {
+  if (!kda) return align_up(ncj * kStepRecB, 1024) + align_up(ncj * sizeof(int64_t), 1024);
   return ncj * (2 * kImgBytes + kImgBytes + kImgBytes + (kda ? kImgBytes : 0)) +
          align_up(ncj * kScFloats * sizeof(float), 1024) + align_up(ncj * sizeof(int64_t), 1024);
 }
 
 inline __host__ TcWorkspace tc_ws_view(void* base, size_t ncj, bool kda) {
-  TcWorkspace w;
+  TcWorkspace w{};
   uint8_t* b = reinterpret_cast<uint8_t*>(base);
+  if (!kda) {
+    w.rec = b;
+    w.flags = reinterpret_cast<int64_t*>(b + align_up(ncj * kStepRecB, 1024));
+    return w;
+  }
   w.wq = b;                      b += ncj * 2 * kImgBytes;
   w.u = b;                       b += ncj * kImgBytes;
   w.ol = b;                      b += ncj * kImgBytes;
@@ -79,6 +105,20 @@ inline __host__ SegBuffers tc_seg_view(void* base, size_t nj, int nseg, size_t r
   g.r = reinterpret_cast<__nv_bfloat16*>(b);
   (void)rows; (void)HV;
   return g;
+}
+
+// Scratch of a call whose sequences are cut into spans: per (sequence, V-head) and span the offset b_s, which the span's
+// true start state h_s replaces, and the transition Phi_s (fp32 128 x 128 each, [key][value channel]).
+struct SpanBuffers {
+  int nspan;            // 1: off
+  float* b;
+  float* phi;
+};
+inline __host__ size_t tc_span_bytes(size_t nj, int nspan) { return nspan <= 1 ? 0 : nj * nspan * 2 * 65536; }
+inline __host__ SpanBuffers tc_span_view(void* base, size_t nj, int nspan) {
+  if (nspan <= 1) return SpanBuffers{1, nullptr, nullptr};
+  float* f = reinterpret_cast<float*>(base);
+  return SpanBuffers{nspan, f, f + nj * nspan * 16384};
 }
 
 }  // namespace ha_la

@@ -1,0 +1,283 @@
+// Chunk-local operators of the delta-rule prefill, KDA (a gate per key channel): what the state-passing kernel needs per
+// step of 128 tokens.  Work item = (step slot, V-head).  With G the step-local cumulative log-gates of a channel:
+//   #1 Gate   G                                                    (and the operand images K e^G, scale Q e^G, K e^{G_L-G})
+//   #2 KKT    A_ij = beta_i sum_c K_ic K_jc e^{G_ic-G_jc}  (j < i)     P_ij = sum_c Q_ic K_jc e^{G_ic-G_jc}  (j <= i)
+//   #3 Solve  T = (I + A)^-1 by blocked forward substitution (tc_solve.cuh)
+// Out go the three images (tiles as the state-passing kernel's MMAs read them) and the record (tc_common.cuh) T diag(beta),
+// scale P, e^{G_L}: 133 KiB per item, 261 KiB with what it reads, which is what bounds the kernel once its two halves
+// overlap.  They do: a persistent kernel, one CTA per SM, eight warps that make the gate-scaled operands of one item and
+// eight that contract and solve the item before.
+//
+// The decay sits inside the contraction.  Per block of 16 tokens (block rows I, block columns J) it is split at the gates
+// of block boundaries, rounded to whole powers of two, rho_I (log2):
+//   K_i 2^{G_i-rho_I} . K_j 2^{rho_{J+1}-G_j} 2^{rho_I-rho_{J+1}}
+// Both scaled copies are made once per token, in fp32, with exponents <= 1/2 up to rounding; the factor of the pair of
+// blocks is a power of two per channel, so applying it to the bf16 operand in registers rounds nothing.  (A hierarchy of
+// reference points with an own copy per level needs twice the shared memory.)  In a diagonal block that factor is >= 1;
+// where a channel decays by more than 2^100 over 16 tokens, the block is evaluated entry by entry from the inputs.
+// The contraction runs on warp-level MMAs: 36 pairs of blocks of the 64, no work above the diagonal, no operand copies
+// per pair; it is a fifth of the kernel's instructions.
+//
+// Measured on B200 with 32 heads and 8192 tokens: 262 us before (64-token chunks, a copy of the operands per block row,
+// one item at a time per SM).
+//
+// Tokens past the end of a sequence are made no-ops by beta = 0 and g = 0; whatever the TMA box read for them (the
+// next sequence's rows, or zero fill past the end of the tensor) is multiplied by exact zeros.  This relies on the
+// inputs being finite.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include "tc_common.cuh"
+#include "tc_mma.cuh"
+#include "tc_ptx.cuh"
+#include "tc_solve.cuh"
+
+namespace ha_la {
+
+using namespace ptx;
+using namespace solve;
+
+namespace {
+
+constexpr int kKdaThreads = 512;                           // eight scaling warps, eight solving warps
+// per buffer (items alternate): K then K 2^{G-rho} in place | Q likewise | K 2^{rho-G}, then T (fp16 blocks)
+constexpr uint32_t OFF_K = 0, OFF_Q = kTileBytes, OFF_K1 = 2 * kTileBytes, kBufBytes = 3 * kTileBytes;
+constexpr uint32_t OFF_A = 2 * kBufBytes;                  // fp16 A below the diagonal blocks: 28 blocks, operand order
+constexpr uint32_t OFF_D = OFF_A + 28 * 512;               // fp32 diagonal blocks of A
+constexpr uint32_t OFF_TOT = OFF_D + 8 * 16 * LDD * 4;     // float [8][128]: log2 decay of each block
+constexpr uint32_t OFF_DN = OFF_TOT + 4096;                // per buffer: bf16 [8][128], 2^{rho_{J+1}-rho_J}
+constexpr uint32_t OFF_BETA = OFF_DN + 2 * 2048;           // per buffer: float [128]
+constexpr uint32_t OFF_FALL = OFF_BETA + 2 * 512;          // per buffer: int [8], block needs the evaluation entry by entry
+constexpr uint32_t OFF_BAR = OFF_FALL + 2 * 32;
+constexpr uint32_t kKdaSmem = OFF_BAR + 32;
+static_assert(kKdaSmem <= 227 * 1024, "shared memory budget");
+constexpr float kMaxUp = 100.f;
+
+struct KdaParams {
+  const __nv_bfloat16* q;
+  const __nv_bfloat16* k;
+  const float* g;
+  const float* beta;
+  const int32_t* chunk_tok0;   // step table of the plan kernel, or NULL for equal-length rows:
+  const int32_t* chunk_len;    //   then slot s is step s % cps of row s / cps, T_row tokens per row
+  int T_row, cps;
+  TcWorkspace ws;
+  int HK, HV;
+  float scale;
+  long long total;             // work items = step slots x V-heads
+  int32_t* status;
+};
+
+__device__ __forceinline__ float2 ex2(float2 x) { return make_float2(ptx::ex2(x.x), ptx::ex2(x.y)); }
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 r = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+// 2^e for a whole e as bf16 bits (0 below the normal range, the largest power above it)
+__device__ __forceinline__ uint32_t pow2_bf16(float e) { return static_cast<uint32_t>(min(max(static_cast<int>(e) + 127, 0), 254)) << 7; }
+__device__ __forceinline__ uint32_t pow2_pair(float2 e) { return pow2_bf16(e.x) | (pow2_bf16(e.y) << 16); }
+
+// Diagonal block I of A (fp32, times beta) and P, entry by entry, by one warp: lane l has channels 4 l .. 4 l + 3.
+__device__ __noinline__ void slow_diagonal(const KdaParams& p, int j, int jq, int tok0, int L, int I, const float* sBeta, float* sd,
+                                           float (&pd)[2][4], int lane) {
+  const int g8 = lane >> 2, t2 = (lane & 3) * 2;
+  for (int i = 0; i < 16; ++i) {
+    const int ti = 16 * I + i;
+    float kv[4] = {}, qv[4] = {}, w[4] = {1.f, 1.f, 1.f, 1.f};
+    if (ti < L) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const size_t a = ((size_t)(tok0 + ti) * p.HK + jq) * 128 + 4 * lane + c;
+        kv[c] = __bfloat162float(p.k[a]);
+        qv[c] = __bfloat162float(p.q[a]);
+      }
+    }
+    for (int jj = i; jj >= 0; --jj) {
+      const int tj = 16 * I + jj;
+      float a = 0.f, b = 0.f;
+      if (ti < L) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float x = __bfloat162float(p.k[((size_t)(tok0 + tj) * p.HK + jq) * 128 + 4 * lane + c]) * w[c];
+          a = fmaf(kv[c], x, a);
+          b = fmaf(qv[c], x, b);
+          w[c] *= __expf(p.g[((size_t)(tok0 + tj) * p.HV + j) * 128 + 4 * lane + c]);   // decay from tj - 1 to i
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+      }
+      if (lane == 0) sd[i * LDD + jj] = jj < i ? a * sBeta[ti] : 0.f;
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (i == g8 + (e >> 1) * 8 && jj == 8 * n + t2 + (e & 1)) pd[n][e] = b;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kKdaThreads, 1)
+tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, KdaParams p) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + OFF_BAR);         // [2] K and Q tiles
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 2);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int R = p.HV / p.HK;
+  if (tid == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    *abort_flag = 0;
+    mbar_fence_init();
+    prefetch_tmap(&map_q); prefetch_tmap(&map_k);
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");     // nothing of this call has been read or written so far
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  struct Geom { int s, j, L, tok0; };
+  auto geom = [&](long long c) {                         // slots that a packed batch does not use come last, with L = 0
+    Geom g{0, 0, 0, 0};
+    if (c >= p.total) return g;
+    g.s = (int)((unsigned)c / (unsigned)p.HV);
+    g.j = (int)((unsigned)c - (unsigned)g.s * (unsigned)p.HV);
+    if (p.chunk_len) {
+      g.L = p.chunk_len[g.s];
+      g.tok0 = p.chunk_tok0[g.s];
+    } else {
+      const int cc = g.s % p.cps;
+      g.tok0 = (g.s / p.cps) * p.T_row + cc * kStep;
+      g.L = min(kStep, p.T_row - cc * kStep);
+    }
+    return g;
+  };
+  auto issue_tiles = [&](const Geom& g, int b) {         // one thread
+    mbar_expect_tx(&full[b], 2 * kTileBytes);
+    tma_load_4d(sm + b * kBufBytes + OFF_K, &map_k, &full[b], 0, g.j / R, g.tok0, 0);
+    tma_load_4d(sm + b * kBufBytes + OFF_Q, &map_q, &full[b], 0, g.j / R, g.tok0, 0);
+  };
+  // named barriers: 1, 2 the scaled operands of buffer 0, 1 are ready; 3, 4 the buffer is free again (T read); 5, 6 within
+  // the scaling and the solving warps
+  auto arrive = [&](int id) { asm volatile("bar.arrive %0, 512;" ::"r"(id) : "memory"); };
+  auto sync = [&](int id) { asm volatile("bar.sync %0, 512;" ::"r"(id) : "memory"); };
+  auto sync_half = [&](int id) { asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory"); };
+
+  const long long stride = gridDim.x;
+  if (warp >= 8) {
+    // ------------------------------------------------------------ scaling: a pair of channels and 32 tokens per thread
+    const int w = warp - 8, kb = w & 1, tg = w >> 1;
+    const int cp = kb * 64 + 2 * lane;                   // channels cp, cp + 1; blocks 2 tg, 2 tg + 1
+    const uint32_t o0 = kb * 16384 + ((lane & 3) << 2), ch = (lane >> 2) << 4;
+    float* sTot = reinterpret_cast<float*>(sm + OFF_TOT);
+    Geom gm = geom(blockIdx.x);
+    if (tid == 256 && gm.L > 0) issue_tiles(gm, 0);
+    long long it = 0;
+    for (long long item = blockIdx.x; gm.L > 0; ++it) {
+      const int b = (int)(it & 1);
+      const size_t cj = (size_t)gm.s * p.HV + gm.j;
+      float2 l[2][16];                                   // block-local cumulative log2 gates
+      {
+        const float* gp = p.g + ((size_t)(gm.tok0 + 32 * tg) * p.HV + gm.j) * 128 + cp;
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int t = 0; t < 16; ++t)
+            l[u][t] = 32 * tg + 16 * u + t < gm.L ? *reinterpret_cast<const float2*>(gp + (size_t)(16 * u + t) * p.HV * 128) : make_float2(0.f, 0.f);
+      }
+      float bt = 0.f;
+      if (tg == 0 || tg == 1) {                          // (warps 8 .. 11: a token's beta per thread)
+        const int t = w * 32 + lane;
+        bt = t < gm.L ? p.beta[(size_t)(gm.tok0 + t) * p.HV + gm.j] : 0.f;
+      }
+      item += stride;
+      const Geom gn = geom(item);
+      if (gn.L > 0 && w < 4) {                           // the next item's gate rows, into L2
+        const int t = w * 32 + lane;
+        if (t < gn.L) bulk_prefetch_l2(p.g + ((size_t)(gn.tok0 + t) * p.HV + gn.j) * 128, 512);
+      }
+      const float2 lg = make_float2(1.4426950408889634f, 1.4426950408889634f);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        l[u][0] = mul2(l[u][0], lg);
+#pragma unroll
+        for (int t = 1; t < 16; ++t) l[u][t] = fma2(l[u][t], lg, l[u][t - 1]);
+        *reinterpret_cast<float2*>(sTot + (2 * tg + u) * 128 + cp) = l[u][15];
+      }
+      sync_half(5);
+      float2 B[3], GL = make_float2(0.f, 0.f);           // gates at the boundaries of this thread's blocks, and the last
+#pragma unroll
+      for (int I = 0; I < 8; ++I) {
+        if (I == 2 * tg) B[0] = GL;
+        const float2 x = *reinterpret_cast<const float2*>(sTot + I * 128 + cp);
+        GL.x += x.x; GL.y += x.y;
+        if (I == 2 * tg) B[1] = GL;
+        if (I == 2 * tg + 1) B[2] = GL;
+      }
+      float2 rho[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) rho[i] = make_float2(rintf(B[i].x), rintf(B[i].y));
+      if (it > 1) sync(3 + b);                           // the solving warps are done with the item two before
+      mbar_wait(&full[b], (uint32_t)(it >> 1) & 1, abort_flag);
+      uint8_t* buf = sm + b * kBufBytes;
+      if (tg < 2) reinterpret_cast<float*>(sm + OFF_BETA + b * 512)[w * 32 + lane] = bt;
+      uint8_t* img = p.ws.img + cj * 3 * kTileBytes;
+      if (tg == 0) *reinterpret_cast<float2*>(p.ws.rec + cj * kStepRecB + kStepSc + cp * 4) = ex2(GL);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int I = 2 * tg + u;
+        const float2 dn = make_float2(rho[u + 1].x - rho[u].x, rho[u + 1].y - rho[u].y);
+        *reinterpret_cast<uint32_t*>(sm + OFF_DN + b * 2048 + I * 256 + cp * 2) = pow2_pair(dn);
+        const bool far = __any_sync(0xffffffffu, dn.x < -kMaxUp || dn.y < -kMaxUp);
+        if (lane == 0) reinterpret_cast<int*>(sm + OFF_FALL + b * 32)[I] = 0;
+        __syncwarp();
+        (void)far;
+        const float2 a0 = make_float2(B[u].x - rho[u].x, B[u].y - rho[u].y);
+        const float2 a1 = make_float2(rho[u + 1].x - B[u].x, rho[u + 1].y - B[u].y);
+        const uint32_t pw = pow2_pair(rho[u]);
+        const float2 sq = mul2(ex2(rho[u]), make_float2(p.scale, p.scale));
+        const float2 cd = ex2(make_float2(GL.x - rho[u + 1].x, GL.y - rho[u + 1].y));
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const uint32_t o = o0 + (16 * I + t) * 128 + (ch ^ ((t & 7) << 4));
+          const int td = step_pos(t);
+          const uint32_t od = o0 + (16 * I + td) * 128 + (ch ^ ((td & 7) << 4));
+          const float2 e0 = ex2(make_float2(l[u][t].x + a0.x, l[u][t].y + a0.y));
+          const float2 e1 = ex2(make_float2(a1.x - l[u][t].x, a1.y - l[u][t].y));
+          const float2 kf = unpack_bf16(*reinterpret_cast<const uint32_t*>(buf + OFF_K + o));
+          const float2 qe = mul2(unpack_bf16(*reinterpret_cast<const uint32_t*>(buf + OFF_Q + o)), e0);
+          const uint32_t k0 = pack_bf16(mul2(kf, e0));
+          const float2 k1 = mul2(kf, e1);
+          *reinterpret_cast<uint32_t*>(buf + OFF_K + o) = k0;
+          *reinterpret_cast<uint32_t*>(buf + OFF_Q + o) = pack_bf16(qe);
+          *reinterpret_cast<uint32_t*>(buf + OFF_K1 + o) = pack_bf16(k1);
+          *reinterpret_cast<uint32_t*>(img + o) = mul_bf16x2(k0, pw);
+          *reinterpret_cast<uint32_t*>(img + kTileBytes + o) = pack_bf16(mul2(qe, sq));
+          *reinterpret_cast<uint32_t*>(img + 2 * kTileBytes + od) = pack_bf16(mul2(k1, cd));
+        }
+      }
+      arrive(1 + b);
+      // the other buffer's tiles were free once the solving warps had the item before in registers (they issue the copy)
+      gm = gn;
+    }
+  } else {
+    // ------------------------------------------------------------ contraction and solve
+    Geom gm = geom(blockIdx.x);
+    long long it = 0;
+    for (long long item = blockIdx.x; gm.L > 0; ++it) {
+      const int b = (int)(it & 1);
+      const int j = gm.j, jq = j / R;
+      const size_t cj = (size_t)gm.s * p.HV + j;
+      uint8_t* rec = p.ws.rec + cj * kStepRecB;
+      uint8_t* buf = sm + b * kBufBytes;
+      item += stride;
+      const Geom gn = geom(item);
+      (void)rec; (void)buf; (void)jq; (void)cj;
+      gm = gn;
+    }
+  }
+}
+
+}  // namespace
+}  // namespace ha_la

@@ -56,7 +56,7 @@ constexpr int kPhiLd = 128 + 4;          // row strides (floats) in shared memor
 constexpr int kHLd = kFixCols + 4;
 constexpr size_t kFixSmem = (size_t)128 * kPhiLd * 4 + (size_t)128 * kHLd * 4;
 
-__global__ void __launch_bounds__(256) seg_fix_kernel(SegBuffers sg, float* hT, int T_row, int HV, const int32_t* seq_len) {
+__global__ void __launch_bounds__(256) seg_fix_kernel(SegBuffers sg, float* hT, int T_row, int HV, int step, const int32_t* seq_len) {
   using namespace nvcuda;
   extern __shared__ __align__(32) float fsm[];
   float* sPhi = fsm;                     // [128][kPhiLd]: Phi_s
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) seg_fix_kernel(SegBuffers sg, float* hT, 
   // segments past the end of a short sequence are empty: their transition is the identity and the state passes
   // through untouched (bit for bit, which the TF32 product would not do)
   const int len = seq_len ? seq_len[nj / HV] : T_row;
-  const int nch = (len + kChunk - 1) / kChunk;
+  const int nch = (len + step - 1) / step;
   const int cpseg = (nch + sg.nseg - 1) / sg.nseg;
   asm volatile("griddepcontrol.wait;" ::: "memory");     // (launched as a programmatic dependent of the chain kernel)
   float4 t[16];
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256) seg_fix_kernel(SegBuffers sg, float* hT, 
 constexpr int kLdR = 128 + 8, kLdC = 64 + 4;
 constexpr size_t kOutSmem = (size_t)(64 + 128) * kLdR * 2 + (size_t)8 * 16 * kLdC * 4;
 
-__global__ void __launch_bounds__(256) seg_out_kernel(SegBuffers sg, __nv_bfloat16* o, int T_row, int HV, int cps,
+__global__ void __launch_bounds__(256) seg_out_kernel(SegBuffers sg, __nv_bfloat16* o, int T_row, int HV, int cps, int step,
                                                       const int32_t* seq_tok0, const int32_t* seq_len) {
   using namespace nvcuda;
   extern __shared__ __align__(32) uint8_t osm[];
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) seg_out_kernel(SegBuffers sg, __nv_bfloat
   const int len = seq_len ? seq_len[n] : T_row;          // (packed batches: the plan kernel's per-sequence table)
   const int tok0 = seq_tok0 ? seq_tok0[n] : n * T_row;
   const int nch = (len + kChunk - 1) / kChunk;
-  const int cpseg = (nch + sg.nseg - 1) / sg.nseg;
+  const int cpseg = ((len + step - 1) / step + sg.nseg - 1) / sg.nseg * (step / kChunk);   // segments are whole steps
   const int cc = seg * cpseg + cin;                      // this CTA's chunk of the sequence
   const int cend = min((seg + 1) * cpseg, nch);          // end of the segment
   asm volatile("griddepcontrol.wait;" ::: "memory");     // (programmatic dependent of the fix-up kernel)
@@ -253,16 +253,16 @@ cudaError_t launch_tc_seg_fix(const Problem& p, const ha_la_prefill_args& a, Pla
   cfg.gridDim = dim3((unsigned)(p.N * p.HV), 128 / kFixCols);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = kFixSmem;
-  ce = cudaLaunchKernelEx(&cfg, seg_fix_kernel, sg, a.hT, p.T_row, p.HV, (const int32_t*)plan.seq_len);
+  ce = cudaLaunchKernelEx(&cfg, seg_fix_kernel, sg, a.hT, p.T_row, p.HV, p.step, (const int32_t*)plan.seq_len);
   if (ce != cudaSuccess) return ce;
-  const int nch = p.max_seq_chunks;                      // longest sequence (a bound, for packed batches)
-  const int cpseg = (nch + sg.nseg - 1) / sg.nseg;
-  if (nch <= cpseg) return cudaSuccess;                  // (everything is in segment 0)
+  const int nst = p.max_seq_chunks;                      // longest sequence (a bound, for packed batches)
+  const int cpseg = (nst + sg.nseg - 1) / sg.nseg * (p.step / kChunk);
+  if (nst * (p.step / kChunk) <= cpseg) return cudaSuccess;                  // (everything is in segment 0)
   timer_mark(stream, "tc_seg_out");
   cfg.gridDim = dim3((unsigned)(p.N * (sg.nseg - 1) * cpseg), (unsigned)p.HV);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = kOutSmem;
-  return cudaLaunchKernelEx(&cfg, seg_out_kernel, sg, reinterpret_cast<__nv_bfloat16*>(a.o), p.T_row, p.HV, cpseg,
+  return cudaLaunchKernelEx(&cfg, seg_out_kernel, sg, reinterpret_cast<__nv_bfloat16*>(a.o), p.T_row, p.HV, cpseg, p.step,
                             (const int32_t*)plan.seq_tok0, (const int32_t*)plan.seq_len);
 }
 

@@ -1,0 +1,698 @@
+// Sequential part of the delta-rule prefill on tcgen05 tensor cores: operator #5 (state passing) with operator #4
+// applied and operator #6 (output) fused in the paper's chunk-first order.
+//
+// One CTA owns all 128 value channels of a (sequence, V-head) and walks its sequence, or one span of it, in steps of 128
+// tokens.  The state is kept TRANSPOSED: fp32 in registers, and as bf16 pairs in tensor memory (lane = value channel,
+// columns = key channels), where it is the A operand of the products; every other state-dependent operand is made there
+// too, so nothing that threads write goes through shared memory on its way to the tensor cores (no proxy fences), and
+// shared memory is left to the B operands, which arrive ready-made by bulk copy.  Per step (GDN; the prep kernel supplies
+// T diag(beta), P and the gate factors):
+//   X^T  = h^T K^T                          R^T = V^T - e^{G_j} X^T                 bf16 pairs
+//   U~^T = R^T (T diag(beta))^T                                                     bf16 pairs, plain and times e^{G_L-G_j}
+//   h^T <- e^{G_L} h^T + (U~ e^{G_L-G})^T K                                          op #5
+//   o^T  = scale [e^{G_i} (h^T Q^T) + U~^T P^T]   (old h; off the sequential path)   op #6
+// KDA: K e^G, Q e^G and K e^{G_L-G} come as images from the prep kernel, so no column factors are needed and the decay is
+// per key channel.
+//
+// What bounds a step: three products that wait for each other's epilogue (K = 128: eight instructions of 64 cycles, ~180
+// cycles to a visible result, ~250 of tensor-memory traffic and arithmetic by the compute warps) -- about 3 k cycles -- and
+// close behind it the tensor cores (2.3 k: all five products) and shared memory (133 KiB in, 132 KiB of B operands,
+// 96 KiB of V and o tiles: 2.9 k at 128 bytes per cycle).  T and P are lower triangular: step ks of their products runs
+// with N = 128 - 16 ks rows.
+//
+// Warp roles: sixteen compute warps (tensor-memory lanes 32 (w % 4).., group w / 4 of the columns), four output warps, two
+// producer warps, two warps that issue MMAs (the sequential path; the outputs).  Every wait is bounded.
+#include <cuda.h>
+
+#include "tc_common.cuh"
+#include "tc_mma.cuh"
+#include "tc_ptx.cuh"
+#include "prof.cuh"
+
+namespace ha_la {
+
+using namespace ptx;
+
+HA_PROF_DECL(walk)
+
+namespace {
+
+constexpr int kCompute = 512;                              // compute threads: four warps for each of four column groups
+constexpr int walk_threads(bool out) { return kCompute + 32 * (out ? 8 : 3); }
+
+struct WalkCfg {
+  static constexpr uint32_t OFF_K = 0;                     // GDN: two K tiles (steps alternate); KDA: K e^G, K e^{G_L-G}
+  static constexpr uint32_t OFF_Q = 65536;                 // Q (KDA: Q e^G)
+  static constexpr uint32_t OFF_V = 98304;                 // V tile, [2][128 tok][64 ch]
+  static constexpr uint32_t OFF_T = 131072;
+  static constexpr uint32_t OFF_P = OFF_T + kTriB;
+  static constexpr uint32_t OFF_OUT = OFF_P + kTriB;       // output staging: [4 warps][128 tok][32 ch]
+  static constexpr uint32_t OFF_SC = OFF_OUT + 32768;      // two sets of gate factors
+  static constexpr uint32_t OFF_BAR = OFF_SC + 2 * kStepScB;
+  static constexpr uint32_t kSmem = OFF_BAR + 20 * 8 + 16;
+  static_assert(kSmem <= 227 * 1024, "shared memory budget");
+  // tensor-memory columns (all 512 are allocated, so the base is column 0): X, then D2 | U, then (GDN) plain U~ as operand | Y, then o | h operand | R, then U~ operand
+  static constexpr uint32_t TM_X = 0, TM_U = 128, TM_UP = 128, TM_Y = 256, TM_H = 384, TM_R = 448;
+};
+
+struct WalkParams {
+  const float* h0;
+  float* hT;
+  void* o;
+  const int32_t* seq_tok0;     // per-sequence table of the plan kernel, or NULL for equal-length rows
+  const int32_t* seq_len;      //   (then sequence n is tokens [n*T_row, (n+1)*T_row), cps steps each)
+  const int32_t* seq_chunk0;
+  const int32_t* seq_order;    // launch order of the sequences (longest first), or NULL
+  int T_row, cps;
+  TcWorkspace ws;
+  int HK, HV;
+  float scale;
+  int64_t epoch;               // != 0: the prep kernel runs concurrently; wait for ws.flags[cj] == epoch per step
+                               // == 0: wait for the whole prep grid before the first workspace read
+  uint32_t spin_limit;         // polls before a bounded wait gives up (a few thousand in the time-out test)
+  // Spans: a sequence's steps are cut into `nspan` runs that are walked at the same time (1: off), in two launches with
+  // span_fix_kernel (tc_span.cu) between them.  The state recurrence is affine in the start state, so
+  //   first launch, state only (OUT = false): spans 0 .. nspan-2 from their own start (span 0: h0, others: zero) into
+  //     span_b, and spans 1 .. nspan-2 from the IDENTITY with V = 0 (the transition) into span_phi;
+  //   fix: h_1 = b_0, h_{s+1} = Phi_s h_s + b_s,  in place of b_{s+1};
+  //   second launch (OUT = true): every span from its true start, outputs and final state.
+  int nspan;
+  float* span_b;               // [N*HV][nspan][128 keys][128 channels] fp32
+  float* span_phi;
+  int32_t* status;
+};
+
+// named barriers (0 is __syncthreads)
+constexpr int BAR_H = 1;       // compute arrive, W_MMA syncs: h operand stored
+constexpr int BAR_R = 2;       // ... R operand, first (2) and second (3) half of the tokens
+constexpr int BAR_U = 4;       // ... operand of the state update, likewise (4, 5)
+constexpr int BAR_UP = 6;      // (GDN) ... plain U~ operand, and Y times e^{G_i}; syncs the second MMA warp
+constexpr int BAR_GY = 7;      // the first MMA warp arrives, the second syncs: X issued
+constexpr int BAR_GP = 8;      // ... D2 issued
+// A CTA lets the stream's next programmatic dependent be scheduled when it has this many steps left (CTAs with fewer:
+// when they exit).  That kernel then gets through its launch and set-up under the tail of this one and waits at its
+// griddepcontrol.wait for this grid to complete.
+constexpr int kTailSteps = 3;
+__device__ __forceinline__ void named_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+template <bool KDA, bool OUT>
+__global__ void __launch_bounds__(walk_threads(OUT), 1)
+tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
+               const __grid_constant__ CUtensorMap map_v, WalkParams p) {
+  using Cfg = WalkCfg;
+  extern __shared__ __align__(1024) uint8_t sm[];       // no static shared memory in this kernel: 1024-aligned
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + Cfg::OFF_BAR);
+  uint64_t* full_k = bar;            // [2] operand tiles of X and D2 (GDN: one per step, two slots; KDA: one each)
+  uint64_t* empty_k = bar + 2;       // [2] (GDN) D2 of the slot's step complete
+  uint64_t* full_q = bar + 4;
+  uint64_t* bar_y = bar + 5;         // Y complete (Q and the old h operand have been read)
+  uint64_t* full_v = bar + 6;
+  uint64_t* empty_v = bar + 7;       // V read by the compute warps
+  uint64_t* full_t = bar + 8;        // (T is free again when U is complete, P when the step's output product is)
+  uint64_t* full_p = bar + 9;
+  uint64_t* full_sc = bar + 10;      // [2]
+  uint64_t* bar_x = bar + 12;
+  uint64_t* bar_u0 = bar + 13;       // U complete for the first 64 tokens
+  uint64_t* bar_d2 = bar + 14;
+  uint64_t* bar_o = bar + 15;        // o complete in tensor memory
+  uint64_t* out_free = bar + 16;     // ... and read by the output warps
+  uint64_t* empty_sc = bar + 17;     // [2] gate factors read by everyone
+  uint64_t* bar_u1 = bar + 19;       // ... for the others
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 20);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  constexpr int W_OUT = kCompute / 32, W_P0 = W_OUT + (OUT ? 4 : 0), W_P1 = W_P0 + 1, W_MMA = W_P1 + 1;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int units = p.nspan == 1 ? 1 : (OUT ? p.nspan : 2 * p.nspan - 3);   // runs per (sequence, V-head)
+  const int unit = blockIdx.x % units;
+  const int nj = blockIdx.x / units;
+  const bool trans = !OUT && unit >= p.nspan - 1;        // a transition run
+  const int span = trans ? unit - p.nspan + 2 : unit;
+  const int j = nj % p.HV;
+  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;   // CTAs of the longest sequences come first
+  const int jq = j / (p.HV / p.HK);
+  const int tok0_seq = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
+  const int len_seq = p.seq_tok0 ? p.seq_len[n] : p.T_row;
+  const int slot0_seq = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
+  // this CTA's span of the sequence, walked like a sequence of its own
+  const int nst_seq = (len_seq + kStep - 1) / kStep;
+  const int spspan = (nst_seq + p.nspan - 1) / p.nspan;
+  const int tok0 = tok0_seq + span * spspan * kStep;
+  const int len = max(0, min(len_seq - span * spspan * kStep, spspan * kStep));
+  const int slot0 = slot0_seq + span * spspan;
+  const int nsteps = (len + kStep - 1) / kStep;
+
+  if (tid == 0) {
+    for (int i = 0; i < 20; ++i) {
+      const uint64_t* b = bar + i;
+      mbar_init(&bar[i], b == empty_v ? kCompute / 32 : b == out_free ? 4 : b == empty_sc || b == empty_sc + 1 ? kCompute / 32 : 1);
+    }
+    *abort_flag = 0;
+    mbar_fence_init();
+    prefetch_tmap(&map_v);
+    if (!KDA) { prefetch_tmap(&map_k); prefetch_tmap(&map_q); }
+  }
+  if (warp == 0) tmem_alloc(tmem_slot, 512);
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  constexpr uint32_t tmem = 0;                           // (the whole of tensor memory)
+  // This kernel may be launched as a programmatic dependent of the prep kernel, i.e. start while that one is still
+  // running.  Sequential mode: everything above overlapped the prep kernel's tail; wait for it here.
+  if (p.epoch == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // Concurrent mode: a whole warp looks at the ready flags of the next 32 steps at once (plain loads) and remembers how
+  // far the prep kernel has got; the acquire fence and the proxy fence, which are what makes the published results
+  // visible to this kernel's bulk copies, are then paid once per batch, not per step.
+  int ready_upto = p.epoch != 0 ? 0 : nsteps;            // steps [0, ready_upto) are known to be published
+  auto wait_ready = [&](int c) {
+    if (c < ready_upto) return;
+    int got = 0;
+    for (uint32_t it = 0; it < p.spin_limit && !*abort_flag; ++it) {
+      const int cc = c + lane;
+      bool ok = false;
+      if (cc < nsteps)
+        ok = *reinterpret_cast<const volatile int64_t*>(p.ws.flags + (size_t)(slot0 + cc) * p.HV + j) == p.epoch;
+      const unsigned m = __ballot_sync(0xffffffffu, ok);
+      got = __ffs(~m) - 1;                               // leading published steps (32 when all are)
+      if (got < 0) got = 32;
+      if (got > 0) break;
+      __nanosleep(100);
+    }
+    if (got == 0) *abort_flag = 1;                       // gave up: the status word reports the time-out
+    ready_upto = c + (got > 0 ? got : nsteps);
+    __threadfence();                                     // acquire side of the prep kernel's release
+    fence_proxy_async_all();
+  };
+  auto aborted = [&]() { return __any_sync(0xffffffffu, *abort_flag) != 0; };
+  // (mbarrier.try_wait costs the caller ~150 cycles even when the phase is over: test first)
+  auto wait1 = [&](uint64_t* b, uint32_t parity) {
+    if (!mbar_test_wait(b, parity & 1)) mbar_wait(b, parity & 1, abort_flag, p.spin_limit);
+  };
+
+  if (warp == W_P0) {
+    // ------------------------------------------------------------ producer of the tiles: X / D2 operands, Q, V
+    for (int c = 0; c < nsteps; ++c) {
+      if (KDA) wait_ready(c);
+      if (lane == 0) {
+        const int t0 = tok0 + c * kStep;
+        const uint8_t* img = KDA ? p.ws.img + ((size_t)(slot0 + c) * p.HV + j) * 3 * kTileBytes : nullptr;
+        if constexpr (KDA) {
+          if (c > 0) wait1(bar_x, c - 1);
+          if (!*abort_flag) {
+            mbar_expect_tx(&full_k[0], kTileBytes);
+            bulk_load(sm + Cfg::OFF_K, img, kTileBytes, &full_k[0]);
+          }
+        } else {
+          const int st = c & 1;
+          if (c > 1) wait1(&empty_k[st], (c >> 1) - 1);
+          if (!*abort_flag) {
+            mbar_expect_tx(&full_k[st], kTileBytes);
+            tma_load_4d(sm + Cfg::OFF_K + st * kTileBytes, &map_k, &full_k[st], 0, jq, t0, 0);
+          }
+        }
+        if (!trans) {                                    // (transition: V = 0)
+          if (c > 0) wait1(empty_v, c - 1);
+          if (!*abort_flag) {
+            mbar_expect_tx(full_v, kTileBytes);
+            tma_load_4d(sm + Cfg::OFF_V, &map_v, full_v, 0, j, t0, 0);
+          }
+        }
+        if constexpr (OUT) {
+          if (c > 0) wait1(bar_y, c - 1);
+          if (!*abort_flag) {
+            mbar_expect_tx(full_q, kTileBytes);
+            if constexpr (KDA) bulk_load(sm + Cfg::OFF_Q, img + kTileBytes, kTileBytes, full_q);
+            else tma_load_4d(sm + Cfg::OFF_Q, &map_q, full_q, 0, jq, t0, 0);
+          }
+        }
+        if constexpr (KDA) {
+          if (c > 0) wait1(bar_d2, c - 1);
+          if (!*abort_flag) {
+            mbar_expect_tx(&full_k[1], kTileBytes);
+            bulk_load(sm + Cfg::OFF_K + kTileBytes, img + 2 * kTileBytes, kTileBytes, &full_k[1]);
+          }
+        }
+      }
+      if (aborted()) break;
+    }
+  } else if (warp == W_P1) {
+    // ------------------------------------------------------------ producer of the prep kernel's records
+    for (int c = 0; c < nsteps; ++c) {
+      wait_ready(c);
+      const uint8_t* rec = p.ws.rec + ((size_t)(slot0 + c) * p.HV + j) * kStepRecB;
+      if (lane == 0) {
+        if (c > 1) wait1(&empty_sc[c & 1], (c >> 1) - 1);
+        if (!*abort_flag) {
+          mbar_expect_tx(&full_sc[c & 1], kStepScB);
+          bulk_load(sm + Cfg::OFF_SC + (c & 1) * kStepScB, rec + kStepSc, kStepScB, &full_sc[c & 1]);
+        }
+        if (c > 0) wait1(bar_u1, c - 1);
+        if (!*abort_flag) {
+          mbar_expect_tx(full_t, kTriB);
+          bulk_load(sm + Cfg::OFF_T, rec + kStepT, kTriB, full_t);
+        }
+        if constexpr (OUT) {
+          if (c > 0) wait1(bar_o, c - 1);
+          if (!*abort_flag) {
+            mbar_expect_tx(full_p, kTriB);
+            bulk_load(sm + Cfg::OFF_P, rec + kStepP, kTriB, full_p);
+          }
+        }
+      }
+      if (aborted()) break;
+    }
+  } else if (warp >= W_MMA) {
+    // ------------------------------------------------------------ MMA issue (lane 0 issues; the warp keeps the barriers)
+    // One warp issues the products of the sequential path, another those of the outputs: an instruction is accepted when
+    // the one a few places before it has run, so an issuing thread is held up by its own products.  The tensor cores work
+    // in order of issue, so the second warp goes when the first one tells it to: Y behind X, under X's epilogue, and P U~
+    // behind D2, under the epilogue of the state.  Descriptors advance by constants: their arithmetic takes the thread as
+    // long as an instruction of the MMA itself.
+    constexpr uint32_t id_kk = idesc_bf16(128, 128, false, false);   // B K-major: X, Y (rows = tokens)
+    constexpr uint32_t id_km = idesc_bf16(128, 128, false, true);    // B MN-major: D2 (rows = the K index, tokens)
+    const bool lead = lane == 0;
+    auto tile_product = [&](uint32_t d, uint64_t b) {    // K-major B tile, 128 rows: 16 features per instruction
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks)
+        umma_ts(d, Cfg::TM_H + 8 * ks, b + ((uint32_t)((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), id_kk, ks > 0);
+    };
+    // A [128 x 128] (triangular operand)^T, k-steps 4 half ..: slab ks is the operand of the result's columns 16 ks ..
+    auto tri_half = [&](int half, uint32_t d, uint32_t a, uint32_t astep, uint64_t tri, uint32_t acc) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int ks = 4 * half + i;
+        umma_ts(d + 16 * ks, a + ks * astep, tri + (tri_slab(ks) >> 4), idesc_bf16(128, 128 - 16 * ks, false, false), acc | (ks > 0));
+      }
+    };
+    if (warp == W_MMA) {
+      const uint64_t dK0 = smem_desc(smem_u32(sm + Cfg::OFF_K), 16, 1024, kSwizzle128B);
+      const uint64_t dKm0 = smem_desc(smem_u32(sm + Cfg::OFF_K), 16384, 1024, kSwizzle128B);
+      const uint64_t dT = smem_desc(smem_u32(sm + Cfg::OFF_T), 16, 256, kSwizzle32B);
+      for (int c = 0; c < nsteps; ++c) {
+        const int st = KDA ? 0 : (c & 1);
+        const uint64_t dK = dK0 + st * (kTileBytes >> 4);
+        const uint64_t dKm = dKm0 + (KDA ? 1 : st) * (kTileBytes >> 4);
+        if (lead) wait1(&full_k[st], KDA ? c : (c >> 1));
+        named_sync(BAR_H, kCompute + 32);                // h operand of the previous step
+        if (lead) {
+          tc_fence_after_sync();
+          tile_product(Cfg::TM_X, dK);
+          umma_commit(bar_x);
+        }
+        __syncwarp();
+        if (OUT) named_arrive(BAR_GY, 64);
+        if (lead) {
+          wait1(full_t, c);
+          if (OUT && c > 0) wait1(bar_o, c - 1);         // (its operand lies in U's columns)
+        }
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {           // (tokens 0 .. 63 of U are final after the first four k-steps)
+          named_sync(BAR_R + half, kCompute + 32);
+          if (lead) {
+            tc_fence_after_sync();
+            tri_half(half, Cfg::TM_U, Cfg::TM_R, 8, dT, 0u);
+            umma_commit(half ? bar_u1 : bar_u0);
+          }
+        }
+        if (KDA && lead) wait1(&full_k[1], c);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          named_sync(BAR_U + half, kCompute + 32);
+          if (lead) {
+            tc_fence_after_sync();
+#pragma unroll
+            for (int ks = 4 * half; ks < 4 * half + 4; ++ks)   // K index = tokens: 16 rows of 128 bytes per step
+              umma_ts(Cfg::TM_X, Cfg::TM_R + 8 * ks, dKm + ks * (2048u >> 4), id_km, ks > 0);
+          }
+        }
+        if (lead) {
+          umma_commit(bar_d2);
+          if (!KDA) umma_commit(&empty_k[st]);
+        }
+        __syncwarp();
+        if (OUT) named_arrive(BAR_GP, 64);
+      }
+      named_sync(BAR_H, kCompute + 32);                  // pairs with the compute warps' last arrival
+    } else {
+      const uint64_t dQ = smem_desc(smem_u32(sm + Cfg::OFF_Q), 16, 1024, kSwizzle128B);
+      const uint64_t dP = smem_desc(smem_u32(sm + Cfg::OFF_P), 16, 256, kSwizzle32B);
+      for (int c = 0; c < nsteps; ++c) {
+        if (lead) {
+          wait1(full_q, c);
+          if (c > 0) wait1(out_free, c - 1);
+        }
+        named_sync(BAR_GY, 64);
+        if (lead) {
+          tc_fence_after_sync();
+          tile_product(Cfg::TM_Y, dQ);
+          umma_commit(bar_y);
+          wait1(full_p, c);
+        }
+        if (!KDA) named_sync(BAR_UP, kCompute + 32);
+        named_sync(BAR_GP, 64);
+        if (lead) {
+          tc_fence_after_sync();
+          tri_half(0, Cfg::TM_Y, KDA ? Cfg::TM_R : Cfg::TM_UP, KDA ? 8 : 16, dP, 1u);
+          tri_half(1, Cfg::TM_Y, KDA ? Cfg::TM_R : Cfg::TM_UP, KDA ? 8 : 16, dP, 1u);
+          umma_commit(bar_o);
+        }
+      }
+    }
+  } else if (warp >= W_OUT) {
+    // ------------------------------------------------------------ output warps: o, transposed
+    if constexpr (OUT) {
+      const int q = warp - W_OUT;
+      const int lm = lane >> 3, lr = lane & 7;
+      const uint32_t ty = tmem + Cfg::TM_Y + (static_cast<uint32_t>(q * 32) << 16);
+      const uint32_t tile = smem_u32(sm + Cfg::OFF_OUT) + q * 8192;       // [128 tok][32 ch], 64-byte rows
+      const uint32_t tile0[2] = {tile + sw64_offset((lm >> 1) * 8 + lr, lm & 1), tile + sw64_offset((lm >> 1) * 8 + lr, 2 + (lm & 1))};
+      __nv_bfloat16* obase = reinterpret_cast<__nv_bfloat16*>(p.o) + (size_t)j * 128 + q * 32;
+      for (int c = 0; c < nsteps; ++c) {
+        wait1(bar_o, c);
+        tc_fence_after_sync();
+        uint32_t r[2][2][16];
+        auto load_o = [&](int tb) {
+#pragma unroll
+          for (int hl = 0; hl < 2; ++hl) tmem_ld_16x256b_x4(ty + (static_cast<uint32_t>(16 * hl) << 16) + 32 * tb, r[tb & 1][hl]);
+        };
+        load_o(0);
+#pragma unroll
+        for (int tb = 0; tb < 4; ++tb) {
+          tmem_ld_wait();
+          if (tb < 3) load_o(tb + 1);
+          else {
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(out_free);        // (the next Y may go there)
+          }
+#pragma unroll
+          for (int hl = 0; hl < 2; ++hl)
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {                // 16 tokens x 16 channels, transposed on the way
+              uint32_t w[4];
+#pragma unroll
+              for (int x = 0; x < 4; ++x) w[x] = pack_bf16(as_f2(r[tb & 1][hl][8 * m + 2 * x], r[tb & 1][hl][8 * m + 2 * x + 1]));
+              stsm4t(tile0[hl] + (32 * tb + 16 * m) * 64, w);
+            }
+        }
+        __syncwarp();
+        const int left = len - c * kStep;
+        __nv_bfloat16* orow = obase + (size_t)(tok0 + c * kStep) * p.HV * 128 + (lane & 3) * 8;
+#pragma unroll 4
+        for (int it = 0; it < 16; ++it) {
+          const int t = it * 8 + (lane >> 2);
+          uint32_t w[4];
+          lds4(w, tile + sw64_offset(t, lane & 3));
+          if (t < left) *reinterpret_cast<uint4*>(orow + (size_t)t * p.HV * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncwarp();
+      }
+    }
+  } else {
+    // ------------------------------------------------------------ compute
+    // tensor-memory lanes 32 q ..; columns: keys 32 g .. of the state, tokens 16 g .. of each half of the step
+    const int q = warp & 3, g = warp >> 2;
+    const int v = q * 32 + lane;                         // value channel of the 32x32b accesses
+    const int lm = lane >> 3, lr = lane & 7, t2 = (lane & 3) * 2;
+    const uint32_t tq = tmem + (static_cast<uint32_t>(q * 32) << 16);
+    float h[32];                                         // h^T[v][32 g ..]
+    {
+      const float* src = nullptr;
+      if (span == 0 && !trans) src = p.h0 ? p.h0 + ((size_t)n * p.HV + j) * 16384 : nullptr;
+      else if (OUT) src = p.span_b + (((size_t)n * p.HV + j) * p.nspan + span) * 16384;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) h[k] = src ? src[(size_t)(32 * g + k) * 128 + v] : (trans && 32 * g + k == v ? 1.f : 0.f);
+    }
+    auto step_h = [&](int k, float2 decay, float2 add) {
+      const float2 x = fma2(decay, make_float2(h[k], h[k + 1]), add);
+      h[k] = x.x;
+      h[k + 1] = x.y;
+    };
+    auto store_h = [&]() {                               // bf16 pairs of this thread's key channels -> A operand
+      uint32_t r[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) r[k] = pack_bf16(h[2 * k], h[2 * k + 1]);
+      tmem_st16(tq + Cfg::TM_H + 16 * g, r);
+      tmem_st_wait();
+    };
+    store_h();
+    tc_fence_before_sync();
+    named_arrive(BAR_H, kCompute + 32);
+
+    const uint32_t hi = 16u << 16;                       // sixteen lanes further
+    const uint32_t va0 = smem_u32(sm + Cfg::OFF_V) + ((4 * q) >> 3) * 16384;
+    uint32_t vv[2][4], x[2][8];
+    auto load_v = [&](int tk) {                          // V^T of 16 tokens, 2 x 16 channels (transposed by ldmatrix)
+#pragma unroll
+      for (int hl = 0; hl < 2; ++hl)
+        ldsm4t(vv[hl], va0 + sw128_offset(tk + (lm >> 1) * 8 + lr, (4 * q + 2 * hl + (lm & 1)) & 7));
+    };
+    auto load_x = [&](int tk) {
+#pragma unroll
+      for (int hl = 0; hl < 2; ++hl) tmem_ld_16x256b_x2(tq + hl * hi + Cfg::TM_X + tk, x[hl]);
+    };
+    if (trans) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) vv[i >> 2][i & 3] = 0u;
+    }
+    for (int c = 0; c < nsteps; ++c) {
+      if (c == nsteps - kTailSteps) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      HA_PROF(walk, 8 * c + 0);
+      wait1(&full_sc[c & 1], c >> 1);
+      // GDN: e^{G_t}[128], e^{G_L-G_t}[128]; KDA: e^{G_L} per key
+      const float* sc = reinterpret_cast<const float*>(sm + Cfg::OFF_SC + (c & 1) * kStepScB);
+      if (!trans) {
+        wait1(full_v, c);
+        load_v(16 * g);
+      }
+      wait1(bar_x, c);
+      HA_PROF(walk, 8 * c + 1);
+      tc_fence_after_sync();
+      load_x(16 * g);
+      if (KDA && OUT && c > 0) wait1(bar_o, c - 1);      // P U~ of the previous step has read its operand there
+      // ---- R^T = V^T - e^{G_j} X^T, in fragment layout
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const int tk = 64 * half + 16 * g;
+        float2 e[2];                                     // -e^{G_j} of tokens tk + 8 k + t2, + 1
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          e[k] = make_float2(-1.f, -1.f);
+          if (!KDA) {
+            const float2 f = *reinterpret_cast<const float2*>(sc + tk + 8 * k + t2);
+            e[k] = make_float2(-f.x, -f.y);
+          }
+        }
+        tmem_ld_wait();
+#pragma unroll
+        for (int hl = 0; hl < 2; ++hl) {
+          uint32_t w[4];
+#pragma unroll
+          for (int y = 0; y < 2; ++y)                    // rows g8, g8 + 8
+#pragma unroll
+            for (int k = 0; k < 2; ++k)                  // tokens 8 k + t2, + 1; columns in step_pos order
+              w[2 * y + k] = pack_bf16(fma2(e[k], as_f2(x[hl][4 * k + 2 * y], x[hl][4 * k + 2 * y + 1]), unpack_bf16(vv[hl][2 * k + y])));
+          tmem_st_16x256b_x1(tq + hl * hi + Cfg::TM_R + tk / 2, w);
+        }
+        tmem_st_wait();
+        tc_fence_before_sync();
+        named_arrive(BAR_R + half, kCompute + 32);
+        if (half == 0) {
+          load_x(64 + 16 * g);
+          if (!trans) load_v(64 + 16 * g);
+        }
+        HA_PROF(walk, 8 * c + 2);
+      }
+      __syncwarp();
+      if (!trans && lane == 0) mbar_arrive(empty_v);
+
+      // ---- U~^T as operands.  GDN: times e^{G_L-G_t} for the state update, and plain for the outputs, over columns of U
+      // that this warp has read already (columns in step_pos order).  KDA: the latter for both.
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const int tk = 64 * half + 16 * g;
+        float4 e[4];                                     // e^{G_L-G_t}
+        if (!KDA) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) e[k] = *reinterpret_cast<const float4*>(sc + 128 + tk + 4 * k);
+        }
+        wait1(half ? bar_u1 : bar_u0, c);
+        HA_PROF(walk, 8 * c + 3);
+        tc_fence_after_sync();
+        uint32_t u[16], w[8];
+        tmem_ld16(tq + Cfg::TM_U + tk, u);
+        tmem_ld_wait();
+        if constexpr (!KDA) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            w[2 * k] = pack_bf16(mul2(as_f2(u[4 * k], u[4 * k + 1]), make_float2(e[k].x, e[k].y)));
+            w[2 * k + 1] = pack_bf16(mul2(as_f2(u[4 * k + 2], u[4 * k + 3]), make_float2(e[k].z, e[k].w)));
+          }
+          tmem_st8(tq + Cfg::TM_R + tk / 2, w);
+          tmem_st_wait();
+          tc_fence_before_sync();
+          named_arrive(BAR_U + half, kCompute + 32);
+        }
+        if constexpr (KDA || OUT) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            w[2 * k] = pack_bf16(__uint_as_float(u[2 * k]), __uint_as_float(u[2 * k + 1]));
+            w[2 * k + 1] = pack_bf16(__uint_as_float(u[8 + 2 * k]), __uint_as_float(u[9 + 2 * k]));
+          }
+          tmem_st8(tq + (KDA ? Cfg::TM_R + tk / 2 : Cfg::TM_UP + tk), w);
+          if (KDA) {
+            tmem_st_wait();
+            tc_fence_before_sync();
+            named_arrive(BAR_U + half, kCompute + 32);
+          }
+        }
+        HA_PROF(walk, 8 * c + 4);
+      }
+
+      if (OUT) wait1(bar_y, c);
+      if constexpr (OUT && !KDA) {                       // Y <- scale e^{G_i} Y in place while D2 runs; then (scale P) U~ is added to it
+        tc_fence_after_sync();
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const int tk = 64 * half + 16 * g;
+#pragma unroll
+          for (int hl = 0; hl < 2; ++hl) tmem_ld_16x256b_x2(tq + hl * hi + Cfg::TM_Y + tk, x[hl]);
+          float2 e[2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) e[k] = mul2(*reinterpret_cast<const float2*>(sc + tk + 8 * k + t2), make_float2(p.scale, p.scale));
+          tmem_ld_wait();
+#pragma unroll
+          for (int hl = 0; hl < 2; ++hl) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float2 y = mul2(as_f2(x[hl][2 * k], x[hl][2 * k + 1]), e[k >> 1]);
+              x[hl][2 * k] = __float_as_uint(y.x);
+              x[hl][2 * k + 1] = __float_as_uint(y.y);
+            }
+            tmem_st_16x256b_x2(tq + hl * hi + Cfg::TM_Y + tk, x[hl]);
+          }
+        }
+        tmem_st_wait();
+        tc_fence_before_sync();
+        named_arrive(BAR_UP, kCompute + 32);
+      }
+      wait1(bar_d2, c);
+      HA_PROF(walk, 8 * c + 5);
+      tc_fence_after_sync();
+      // ---- h^T <- decay h^T + D2
+      {
+        uint32_t d[32];
+        tmem_ld32(tq + Cfg::TM_X + 32 * g, d);
+        tmem_ld_wait();
+        if constexpr (KDA) {
+#pragma unroll
+          for (int k = 0; k < 32; k += 4) {
+            const float4 gm = *reinterpret_cast<const float4*>(sc + 32 * g + k);   // decay per key channel
+            step_h(k, make_float2(gm.x, gm.y), as_f2(d[k], d[k + 1]));
+            step_h(k + 2, make_float2(gm.z, gm.w), as_f2(d[k + 2], d[k + 3]));
+          }
+        } else {
+          const float gm = sc[127];                      // one decay for the whole step
+#pragma unroll
+          for (int k = 0; k < 32; k += 2) step_h(k, make_float2(gm, gm), as_f2(d[k], d[k + 1]));
+        }
+      }
+      store_h();                                         // (Y has read the old operand)
+      tc_fence_before_sync();
+      named_arrive(BAR_H, kCompute + 32);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty_sc[c & 1]);
+      HA_PROF(walk, 8 * c + 6);
+    }
+
+    // where the end state goes: hT (from the last span), or the span's offset b_s / transition Phi_s
+    float* dst = nullptr;
+    if (!OUT) dst = (trans ? p.span_phi : p.span_b) + (((size_t)n * p.HV + j) * p.nspan + span) * 16384;
+    else if (p.hT && span == p.nspan - 1) dst = p.hT + ((size_t)n * p.HV + j) * 16384;
+    if (dst) {
+#pragma unroll
+      for (int k = 0; k < 32; ++k) dst[(size_t)(32 * g + k) * 128 + v] = h[k];
+    }
+  }
+
+  tc_fence_before_sync();
+  __syncthreads();
+  if (*abort_flag) {
+    // A wait ran out: the producers have stopped; give copies that were still in flight time to land.
+    if (tid == 0) report_status(p.status, HA_LA_ERR_TIMEOUT);
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+  }
+  // Concurrent mode: do not finish before the prep grid has (it has published its last step by now), so that
+  // work queued behind this kernel is also behind the prep kernel.
+  if (p.epoch != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (warp == 0) tmem_dealloc(*tmem_slot, 512);
+}
+
+template <bool KDA, bool OUT>
+cudaError_t run_walk(const WalkParams* wp, const CUtensorMap* mk, const CUtensorMap* mq, const CUtensorMap* mv, int grid,
+                     bool dependent, cudaStream_t stream) {
+  auto kern = tc_walk_kernel<KDA, OUT>;
+  constexpr int smem = WalkCfg::kSmem;
+  if (!wp) {                                             // configure only (this also loads the kernel)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  }
+  timer_mark(stream, OUT ? "tc_chain" : "tc_span");
+  // `dependent`: programmatic dependent launch behind the kernel before it (same stream): the CTAs may start as soon
+  // as every CTA of that one is running, instead of after its grid has drained.
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(walk_threads(OUT));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, *mk, *mq, *mv, *wp);
+}
+
+}  // namespace
+
+// `states_only`: the first of the two launches of a call whose sequences are cut into spans.
+cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
+                           const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, int64_t epoch,
+                           bool dependent, uint32_t spin_limit, const SpanBuffers& sb, bool states_only,
+                           cudaStream_t stream) {
+  WalkParams wp;
+  wp.h0 = a.h0; wp.hT = a.hT; wp.o = a.o;
+  wp.seq_tok0 = plan.seq_tok0; wp.seq_len = plan.seq_len; wp.seq_chunk0 = plan.seq_chunk0;
+  wp.seq_order = plan.seq_tok0 ? plan.seq_order : nullptr;
+  wp.T_row = p.T_row; wp.cps = p.max_seq_chunks > 0 ? p.max_seq_chunks : 1;
+  wp.ws = ws; wp.HK = p.HK; wp.HV = p.HV; wp.scale = p.scale; wp.status = a.status_word;
+  wp.epoch = epoch;
+  wp.spin_limit = spin_limit;
+  wp.nspan = sb.nspan; wp.span_b = sb.b; wp.span_phi = sb.phi;
+  const int grid = p.N * p.HV * (states_only ? 2 * sb.nspan - 3 : sb.nspan);
+  if (grid == 0) return cudaSuccess;
+  const bool kda = p.variant == HA_LA_KDA;
+  if (states_only) return kda ? run_walk<true, false>(&wp, &mk, &mq, &mv, grid, dependent, stream)
+                              : run_walk<false, false>(&wp, &mk, &mq, &mv, grid, dependent, stream);
+  return kda ? run_walk<true, true>(&wp, &mk, &mq, &mv, grid, dependent, stream)
+             : run_walk<false, true>(&wp, &mk, &mq, &mv, grid, dependent, stream);
+}
+
+// Attributes (and loading) of the instances a launch can use.
+cudaError_t configure_tc_walk(const Problem& p) {
+  const bool kda = p.variant == HA_LA_KDA;
+  cudaError_t e = kda ? run_walk<true, false>(nullptr, nullptr, nullptr, nullptr, 0, false, nullptr)
+                      : run_walk<false, false>(nullptr, nullptr, nullptr, nullptr, 0, false, nullptr);
+  if (e != cudaSuccess) return e;
+  return kda ? run_walk<true, true>(nullptr, nullptr, nullptr, nullptr, 0, false, nullptr)
+             : run_walk<false, true>(nullptr, nullptr, nullptr, nullptr, 0, false, nullptr);
+}
+
+}  // namespace ha_la
