@@ -151,9 +151,10 @@ int forced_segments() {
 
 // Spans per sequence of the step path (tc_walk.cu): with few (sequence, head) pairs a sequence is cut into S runs that
 // are walked at the same time, in two launches, 2 S - 3 state-only runs and then S runs with outputs, with S - 2
-// products of 128^3 between them.  Costs measured on B200: 2.0 us per state-only step, 2.45 per step with outputs, 1.25
-// per product and about 8 for the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack
-// (the longest first) to within some 15 %.
+// products of 128^3 between them.  Costs measured on B200: 2.0 us per state-only step, 2.45 per step with outputs, 5 for
+// a CTA's start and end, 1.25 per product (5 when the products' 8 CTAs per pair do not all have an SM) and about 8 for
+// the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
+// within some 15 %.
 int plan_spans(const Problem& p) {
   const long long chains = (long long)p.N * p.HV;
   const int sms = sm_count(), longest = (p.max_len + kStep - 1) / kStep;
@@ -163,15 +164,15 @@ int plan_spans(const Problem& p) {
   auto launch_us = [&](int runs, int spans, double step_us) {
     const int cps = (longest + spans - 1) / spans;
     const long long ctas = chains * runs;
-    if (ctas <= sms) return cps * step_us;
-    if (even) return cps * step_us * (double)((ctas + sms - 1) / sms);
+    if (ctas <= sms) return cps * step_us + 5.0;
+    if (even) return (cps * step_us + 5.0) * (double)((ctas + sms - 1) / sms);
     const double spread = 1.15 * total * runs / spans / sms;
-    return (spread > cps ? spread : cps) * step_us;
+    return (spread > cps ? spread : cps) * step_us + 5.0 * (double)ctas / sms;
   };
   int best_s = 1;
   double best = launch_us(1, 1, 2.45);
   for (int S = 2; S <= 32 && S <= longest; ++S) {
-    const double t = launch_us(2 * S - 3, S, 2.0) + launch_us(S, S, 2.45) + 1.25 * (S - 2) + 8.0;
+    const double t = launch_us(2 * S - 3, S, 2.0) + launch_us(S, S, 2.45) + (8 * chains <= sms ? 1.25 : 5.0) * (S - 2) + 8.0;
     if (t < best) { best = t; best_s = S; }
   }
   return best_s;
