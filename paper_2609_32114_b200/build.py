@@ -26,8 +26,8 @@ TORCH_CALL = os.path.join(PKG, "ha_la_torch_call.so")   # binding.py's native ha
 INCLUDE = os.path.join(ROOT, "include")
 
 # (object name, source, extra flags)
-UNITS = [("api", "api.cu", []), ("plan", "plan.cu", []), ("tc", "tc.cu", []), ("tc_prep", "tc_prep.cu", []), ("tc_chain", "tc_chain.cu", []), ("tc_seg", "tc_seg.cu", []),
-         ("tc_tp", "tc_tp.cu", []), ("tc_walk", "tc_walk.cu", []), ("tc_span", "tc_span.cu", []),
+UNITS = [("api", "api.cu", []), ("plan", "plan.cu", []), ("tc", "tc.cu", []), ("tc_tp", "tc_tp.cu", []), ("tc_kda", "tc_kda.cu", []),
+         ("tc_walk", "tc_walk.cu", []), ("tc_span", "tc_span.cu", []),
          ("noalloc", "noalloc.cu", []), ("decode", "decode.cu", [])] + [
     (f"simt{u}", "simt.cu", [f"-DHA_LA_SIMT_UNIT={u}"]) for u in range(5)
 ] + [

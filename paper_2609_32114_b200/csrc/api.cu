@@ -52,7 +52,7 @@ int make_problem(const ha_la_prefill_args* a, Problem* p) {
   p->dv = a->d_v;
   p->scale = a->scale;
   p->varlen = varlen ? 1 : 0;
-  p->step = use_tc(*p) && p->variant == HA_LA_GDN ? 128 : kChunk;
+  p->step = use_tc(*p) ? 128 : kChunk;
   if (varlen) {
     p->max_len = (a->max_seqlen > 0 && a->max_seqlen < a->seqlen) ? a->max_seqlen : a->seqlen;
     p->max_chunks = (int)(((long long)p->T_total + (p->step - 1LL) * p->N) / p->step);

@@ -1,15 +1,8 @@
-// Tensor-core (tcgen05) path, host side: tensor maps, workspace carving, slice-width choice, launches.
+// Tensor-core (tcgen05) path, host side: tensor maps, workspace carving, spans, launches.
 //
-// Both kernels go on the caller's stream; the chain kernel is launched as a programmatic dependent of the
-// prep kernel, so it may start once every prep CTA is running.  Two modes:
-//   sequential: the chain kernel sets itself up under the prep kernel's tail and then waits for that whole grid;
-//   concurrent: when the chain CTAs need at most half of the SMs and the cost model below expects a gain, the
-//     prep kernel is sized to the other SMs
-//     (one CTA per SM) and the chain kernel consumes each chunk as soon as the prep work group of that chunk
-//     has published it (release/acquire flag per chunk in the workspace, stamped with a per-call epoch so that
-//     nothing has to be cleared).  The flags' producer is running (or done) before a consumer starts, whatever
-//     else the GPU is doing, so the consumer's bounded waits cannot starve.
-// HA_LA_TC_OVERLAP=0 forces the sequential mode, =2 the concurrent one wherever it is legal.
+// The chunk-local kernel (tc_tp.cu, KDA: tc_kda.cu) and the state-passing kernel (tc_walk.cu) go on the caller's stream one
+// behind the other, both in steps of 128 tokens; where sequences are cut into spans, the latter runs twice with the spans'
+// start states (tc_span.cu) between.  Each is a programmatic dependent of the one before: it is set up under its tail.
 #include <cuda.h>
 #include <stdlib.h>
 
@@ -20,17 +13,10 @@
 
 namespace ha_la {
 
-cudaError_t launch_tc_prep(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                           const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, int64_t epoch,
-                           int reserved_sms, cudaStream_t stream);
-cudaError_t launch_tc_chain(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                            const CUtensorMap& mk, const CUtensorMap& mo, int nv, int64_t epoch, bool dependent,
-                            uint32_t spin_limit, const SegBuffers& sg, cudaStream_t stream);
-cudaError_t launch_tc_seg_fix(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const SegBuffers& sg,
-                              cudaStream_t stream);
-
 cudaError_t launch_tc_tp(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                         const CUtensorMap& mq, const CUtensorMap& mk, int64_t epoch, int ctas, cudaStream_t stream);
+                         const CUtensorMap& mq, const CUtensorMap& mk, int ctas, cudaStream_t stream);
+cudaError_t launch_tc_kda(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
+                          const CUtensorMap& mq, const CUtensorMap& mk, int ctas, cudaStream_t stream);
 cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
                            const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, int64_t epoch,
                            bool dependent, uint32_t spin_limit, const SpanBuffers& sb, bool states_only,
@@ -39,8 +25,7 @@ cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& 
 cudaError_t configure_span_fix();
 cudaError_t configure_tc_tp();
 cudaError_t configure_tc_walk(const Problem& p);
-cudaError_t configure_tc_prep(const Problem& p);
-cudaError_t configure_tc_chain(const Problem& p, int nv);
+cudaError_t configure_tc_kda();
 
 namespace {
 
@@ -59,21 +44,7 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// [T][H][128] bf16 token-major tensor; box = 64 features x 1 head x 64 tokens, 128-byte swizzle.
-// The innermost coordinate of every load is 0 or 64 elements (a multiple of 16 bytes).
-bool make_map(CUtensorMap* m, const void* base, int T, int H) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return false;
-  const cuuint64_t dims[3] = {128, (cuuint64_t)H, (cuuint64_t)(T > 0 ? T : 1)};
-  const cuuint64_t strides[2] = {128 * 2, (cuuint64_t)H * 128 * 2};
-  const cuuint32_t box[3] = {64, 1, 64};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// The same tensor in tiles of 128 features x 1 head x 128 tokens, as two 64-feature halves of 128-byte rows one after the
+// [T][H][128] bf16 token-major tensor, in tiles of 128 features x 1 head x 128 tokens, as two 64-feature halves of 128-byte rows one after the
 // other ([kb][128 tok][64 feat], 128-byte swizzle): the feature halves are the outermost dimension of the map.
 bool make_map_tile(CUtensorMap* m, const void* base, int T, int H) {
   EncodeTiledFn enc = encode_fn();
@@ -85,20 +56,6 @@ bool make_map_tile(CUtensorMap* m, const void* base, int T, int H) {
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// The output o as the chain kernel stores it: box = one slice block (nv <= 64 channels) x 1 head x 64 tokens,
-// swizzled like the kernel's staging tile.  Store coordinates are multiples of 32 channels (64 bytes).
-bool make_map_o(CUtensorMap* m, const void* base, int T, int H, int nv) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return false;
-  const cuuint64_t dims[3] = {128, (cuuint64_t)H, (cuuint64_t)(T > 0 ? T : 1)};
-  const cuuint64_t strides[2] = {128 * 2, (cuuint64_t)H * 128 * 2};
-  const cuuint32_t box[3] = {(cuuint32_t)(nv < 64 ? nv : 64), 1, 64};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, nv < 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int sm_count() {
@@ -264,13 +221,11 @@ bool tc_supported(const Problem& p) {
   return p.dtype == HA_LA_BF16 && p.dk == 128 && p.dv == 128;
 }
 
-// Images or step records, the scratch of the planned spans (GDN), and, when the planner cuts the sequences into segments,
-// the segment scratch for that many.  (The call
-// checks the caller's size against this same function, so an environment switch that is changed between sizing and
-// calling ends in HA_LA_ERR_WORKSPACE, not in an overrun.)
+// Step records (and images), the scratch of the planned spans, and, when the planner below cuts the sequences into segments,
+// the segment scratch for that many.  (The call checks the caller's size against this same function, so an environment
+// switch that is changed between sizing and calling ends in HA_LA_ERR_WORKSPACE, not in an overrun.)
 static size_t tc_base_bytes(const Problem& p) {
-  const bool kda = p.variant == HA_LA_KDA;
-  return tc_ws_bytes_for((size_t)p.max_chunks * p.HV, kda) + (kda ? 0 : tc_span_bytes((size_t)p.N * p.HV, plan_spans(p)));
+  return tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA) + tc_span_bytes((size_t)p.N * p.HV, plan_spans(p));
 }
 
 size_t tc_workspace_bytes(const Problem& p) {
@@ -278,18 +233,17 @@ size_t tc_workspace_bytes(const Problem& p) {
 }
 
 // HA_LA_TC_SEGMENTS forces the spans too (1: none); their scratch is then the segment scratch, which is larger.
-static SpanBuffers gdn_spans(const Problem& p, const TcPlan& tp, void* tc_ws) {
+static SpanBuffers call_spans(const Problem& p, const TcPlan& tp, void* tc_ws) {
   uint8_t* b = reinterpret_cast<uint8_t*>(tc_ws);
   const size_t nj = (size_t)p.N * p.HV;
   const int forced = forced_segments();
   if (forced == 1) return tc_span_view(nullptr, nj, 1);
   if (forced > 1 && tp.nseg > 1) return tc_span_view(b + tc_base_bytes(p), nj, tp.nseg);
-  return tc_span_view(b + tc_ws_bytes_for((size_t)p.max_chunks * p.HV, false), nj, plan_spans(p));
+  return tc_span_view(b + tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA), nj, plan_spans(p));
 }
 
 int tc_num_launches(const Problem& p) {
   const int nseg = plan_tc(p).nseg;
-  if (p.variant == HA_LA_KDA) return nseg > 1 ? 4 : 2;
   const int forced = forced_segments();
   return (forced == 1 ? 1 : forced > 1 && nseg > 1 ? nseg : plan_spans(p)) > 1 ? 4 : 2;
 }
@@ -302,116 +256,48 @@ void tc_launch_plan(const Problem& p, int* slice_width, int* concurrent) {
   *concurrent = tp.concurrent ? 1 : 0;
 }
 
-static cudaError_t launch_tc_gdn(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                                 const SpanBuffers& sb, cudaStream_t stream) {
+cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* tc_ws, cudaStream_t stream) {
+  const bool kda = p.variant == HA_LA_KDA;
+  const TcWorkspace ws = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, kda);
+  const SpanBuffers sb = call_spans(p, plan_tc(p), tc_ws);
   CUtensorMap mq, mk, mv;
   if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk, a.k, p.T_total, p.HK) ||
       !make_map_tile(&mv, a.v, p.T_total, p.HV))
     return cudaErrorInvalidValue;
+  // Once per device: the attributes stick, and the calls are not free on the host.
   static std::atomic<uint32_t> configured[kMaxDevices];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-  const uint32_t bit = 1u << (p.variant == HA_LA_KDA ? 1 : 0);
+  const uint32_t bit = kda ? 2u : 1u;
   if (dev < 0 || dev >= kMaxDevices || !(configured[dev].load() & bit)) {
-    cudaError_t ce = configure_tc_tp();
-    if (ce != cudaSuccess) return ce;
-    ce = configure_tc_walk(p);
-    if (ce != cudaSuccess) return ce;
-    ce = configure_span_fix();
+    cudaError_t ce = kda ? configure_tc_kda() : configure_tc_tp();
+    if (ce == cudaSuccess) ce = configure_tc_walk(p);
+    if (ce == cudaSuccess) ce = configure_span_fix();
     if (ce != cudaSuccess) return ce;
     if (dev >= 0 && dev < kMaxDevices) configured[dev].fetch_or(bit);
   }
-  const bool dependent = g_timer == nullptr;
-  cudaError_t e = launch_tc_tp(p, a, plan, ws, mq, mk, 0, sm_count(), stream);
-  if (e != cudaSuccess) return e;
-  if (sb.nspan > 1) {
+  const bool dependent = g_timer == nullptr;             // (per-kernel timing wants one kernel at a time)
+  cudaError_t e = kda ? launch_tc_kda(p, a, plan, ws, mq, mk, sm_count(), stream) : launch_tc_tp(p, a, plan, ws, mq, mk, sm_count(), stream);
+  if (e == cudaSuccess && sb.nspan > 1) {
     e = launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, true, stream);
-    if (e != cudaSuccess) return e;
-    e = launch_span_fix(p, plan, sb, a.status_word, stream);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = launch_span_fix(p, plan, sb, a.status_word, stream);
   }
-  return launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, false, stream);
+  return e != cudaSuccess ? e : launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, false, stream);
 }
 
-cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* tc_ws, cudaStream_t stream) {
-  const TcPlan tp = plan_tc(p);
-  if (p.variant != HA_LA_KDA)
-    return launch_tc_gdn(p, a, plan, tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, false), gdn_spans(p, tp, tc_ws), stream);
-  const int nv = tp.nv;
-  CUtensorMap mq, mk, mv, mo;
-  if (!make_map(&mq, a.q, p.T_total, p.HK) || !make_map(&mk, a.k, p.T_total, p.HK) ||
-      !make_map(&mv, a.v, p.T_total, p.HV) || !make_map_o(&mo, a.o, p.T_total, p.HV, nv))
-    return cudaErrorInvalidValue;
-  const size_t ncj = (size_t)p.max_chunks * p.HV;
-  const TcWorkspace ws = tc_ws_view(tc_ws, ncj, p.variant == HA_LA_KDA);
-  const SegBuffers sg = tc_seg_view(reinterpret_cast<uint8_t*>(tc_ws) + tc_ws_bytes_for(ncj, p.variant == HA_LA_KDA),
-                                    (size_t)p.N * p.HV, tp.nseg, (size_t)p.T_total, p.HV);
-  const bool concurrent = tp.concurrent && !g_timer;     // (per-kernel timing wants one kernel at a time)
-  // Configure (and load) both kernels before anything is enqueued: loading a kernel for the first time can
-  // wait for the device, and in the concurrent mode the chain kernel would be spinning meanwhile.
-  // (Once per device and kernel instance: the attributes stick, and the calls are not free on the host.)
-  static std::atomic<uint32_t> configured[kMaxDevices];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-  const uint32_t bit = 1u << ((p.variant == HA_LA_KDA ? 3 : 0) + (nv == 32 ? 0 : (nv == 64 ? 1 : 2)));
-  if (dev < 0 || dev >= kMaxDevices || !(configured[dev].load() & bit)) {
-    cudaError_t ce = configure_tc_prep(p);
-    if (ce != cudaSuccess) return ce;
-    ce = configure_tc_chain(p, nv);
-    if (ce != cudaSuccess) return ce;
-    if (dev >= 0 && dev < kMaxDevices) configured[dev].fetch_or(bit);
-  }
-  int64_t epoch = 0;                                     // 0 means "sequential"
-  int reserved_sms = 0;
-  if (concurrent) {
-    epoch = next_epoch();
-    reserved_sms = p.N * p.HV * (128 / nv);              // a chain CTA fills its SM
-  }
-  if (concurrent) {
-    // A call captured into a CUDA graph is replayed with the epoch it was captured with, and the flags its last
-    // replay left behind carry exactly that epoch: the chain kernel would run ahead of the prep kernel on stale
-    // images.  Under capture the flags are therefore cleared first (a memset node, replayed with the rest).
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) {
-      (void)cudaGetLastError();
-      cs = cudaStreamCaptureStatusNone;
-    }
-    if (cs == cudaStreamCaptureStatusActive) {
-      const cudaError_t me = cudaMemsetAsync(ws.flags, 0, ncj * sizeof(int64_t), stream);
-      if (me != cudaSuccess) return me;
-    }
-  }
-  cudaError_t e = launch_tc_prep(p, a, plan, ws, mq, mk, mv, epoch, reserved_sms, stream);
-  if (e != cudaSuccess) return e;
-  e = launch_tc_chain(p, a, plan, ws, mk, mo, nv, epoch, /*dependent=*/g_timer == nullptr, kDefaultSpinLimit, sg, stream);
-  if (e != cudaSuccess) return e;
-  return launch_tc_seg_fix(p, a, plan, sg, stream);
-}
-
-// Test hook behind ha_la_debug_wait_timeout: the sequential kernel alone, in the concurrent mode, with an epoch that
-// nothing will ever publish and a small poll limit.  Its first flag wait runs out, it records the time-out, and then
-// walks the chunks on whatever the workspace holds (valid memory, meaningless numbers) to a normal exit.
+// Test hook behind ha_la_debug_wait_timeout: the state-passing kernel alone, waiting for steps to be published, with an
+// epoch that nothing will ever publish and a small poll limit.  Its first flag wait runs out, it records the time-out, and
+// runs its barriers to a normal exit.
 cudaError_t launch_tc_chain_unpublished(const Problem& p, const ha_la_prefill_args& a, void* tc_ws, uint32_t spin_limit,
                                         cudaStream_t stream) {
-  const int nv = 32;
-  if (p.variant != HA_LA_KDA) {
-    CUtensorMap mq, mk2, mv;
-    if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk2, a.k, p.T_total, p.HK) ||
-        !make_map_tile(&mv, a.v, p.T_total, p.HV))
-      return cudaErrorInvalidValue;
-    const TcWorkspace w = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, false);
-    cudaError_t ce2 = configure_tc_walk(p);
-    if (ce2 != cudaSuccess) return ce2;
-    return launch_tc_walk(p, a, PlanView{}, w, mk2, mq, mv, next_epoch(), false, spin_limit,
-                          SpanBuffers{1, nullptr, nullptr}, false, stream);
-  }
-  CUtensorMap mk, mo;
-  if (!make_map(&mk, a.k, p.T_total, p.HK) || !make_map_o(&mo, a.o, p.T_total, p.HV, nv)) return cudaErrorInvalidValue;
+  CUtensorMap mq, mk, mv;
+  if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk, a.k, p.T_total, p.HK) ||
+      !make_map_tile(&mv, a.v, p.T_total, p.HV))
+    return cudaErrorInvalidValue;
   const TcWorkspace ws = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA);
-  cudaError_t ce = configure_tc_chain(p, nv);
-  if (ce != cudaSuccess) return ce;
-  return launch_tc_chain(p, a, PlanView{}, ws, mk, mo, nv, next_epoch(), /*dependent=*/false, spin_limit,
-                         SegBuffers{1, nullptr, nullptr, nullptr, nullptr}, stream);
+  cudaError_t e = configure_tc_walk(p);
+  if (e != cudaSuccess) return e;
+  return launch_tc_walk(p, a, PlanView{}, ws, mk, mq, mv, next_epoch(), false, spin_limit, SpanBuffers{1, nullptr, nullptr}, false, stream);
 }
 
 }  // namespace ha_la

@@ -18,8 +18,8 @@
 // The contraction runs on warp-level MMAs: 36 pairs of blocks of the 64, no work above the diagonal, no operand copies
 // per pair; it is a fifth of the kernel's instructions.
 //
-// Measured on B200 with 32 heads and 8192 tokens: 262 us before (64-token chunks, a copy of the operands per block row,
-// one item at a time per SM).
+// Measured on B200 with 32 heads and 8192 tokens: 162 us; with 64-token chunks, a copy of the operands per block row and
+// one item at a time per SM it was 262 us.
 //
 // Tokens past the end of a sequence are made no-ops by beta = 0 and g = 0; whatever the TMA box read for them (the
 // next sequence's rows, or zero fill past the end of the tensor) is multiplied by exact zeros.  This relies on the
@@ -47,8 +47,8 @@ constexpr uint32_t OFF_D = OFF_A + 28 * 512;               // fp32 diagonal bloc
 constexpr uint32_t OFF_TOT = OFF_D + 8 * 16 * LDD * 4;     // float [8][128]: log2 decay of each block
 constexpr uint32_t OFF_DN = OFF_TOT + 4096;                // per buffer: bf16 [8][128], 2^{rho_{J+1}-rho_J}
 constexpr uint32_t OFF_BETA = OFF_DN + 2 * 2048;           // per buffer: float [128]
-constexpr uint32_t OFF_FALL = OFF_BETA + 2 * 512;          // per buffer: int [8], block needs the evaluation entry by entry
-constexpr uint32_t OFF_BAR = OFF_FALL + 2 * 32;
+constexpr uint32_t OFF_FALL = OFF_BETA + 2 * 512;          // per buffer: int [8][2] (channel halves), block needs the evaluation entry by entry
+constexpr uint32_t OFF_BAR = OFF_FALL + 2 * 64;
 constexpr uint32_t kKdaSmem = OFF_BAR + 32;
 static_assert(kKdaSmem <= 227 * 1024, "shared memory budget");
 constexpr float kMaxUp = 100.f;
@@ -77,31 +77,30 @@ __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
 __device__ __forceinline__ uint32_t pow2_bf16(float e) { return static_cast<uint32_t>(min(max(static_cast<int>(e) + 127, 0), 254)) << 7; }
 __device__ __forceinline__ uint32_t pow2_pair(float2 e) { return pow2_bf16(e.x) | (pow2_bf16(e.y) << 16); }
 
-// Diagonal block I of A (fp32, times beta) and P, entry by entry, by one warp: lane l has channels 4 l .. 4 l + 3.
-__device__ __noinline__ void slow_diagonal(const KdaParams& p, int j, int jq, int tok0, int L, int I, const float* sBeta, float* sd,
-                                           float (&pd)[2][4], int lane) {
-  const int g8 = lane >> 2, t2 = (lane & 3) * 2;
+// Diagonal block I of A (fp32, times beta) and scale P (to its operand dst), entry by entry, by one warp: lane l has
+// channels 4 l .. 4 l + 3.  (k, q, g: the head's first channel of the step's first token; token strides sk, sg.)
+__device__ __noinline__ void slow_diagonal(const __nv_bfloat16* k, const __nv_bfloat16* q, size_t sk, const float* g, size_t sg,
+                                           int L, int I, const float* sBeta, float* sd, uint8_t* dst, float scale, int lane) {
   for (int i = 0; i < 16; ++i) {
     const int ti = 16 * I + i;
     float kv[4] = {}, qv[4] = {}, w[4] = {1.f, 1.f, 1.f, 1.f};
     if (ti < L) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const size_t a = ((size_t)(tok0 + ti) * p.HK + jq) * 128 + 4 * lane + c;
-        kv[c] = __bfloat162float(p.k[a]);
-        qv[c] = __bfloat162float(p.q[a]);
+        kv[c] = __bfloat162float(k[ti * sk + 4 * lane + c]);
+        qv[c] = __bfloat162float(q[ti * sk + 4 * lane + c]);
       }
     }
-    for (int jj = i; jj >= 0; --jj) {
+    for (int jj = 15; jj >= 0; --jj) {
       const int tj = 16 * I + jj;
       float a = 0.f, b = 0.f;
-      if (ti < L) {
+      if (ti < L && jj <= i) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const float x = __bfloat162float(p.k[((size_t)(tok0 + tj) * p.HK + jq) * 128 + 4 * lane + c]) * w[c];
+          const float x = __bfloat162float(k[tj * sk + 4 * lane + c]) * w[c];
           a = fmaf(kv[c], x, a);
           b = fmaf(qv[c], x, b);
-          w[c] *= __expf(p.g[((size_t)(tok0 + tj) * p.HV + j) * 128 + 4 * lane + c]);   // decay from tj - 1 to i
+          w[c] *= __expf(g[tj * sg + 4 * lane + c]);     // decay from tj - 1 to i
         }
       }
 #pragma unroll
@@ -109,12 +108,12 @@ __device__ __noinline__ void slow_diagonal(const KdaParams& p, int j, int jq, in
         a += __shfl_xor_sync(0xffffffffu, a, o);
         b += __shfl_xor_sync(0xffffffffu, b, o);
       }
-      if (lane == 0) sd[i * LDD + jj] = jj < i ? a * sBeta[ti] : 0.f;
-#pragma unroll
-      for (int n = 0; n < 2; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (i == g8 + (e >> 1) * 8 && jj == 8 * n + t2 + (e & 1)) pd[n][e] = b;
+      if (lane == 0) {
+        sd[i * LDD + jj] = jj < i ? a * sBeta[ti] : 0.f;
+        const int t = (jj & 7) >> 1;                     // (store_tri_block's place for column jj)
+        *reinterpret_cast<__nv_bfloat16*>(dst + tri_row(ti, I) + (((t >> 1) ^ ((i & 7) >> 2)) << 4) + (t & 1) * 8 + (jj >> 3) * 4 + (jj & 1) * 2) =
+            __float2bfloat16_rn(scale * b);
+      }
     }
   }
 }
@@ -172,7 +171,11 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     const uint32_t o0 = kb * 16384 + ((lane & 3) << 2), ch = (lane >> 2) << 4;
     float* sTot = reinterpret_cast<float*>(sm + OFF_TOT);
     Geom gm = geom(blockIdx.x);
-    if (tid == 256 && gm.L > 0) issue_tiles(gm, 0);
+    if (tid == 256 && gm.L > 0) {                        // (later tiles are issued by the solving warps)
+      issue_tiles(gm, 0);
+      const Geom g1 = geom(blockIdx.x + stride);
+      if (g1.L > 0) issue_tiles(g1, 1);
+    }
     long long it = 0;
     for (long long item = blockIdx.x; gm.L > 0; ++it) {
       const int b = (int)(it & 1);
@@ -219,6 +222,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
 #pragma unroll
       for (int i = 0; i < 3; ++i) rho[i] = make_float2(rintf(B[i].x), rintf(B[i].y));
       if (it > 1) sync(3 + b);                           // the solving warps are done with the item two before
+      else sync_half(5);                                 // (either way: the totals have been read)
       mbar_wait(&full[b], (uint32_t)(it >> 1) & 1, abort_flag);
       uint8_t* buf = sm + b * kBufBytes;
       if (tg < 2) reinterpret_cast<float*>(sm + OFF_BETA + b * 512)[w * 32 + lane] = bt;
@@ -230,9 +234,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         const float2 dn = make_float2(rho[u + 1].x - rho[u].x, rho[u + 1].y - rho[u].y);
         *reinterpret_cast<uint32_t*>(sm + OFF_DN + b * 2048 + I * 256 + cp * 2) = pow2_pair(dn);
         const bool far = __any_sync(0xffffffffu, dn.x < -kMaxUp || dn.y < -kMaxUp);
-        if (lane == 0) reinterpret_cast<int*>(sm + OFF_FALL + b * 32)[I] = 0;
-        __syncwarp();
-        (void)far;
+        if (lane == 0) reinterpret_cast<int*>(sm + OFF_FALL + b * 64)[2 * I + kb] = far;
         const float2 a0 = make_float2(B[u].x - rho[u].x, B[u].y - rho[u].y);
         const float2 a1 = make_float2(rho[u + 1].x - B[u].x, rho[u + 1].y - B[u].y);
         const uint32_t pw = pow2_pair(rho[u]);
@@ -258,26 +260,146 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         }
       }
       arrive(1 + b);
-      // the other buffer's tiles were free once the solving warps had the item before in registers (they issue the copy)
       gm = gn;
     }
+    for (long long i = it > 2 ? it - 2 : 0; i < it; ++i) sync(3 + (int)(i & 1));   // pair with the last arrivals
   } else {
     // ------------------------------------------------------------ contraction and solve
+    // Runs of blocks, (block row, first and last block column) per warp: at most five of the 36 each.
+    const int I0 = (0x34556677 >> (4 * warp)) & 7, hi0 = (0x34152637 >> (4 * warp)) & 7, lo0 = (0x00020304 >> (4 * warp)) & 7;
+    const int I1 = warp == 3 ? 1 : warp == 5 ? 2 : warp == 7 ? 0 : -1;
+    const uint32_t sA = smem_u32(sm + OFF_A);
+    float* sD = reinterpret_cast<float*>(sm + OFF_D);
+    const int g8 = lane >> 2, t2 = (lane & 3) * 2;
+    const int lrow = lane & 15, lch = lane >> 4;         // ldmatrix: row of a 16-row tile, 16-byte piece of a k-step
     Geom gm = geom(blockIdx.x);
     long long it = 0;
     for (long long item = blockIdx.x; gm.L > 0; ++it) {
       const int b = (int)(it & 1);
-      const int j = gm.j, jq = j / R;
-      const size_t cj = (size_t)gm.s * p.HV + j;
+      const size_t cj = (size_t)gm.s * p.HV + gm.j;
       uint8_t* rec = p.ws.rec + cj * kStepRecB;
-      uint8_t* buf = sm + b * kBufBytes;
+      const uint32_t sbuf = smem_u32(sm + b * kBufBytes);
+      const float* sBeta = reinterpret_cast<const float*>(sm + OFF_BETA + b * 512);
+      const uint32_t* dn = reinterpret_cast<const uint32_t*>(sm + OFF_DN + b * 2048) + (lane & 3);
+      const int* fall = reinterpret_cast<const int*>(sm + OFF_FALL + b * 64);
+      auto frag = [&](uint32_t (&r)[4], uint32_t tile, int I, int k) {    // 16 rows of block I, 16 channels of k-step k
+        ldsm4(r, tile + (k >> 2) * 16384 + sw128_offset(16 * I + lrow, (k & 3) * 2 + lch));
+      };
+      sync(1 + b);
+#pragma unroll 1
+      for (int sg = 0; sg < 2; ++sg) {
+        const int I = sg ? I1 : I0, hi = sg ? I1 : hi0, lo = sg ? 0 : lo0;
+        if (I < 0) break;
+        uint32_t kf[8][4], m[8][2];                      // m: 2^{rho_I - rho_{J+1}} of this lane's channels
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          frag(kf[k], sbuf + OFF_K, I, k);
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int c = 8 * k + 4 * e;
+            if (hi == I) {
+              m[k][e] = 0x7f007f00u - dn[64 * I + c];    // (the reciprocal of a power of two)
+            } else {
+              m[k][e] = 0x3f803f80u;
+              for (int J = hi + 1; J < I; ++J) m[k][e] = mul_bf16x2(m[k][e], dn[64 * J + c]);
+            }
+          }
+        }
+        const float b0 = sBeta[16 * I + g8], b1 = sBeta[16 * I + 8 + g8];
+#pragma unroll 1
+        for (int J = hi; J >= lo; --J) {
+          float a[2][4] = {}, pq[2][4] = {};
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            uint32_t r[4], qf[4];
+            frag(r, sbuf + OFF_K1, J, k);
+            frag(qf, sbuf + OFF_Q, I, k);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[e] = mul_bf16x2(r[e], m[k][e >> 1]);
+            mma_bf16(a[0], kf[k], r[0], r[2]);
+            mma_bf16(a[1], kf[k], r[1], r[3]);
+            mma_bf16(pq[0], qf, r[0], r[2]);
+            mma_bf16(pq[1], qf, r[1], r[3]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e)                  // for the block column to the left
+              m[k][e] = J == I ? 0x3f803f80u : mul_bf16x2(m[k][e], dn[64 * J + 8 * k + 4 * e]);
+          }
+          if (J == I) {
+            float* sd = sD + I * 16 * LDD;
+            if (fall[2 * I] | fall[2 * I + 1]) {
+              const size_t jq = gm.j / R;
+              slow_diagonal(p.k + ((size_t)gm.tok0 * p.HK + jq) * 128, p.q + ((size_t)gm.tok0 * p.HK + jq) * 128, (size_t)p.HK * 128,
+                            p.g + ((size_t)gm.tok0 * p.HV + gm.j) * 128, (size_t)p.HV * 128, gm.L, I, sBeta, sd, rec + kStepP, p.scale, lane);
+              continue;
+            }
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {                // (the substitution reads the strictly lower entries only)
+              *reinterpret_cast<float2*>(sd + g8 * LDD + 8 * n + t2) = make_float2(b0 * a[n][0], b0 * a[n][1]);
+              *reinterpret_cast<float2*>(sd + (g8 + 8) * LDD + 8 * n + t2) = make_float2(b1 * a[n][2], b1 * a[n][3]);
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (8 * n + t2 + (e & 1) > g8 + (e >> 1) * 8) pq[n][e] = 0.f;
+            }
+          } else {
+            const uint32_t f[4] = {pack_f16(b0 * a[0][0], b0 * a[0][1]), pack_f16(b0 * a[1][0], b0 * a[1][1]),
+                                   pack_f16(b1 * a[0][2], b1 * a[0][3]), pack_f16(b1 * a[1][2], b1 * a[1][3])};
+            sts4(sA + off_block(I, J) * 512 + lane * 16, f);
+          }
+          const uint32_t f[4] = {pack_bf16(p.scale * pq[0][0], p.scale * pq[0][1]), pack_bf16(p.scale * pq[1][0], p.scale * pq[1][1]),
+                                 pack_bf16(p.scale * pq[0][2], p.scale * pq[0][3]), pack_bf16(p.scale * pq[1][2], p.scale * pq[1][3])};
+          store_tri_block(rec + kStepP, I, J, lane, f);
+        }
+      }
+      sync_half(6);
+      if (tid == 0) {                                    // the tiles of this buffer have been read: the item after next
+        const Geom g2 = geom(item + 2 * stride);
+        if (g2.L > 0) {
+          fence_proxy_async_smem();
+          issue_tiles(g2, b);
+        }
+      }
+      const bool bad = solve_and_emit(rec + kStepT, sbuf + OFF_K1, sA, sD, smem_u32(sD), sBeta, warp, lane,
+                                      [&]() { sync_half(6); }, [](int) {});
+      if (bad) report_status(p.status, HA_LA_ERR_DEVICE_CHECK);
+      arrive(3 + b);
       item += stride;
-      const Geom gn = geom(item);
-      (void)rec; (void)buf; (void)jq; (void)cj;
-      gm = gn;
+      gm = geom(item);
     }
   }
+  if (tid == 256 && *abort_flag) report_status(p.status, HA_LA_ERR_TIMEOUT);
 }
 
 }  // namespace
+
+cudaError_t configure_tc_kda() {
+  cudaError_t e = cudaFuncSetAttribute(tc_kda_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kKdaSmem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(tc_kda_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
+cudaError_t launch_tc_kda(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
+                          const CUtensorMap& mq, const CUtensorMap& mk, int ctas, cudaStream_t stream) {
+  KdaParams kp;
+  kp.q = reinterpret_cast<const __nv_bfloat16*>(a.q);
+  kp.k = reinterpret_cast<const __nv_bfloat16*>(a.k);
+  kp.g = a.g; kp.beta = a.beta;
+  kp.chunk_tok0 = plan.chunk_tok0; kp.chunk_len = plan.chunk_len;
+  kp.T_row = p.T_row; kp.cps = p.max_seq_chunks > 0 ? p.max_seq_chunks : 1;
+  kp.ws = ws; kp.HK = p.HK; kp.HV = p.HV; kp.scale = p.scale; kp.status = a.status_word;
+  kp.total = (long long)p.max_chunks * p.HV;
+  if (kp.total == 0) return cudaSuccess;
+  timer_mark(stream, "tc_prep");
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(kp.total < ctas ? kp.total : ctas));
+  cfg.blockDim = dim3(kKdaThreads);
+  cfg.dynamicSmemBytes = kKdaSmem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = g_timer ? 0 : 1;                        // (per-kernel timing wants one kernel at a time)
+  return cudaLaunchKernelEx(&cfg, tc_kda_kernel, mq, mk, kp);
+}
+
 }  // namespace ha_la

@@ -62,7 +62,6 @@ struct TpParams {
   int HK, HV;
   float scale;                 // of the outputs: P comes times `scale`
   long long total;             // work items = step slots x q/k heads
-  int64_t epoch;               // published to ws.flags[cj] when the record is in memory (0: do not publish)
   int32_t* status;
 };
 
@@ -95,8 +94,8 @@ tc_tp_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
   // call's state-passing kernel, which lets its dependents go a few steps before its end, everything above ran under
   // that kernel's tail.  Nothing of this call has been read or written so far: wait for the stream's earlier work here.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  // Every CTA of this grid is running now: a dependent launch (the state-passing kernel) may be scheduled.  It either
-  // waits for this grid to finish or consumes steps as they are published.
+  // Every CTA of this grid is running now: a dependent launch (the state-passing kernel) may be scheduled.  It
+  // waits for this grid to finish.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // an item's step slot, q/k head, tokens, first token row; slots that a packed batch does not use come last
@@ -312,10 +311,6 @@ tc_tp_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
       }
       set ^= 1;
       gsync();
-      if (tid == 0 && p.epoch != 0) {                    // hand-over to a concurrently running state-passing kernel
-        __threadfence();
-        st_release_gpu(p.ws.flags + cj, p.epoch);
-      }
     }
     s = sn; jq = jqn; L = Ln; tok0 = tok0n; have = haven;
   }
@@ -335,11 +330,10 @@ cudaError_t configure_tc_tp() {
   return cudaFuncSetAttribute(tc_tp_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
 }
 
-// `ctas`: at most so many CTAs (the SMs that are not reserved for a concurrent state-passing kernel)
+// `ctas`: at most so many CTAs, one per SM
 cudaError_t launch_tc_tp(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                         const CUtensorMap& mq, const CUtensorMap& mk, int64_t epoch, int ctas, cudaStream_t stream) {
+                         const CUtensorMap& mq, const CUtensorMap& mk, int ctas, cudaStream_t stream) {
   TpParams pp;
-  pp.epoch = epoch;
   pp.g = a.g; pp.beta = a.beta;
   pp.chunk_tok0 = plan.chunk_tok0; pp.chunk_len = plan.chunk_len;
   pp.T_row = p.T_row; pp.cps = p.max_seq_chunks > 0 ? p.max_seq_chunks : 1;
