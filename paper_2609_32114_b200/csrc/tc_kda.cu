@@ -18,7 +18,7 @@
 // The contraction runs on warp-level MMAs: 36 pairs of blocks of the 64, no work above the diagonal, no operand copies
 // per pair; it is a fifth of the kernel's instructions.
 //
-// Measured on B200 with 32 heads and 8192 tokens: 162 us; with 64-token chunks, a copy of the operands per block row and
+// Measured on B200 with 32 heads and 8192 tokens: 131 us; with 64-token chunks, a copy of the operands per block row and
 // one item at a time per SM it was 262 us.
 //
 // Tokens past the end of a sequence are made no-ops by beta = 0 and g = 0; whatever the TMA box read for them (the
@@ -45,8 +45,8 @@ constexpr uint32_t OFF_K = 0, OFF_Q = kTileBytes, OFF_K1 = 2 * kTileBytes, kBufB
 constexpr uint32_t OFF_A = 2 * kBufBytes;                  // fp16 A below the diagonal blocks: 28 blocks, operand order
 constexpr uint32_t OFF_D = OFF_A + 28 * 512;               // fp32 diagonal blocks of A
 constexpr uint32_t OFF_TOT = OFF_D + 8 * 16 * LDD * 4;     // float [8][128]: log2 decay of each block
-constexpr uint32_t OFF_DN = OFF_TOT + 4096;                // per buffer: bf16 [8][128], 2^{rho_{J+1}-rho_J}
-constexpr uint32_t OFF_BETA = OFF_DN + 2 * 2048;           // per buffer: float [128]
+constexpr uint32_t OFF_RHO = OFF_TOT + 4096;               // per buffer: int16 [9][rho_slot(channel pair)][2], rho_J
+constexpr uint32_t OFF_BETA = OFF_RHO + 2 * 9 * 256;       // per buffer: float [128]
 constexpr uint32_t OFF_FALL = OFF_BETA + 2 * 512;          // per buffer: int [8][2] (channel halves), block needs the evaluation entry by entry
 constexpr uint32_t OFF_BAR = OFF_FALL + 2 * 64;
 constexpr uint32_t kKdaSmem = OFF_BAR + 32;
@@ -76,6 +76,13 @@ __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
 // 2^e for a whole e as bf16 bits (0 below the normal range, the largest power above it)
 __device__ __forceinline__ uint32_t pow2_bf16(float e) { return static_cast<uint32_t>(min(max(static_cast<int>(e) + 127, 0), 254)) << 7; }
 __device__ __forceinline__ uint32_t pow2_pair(float2 e) { return pow2_bf16(e.x) | (pow2_bf16(e.y) << 16); }
+// rho is kept as int16, as the sum of its steps from block to block clamped to +-kMaxStep: a difference of two is either
+// exact or, like the true one, far outside the exponents of bf16.
+constexpr float kMaxStep = 300.f;
+__device__ __forceinline__ uint32_t pack_s16(float2 e) { return (static_cast<uint32_t>(static_cast<int>(e.x)) & 0xffffu) | (static_cast<uint32_t>(static_cast<int>(e.y)) << 16); }
+// 2^(a + b) per half as bf16, a with the exponent bias added
+__device__ __forceinline__ uint32_t pow2_sum(uint32_t a, uint32_t b) { return __vmins2(__viaddmax_s16x2(a, b, 0u), 0x00fe00feu) << 7; }
+__device__ __forceinline__ int rho_slot(int pair) { return (pair & 3) * 16 + (pair >> 2); }   // a lane's sixteen pairs are neighbours
 
 // Diagonal block I of A (fp32, times beta) and scale P (to its operand dst), entry by entry, by one warp: lane l has
 // channels 4 l .. 4 l + 3.  (k, q, g: the head's first channel of the step's first token; token strides sk, sg.)
@@ -196,9 +203,13 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       }
       item += stride;
       const Geom gn = geom(item);
-      if (gn.L > 0 && w < 4) {                           // the next item's gate rows, into L2
-        const int t = w * 32 + lane;
-        if (t < gn.L) bulk_prefetch_l2(p.g + ((size_t)(gn.tok0 + t) * p.HV + gn.j) * 128, 512);
+      if (gn.L > 0) {                                    // the next item's gate rows, into L2 (line by line: 128 bulk
+        const int t = (tid - 256) >> 1;                  // prefetches of 512 bytes held the copy engine for 6 k cycles)
+        const float* g0 = p.g + ((size_t)(gn.tok0 + t) * p.HV + gn.j) * 128 + (tid & 1) * 64;
+        if (t < gn.L) {
+          prefetch_l2(g0);
+          prefetch_l2(g0 + 32);
+        }
       }
       const float2 lg = make_float2(1.4426950408889634f, 1.4426950408889634f);
 #pragma unroll
@@ -209,22 +220,33 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         *reinterpret_cast<float2*>(sTot + (2 * tg + u) * 128 + cp) = l[u][15];
       }
       sync_half(5);
-      float2 B[3], GL = make_float2(0.f, 0.f);           // gates at the boundaries of this thread's blocks, and the last
+      float2 B[2], GL = make_float2(0.f, 0.f);           // gates at the start of this thread's blocks, and the last
+      float2 rho[3];                                     // rounded, at the boundaries
+      uint32_t rc[3];
+      {
+        float2 r = GL, x = GL;                           // ... and as they are kept
 #pragma unroll
-      for (int I = 0; I < 8; ++I) {
-        if (I == 2 * tg) B[0] = GL;
-        const float2 x = *reinterpret_cast<const float2*>(sTot + I * 128 + cp);
-        GL.x += x.x; GL.y += x.y;
-        if (I == 2 * tg) B[1] = GL;
-        if (I == 2 * tg + 1) B[2] = GL;
+        for (int I = 0; I < 8; ++I) {
+          if (I == 2 * tg) { B[0] = GL; rho[0] = r; rc[0] = pack_s16(x); }
+          if (I == 2 * tg + 1) B[1] = GL;
+          const float2 y = *reinterpret_cast<const float2*>(sTot + I * 128 + cp);
+          GL.x += y.x; GL.y += y.y;
+          const float2 rn = make_float2(rintf(GL.x), rintf(GL.y));
+          x.x += fminf(fmaxf(rn.x - r.x, -kMaxStep), kMaxStep);
+          x.y += fminf(fmaxf(rn.y - r.y, -kMaxStep), kMaxStep);
+          r = rn;
+          if (I == 2 * tg) { rho[1] = r; rc[1] = pack_s16(x); }
+          if (I == 2 * tg + 1) { rho[2] = r; rc[2] = pack_s16(x); }
+        }
       }
-      float2 rho[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) rho[i] = make_float2(rintf(B[i].x), rintf(B[i].y));
       if (it > 1) sync(3 + b);                           // the solving warps are done with the item two before
       else sync_half(5);                                 // (either way: the totals have been read)
       mbar_wait(&full[b], (uint32_t)(it >> 1) & 1, abort_flag);
       uint8_t* buf = sm + b * kBufBytes;
+      uint32_t* kept = reinterpret_cast<uint32_t*>(sm + OFF_RHO + b * 2304) + 128 * tg + rho_slot(cp >> 1);
+      if (tg == 0) kept[0] = rc[0];
+      kept[64] = rc[1];
+      kept[128] = rc[2];
       if (tg < 2) reinterpret_cast<float*>(sm + OFF_BETA + b * 512)[w * 32 + lane] = bt;
       uint8_t* img = p.ws.img + cj * 3 * kTileBytes;
       if (tg == 0) *reinterpret_cast<float2*>(p.ws.rec + cj * kStepRecB + kStepSc + cp * 4) = ex2(GL);
@@ -232,7 +254,6 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       for (int u = 0; u < 2; ++u) {
         const int I = 2 * tg + u;
         const float2 dn = make_float2(rho[u + 1].x - rho[u].x, rho[u + 1].y - rho[u].y);
-        *reinterpret_cast<uint32_t*>(sm + OFF_DN + b * 2048 + I * 256 + cp * 2) = pow2_pair(dn);
         const bool far = __any_sync(0xffffffffu, dn.x < -kMaxUp || dn.y < -kMaxUp);
         if (lane == 0) reinterpret_cast<int*>(sm + OFF_FALL + b * 64)[2 * I + kb] = far;
         const float2 a0 = make_float2(B[u].x - rho[u].x, B[u].y - rho[u].y);
@@ -280,7 +301,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       uint8_t* rec = p.ws.rec + cj * kStepRecB;
       const uint32_t sbuf = smem_u32(sm + b * kBufBytes);
       const float* sBeta = reinterpret_cast<const float*>(sm + OFF_BETA + b * 512);
-      const uint32_t* dn = reinterpret_cast<const uint32_t*>(sm + OFF_DN + b * 2048) + (lane & 3);
+      const uint32_t* srho = reinterpret_cast<const uint32_t*>(sm + OFF_RHO + b * 2304) + (lane & 3) * 16;
       const int* fall = reinterpret_cast<const int*>(sm + OFF_FALL + b * 64);
       auto frag = [&](uint32_t (&r)[4], uint32_t tile, int I, int k) {    // 16 rows of block I, 16 channels of k-step k
         ldsm4(r, tile + (k >> 2) * 16384 + sw128_offset(16 * I + lrow, (k & 3) * 2 + lch));
@@ -290,39 +311,38 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       for (int sg = 0; sg < 2; ++sg) {
         const int I = sg ? I1 : I0, hi = sg ? I1 : hi0, lo = sg ? 0 : lo0;
         if (I < 0) break;
-        uint32_t kf[8][4], m[8][2];                      // m: 2^{rho_I - rho_{J+1}} of this lane's channels
+        uint32_t rI[16];                                 // 127 + rho_I of this lane's channels
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          frag(kf[k], sbuf + OFF_K, I, k);
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int c = 8 * k + 4 * e;
-            if (hi == I) {
-              m[k][e] = 0x7f007f00u - dn[64 * I + c];    // (the reciprocal of a power of two)
-            } else {
-              m[k][e] = 0x3f803f80u;
-              for (int J = hi + 1; J < I; ++J) m[k][e] = mul_bf16x2(m[k][e], dn[64 * J + c]);
-            }
-          }
+        for (int x = 0; x < 16; x += 4) {
+          const uint4 y = *reinterpret_cast<const uint4*>(srho + 64 * I + x);
+          rI[x] = __vadd2(y.x, 0x007f007fu); rI[x + 1] = __vadd2(y.y, 0x007f007fu);
+          rI[x + 2] = __vadd2(y.z, 0x007f007fu); rI[x + 3] = __vadd2(y.w, 0x007f007fu);
         }
         const float b0 = sBeta[16 * I + g8], b1 = sBeta[16 * I + 8 + g8];
 #pragma unroll 1
         for (int J = hi; J >= lo; --J) {
           float a[2][4] = {}, pq[2][4] = {};
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            uint32_t r[4], qf[4];
-            frag(r, sbuf + OFF_K1, J, k);
-            frag(qf, sbuf + OFF_Q, I, k);
+          for (int k = 0; k < 8; k += 2) {               // (k-steps in pairs: one 16-byte read of the block's gates)
+            const uint4 y = *reinterpret_cast<const uint4*>(srho + 64 * (J + 1) + 2 * k);
+            const uint32_t yy[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) r[e] = mul_bf16x2(r[e], m[k][e >> 1]);
-            mma_bf16(a[0], kf[k], r[0], r[2]);
-            mma_bf16(a[1], kf[k], r[1], r[3]);
-            mma_bf16(pq[0], qf, r[0], r[2]);
-            mma_bf16(pq[1], qf, r[1], r[3]);
+            for (int i = 0; i < 2; ++i) {
+              uint32_t r[4], kf[4], qf[4];
+              frag(r, sbuf + OFF_K1, J, k + i);
+              frag(kf, sbuf + OFF_K, I, k + i);
+              frag(qf, sbuf + OFF_Q, I, k + i);
 #pragma unroll
-            for (int e = 0; e < 2; ++e)                  // for the block column to the left
-              m[k][e] = J == I ? 0x3f803f80u : mul_bf16x2(m[k][e], dn[64 * J + 8 * k + 4 * e]);
+              for (int e = 0; e < 2; ++e) {              // 2^(rho_I - rho_{J+1})
+                const uint32_t m = pow2_sum(rI[2 * (k + i) + e], __vneg2(yy[2 * i + e]));
+                r[2 * e] = mul_bf16x2(r[2 * e], m);
+                r[2 * e + 1] = mul_bf16x2(r[2 * e + 1], m);
+              }
+              mma_bf16(a[0], kf, r[0], r[2]);
+              mma_bf16(a[1], kf, r[1], r[3]);
+              mma_bf16(pq[0], qf, r[0], r[2]);
+              mma_bf16(pq[1], qf, r[1], r[3]);
+            }
           }
           if (J == I) {
             float* sd = sD + I * 16 * LDD;
