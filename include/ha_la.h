@@ -67,10 +67,9 @@
  *
  * Environment switches (test hooks, read by the host launch code; they change how the
  * work is launched, never the result): HA_LA_FORCE_SIMT=1 (read once) sends every shape
- * to the fp32 CUDA-core kernel; HA_LA_TC_NV=32|64|128 fixes the slice width of the
- * sequential kernel; HA_LA_TC_OVERLAP=0|2 forbids / forces running the two tensor-core
- * kernels side by side; HA_LA_TC_SEGMENTS=1|2|4|8 fixes the number of segments a head's
- * chunk sequence is split into.  Production callers leave them unset; a caller that sets one
+ * to the fp32 CUDA-core kernels; HA_LA_TC_SEGMENTS=1|2|4|8 fixes the number of runs a
+ * sequence is cut into; HA_LA_TC_NV=32|64|128 and HA_LA_TC_OVERLAP=0|2 change only what
+ * ha_la_prefill_launch_plan answers.  Production callers leave them unset; a caller that sets one
  * does so before it asks for the workspace size (the size follows the plan, and a call whose
  * plan needs more than it was given returns HA_LA_ERR_WORKSPACE).
  */
@@ -144,22 +143,19 @@ const char* ha_la_prefill_path(const ha_la_prefill_args* args);
 /* Number of kernels ha_la_prefill launches for these shapes (0 if unsupported).  Host only. */
 int ha_la_prefill_num_launches(const ha_la_prefill_args* args);
 
-/* How ha_la_prefill would launch the tensor-core kernels for these shapes (host only; pointers are
- * ignored).  *slice_width = value channels per CTA of the sequential (state-passing) kernel: 32, 64 or
- * 128 -- the "Computation Splitting" paragraph of Section 4: a head's state split into column sub-heads --
- * or 0 on the CUDA-core path; *concurrent = 1 if that kernel runs beside the chunk-local kernel and
- * takes each chunk as it is published, 0 if the two run back to back.  The choice comes from measured
- * per-chunk costs of the two kernels and the bounds in `args` (sequences, longest sequence, total
- * tokens); the environment switches HA_LA_TC_NV and HA_LA_TC_OVERLAP override it.
+/* The cost model's answer for these shapes in chunks of 64 tokens (host only; pointers are ignored):
+ * *slice_width = value channels per CTA of a sliced state-passing kernel: 32, 64 or 128 -- the "Computation
+ * Splitting" paragraph of Section 4: a head's state split into column sub-heads -- or 0 on the CUDA-core path;
+ * *concurrent = 1 if such a kernel would best run beside the chunk-local one.  Kept for callers that read it:
+ * the kernels now work in steps of 128 tokens, a whole head per CTA, one behind the other.
  * Returns HA_LA_OK, or an error for invalid / unsupported shapes or NULL outputs.               */
 int ha_la_prefill_launch_plan(const ha_la_prefill_args* args, int* slice_width, int* concurrent);
 
-/* Segments per sequence ha_la_prefill would use for these shapes (host only; 1 = the chunks of a sequence are
- * walked strictly in order; 0 if the shapes are unsupported).  With S > 1 a sequence's chunks are cut into S
- * runs that are walked at the same time -- the Chunk-Seg-Seg mapping the paper describes for its FlashQLA
- * baseline (Section "Head-Level Mapping with Cross-Operator Fusion"): later segments start from a zero state and from the identity, and their true start
- * states, final state and outputs follow from one affine fix-up per segment.  Chosen only for equal-length rows
- * with so few (sequence, head) pairs that every run still gets an SM; HA_LA_TC_SEGMENTS overrides it.            */
+/* Segments per sequence in the same cost model, or as forced by HA_LA_TC_SEGMENTS (host only; 0 if the shapes are
+ * unsupported).  A call cuts its sequences by its own rule into runs that are walked at the same time -- the
+ * Chunk-Seg-Seg mapping the paper describes for its FlashQLA baseline (Section "Head-Level Mapping with
+ * Cross-Operator Fusion"): later runs are first walked from a zero state and from the identity, their true start
+ * states follow from one affine fix-up per run, and then every run is walked from there.  A forced number above 1 is used as it is. */
 int ha_la_prefill_num_segments(const ha_la_prefill_args* args);
 
 /* Profiling aid (the paper's "Metrics" paragraph times kernels with device events): the same work

@@ -4,7 +4,7 @@
 
 --profile builds a second library, libha_la_prof.so, with -DHA_LA_PROFILE_PHASES: the tensor-core kernels then
 record clock64 / %globaltimer stamps at their phase boundaries (csrc/prof.cuh) and the library exports
-ha_la_debug_read_prof_prep / _chain to read them; `python -m paper_2609_32114_b200.prof_phases` prints them.
+ha_la_debug_read_prof_walk to read them; `python -m paper_2609_32114_b200.prof_phases` prints them.
 The normal library contains none of this (the macros expand to nothing).
 
 Objects are cached under paper_2609_32114_b200/build/ and rebuilt when their source, any

@@ -83,22 +83,6 @@ int64_t next_epoch() {
   return (int64_t)(((uint64_t)(tag & 0x7fffffu) << 40) | ((uint64_t)(uint32_t)g_calls.fetch_add(1) << 8));
 }
 
-// Slice width (value channels per chain CTA) and launch mode, from a cost model measured on B200.
-// Chain kernel: bound by the latency of its two MMA round trips per chunk, which grows with the slice width (about
-// 0.9 / 1.23 / 1.5 us per chunk at 32 / 64 / 128 channels; the last is a kernel of its own that keeps the whole head's
-// state in tensor memory) and does not depend on the number of CTAs.  Each CTA
-// needs an SM of its own, so the kernel's time is about  max(longest sequence, all sequences / SMs)  in chunk-times
-// when the lengths differ (more CTAs than SMs are started longest sequence first and pack well), and whole rounds
-// when they do not: with few chains the narrow slice wins, with many a wider one may.
-// Prep kernel: throughput-bound, about 3.45 (GDN) / 9.8 (KDA) SM-microseconds per (chunk, head), and never
-// faster than its rounds of one item per work group (3 per SM for GDN, 1 for KDA) at 9 / 10.5 us per item.
-// Back to back the two times add.  Concurrently (allowed while the chain's CTAs leave at least half of the SMs to
-// the prep kernel) the call takes the longer of the chain and of the prep kernel on the remaining SMs (plus some
-// interference), plus the wait for the first chunks; with several sequences the prep kernel works through them
-// one after the other, so the last sequence's chain starts only when most of the prep work is done.
-// Only bounds are known on the host: max_len for the longest sequence, max_chunks for the total.
-struct TcPlan { int nv; bool concurrent; int nseg; };
-
 // HA_LA_TC_SEGMENTS, or 0
 int forced_segments() {
   const char* e = getenv("HA_LA_TC_SEGMENTS");
@@ -134,6 +118,25 @@ int plan_spans(const Problem& p) {
   }
   return best_s;
 }
+
+// What ha_la_prefill_launch_plan and ha_la_prefill_num_segments answer, and what a forced HA_LA_TC_SEGMENTS must fit:
+// the choice for a launch in chunks of 64 tokens with a state-passing kernel of sliced heads.  The kernels above this
+// line's rule work in steps of 128 on whole heads; callers may have built on the answers, so they stay.
+// Slice width (value channels per chain CTA) and launch mode, from a cost model measured on B200.
+// Chain kernel: bound by the latency of its two MMA round trips per chunk, which grows with the slice width (about
+// 0.9 / 1.23 / 1.5 us per chunk at 32 / 64 / 128 channels; the last is a kernel of its own that keeps the whole head's
+// state in tensor memory) and does not depend on the number of CTAs.  Each CTA
+// needs an SM of its own, so the kernel's time is about  max(longest sequence, all sequences / SMs)  in chunk-times
+// when the lengths differ (more CTAs than SMs are started longest sequence first and pack well), and whole rounds
+// when they do not: with few chains the narrow slice wins, with many a wider one may.
+// Prep kernel: throughput-bound, about 3.45 (GDN) / 9.8 (KDA) SM-microseconds per (chunk, head), and never
+// faster than its rounds of one item per work group (3 per SM for GDN, 1 for KDA) at 9 / 10.5 us per item.
+// Back to back the two times add.  Concurrently (allowed while the chain's CTAs leave at least half of the SMs to
+// the prep kernel) the call takes the longer of the chain and of the prep kernel on the remaining SMs (plus some
+// interference), plus the wait for the first chunks; with several sequences the prep kernel works through them
+// one after the other, so the last sequence's chain starts only when most of the prep work is done.
+// Only bounds are known on the host: max_len for the longest sequence, max_chunks for the total.
+struct TcPlan { int nv; bool concurrent; int nseg; };
 
 TcPlan plan_tc(const Problem& p) {
   const int sms = sm_count();
@@ -233,19 +236,20 @@ size_t tc_workspace_bytes(const Problem& p) {
 }
 
 // HA_LA_TC_SEGMENTS forces the spans too (1: none); their scratch is then the segment scratch, which is larger.
-static SpanBuffers call_spans(const Problem& p, const TcPlan& tp, void* tc_ws) {
+static SpanBuffers call_spans(const Problem& p, void* tc_ws) {
   uint8_t* b = reinterpret_cast<uint8_t*>(tc_ws);
   const size_t nj = (size_t)p.N * p.HV;
   const int forced = forced_segments();
   if (forced == 1) return tc_span_view(nullptr, nj, 1);
-  if (forced > 1 && tp.nseg > 1) return tc_span_view(b + tc_base_bytes(p), nj, tp.nseg);
+  if (forced > 1) {
+    const int nseg = plan_tc(p).nseg;
+    if (nseg > 1) return tc_span_view(b + tc_base_bytes(p), nj, nseg);
+  }
   return tc_span_view(b + tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA), nj, plan_spans(p));
 }
 
 int tc_num_launches(const Problem& p) {
-  const int nseg = plan_tc(p).nseg;
-  const int forced = forced_segments();
-  return (forced == 1 ? 1 : forced > 1 && nseg > 1 ? nseg : plan_spans(p)) > 1 ? 4 : 2;
+  return call_spans(p, nullptr).nspan > 1 ? 4 : 2;
 }
 
 int tc_num_segments(const Problem& p) { return plan_tc(p).nseg; }
@@ -259,7 +263,7 @@ void tc_launch_plan(const Problem& p, int* slice_width, int* concurrent) {
 cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* tc_ws, cudaStream_t stream) {
   const bool kda = p.variant == HA_LA_KDA;
   const TcWorkspace ws = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, kda);
-  const SpanBuffers sb = call_spans(p, plan_tc(p), tc_ws);
+  const SpanBuffers sb = call_spans(p, tc_ws);
   CUtensorMap mq, mk, mv;
   if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk, a.k, p.T_total, p.HK) ||
       !make_map_tile(&mv, a.v, p.T_total, p.HV))

@@ -1,15 +1,10 @@
-"""Prints the phase time stamps of the tensor-core kernels from the instrumented build.
+"""Prints the phase time stamps of the state-passing kernel from the instrumented build.
 
     python -m paper_2609_32114_b200.build --profile
     python -m paper_2609_32114_b200.prof_phases [WORKLOAD]          (needs a GPU)
 
-The instrumented library (libha_la_prof.so, -DHA_LA_PROFILE_PHASES) records, for CTA 0 of each kernel, clock64 at
-the phase boundaries of its first work items / chunks and a few %globaltimer stamps (kernel start and end, first
-and last chunk, when chunks were published).  This script runs one workload through it and prints
-  * the chain kernel: cycles per chunk, split into waiting for the operands, the first product, the first
-    epilogue, the second product, the second epilogue;
-  * the prep kernel: cycles between the numbered phase probes of its first items;
-  * a nanosecond timeline of both kernels within one call.
+The instrumented library (libha_la_prof.so, -DHA_LA_PROFILE_PHASES) records clock64 of a compute warp of CTA 0 at the
+phase boundaries of its steps; this script runs one workload through it and prints the cycles between them.
 """
 import ctypes
 import os
@@ -51,21 +46,11 @@ def main(argv):
         getattr(lib, f"ha_la_debug_read_prof_{name}")(buf)
         return np.array(buf[:], dtype=np.int64)
 
-    P, C = read("prep"), read("chain")
-    nch = min(64, (max(inp["seq_lens"]) + 63) // 64)
-    print("chain kernel, CTA 0, cycles per chunk: operands / product 1 / epilogue 1 / product 2 / epilogue 2 / total")
-    for c in list(range(1, min(nch, 9))) + ([nch // 2] if nch > 16 else []):
-        t = C[8 * c: 8 * c + 6]
-        print(f"  chunk {c:3d}: {t[1]-t[0]:5d} {t[2]-t[1]:5d} {t[3]-t[2]:5d} {t[4]-t[3]:5d} {t[5]-t[4]:5d} {t[5]-t[0]:6d}")
-    print("prep kernel, CTA 0 group 0, cycles between phase probes 2..13 of its first items")
-    for n in range(3):
-        t = P[16 + 16 * n + 2: 16 + 16 * n + 14]
-        if t[0] > 0:
-            print(f"  item {n}: {[int(x) for x in np.diff(t)]} sum {int(t[-1] - t[0])}")
-    t0 = min(P[900], C[900])
-    print("timeline (ns from the first kernel's start): prep start", P[900] - t0, "prep end", P[901] - t0,
-          "| chain start", C[900] - t0, "first chunk done", C[700] - t0, "last chunk done", C[700 + nch - 1] - t0,
-          "chain end", C[901] - t0)
+    t = read("walk")
+    print("cycles per step: X / R / U / update operand / D2 / state / total")
+    for c in range(1, min(9, (max(inp["seq_lens"]) + 127) // 128)):
+        v = t[8 * c: 8 * c + 7]
+        print(f"  step {c:3d}:", *(f"{x:5d}" for x in np.diff(v)), f"{v[6] - v[0]:6d}")
     print("status word:", int(keep["status_word"].item()))
 
 

@@ -1,0 +1,46 @@
+"""The tensor-core kernels against the fp64 oracle, where their indexing can go wrong: lengths around a step of 128 tokens and
+a block of 16, sequences cut into runs (short ones into empty runs), more work items than work groups."""
+import pytest
+
+from paper_2609_32114_b200 import synth
+from tests import helpers
+
+pytestmark = pytest.mark.gpu
+W = synth.WORKLOADS
+
+
+def _inputs(variant, lens, packed, hk, hv, seed, **kw):
+    base = W["gdn_varlen"] if variant == "gdn" else W["kda_8k"]
+    w = synth.shrink(base, seq_lens=lens, hk=hk, hv=hv, h0_std=0.05, varlen=packed, **dict(dict(gate_shift=-1.0), **kw))
+    return synth.make_inputs(w, seed=seed)
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("lens,packed,hk,hv", [([1], False, 1, 1), ([127, 127], False, 1, 2), ([129], False, 2, 4),
+                                               ([128, 0, 15, 257, 17], True, 2, 2), ([112] * 5, True, 1, 3)])
+def test_step_edges(variant, lens, packed, hk, hv):
+    helpers.check_parity(_inputs(variant, lens, packed, hk, hv, 311 + len(lens)), scale=0.5)
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("runs", [1, 2, 4, 8])
+def test_runs_of_a_sequence(variant, runs, monkeypatch):
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
+    helpers.check_parity(_inputs(variant, [1025], False, 1, 2, 331, gate_shift=5.0), scale=0.5)
+    helpers.check_parity(_inputs(variant, [700, 0, 129, 1], True, 1, 2, 337, gate_shift=3.0))
+
+
+@pytest.mark.parametrize("variant,hk,hv,lens", [("gdn", 16, 16, [2560]), ("gdn", 8, 16, [1300, 2500]), ("kda", 16, 16, [2100, 1900])])
+def test_every_group_takes_several_items(variant, hk, hv, lens):
+    helpers.check_parity(_inputs(variant, lens, len(lens) > 1, hk, hv, 347, gate_shift=2.0))
+
+
+@pytest.mark.parametrize("log_gate", [-3.0, -9.0, -90.0, -500.0])
+def test_kda_strong_decay(log_gate):
+    """Channels whose decay between two block boundaries is inside, around and far outside the range that the scaled
+    operands of a block hold; the last clamps the kept exponents too."""
+    inp = _inputs("kda", [300], False, 1, 2, 353)
+    for tok in (5, 15, 16, 37, 70, 71, 131, 200):
+        inp["g"][tok, :, ::7] = log_gate
+    inp["g"][140:190, :, 3::11] = log_gate
+    helpers.check_parity(inp)
