@@ -491,15 +491,16 @@ def measure(ha, helpers, w, inp, steps, warmup, dev, local_rank, dist, peaks, wo
     # g, beta; the chain kernel reads h0 and writes o and hT; the operand images between them are not algorithmic)
     e = 2 if w.dtype == "bf16" else 4
     in_bytes = T * (2 * w.hk * w.dk * e + w.hv * w.dv * e + w.hv * 4 * (1 + (w.dk if w.variant == "kda" else 1)))
-    kernel_alg_bytes = {"simt_prefill": alg_bytes, "tc_prep": in_bytes, "tc_chain": alg_bytes - in_bytes, "plan": 0.0}
+    kernel_alg_bytes = {"simt_prefill": alg_bytes, "tc_prep": in_bytes, "tc_chain": alg_bytes - in_bytes,
+                        "tc_span": 0.0, "tc_span_fix": 0.0, "plan": 0.0}
     dom_s = kernel_ms[dom] / 1e3
     achieved = alg_bytes / dom_s / 1e9                   # the path's bytes over the dominant kernel's time
     t_hbm = alg_bytes / (peaks["hbm_gbs"] * 1e9)
     t_flop = alg_flops / (peaks["bf16_tflops"] * 1e12)
     path_s = ms_per_step / 1e3
-    nv_plan, conc_plan = ha.ha_la_prefill_launch_plan(sets[0][0])
-    launch_mode = ("fp32 CUDA-core kernel" if nv_plan == 0 else
-                   f"{nv_plan}-channel slices, prep and chain kernels " + ("side by side" if conc_plan else "back to back"))
+    launches = ha.ha_la_prefill_num_launches(sets[0][0])
+    launch_mode = ("fp32 kernels" if ha.ha_la_prefill_path(sets[0][0]) != "tc" else
+                   "one state-passing launch" if launches == 2 else "sequences cut into runs, two state-passing launches")
     roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(w.name, dom),
                 "alg_bytes": alg_bytes, "peak_source": peaks["source"],
@@ -541,9 +542,8 @@ def profile_range(ha, helpers, w, inp, warmup, dev):
     e1.record()
     torch.cuda.synchronize(dev)
     torch.cuda.profiler.stop()
-    nv, conc = ha.ha_la_prefill_launch_plan(a)
     print(json.dumps({"profile_range": w.name, "tokens": inp["T"], "rc": rc, "status": int(keep["status_word"].item()),
-                      "ms": e0.elapsed_time(e1), "slice_width": nv, "side_by_side": bool(conc),
+                      "ms": e0.elapsed_time(e1), "launches": ha.ha_la_prefill_num_launches(a),
                       "alg_bytes": synth.algorithmic_bytes(w, inp["T"], inp["N"])}), flush=True)
 
 
