@@ -95,25 +95,36 @@ int forced_segments() {
 // products of 128^3 between them.  Costs measured on B200: 2.0 us per state-only step, 2.45 per step with outputs, 5 for
 // a CTA's start and end, 1.25 per product (5 when the products' 8 CTAs per pair do not all have an SM) and about 8 for
 // the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
-// within some 15 %.
+// within some 15 %.  And no launch beats HBM, at 6 TB/s, once its operands do not stay in L2: 8 sequences of 139 k tokens
+// in all were cut in two for a second launch of 470 us, 444 of them HBM's, after a first of 250; uncut they take 575.
 int plan_spans(const Problem& p) {
   const long long chains = (long long)p.N * p.HV;
   const int sms = sm_count(), longest = (p.max_len + kStep - 1) / kStep;
   const double avg_len = p.N > 0 ? (double)p.T_total / p.N : 0.0;
   const bool even = p.max_len < 1.5 * avg_len;
   const double total = (double)p.max_chunks * p.HV;
-  auto launch_us = [&](int runs, int spans, double step_us) {
+  const bool kda = p.variant == HA_LA_KDA;
+  auto launch_us = [&](int runs, int spans, bool out) {
+    const double step_us = out ? 2.45 : 2.0;
     const int cps = (longest + spans - 1) / spans;
     const long long ctas = chains * runs;
-    if (ctas <= sms) return cps * step_us + 5.0;
-    if (even) return (cps * step_us + 5.0) * (double)((ctas + sms - 1) / sms);
-    const double spread = 1.15 * total * runs / spans / sms;
-    return (spread > cps ? spread : cps) * step_us + 5.0 * (double)ctas / sms;
+    double t = cps * step_us + 5.0;
+    if (ctas > sms && even) {
+      t *= (double)((ctas + sms - 1) / sms);
+    } else if (ctas > sms) {
+      const double spread = 1.15 * total * runs / spans / sms;
+      t = (spread > cps ? spread : cps) * step_us + 5.0 * (double)ctas / sms;
+    }
+    // bytes of a step: the tiles (GDN: K and Q once per group of heads), V, the record, the outputs
+    const double qk = kda ? 1.0 : (double)p.HK / p.HV;
+    const double bytes = kTileBytes * (qk * (kda ? 2 + out : 1 + out) + 1 + out) + kTriB * (1 + out) + kStepScB;
+    const double moved = total * runs / spans * bytes;
+    return moved > 126e6 && moved / 6e6 > t ? moved / 6e6 : t;
   };
   int best_s = 1;
-  double best = launch_us(1, 1, 2.45);
+  double best = launch_us(1, 1, true);
   for (int S = 2; S <= 32 && S <= longest; ++S) {
-    const double t = launch_us(2 * S - 3, S, 2.0) + launch_us(S, S, 2.45) + (8 * chains <= sms ? 1.25 : 5.0) * (S - 2) + 8.0;
+    const double t = launch_us(2 * S - 3, S, false) + launch_us(S, S, true) + (8 * chains <= sms ? 1.25 : 5.0) * (S - 2) + 8.0;
     if (t < best) { best = t; best_s = S; }
   }
   return best_s;
