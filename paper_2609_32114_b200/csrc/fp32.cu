@@ -13,9 +13,9 @@
 // and the walk does    U~ = U - W h;   o = scale (QG h + P U~);   h <- e^{G_L} h + KD^T U~.
 //
 // What bounds it: shared-memory reads (a 16-byte read costs four cycles of the SM's 128 bytes whatever is shared between
-// lanes; the thread tiles here do 16 multiply-adds for five of them: 4.2 k cycles per chunk of the d = 64 walk, 76 % of its
-// time), and for short sequences the walk's chain of chunks.  One call with T = 256, one head, d = 64: one CTA for
-// everything took 237 us, split like this 21.6 us; d = 64, 8 heads, T = 1000: 924 us -> 53.7 us.
+// lanes), the walk's two barriers per chunk, and for short sequences its chain of chunks: 2.2 us each at d = 64.  One call
+// with T = 256, one head, d = 64: one CTA for everything took 237 us, split like this 19.0 us; d = 64, 8 heads, T = 1000:
+// 924 us -> 42.8 us.
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -356,19 +356,32 @@ template <int D> struct WalkSmem {
   static constexpr int BAR = (Y + C * (kNV + 1) + 3) / 4 * 4;
   static constexpr size_t bytes = (size_t)BAR * 4 + 32;
 };
-// Threads: the first kUpd<D> update the state (four keys of NV / 8 channels, over half of the tokens each), then 256 for the
-// outputs (four rows, over half of the tokens); the first 512 compute W h and QG h (two tokens, over half of the keys).
-// Neighbouring lanes hold the two halves of a sum: enough warps to cover the shared-memory latency of a CTA that has an
-// SM to itself.
+// Threads: the first kUpd<D> update the state, then 256 form the outputs; the first 512 compute W h and QG h.  A thread makes
+// four rows (tokens, keys) by NV / 2 channels of a product over an eighth of its depth: sixteen and more multiply-adds for
+// every two 16-byte reads, where reads bound the kernel.  The eight parts of a sum sit in neighbouring lanes, which add
+// them up so that each ends with one row and NV / 4 channels.  (Two rows by one or two channels over half of the depth:
+// 53.7 us for d = 64, 8 heads, T = 1000; 42.8 like this.)
 template <int D> constexpr int kUpd = D * 4;
 template <int D> constexpr int kWalkThreads = kUpd<D> + 256;
-__device__ __forceinline__ float pair_sum(float x) { return x + __shfl_xor_sync(0xffffffffu, x, 1); }
+// v[N] summed over eight neighbouring lanes; lane l keeps the sums N / 8 (l % 8) .. in v[0 .. N / 8)
+template <int N> __device__ __forceinline__ void scatter_sum(float (&v)[N], int lane) {
+#pragma unroll
+  for (int b = 4, n = N / 2; b > 0; b >>= 1, n /= 2) {
+    const bool up = lane & b;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      if (i >= n) break;
+      const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, b);
+    }
+  }
+}
 
 template <typename In, int D, int NV>
 __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Params p) {
   using S = WalkSmem<D>;
   using R = Rec<D>;
-  constexpr int LD = D + 4, NSL = D / NV, E = NV / 8;     // E channels per thread: cg, cg + 8
+  constexpr int LD = D + 4, NSL = D / NV, H = NV / 2, E = NV / 4;   // channels of a thread's products; of its sums
   extern __shared__ __align__(16) float sf[];
   constexpr int ST = S::kStages;
   float* sH = sf + S::HT;
@@ -376,7 +389,8 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   float* sY = sf + S::Y;
   uint64_t* bar1 = reinterpret_cast<uint64_t*>(sf + S::BAR);   // [stages] W, QG, U
   uint64_t* bar3 = bar1 + 2;                                   // [stages] KD, P, e^{G_L}
-  const int tid = threadIdx.x, half = tid & 1, cg = (tid >> 1) & 7;
+  const int tid = threadIdx.x, part = tid & 7, ch0 = ((tid >> 3) & 1) * H, grp = tid >> 4;
+  const int row = part >> 1, ch = ch0 + (part & 1) * E;   // this thread's row of four and first channel, once summed up
   const int slice = blockIdx.x % NSL, nj = blockIdx.x / NSL, j = nj % p.HV;
   const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;
   const int tok0 = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
@@ -387,24 +401,21 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
     for (int i = 0; i < ST; ++i) { mbar_init(&bar1[i], 1); mbar_init(&bar3[i], 1); }
     mbar_fence_init();
   }
-  // state: thread -> four keys, its channels of the slice (held by both lanes of a pair)
-  const int kg = tid >> 4;
+  // state: thread -> key 4 grp + row, its E channels of the slice
   const bool upd = tid < kUpd<D>;
-  const size_t hbase = (((size_t)n * p.HV + j) * D + 4 * kg) * D + slice * NV + cg;
-  const int uc = (NV == kNV ? 0 : (slice & 1) * NV) + cg;      // first channel within the record's U slice
-  float h[E][4];
+  const int key = 4 * grp + row;
+  const size_t hbase = (((size_t)n * p.HV + j) * D + key) * D + slice * NV + ch;
+  const int uc = NV == kNV ? 0 : (slice & 1) * NV;       // first channel within the record's U slice
+  float h[E];
 #pragma unroll
-  for (int e = 0; e < E; ++e)
-#pragma unroll
-    for (int x = 0; x < 4; ++x) h[e][x] = 0.f;
+  for (int e = 0; e < E; ++e) h[e] = 0.f;
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (upd) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-#pragma unroll
-      for (int x = 0; x < 4; ++x) h[e][x] = p.h0 ? p.h0[hbase + (size_t)x * D + 8 * e] : 0.f;
-      *reinterpret_cast<float4*>(sH + (cg + 8 * e) * LD + 4 * kg) = make_float4(h[e][0], h[e][1], h[e][2], h[e][3]);
+      h[e] = p.h0 ? p.h0[hbase + e] : 0.f;
+      sH[(ch + e) * LD + key] = h[e];
     }
   }
   auto load1 = [&](int c) {
@@ -430,113 +441,91 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
 
   for (int c = 0; c < nch; ++c) {
     const float* sW = sf + (c % ST) * S::kStage + S::WQ;
-    const float* sQ = sW + C * LD;
-    const float* sK = sf + (c % ST) * S::kStage + S::KP;
+    const float* sK = sf + (c % ST) * S::kStage + S::KP;   // (QG follows W: rows 64 .. 127 of one operand)
     const float* sP = sK + C * LD;
     const float* sGam = sP + C * LDP;
     const float* sU = sf + (c % ST) * S::kStage + S::U;
-    // ---- W h and QG h: 64 tokens x NV channels each; token rows rg, rg + 32
+    // ---- [W; QG] h: 128 rows x NV channels; rows grp + 32 i
     if (tid < 512) {
       if (!mbar_test_wait(&bar1[c % ST], (c / ST) & 1)) mbar_wait(&bar1[c % ST], (c / ST) & 1, abort_flag);
-      const int rg = tid >> 4;
-      float x[2][E] = {}, y[2][E] = {};
-#pragma unroll 4
-      for (int k = 4 * half; k < D; k += 8) {
-        float4 hv[E];
+      float x[4 * H] = {};
+#pragma unroll 2
+      for (int k = 4 * part; k < D; k += 32) {
+        float4 w[4];
 #pragma unroll
-        for (int e = 0; e < E; ++e) hv[e] = ld4(sH + (cg + 8 * e) * LD + k);
+        for (int i = 0; i < 4; ++i) w[i] = ld4(sW + (grp + 32 * i) * LD + k);
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const float4 w = ld4(sW + (rg + 32 * r) * LD + k), q = ld4(sQ + (rg + 32 * r) * LD + k);
+        for (int e = 0; e < H; ++e) {
+          const float4 hv = ld4(sH + (ch0 + e) * LD + k);
 #pragma unroll
-          for (int e = 0; e < E; ++e) {
-            x[r][e] = dot4(w, hv[e], x[r][e]);
-            y[r][e] = dot4(q, hv[e], y[r][e]);
-          }
+          for (int i = 0; i < 4; ++i) x[i * H + e] = dot4(w[i], hv, x[i * H + e]);
         }
       }
+      scatter_sum(x, part);
+      const int t = grp + 32 * (row & 1);
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const int t = rg + 32 * r, ch = cg + 8 * e;
-          const float xs = pair_sum(x[r][e]), ys = pair_sum(y[r][e]);
-          if (half == 0) sT[ch * LDP + t] = sU[t * kNV + uc + 8 * e] - xs;
-          else sY[t * (kNV + 1) + ch] = ys;
-        }
+      for (int e = 0; e < E; ++e) {
+        if (row < 2) sT[(ch + e) * LDP + t] = sU[t * kNV + uc + ch + e] - x[e];
+        else sY[t * (kNV + 1) + ch + e] = x[e];
+      }
     }
     __syncthreads();                                     // U~ and QG h are complete; W, QG, U and the old state are free
     if (tid == 0 && c + ST < nch) load1(c + ST);
     if (!mbar_test_wait(&bar3[c % ST], (c / ST) & 1)) mbar_wait(&bar3[c % ST], (c / ST) & 1, abort_flag);
     if (upd) {
-      // ---- h <- e^{G_L} h + KD^T U~
-      float d[E][4] = {};
+      // ---- h <- e^{G_L} h + KD^T U~: keys 4 grp .., tokens part + 8 m
+      float d[4 * H] = {};
 #pragma unroll 4
-      for (int t = 4 * half; t < C; t += 8) {
-        float uu[E][4];
+      for (int t = part; t < C; t += 8) {
+        const float4 k4 = ld4(sK + t * LD + 4 * grp);
 #pragma unroll
-        for (int e = 0; e < E; ++e) *reinterpret_cast<float4*>(uu[e]) = ld4(sT + (cg + 8 * e) * LDP + t);
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          const float4 k4 = ld4(sK + (t + s) * LD + 4 * kg);
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            d[e][0] = fmaf(k4.x, uu[e][s], d[e][0]);
-            d[e][1] = fmaf(k4.y, uu[e][s], d[e][1]);
-            d[e][2] = fmaf(k4.z, uu[e][s], d[e][2]);
-            d[e][3] = fmaf(k4.w, uu[e][s], d[e][3]);
-          }
+        for (int e = 0; e < H; ++e) {
+          const float u = sT[(ch0 + e) * LDP + t];
+          d[e] = fmaf(k4.x, u, d[e]);
+          d[H + e] = fmaf(k4.y, u, d[H + e]);
+          d[2 * H + e] = fmaf(k4.z, u, d[2 * H + e]);
+          d[3 * H + e] = fmaf(k4.w, u, d[3 * H + e]);
         }
       }
-      const float4 gm = ld4(sGam + 4 * kg);
+      scatter_sum(d, part);
+      const float gm = sGam[key];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        h[e][0] = fmaf(gm.x, h[e][0], pair_sum(d[e][0]));
-        h[e][1] = fmaf(gm.y, h[e][1], pair_sum(d[e][1]));
-        h[e][2] = fmaf(gm.z, h[e][2], pair_sum(d[e][2]));
-        h[e][3] = fmaf(gm.w, h[e][3], pair_sum(d[e][3]));
-        if (half == 0)
-          *reinterpret_cast<float4*>(sH + (cg + 8 * e) * LD + 4 * kg) = make_float4(h[e][0], h[e][1], h[e][2], h[e][3]);
+        h[e] = fmaf(gm, h[e], d[e]);
+        sH[(ch + e) * LD + key] = h[e];
       }
     } else {
-      // ---- o = scale (QG h + P U~): rows rg, rg + 16, ..; P is lower triangular
-      const int rg = (tid - kUpd<D>) >> 4;
-      float s[4][E] = {};
+      // ---- o = scale (QG h + P U~): rows rg + 16 i, tokens 4 part + 32 m; P's blocks of 16 above the diagonal are not there
+      const int rg = grp - kUpd<D> / 16;
+      float s[4 * H] = {};
 #pragma unroll
-      for (int b = 0; b < 4; ++b)
+      for (int m = 0; m < 2; ++m) {
+        const int t = 4 * part + 32 * m;
+        float4 q[4];
 #pragma unroll
-        for (int t = 16 * b; t < 16 * b + 16; t += 8) {
-          float4 u[E];
+        for (int i = 2 * m; i < 4; ++i) q[i] = t < 16 * (i + 1) ? ld4(sP + (rg + 16 * i) * LDP + t) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < E; ++e) u[e] = ld4(sT + (cg + 8 * e) * LDP + t + 4 * half);
+        for (int e = 0; e < H; ++e) {
+          const float4 u = ld4(sT + (ch0 + e) * LDP + t);
 #pragma unroll
-          for (int r = b; r < 4; ++r) {
-            const float4 q = ld4(sP + (rg + 16 * r) * LDP + t + 4 * half);
-#pragma unroll
-            for (int e = 0; e < E; ++e) s[r][e] = dot4(q, u[e], s[r][e]);
-          }
+          for (int i = 2 * m; i < 4; ++i) s[i * H + e] = dot4(q[i], u, s[i * H + e]);
         }
-      In* go = reinterpret_cast<In*>(p.o) + ((size_t)(tok0 + c * C) * p.HV + j) * D + slice * NV + cg;
-      const int left = len - c * C;
+      }
+      scatter_sum(s, part);
+      const int t = rg + 16 * row;
+      In* go = reinterpret_cast<In*>(p.o) + ((size_t)(tok0 + c * C + t) * p.HV + j) * D + slice * NV + ch;
+      if (t < len - c * C) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int t = rg + 16 * r;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const float o = sY[t * (kNV + 1) + cg + 8 * e] + pair_sum(s[r][e]);
-          if (t < left && half == 0) go[(size_t)t * p.HV * D + 8 * e] = from_f32<In>(p.scale * o);
-        }
+        for (int e = 0; e < E; ++e) go[e] = from_f32<In>(p.scale * (sY[t * (kNV + 1) + ch + e] + s[e]));
       }
     }
     __syncthreads();                                     // the new state is complete; KD, P, U~ and QG h are free
     if (tid == 0 && c + ST < nch) load3(c + ST);
   }
   if (gave_up) report_status(p.status, HA_LA_ERR_TIMEOUT);
-  if (p.hT && upd && half == 0) {
+  if (p.hT && upd) {
 #pragma unroll
-    for (int e = 0; e < E; ++e)
-#pragma unroll
-      for (int x = 0; x < 4; ++x) p.hT[hbase + (size_t)x * D + 8 * e] = h[e][x];
+    for (int e = 0; e < E; ++e) p.hT[hbase + e] = h[e];
   }
 }
 
