@@ -4,7 +4,7 @@
 //   fp32_prep_kernel   one CTA per (chunk, V-head): operators #1-#4 of the paper's pipeline (Section 2.1, "Chunkwise
 //                      Map-Reduce-Map Execution").  Chunks are independent here, so a single short sequence already
 //                      keeps several SMs busy instead of one.
-//   fp32_walk_kernel   one CTA per (sequence, V-head, 8 or 16 value channels) walks the chunks in order: operator #5 with #6 in
+//   fp32_walk_kernel   one CTA per (sequence, V-head, 4, 8 or 16 value channels) walks the chunks in order: operator #5 with #6 in
 //                      the paper's chunk-first order.  Value channels are independent ("Computation Splitting"), so the
 //                      sequential part of a head is spread over several SMs.
 //
@@ -13,9 +13,9 @@
 // and the walk does    U~ = U - W h;   o = scale (QG h + P U~);   h <- e^{G_L} h + KD^T U~.
 //
 // What bounds it: shared-memory reads (a 16-byte read costs four cycles of the SM's 128 bytes whatever is shared between
-// lanes), the walk's two barriers per chunk, and for short sequences its chain of chunks: 2.2 us each at d = 64.  One call
-// with T = 256, one head, d = 64: one CTA for everything took 237 us, split like this 19.0 us; d = 64, 8 heads, T = 1000:
-// 924 us -> 42.8 us.
+// lanes), the walk's two barriers per chunk, and for short sequences its chain of chunks: 1.6 us each at d = 64.  One call
+// with T = 256, one head, d = 64: one CTA for everything took 237 us, split like this 16.8 us; d = 64, 8 heads, T = 1000:
+// 924 us -> 35.0 us.
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   const bool upd = tid < kUpd<D>;
   const int key = 4 * grp + row;
   const size_t hbase = (((size_t)n * p.HV + j) * D + key) * D + slice * NV + ch;
-  const int uc = NV == kNV ? 0 : (slice & 1) * NV;       // first channel within the record's U slice
+  const int uc = slice % (kNV / NV) * NV;       // first channel within the record's U slice
   float h[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) h[e] = 0.f;
@@ -563,9 +563,11 @@ cudaError_t run(const Problem& p, const Fp32Params& fp, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
   }
   timer_mark(stream, "simt_prefill");
-  // Slices of 8 channels while that leaves every CTA an SM (a chunk then takes about 0.6 of the time), else of 16 (fewer
-  // reads of the shared operands per channel).
+  // The narrowest slices that leave every CTA an SM: a chunk takes 2.2 us with 8 channels and 1.6 with 4 (d = 64); else 16
+  // (fewer reads of the shared operands per channel).
   const long long heads = (long long)p.N * p.HV;
+  if (heads * (D / 4) <= 148)
+    return launch<fp32_walk_kernel<In, D, 4>>((unsigned)(heads * (D / 4)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
   if (heads * (D / 8) <= 148)
     return launch<fp32_walk_kernel<In, D, 8>>((unsigned)(heads * (D / 8)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
   return launch<fp32_walk_kernel<In, D, 16>>((unsigned)(heads * (D / 16)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);

@@ -26,3 +26,11 @@ def test_fp32_kda_strong_decay_inside_a_block():
     for tok in (5, 37, 70, 71):
         inp["g"][tok, :, ::7] = -90.0
     helpers.check_parity(inp)
+
+
+@pytest.mark.parametrize("dtype,d,lens,hk,hv", [("fp32", 64, [65, 64, 1], 2, 4), ("bf16", 64, [100, 130], 5, 5),
+                                                ("fp32", 128, [40, 70], 4, 4), ("fp32", 64, [150], 9, 9)])
+def test_fp32_slice_widths(dtype, d, lens, hk, hv):
+    """Numbers of heads on either side of where the sequential kernel's slices get wider."""
+    w = synth.shrink(W["gdn_varlen"], seq_lens=lens, hk=hk, hv=hv, dtype=dtype, dk=d, dv=d, h0_std=0.05, varlen=len(lens) > 1)
+    helpers.check_parity(synth.make_inputs(w, seed=239))
