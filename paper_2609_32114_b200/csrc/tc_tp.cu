@@ -23,6 +23,10 @@
 // operator anyway); this assumes the delta rule's usual normalisation (beta |k|^2 of order one), far inside the fp16
 // range, and a result outside it is reported.
 //
+// What bounds it: the solve's dependent phases and the instructions of the masks (10 k warp instructions per unit, 5.6 k
+// SM-cycles with two units in flight).  Measured on B200, with the W, U, Q~ and O_loc images of 64-token chunks before: 16
+// heads, T = 4096 36 -> 21 us; 32 heads, T = 16384 188 -> 91; 8 sequences of 136 k tokens, 16 heads 800 -> 384.
+//
 // Tokens past the end of a sequence are made no-ops by beta = 0 and g = 0; whatever the TMA box read for them (the
 // next sequence's rows, or zero fill past the end of the tensor) is multiplied by exact zeros.  This relies on the
 // inputs being finite.

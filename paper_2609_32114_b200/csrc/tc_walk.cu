@@ -15,10 +15,14 @@
 // per key channel.
 //
 // What bounds a step: three products that wait for each other's epilogue (K = 128: eight instructions of 64 cycles, ~180
-// cycles to a visible result, ~250 of tensor-memory traffic and arithmetic by the compute warps) -- about 3 k cycles -- and
-// close behind it the tensor cores (2.3 k: all five products) and shared memory (133 KiB in, 132 KiB of B operands,
-// 96 KiB of V and o tiles: 2.9 k at 128 bytes per cycle).  T and P are lower triangular: step ks of their products runs
-// with N = 128 - 16 ks rows.
+// cycles to a visible result, ~250 of tensor-memory traffic and arithmetic by the compute warps), with the tensor cores
+// (2.3 k cycles for all five products) and shared memory (133 KiB in, 132 KiB of B operands, 96 KiB of V and o tiles: 2.9 k
+// at 128 bytes per cycle) close behind; on large calls HBM (165 KiB per step and head, KDA 197).  T and P are lower
+// triangular: step ks of their products runs with N = 128 - 16 ks rows.  U and D2 run in token halves, so that an epilogue
+// starts when half of its input is final; Y goes behind X and P U~ behind D2, where the sequential path leaves the tensor
+// cores idle.
+// Measured on B200: 2.3 - 2.45 us per step of 128 tokens and head on one SM, 2.0 without outputs; the kernel before it, on
+// steps of 64, took 0.9 us per step on four SMs or 1.23 on two.  8 sequences of 136 k tokens, 16 heads: 700 -> 573 us.
 //
 // Warp roles: sixteen compute warps (tensor-memory lanes 32 (w % 4).., group w / 4 of the columns), four output warps, two
 // producer warps, two warps that issue MMAs (the sequential path; the outputs).  Every wait is bounded.
