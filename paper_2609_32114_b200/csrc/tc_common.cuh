@@ -49,7 +49,8 @@ inline __host__ size_t tc_seg_bytes(size_t nj, int nseg, size_t rows, int HV) {
 }
 
 // Scratch of a call whose sequences are cut into spans: per (sequence, V-head) and span the offset b_s, which the span's
-// true start state h_s replaces, and the transition Phi_s (fp32 128 x 128 each, [key][value channel]).
+// true start state h_s replaces, and the transition Phi_s (fp32 128 x 128 each, [key][value channel]; span 0 has none: its
+// place keeps h0 in a call that works in place).
 struct SpanBuffers {
   int nspan;            // 1: off
   float* b;

@@ -78,6 +78,8 @@ struct WalkParams {
   // span_fix_kernel (tc_span.cu) between them.  The state recurrence is affine in the start state, so
   //   first launch, state only (OUT = false): spans 0 .. nspan-2 from their own start (span 0: h0, others: zero) into
   //     span_b, and spans 1 .. nspan-2 from the IDENTITY with V = 0 (the transition) into span_phi;
+  //     in place (hT = h0), span 0 also leaves h0 in span_phi[0], which no transition uses: the second launch's last
+  //     span may have stored hT before a CTA of its span 0 gets an SM;
   //   fix: h_1 = b_0, h_{s+1} = Phi_s h_s + b_s,  in place of b_{s+1};
   //   second launch (OUT = true): every span from its true start, outputs and final state.
   int nspan;
@@ -427,11 +429,17 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     const uint32_t tq = tmem + (static_cast<uint32_t>(q * 32) << 16);
     float h[32];                                         // h^T[v][32 g ..]
     {
+      const size_t nh = (size_t)n * p.HV + j;
+      float* const kept = p.nspan > 1 && p.h0 && p.h0 == p.hT && span == 0 && !trans ? p.span_phi + nh * p.nspan * 16384 : nullptr;
       const float* src = nullptr;
-      if (span == 0 && !trans) src = p.h0 ? p.h0 + ((size_t)n * p.HV + j) * 16384 : nullptr;
-      else if (OUT) src = p.span_b + (((size_t)n * p.HV + j) * p.nspan + span) * 16384;
+      if (span == 0 && !trans) src = OUT && kept ? kept : p.h0 ? p.h0 + nh * 16384 : nullptr;
+      else if (OUT) src = p.span_b + (nh * p.nspan + span) * 16384;
 #pragma unroll
       for (int k = 0; k < 32; ++k) h[k] = src ? src[(size_t)(32 * g + k) * 128 + v] : (trans && 32 * g + k == v ? 1.f : 0.f);
+      if (!OUT && kept) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) kept[(size_t)(32 * g + k) * 128 + v] = h[k];
+      }
     }
     auto step_h = [&](int k, float2 decay, float2 add) {
       const float2 x = fma2(decay, make_float2(h[k], h[k + 1]), add);

@@ -44,3 +44,28 @@ def test_kda_strong_decay(log_gate):
         inp["g"][tok, :, ::7] = log_gate
     inp["g"][140:190, :, 3::11] = log_gate
     helpers.check_parity(inp)
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("runs,lens,hv", [(8, [1500, 100, 1, 0, 700, 130, 900], 8), (4, [0, 3000, 129, 1, 513], 16), (2, [5, 2000], 2)])
+def test_runs_in_place(variant, runs, lens, hv, monkeypatch):
+    """h0 = hT with sequences cut into runs, some shorter than the number of runs (their last runs are empty and have the end
+    state at once), with more CTAs than SMs in all but the last case: the same call out of place, bit for bit, every time."""
+    import torch
+    import paper_2609_32114_b200 as ha
+
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
+    inp = _inputs(variant, lens, True, hv // 2, hv, 359)
+    d = helpers.to_device(inp)
+    a, keep = ha.prepare_args(d["q"], d["k"], d["v"], d["g"], d["beta"], variant=variant, h0=d["h0"],
+                              cu_seqlens=d["cu_seqlens"], max_seqlen=d["max_seqlen"])
+    assert ha.ha_la_prefill_num_launches(a) == 5           # plan, chunk-local, states only, start states, outputs
+    assert ha.ha_la_prefill_raw(a, torch.cuda.current_stream().cuda_stream) == 0
+    for _ in range(8):
+        state = d["h0"].clone()
+        o, hT, st, _ = ha.ha_la_prefill(d["q"], d["k"], d["v"], d["g"], d["beta"], variant=variant, h0=state, hT=state,
+                                        cu_seqlens=d["cu_seqlens"], max_seqlen=d["max_seqlen"], workspace=keep["workspace"])
+        torch.cuda.synchronize()
+        assert hT is state and int(st.item()) == 0 and int(keep["status_word"].item()) == 0
+        assert torch.equal(o, keep["o"][0]) and torch.equal(state, keep["hT"])
+    helpers.check_parity(inp)
