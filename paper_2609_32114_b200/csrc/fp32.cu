@@ -392,11 +392,6 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   const int tid = threadIdx.x, part = tid & 7, ch0 = ((tid >> 3) & 1) * H, grp = tid >> 4;
   const int row = part >> 1, ch = ch0 + (part & 1) * E;   // this thread's row of four and first channel, once summed up
   const int slice = blockIdx.x % NSL, nj = blockIdx.x / NSL, j = nj % p.HV;
-  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;
-  const int tok0 = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
-  const int len = p.seq_tok0 ? p.seq_len[n] : p.T_row;
-  const int slot0 = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
-  const int nch = (len + C - 1) / C;
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) { mbar_init(&bar1[i], 1); mbar_init(&bar3[i], 1); }
     mbar_fence_init();
@@ -404,13 +399,19 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   // state: thread -> key 4 grp + row, its E channels of the slice
   const bool upd = tid < kUpd<D>;
   const int key = 4 * grp + row;
-  const size_t hbase = (((size_t)n * p.HV + j) * D + key) * D + slice * NV + ch;
   const int uc = slice % (kNV / NV) * NV;       // first channel within the record's U slice
   float h[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) h[e] = 0.f;
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // (the plan kernel's tables among what is read from here on: a batch without a token has no kernel between that one and this)
+  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;
+  const int tok0 = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
+  const int len = p.seq_tok0 ? p.seq_len[n] : p.T_row;
+  const int slot0 = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
+  const int nch = (len + C - 1) / C;
+  const size_t hbase = (((size_t)n * p.HV + j) * D + key) * D + slice * NV + ch;
   if (upd) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {

@@ -139,19 +139,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   const int nj = blockIdx.x / units;
   const bool trans = !OUT && unit >= p.nspan - 1;        // a transition run
   const int span = trans ? unit - p.nspan + 2 : unit;
-  const int j = nj % p.HV;
-  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;   // CTAs of the longest sequences come first
-  const int jq = j / (p.HV / p.HK);
-  const int tok0_seq = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
-  const int len_seq = p.seq_tok0 ? p.seq_len[n] : p.T_row;
-  const int slot0_seq = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
-  // this CTA's span of the sequence, walked like a sequence of its own
-  const int nst_seq = (len_seq + kStep - 1) / kStep;
-  const int spspan = (nst_seq + p.nspan - 1) / p.nspan;
-  const int tok0 = tok0_seq + span * spspan * kStep;
-  const int len = max(0, min(len_seq - span * spspan * kStep, spspan * kStep));
-  const int slot0 = slot0_seq + span * spspan;
-  const int nsteps = (len + kStep - 1) / kStep;
 
   if (tid == 0) {
     for (int i = 0; i < 20; ++i) {
@@ -171,6 +158,22 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   // This kernel may be launched as a programmatic dependent of the prep kernel, i.e. start while that one is still
   // running.  Sequential mode: everything above overlapped the prep kernel's tail; wait for it here.
   if (p.epoch == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // (The plan kernel's tables too are read behind the wait only: in a batch without a token there is no chunk-local kernel
+  // between that kernel, which lets its dependents go before it writes them, and this one.)
+  const int j = nj % p.HV;
+  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;   // CTAs of the longest sequences come first
+  const int jq = j / (p.HV / p.HK);
+  const int tok0_seq = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
+  const int len_seq = p.seq_tok0 ? p.seq_len[n] : p.T_row;
+  const int slot0_seq = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
+  // this CTA's span of the sequence, walked like a sequence of its own
+  const int nst_seq = (len_seq + kStep - 1) / kStep;
+  const int spspan = (nst_seq + p.nspan - 1) / p.nspan;
+  const int tok0 = tok0_seq + span * spspan * kStep;
+  const int len = max(0, min(len_seq - span * spspan * kStep, spspan * kStep));
+  const int slot0 = slot0_seq + span * spspan;
+  const int nsteps = (len + kStep - 1) / kStep;
 
   // Concurrent mode: a whole warp looks at the ready flags of the next 32 steps at once (plain loads) and remembers how
   // far the prep kernel has got; the acquire fence and the proxy fence, which are what makes the published results

@@ -69,3 +69,30 @@ def test_runs_in_place(variant, runs, lens, hv, monkeypatch):
         assert hT is state and int(st.item()) == 0 and int(keep["status_word"].item()) == 0
         assert torch.equal(o, keep["o"][0]) and torch.equal(state, keep["hT"])
     helpers.check_parity(inp)
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("bf16", 64), ("fp32", 128)])
+@pytest.mark.parametrize("seqs", [1, 2])
+def test_packed_batch_without_a_token(variant, dtype, d, seqs):
+    """Through the C ABI (torch has no pointers for empty tensors): a packed batch of empty sequences hands the states on.  With
+    one sequence there are no chunk slots, so nothing runs between the plan kernel and the state-passing kernel."""
+    import torch
+    import paper_2609_32114_b200 as ha
+
+    any_ = torch.zeros(4096, device="cuda")                # in the place of q, k, v, g, beta, o: no token of them is touched
+    cu = torch.zeros(seqs + 1, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    h0 = torch.randn(seqs, 3, d, d, device="cuda")
+    p = any_.data_ptr()
+    for start in (h0, None):
+        hT = torch.full_like(h0, float("nan"))
+        a = ha.make_args(variant=variant, dtype=dtype, batch=1, seqlen=0, hk=1, hv=3, dk=d, dv=d, num_seqs=seqs, q=p, k=p, v=p, g=p,
+                         beta=p, o=p, h0=0 if start is None else start.data_ptr(), cu_seqlens=cu.data_ptr(), hT=hT.data_ptr(),
+                         status_word=status.data_ptr())
+        need = ha.ha_la_prefill_workspace_bytes(a)
+        ws = torch.full((need + 256,), 0x7f, dtype=torch.uint8, device="cuda")    # lengths of two thousand million, if they were read
+        a.workspace, a.workspace_bytes = (ws.data_ptr() + 255) // 256 * 256, need
+        assert ha.ha_la_prefill_raw(a, torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and torch.equal(hT, torch.zeros_like(h0) if start is None else start)

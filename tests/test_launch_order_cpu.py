@@ -1,0 +1,33 @@
+"""Kernels that are launched as programmatic dependents may run before the kernel ahead of them in the stream has written
+anything, so each has to execute griddepcontrol.wait before its first access to what another kernel writes: the plan kernel's
+tables above all, which lie in workspace memory that holds anything until then.  Checked on the sources, without a GPU."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_32114_b200", "csrc")
+TABLES = r"\b(?:seq_order|seq_tok0|seq_len|seq_chunk0|chunk_seq|chunk_tok0|chunk_len|cu)\s*\["
+INPUTS = r"\bp\.(?:q|k|v|g|beta|h0|h_in|o|hT|h_out|rec)\s*\["
+
+
+def _kernels():
+    for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        src = re.sub(r"//[^\n]*", "", open(f).read())
+        for part in src.split("__global__")[1:]:
+            name = re.search(r"(\w+_kernel)\s*\(", part)
+            if name and "griddepcontrol.wait" in part:
+                yield os.path.basename(f), name.group(1), part
+
+
+def test_the_dependent_kernels_are_found():
+    names = {k for _, k, _ in _kernels()}
+    assert {"plan_kernel", "tc_tp_kernel", "tc_kda_kernel", "tc_walk_kernel", "span_fix_kernel", "fp32_prep_kernel",
+            "fp32_walk_kernel", "decode_kernel"} <= names
+
+
+@pytest.mark.parametrize("file,kernel,body", list(_kernels()), ids=lambda x: x if isinstance(x, str) and len(x) < 30 else "")
+def test_nothing_is_read_before_the_wait(file, kernel, body):
+    before = body[:body.index("griddepcontrol.wait")]
+    assert re.findall(TABLES, before) == [] and re.findall(INPUTS, before) == [], f"{kernel} in {file}"
