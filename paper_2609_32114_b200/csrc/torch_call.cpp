@@ -133,7 +133,9 @@ PyObject* prefill(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int rc = g_prefill_bytes(&d, &need);
   if (rc != HA_LA_OK) Py_RETURN_NONE;                     // (binding.py words the error)
   at::Tensor o_new, h_new, w_new, s_new;
-  const bool want_hT = a[13] == Py_True;
+  // (asked for its truth value only where the call has to know: when it brings no hT)
+  const int want_hT = hT ? 0 : PyObject_IsTrue(a[13]);
+  if (want_hT < 0) return nullptr;
   try {
     if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
     if (!hT && want_hT) { h_new = at::empty({N, v->size(2), q->size(3), v->size(3)}, g->options()); hT = &h_new; }

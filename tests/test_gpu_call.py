@@ -82,3 +82,35 @@ def test_decode_steps_queued_in_place(variant, dtype, d, n, hk, hv):
     o = torch.stack(outs, 1).float().cpu().numpy().reshape(o_ref.shape)
     assert helpers.rel_max_err(o, o_ref) <= helpers.TOL[dtype]
     assert helpers.rel_max_err(state.cpu().numpy().astype(np.float64), h_ref) <= 1e-5
+
+
+@pytest.mark.parametrize("want,given", [(1, True), (0, False), ("numpy", True), ([], False)])
+def test_want_hT_is_any_true_value(want, given):
+    import numpy as np
+    import torch
+    import paper_2609_32114_b200 as ha
+
+    t = _inputs()
+    ref = ha.ha_la_prefill(*t)
+    r = ha.ha_la_prefill(*t, want_hT=np.bool_(True) if want == "numpy" else want)
+    torch.cuda.synchronize()
+    assert (r[1] is not None) == given and torch.equal(r[0], ref[0])
+    if given:
+        assert torch.equal(r[1], ref[1])
+
+
+def test_want_hT_is_not_asked_of_a_call_that_brings_its_own():
+    """An object without a truth value is an error where the call has to know (as it is in Python), and only there."""
+    import torch
+    import paper_2609_32114_b200 as ha
+
+    class NoTruth:
+        def __bool__(self):
+            raise ValueError("no truth value")
+
+    t = _inputs()
+    with pytest.raises(ValueError):
+        ha.ha_la_prefill(*t, want_hT=NoTruth())
+    mine = torch.empty_like(ha.ha_la_prefill(*t)[1])
+    assert ha.ha_la_prefill(*t, hT=mine, want_hT=NoTruth())[1] is mine
+    torch.cuda.synchronize()
