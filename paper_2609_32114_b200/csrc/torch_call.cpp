@@ -7,6 +7,7 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "ha_la.h"
@@ -52,7 +53,7 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 // decode(q, k, v, g, beta, state, stream, kda, scale, o, state_out) -> (o, state_out) | status | None
-PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
+PyObject* decode_call(PyObject* const* a, Py_ssize_t n) {
   if (n != 11 || !g_decode) { PyErr_SetString(PyExc_TypeError, "eleven arguments"); return nullptr; }
   const at::Tensor *q, *k, *v, *g, *beta, *st, *o, *so;
   const bool kda = a[7] == Py_True;
@@ -70,15 +71,10 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
   d.scale = (float)PyFloat_AsDouble(a[8]);
   if (PyErr_Occurred()) return nullptr;
   at::Tensor o_new, s_new;
-  try {
-    if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
-    if (!so) {
-      if (st) so = st;
-      else { s_new = at::empty({d.num_seqs, d.num_v_heads, d.d_k, d.d_k}, g->options()); so = &s_new; }
-    }
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
+  if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
+  if (!so) {
+    if (st) so = st;
+    else { s_new = at::empty({d.num_seqs, d.num_v_heads, d.d_k, d.d_k}, g->options()); so = &s_new; }
   }
   d.q = ptr(q); d.k = ptr(k); d.v = ptr(v);
   d.g = (const float*)ptr(g); d.beta = (const float*)ptr(beta);
@@ -100,7 +96,7 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 // prefill(q, k, v, g, beta, h0, cu_seqlens, max_seqlen, stream, kda, scale, o, hT, want_hT, workspace, status_word)
 //   -> (o, hT | None, status_word, workspace) | status | None
-PyObject* prefill(PyObject*, PyObject* const* a, Py_ssize_t n) {
+PyObject* prefill_call(PyObject* const* a, Py_ssize_t n) {
   if (n != 16 || !g_prefill) { PyErr_SetString(PyExc_TypeError, "sixteen arguments"); return nullptr; }
   const at::Tensor *q, *k, *v, *g, *beta, *h0, *cu, *o, *hT, *ws, *sw;
   if (a[9] != Py_True && a[9] != Py_False) Py_RETURN_NONE;
@@ -136,15 +132,10 @@ PyObject* prefill(PyObject*, PyObject* const* a, Py_ssize_t n) {
   // (asked for its truth value only where the call has to know: when it brings no hT)
   const int want_hT = hT ? 0 : PyObject_IsTrue(a[13]);
   if (want_hT < 0) return nullptr;
-  try {
-    if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
-    if (!hT && want_hT) { h_new = at::empty({N, v->size(2), q->size(3), v->size(3)}, g->options()); hT = &h_new; }
-    if (!ws) { w_new = at::empty({(int64_t)need + 256}, g->options().dtype(at::kByte)); ws = &w_new; }
-    if (!sw) { s_new = at::zeros({1}, g->options().dtype(at::kInt)); sw = &s_new; }
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
-  }
+  if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
+  if (!hT && want_hT) { h_new = at::empty({N, v->size(2), q->size(3), v->size(3)}, g->options()); hT = &h_new; }
+  if (!ws) { w_new = at::empty({(int64_t)need + 256}, g->options().dtype(at::kByte)); ws = &w_new; }
+  if (!sw) { s_new = at::zeros({1}, g->options().dtype(at::kInt)); sw = &s_new; }
   d.o = ptr(o); d.hT = (float*)ptr(hT); d.status_word = (int32_t*)ptr(sw);
   const uintptr_t base = (uintptr_t)ws->data_ptr(), al = (base + 255) / 256 * 256;
   d.workspace = (void*)al;
@@ -164,10 +155,20 @@ PyObject* prefill(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return r;
 }
 
+// torch's C++ calls throw (no memory, no driver, a tensor without storage).  An exception that left these functions would go
+// through the interpreter's C frames and end the process; torch's own translation gives the caller the type that the same
+// call raises in Python.
+template <PyObject* (*call)(PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  return call(a, n);
+  END_HANDLE_TH_ERRORS
+}
+
 PyMethodDef kMethods[] = {
     {"bind", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&bind)), METH_FASTCALL, nullptr},
-    {"decode", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&decode)), METH_FASTCALL, nullptr},
-    {"prefill", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&prefill)), METH_FASTCALL, nullptr},
+    {"decode", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&guarded<decode_call>)), METH_FASTCALL, nullptr},
+    {"prefill", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(&guarded<prefill_call>)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "ha_la_torch_call", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 
