@@ -523,7 +523,10 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
     __syncthreads();                                     // the new state is complete; KD, P, U~ and QG h are free
     if (tid == 0 && c + ST < nch) load3(c + ST);
   }
-  if (gave_up) report_status(p.status, HA_LA_ERR_TIMEOUT);
+  if (gave_up) {
+    report_status(p.status, HA_LA_ERR_TIMEOUT);
+    settle_copies();
+  }
   if (p.hT && upd) {
 #pragma unroll
     for (int e = 0; e < E; ++e) p.hT[hbase + e] = h[e];

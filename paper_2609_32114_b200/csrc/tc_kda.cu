@@ -386,7 +386,10 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
       gm = geom(item);
     }
   }
-  if (tid == 256 && *abort_flag) report_status(p.status, HA_LA_ERR_TIMEOUT);
+  if (tid == 256 && *abort_flag) {
+    report_status(p.status, HA_LA_ERR_TIMEOUT);
+    settle_copies();
+  }
 }
 
 }  // namespace

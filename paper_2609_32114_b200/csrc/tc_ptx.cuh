@@ -67,6 +67,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// For a CTA in which a wait ran out: gives its copies that may still be in flight time to land (64 us and more), so that
+// they do not end in the shared memory of whatever runs on this SM next.
+__device__ __forceinline__ void settle_copies() {
+  for (int i = 0; i < 64; ++i) __nanosleep(1000);
+}
+
 // ---------------------------------------------------------------- proxies and fences
 
 __device__ __forceinline__ void fence_proxy_async_smem() {

@@ -128,7 +128,10 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
         h[n][e] = make_float2(o[n][e].x + (c[n][0][2 * e] + (c[n][1][2 * e] + c[n][2][2 * e])),
                               o[n][e].y + (c[n][0][2 * e + 1] + (c[n][1][2 * e + 1] + c[n][2][2 * e + 1])));
   }
-  if (threadIdx.x == 0 && *abort_flag) report_status(status, HA_LA_ERR_TIMEOUT);
+  if (threadIdx.x == 0 && *abort_flag) {
+    report_status(status, HA_LA_ERR_TIMEOUT);
+    settle_copies();
+  }
 }
 
 }  // namespace

@@ -318,7 +318,10 @@ tc_tp_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     }
     s = sn; jq = jqn; L = Ln; tok0 = tok0n; have = haven;
   }
-  if (tid == 0 && *abort_flag) report_status(p.status, HA_LA_ERR_TIMEOUT);
+  if (tid == 0 && *abort_flag) {
+    report_status(p.status, HA_LA_ERR_TIMEOUT);
+    settle_copies();
+  }
   tc_fence_before_sync();
   __syncthreads();
   if (threadIdx.x < 32) tmem_dealloc(*tmem_slot, 512);

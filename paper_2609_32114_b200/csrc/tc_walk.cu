@@ -639,9 +639,9 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   tc_fence_before_sync();
   __syncthreads();
   if (*abort_flag) {
-    // A wait ran out: the producers have stopped; give copies that were still in flight time to land.
+    // A wait ran out: the producers have stopped.
     if (tid == 0) report_status(p.status, HA_LA_ERR_TIMEOUT);
-    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    settle_copies();
   }
   // Concurrent mode: do not finish before the prep grid has (it has published its last step by now), so that
   // work queued behind this kernel is also behind the prep kernel.

@@ -1,6 +1,9 @@
-"""Kernels that are launched as programmatic dependents may run before the kernel ahead of them in the stream has written
+"""What a kernel owes the ones around it, checked on the sources, without a GPU.
+
+Kernels that are launched as programmatic dependents may run before the kernel ahead of them in the stream has written
 anything, so each has to execute griddepcontrol.wait before its first access to what another kernel writes: the plan kernel's
-tables above all, which lie in workspace memory that holds anything until then.  Checked on the sources, without a GPU."""
+tables above all, which lie in workspace memory that holds anything until then.  And a kernel in which a bounded wait ran out
+lets its own copies land before it gives its shared memory back."""
 import glob
 import os
 import re
@@ -31,3 +34,13 @@ def test_the_dependent_kernels_are_found():
 def test_nothing_is_read_before_the_wait(file, kernel, body):
     before = body[:body.index("griddepcontrol.wait")]
     assert re.findall(TABLES, before) == [] and re.findall(INPUTS, before) == [], f"{kernel} in {file}"
+
+
+def test_a_kernel_that_gave_up_waiting_lets_its_copies_land():
+    found = 0
+    for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        src = re.sub(r"//[^\n]*", "", open(f).read())
+        for m in re.finditer(r"report_status\([^;]*HA_LA_ERR_TIMEOUT\);", src):
+            assert src[m.end():].split("}")[0].strip() == "settle_copies();", os.path.basename(f)
+            found += 1
+    assert found == 5                                      # every kernel that copies in bulk
