@@ -392,6 +392,8 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   const int tid = threadIdx.x, part = tid & 7, ch0 = ((tid >> 3) & 1) * H, grp = tid >> 4;
   const int row = part >> 1, ch = ch0 + (part & 1) * E;   // this thread's row of four and first channel, once summed up
   const int slice = blockIdx.x % NSL, nj = blockIdx.x / NSL, j = nj % p.HV;
+  const bool packed = p.seq_tok0 != nullptr;
+  int n = nj / p.HV, tok0 = packed ? 0 : n * p.T_row, slot0 = packed ? 0 : n * p.cps, len = p.T_row, nch = (len + C - 1) / C;
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) { mbar_init(&bar1[i], 1); mbar_init(&bar3[i], 1); }
     mbar_fence_init();
@@ -405,12 +407,13 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   for (int e = 0; e < E; ++e) h[e] = 0.f;
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  // (the plan kernel's tables among what is read from here on: a batch without a token has no kernel between that one and this)
-  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;
-  const int tok0 = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
-  const int len = p.seq_tok0 ? p.seq_len[n] : p.T_row;
-  const int slot0 = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
-  const int nch = (len + C - 1) / C;
+  if (packed) {                                          // (a batch without a token has no kernel between the plan kernel and this one)
+    if (p.seq_order) n = p.seq_order[n];
+    tok0 = p.seq_tok0[n];
+    slot0 = p.seq_chunk0[n];
+    len = p.seq_len[n];
+    nch = (len + C - 1) / C;
+  }
   const size_t hbase = (((size_t)n * p.HV + j) * D + key) * D + slice * NV + ch;
   if (upd) {
 #pragma unroll

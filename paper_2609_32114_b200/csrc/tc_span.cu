@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
   const float* phi = sb.phi + (size_t)nj * sb.nspan * stride;
   const size_t tile = (size_t)nj * sb.nspan * stride + (size_t)r0 * 128 + blockIdx.y * kFixCols + 2 * t;
   float* b = sb.b + tile;                                // h_s replaces b_s: the same thread reads the one and writes the other
+  const int32_t* my_len = seq_len ? seq_len + nj / HV : nullptr;
   if (threadIdx.x == 0) {
     mbar_init(&full[0], 1);
     mbar_init(&full[1], 1);
@@ -48,7 +49,7 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
   asm volatile("griddepcontrol.wait;" ::: "memory");     // (launched as a programmatic dependent of the states-only walk)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // spans past the end of a short sequence are empty: the state passes through untouched, bit for bit
-  const int len = seq_len ? seq_len[nj / HV] : T_row;
+  const int len = my_len ? *my_len : T_row;              // (another kernel's table: read behind the wait)
   const int nst = (len + kStep - 1) / kStep;
   const int spspan = (nst + sb.nspan - 1) / sb.nspan;
   auto fetch = [&](int s) {                              // one thread

@@ -60,7 +60,8 @@ struct WalkCfg {
 };
 
 struct WalkParams {
-  const float* h0;
+  const float* h0;             // start states, h0_stride floats from one (sequence, V-head) to the next, or NULL (zeros)
+  size_t h0_stride;
   float* hT;
   void* o;
   const int32_t* seq_tok0;     // per-sequence table of the plan kernel, or NULL for equal-length rows
@@ -78,11 +79,12 @@ struct WalkParams {
   // span_fix_kernel (tc_span.cu) between them.  The state recurrence is affine in the start state, so
   //   first launch, state only (OUT = false): spans 0 .. nspan-2 from their own start (span 0: h0, others: zero) into
   //     span_b, and spans 1 .. nspan-2 from the IDENTITY with V = 0 (the transition) into span_phi;
-  //     in place (hT = h0), span 0 also leaves h0 in span_phi[0], which no transition uses: the second launch's last
-  //     span may have stored hT before a CTA of its span 0 gets an SM;
+  //     in place (hT = h0), span 0 also leaves h0 in span_phi[0], which no transition uses, for the second launch to
+  //     start from: its last span may have stored hT before a CTA of its span 0 gets an SM;
   //   fix: h_1 = b_0, h_{s+1} = Phi_s h_s + b_s,  in place of b_{s+1};
   //   second launch (OUT = true): every span from its true start, outputs and final state.
   int nspan;
+  bool keep_h0;
   float* span_b;               // [N*HV][nspan][128 keys][128 channels] fp32
   float* span_phi;
   int32_t* status;
@@ -139,6 +141,18 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   const int nj = blockIdx.x / units;
   const bool trans = !OUT && unit >= p.nspan - 1;        // a transition run
   const int span = trans ? unit - p.nspan + 2 : unit;
+  const int j = nj % p.HV, jq = j / (p.HV / p.HK);
+  const bool packed = p.seq_tok0 != nullptr;
+  int n = nj / p.HV, tok0 = packed ? 0 : n * p.T_row, len = p.T_row, slot0 = packed ? 0 : n * p.cps, nsteps;
+  auto take_span = [&]() {                               // this CTA's span of the sequence, walked like a sequence of its own
+    const int nst = (len + kStep - 1) / kStep;
+    const int spspan = (nst + p.nspan - 1) / p.nspan;
+    tok0 += span * spspan * kStep;
+    slot0 += span * spspan;
+    len = max(0, min(len - span * spspan * kStep, spspan * kStep));
+    nsteps = (len + kStep - 1) / kStep;
+  };
+  take_span();
 
   if (tid == 0) {
     for (int i = 0; i < 20; ++i) {
@@ -159,21 +173,15 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   // running.  Sequential mode: everything above overlapped the prep kernel's tail; wait for it here.
   if (p.epoch == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // (The plan kernel's tables too are read behind the wait only: in a batch without a token there is no chunk-local kernel
-  // between that kernel, which lets its dependents go before it writes them, and this one.)
-  const int j = nj % p.HV;
-  const int n = p.seq_order ? p.seq_order[nj / p.HV] : nj / p.HV;   // CTAs of the longest sequences come first
-  const int jq = j / (p.HV / p.HK);
-  const int tok0_seq = p.seq_tok0 ? p.seq_tok0[n] : n * p.T_row;
-  const int len_seq = p.seq_tok0 ? p.seq_len[n] : p.T_row;
-  const int slot0_seq = p.seq_tok0 ? p.seq_chunk0[n] : n * p.cps;
-  // this CTA's span of the sequence, walked like a sequence of its own
-  const int nst_seq = (len_seq + kStep - 1) / kStep;
-  const int spspan = (nst_seq + p.nspan - 1) / p.nspan;
-  const int tok0 = tok0_seq + span * spspan * kStep;
-  const int len = max(0, min(len_seq - span * spspan * kStep, spspan * kStep));
-  const int slot0 = slot0_seq + span * spspan;
-  const int nsteps = (len + kStep - 1) / kStep;
+  if (packed) {
+    // (These tables too are read behind the wait only: in a batch without a token there is no chunk-local kernel between the
+    // plan kernel, which lets its dependents go before it writes them, and this one.)
+    if (p.seq_order) n = p.seq_order[n];                 // CTAs of the longest sequences come first
+    tok0 = p.seq_tok0[n];
+    len = p.seq_len[n];
+    slot0 = p.seq_chunk0[n];
+    take_span();
+  }
 
   // Concurrent mode: a whole warp looks at the ready flags of the next 32 steps at once (plain loads) and remembers how
   // far the prep kernel has got; the acquire fence and the proxy fence, which are what makes the published results
@@ -432,16 +440,15 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     const uint32_t tq = tmem + (static_cast<uint32_t>(q * 32) << 16);
     float h[32];                                         // h^T[v][32 g ..]
     {
-      const size_t nh = (size_t)n * p.HV + j;
-      float* const kept = p.nspan > 1 && p.h0 && p.h0 == p.hT && span == 0 && !trans ? p.span_phi + nh * p.nspan * 16384 : nullptr;
       const float* src = nullptr;
-      if (span == 0 && !trans) src = OUT && kept ? kept : p.h0 ? p.h0 + nh * 16384 : nullptr;
-      else if (OUT) src = p.span_b + (nh * p.nspan + span) * 16384;
+      if (span == 0 && !trans) src = p.h0 ? p.h0 + ((size_t)n * p.HV + j) * p.h0_stride : nullptr;
+      else if (OUT) src = p.span_b + (((size_t)n * p.HV + j) * p.nspan + span) * 16384;
 #pragma unroll
       for (int k = 0; k < 32; ++k) h[k] = src ? src[(size_t)(32 * g + k) * 128 + v] : (trans && 32 * g + k == v ? 1.f : 0.f);
-      if (!OUT && kept) {
+      if (!OUT && p.keep_h0 && span == 0 && !trans) {
+        float* keep = p.span_phi + ((size_t)n * p.HV + j) * p.nspan * 16384;
 #pragma unroll
-        for (int k = 0; k < 32; ++k) kept[(size_t)(32 * g + k) * 128 + v] = h[k];
+        for (int k = 0; k < 32; ++k) keep[(size_t)(32 * g + k) * 128 + v] = h[k];
       }
     }
     auto step_h = [&](int k, float2 decay, float2 add) {
@@ -683,7 +690,11 @@ cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanVi
                            bool dependent, uint32_t spin_limit, const SpanBuffers& sb, bool states_only,
                            cudaStream_t stream) {
   WalkParams wp;
-  wp.h0 = a.h0; wp.hT = a.hT; wp.o = a.o;
+  const bool in_place = sb.nspan > 1 && a.h0 && a.h0 == a.hT;
+  wp.keep_h0 = in_place && states_only;
+  wp.h0 = in_place && !states_only ? sb.phi : a.h0;
+  wp.h0_stride = in_place && !states_only ? (size_t)sb.nspan * 16384 : 16384;
+  wp.hT = a.hT; wp.o = a.o;
   wp.seq_tok0 = plan.seq_tok0; wp.seq_len = plan.seq_len; wp.seq_chunk0 = plan.seq_chunk0;
   wp.seq_order = plan.seq_tok0 ? plan.seq_order : nullptr;
   wp.T_row = p.T_row; wp.cps = p.max_seq_chunks > 0 ? p.max_seq_chunks : 1;

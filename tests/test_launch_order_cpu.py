@@ -11,7 +11,7 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_32114_b200", "csrc")
-TABLES = r"\b(?:seq_order|seq_tok0|seq_len|seq_chunk0|chunk_seq|chunk_tok0|chunk_len|cu)\s*\["
+TABLES = r"\b(?:seq_order|seq_tok0|seq_len|seq_chunk0|chunk_seq|chunk_tok0|chunk_len|cu)\s*\[|\*my_len"
 INPUTS = r"\bp\.(?:q|k|v|g|beta|h0|h_in|o|hT|h_out|rec)\s*\["
 
 
