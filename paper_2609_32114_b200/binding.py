@@ -231,7 +231,7 @@ def ha_la_prefill_noalloc(args: ha_la_prefill_args, stream: int = 0) -> int:
 
 
 def ha_la_debug_wait_timeout(args: ha_la_prefill_args, stream: int = 0, spin_limit: int = 4096) -> int:
-    """Test hook: the sequential kernel alone, waiting for flags nothing publishes; returns the status code."""
+    """Test hook: the sequential kernel alone with its copies withheld, so that its waits run out; returns the status code."""
     return load_library().ha_la_debug_wait_timeout(ctypes.byref(args), ctypes.c_void_p(stream) if stream else None,
                                                    ctypes.c_uint(spin_limit))
 

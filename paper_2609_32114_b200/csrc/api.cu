@@ -187,7 +187,7 @@ int ha_la_debug_wait_timeout(const ha_la_prefill_args* a, void* cuda_stream, uns
   if (rc != HA_LA_OK) return rc;
   if (!a->workspace || ((uintptr_t)a->workspace & 255) || a->workspace_bytes < need) return HA_LA_ERR_WORKSPACE;
   void* tc_ws = reinterpret_cast<char*>(a->workspace) + plan_bytes(p);
-  return launch_tc_chain_unpublished(p, *a, tc_ws, spin_limit, reinterpret_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
+  return launch_tc_withheld(p, *a, tc_ws, spin_limit, reinterpret_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
              ? HA_LA_OK : HA_LA_ERR_CUDA;
 }
 

@@ -7,7 +7,6 @@
 #include <stdlib.h>
 
 #include <atomic>
-#include <random>
 
 #include "tc_common.cuh"
 
@@ -18,7 +17,7 @@ cudaError_t launch_tc_tp(const Problem& p, const ha_la_prefill_args& a, PlanView
 cudaError_t launch_tc_kda(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
                           const CUtensorMap& mq, const CUtensorMap& mk, int ctas, cudaStream_t stream);
 cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                           const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, int64_t epoch,
+                           const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, bool withhold,
                            bool dependent, uint32_t spin_limit, const SpanBuffers& sb, bool states_only,
                            cudaStream_t stream);
 cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& sb, int32_t* status, cudaStream_t stream);
@@ -70,18 +69,6 @@ int sm_count() {
 
 constexpr int kMaxDevices = 64;
 constexpr uint32_t kDefaultSpinLimit = 4u << 20;      // polls before a device-side bounded wait gives up
-std::atomic<uint32_t> g_calls{0};
-
-// Epoch of a concurrent-mode call: (random per-process tag, never 0) << 40 | call counter << 8; the low byte is zero
-// (the chain kernel's slices count in it).
-int64_t next_epoch() {
-  static const uint32_t tag = [] {
-    std::random_device rd;
-    uint32_t t = rd();
-    return (t & 0x7fffffu) ? t : 0x9e3779b9u;
-  }();
-  return (int64_t)(((uint64_t)(tag & 0x7fffffu) << 40) | ((uint64_t)(uint32_t)g_calls.fetch_add(1) << 8));
-}
 
 // HA_LA_TC_SEGMENTS, or 0
 int forced_segments() {
@@ -294,17 +281,16 @@ cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView pl
   const bool dependent = g_timer == nullptr;             // (per-kernel timing wants one kernel at a time)
   cudaError_t e = kda ? launch_tc_kda(p, a, plan, ws, mq, mk, sm_count(), stream) : launch_tc_tp(p, a, plan, ws, mq, mk, sm_count(), stream);
   if (e == cudaSuccess && sb.nspan > 1) {
-    e = launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, true, stream);
+    e = launch_tc_walk(p, a, plan, ws, mk, mq, mv, false, dependent, kDefaultSpinLimit, sb, true, stream);
     if (e == cudaSuccess) e = launch_span_fix(p, plan, sb, a.status_word, stream);
   }
-  return e != cudaSuccess ? e : launch_tc_walk(p, a, plan, ws, mk, mq, mv, 0, dependent, kDefaultSpinLimit, sb, false, stream);
+  return e != cudaSuccess ? e : launch_tc_walk(p, a, plan, ws, mk, mq, mv, false, dependent, kDefaultSpinLimit, sb, false, stream);
 }
 
-// Test hook behind ha_la_debug_wait_timeout: the state-passing kernel alone, waiting for steps to be published, with an
-// epoch that nothing will ever publish and a small poll limit.  Its first flag wait runs out, it records the time-out, and
-// runs its barriers to a normal exit.
-cudaError_t launch_tc_chain_unpublished(const Problem& p, const ha_la_prefill_args& a, void* tc_ws, uint32_t spin_limit,
-                                        cudaStream_t stream) {
+// Test hook behind ha_la_debug_wait_timeout: the state-passing kernel alone, with its copies withheld and a small poll limit.
+// Its waits for the tiles run out, it records the time-out and runs its barriers to a normal exit.
+cudaError_t launch_tc_withheld(const Problem& p, const ha_la_prefill_args& a, void* tc_ws, uint32_t spin_limit,
+                               cudaStream_t stream) {
   CUtensorMap mq, mk, mv;
   if (!make_map_tile(&mq, a.q, p.T_total, p.HK) || !make_map_tile(&mk, a.k, p.T_total, p.HK) ||
       !make_map_tile(&mv, a.v, p.T_total, p.HV))
@@ -312,7 +298,7 @@ cudaError_t launch_tc_chain_unpublished(const Problem& p, const ha_la_prefill_ar
   const TcWorkspace ws = tc_ws_view(tc_ws, (size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA);
   cudaError_t e = configure_tc_walk(p);
   if (e != cudaSuccess) return e;
-  return launch_tc_walk(p, a, PlanView{}, ws, mk, mq, mv, next_epoch(), false, spin_limit, SpanBuffers{1, nullptr, nullptr}, false, stream);
+  return launch_tc_walk(p, a, PlanView{}, ws, mk, mq, mv, true, false, spin_limit, SpanBuffers{1, nullptr, nullptr}, false, stream);
 }
 
 }  // namespace ha_la

@@ -27,18 +27,15 @@ constexpr __host__ __device__ int step_pos(int t) {                // stored pos
 struct TcWorkspace {
   uint8_t* img;     // KDA only: [slot][V-head] three tiles
   uint8_t* rec;     // [slot][V-head] records
-  int64_t* flags;   // [slot][V-head], for a state-passing kernel that waits for steps to be published
 };
 
 inline __host__ size_t tc_ws_bytes_for(size_t ncj, bool kda) {
-  return ncj * (kda ? 3 * kTileBytes : 0) + align_up(ncj * kStepRecB, 1024) + align_up(ncj * sizeof(int64_t), 1024);
+  return ncj * (kda ? 3 * kTileBytes : 0) + align_up(ncj * kStepRecB, 1024);
 }
 
 inline __host__ TcWorkspace tc_ws_view(void* base, size_t ncj, bool kda) {
   uint8_t* b = reinterpret_cast<uint8_t*>(base);
-  TcWorkspace w{b, b + ncj * (kda ? 3 * kTileBytes : 0), nullptr};
-  w.flags = reinterpret_cast<int64_t*>(w.rec + align_up(ncj * kStepRecB, 1024));
-  return w;
+  return TcWorkspace{b, b + ncj * (kda ? 3 * kTileBytes : 0)};
 }
 
 // What HA_LA_TC_SEGMENTS or the 64-token planner's segments add to the workspace (spans forced that way use it): per

@@ -52,11 +52,7 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // Bounded wait.  Gives up after `kSpinLimit` polls (or at once when *abort is already set), sets
 // *abort and returns false; the caller carries on with the same control flow (results are then
 // unspecified and the status word reports HA_LA_ERR_TIMEOUT), so no barrier count ever diverges.
-#ifdef HA_EXP_SPIN
-constexpr uint32_t kSpinLimit = HA_EXP_SPIN;   // (developer experiments: give up quickly)
-#else
 constexpr uint32_t kSpinLimit = 4u << 20;
-#endif
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           uint32_t limit = kSpinLimit) {
   for (uint32_t it = 0; it < limit; ++it) {
@@ -109,9 +105,7 @@ __device__ __forceinline__ void prefetch_l2(const void* src) {     // the 128-by
   asm volatile("prefetch.global.L2 [%0];" ::"l"(src) : "memory");
 }
 
-// Cross-kernel hand-over of data moved by the async proxy (bulk copies): the writer waits for its bulk
-// stores, fences the proxies and publishes a flag with release semantics; the reader acquires the
-// flag, fences the proxies and only then issues its bulk loads.
+// Between this thread's view of memory and copies that it issues afterwards.
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
 // ---------------------------------------------------------------- tensor memory

@@ -72,9 +72,8 @@ struct WalkParams {
   TcWorkspace ws;
   int HK, HV;
   float scale;
-  int64_t epoch;               // != 0: the prep kernel runs concurrently; wait for ws.flags[cj] == epoch per step
-                               // == 0: wait for the whole prep grid before the first workspace read
-  uint32_t spin_limit;         // polls before a bounded wait gives up (a few thousand in the time-out test)
+  bool withhold;               // test hook: the producers copy nothing, so that the waits for their tiles run out
+  uint32_t spin_limit;         // polls before a bounded wait gives up (a few thousand in that test)
   // Spans: a sequence's steps are cut into `nspan` runs that are walked at the same time (1: off), in two launches with
   // span_fix_kernel (tc_span.cu) between them.  The state recurrence is affine in the start state, so
   //   first launch, state only (OUT = false): spans 0 .. nspan-2 from their own start (span 0: h0, others: zero) into
@@ -169,10 +168,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   __syncthreads();
   tc_fence_after_sync();
   constexpr uint32_t tmem = 0;                           // (the whole of tensor memory)
-  // This kernel may be launched as a programmatic dependent of the prep kernel, i.e. start while that one is still
-  // running.  Sequential mode: everything above overlapped the prep kernel's tail; wait for it here.
-  if (p.epoch == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-
+  // Launched as a programmatic dependent: everything above ran under the tail of the kernel before; wait for it here.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (packed) {
     // (These tables too are read behind the wait only: in a batch without a token there is no chunk-local kernel between the
     // plan kernel, which lets its dependents go before it writes them, and this one.)
@@ -183,29 +180,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     take_span();
   }
 
-  // Concurrent mode: a whole warp looks at the ready flags of the next 32 steps at once (plain loads) and remembers how
-  // far the prep kernel has got; the acquire fence and the proxy fence, which are what makes the published results
-  // visible to this kernel's bulk copies, are then paid once per batch, not per step.
-  int ready_upto = p.epoch != 0 ? 0 : nsteps;            // steps [0, ready_upto) are known to be published
-  auto wait_ready = [&](int c) {
-    if (c < ready_upto) return;
-    int got = 0;
-    for (uint32_t it = 0; it < p.spin_limit && !*abort_flag; ++it) {
-      const int cc = c + lane;
-      bool ok = false;
-      if (cc < nsteps)
-        ok = *reinterpret_cast<const volatile int64_t*>(p.ws.flags + (size_t)(slot0 + cc) * p.HV + j) == p.epoch;
-      const unsigned m = __ballot_sync(0xffffffffu, ok);
-      got = __ffs(~m) - 1;                               // leading published steps (32 when all are)
-      if (got < 0) got = 32;
-      if (got > 0) break;
-      __nanosleep(100);
-    }
-    if (got == 0) *abort_flag = 1;                       // gave up: the status word reports the time-out
-    ready_upto = c + (got > 0 ? got : nsteps);
-    __threadfence();                                     // acquire side of the prep kernel's release
-    fence_proxy_async_all();
-  };
+  const int ncopied = p.withhold ? 0 : nsteps;
   auto aborted = [&]() { return __any_sync(0xffffffffu, *abort_flag) != 0; };
   // (mbarrier.try_wait costs the caller ~150 cycles even when the phase is over: test first)
   auto wait1 = [&](uint64_t* b, uint32_t parity) {
@@ -214,8 +189,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
 
   if (warp == W_P0) {
     // ------------------------------------------------------------ producer of the tiles: X / D2 operands, Q, V
-    for (int c = 0; c < nsteps; ++c) {
-      if (KDA) wait_ready(c);
+    for (int c = 0; c < ncopied; ++c) {
       if (lane == 0) {
         const int t0 = tok0 + c * kStep;
         const uint8_t* img = KDA ? p.ws.img + ((size_t)(slot0 + c) * p.HV + j) * 3 * kTileBytes : nullptr;
@@ -260,8 +234,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     }
   } else if (warp == W_P1) {
     // ------------------------------------------------------------ producer of the prep kernel's records
-    for (int c = 0; c < nsteps; ++c) {
-      wait_ready(c);
+    for (int c = 0; c < ncopied; ++c) {
       const uint8_t* rec = p.ws.rec + ((size_t)(slot0 + c) * p.HV + j) * kStepRecB;
       if (lane == 0) {
         if (c > 1) wait1(&empty_sc[c & 1], (c >> 1) - 1);
@@ -650,9 +623,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     if (tid == 0) report_status(p.status, HA_LA_ERR_TIMEOUT);
     settle_copies();
   }
-  // Concurrent mode: do not finish before the prep grid has (it has published its last step by now), so that
-  // work queued behind this kernel is also behind the prep kernel.
-  if (p.epoch != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 0) tmem_dealloc(*tmem_slot, 512);
 }
 
@@ -686,7 +656,7 @@ cudaError_t run_walk(const WalkParams* wp, const CUtensorMap* mk, const CUtensor
 
 // `states_only`: the first of the two launches of a call whose sequences are cut into spans.
 cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanView plan, const TcWorkspace& ws,
-                           const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, int64_t epoch,
+                           const CUtensorMap& mk, const CUtensorMap& mq, const CUtensorMap& mv, bool withhold,
                            bool dependent, uint32_t spin_limit, const SpanBuffers& sb, bool states_only,
                            cudaStream_t stream) {
   WalkParams wp;
@@ -699,7 +669,7 @@ cudaError_t launch_tc_walk(const Problem& p, const ha_la_prefill_args& a, PlanVi
   wp.seq_order = plan.seq_tok0 ? plan.seq_order : nullptr;
   wp.T_row = p.T_row; wp.cps = p.max_seq_chunks > 0 ? p.max_seq_chunks : 1;
   wp.ws = ws; wp.HK = p.HK; wp.HV = p.HV; wp.scale = p.scale; wp.status = a.status_word;
-  wp.epoch = epoch;
+  wp.withhold = withhold;
   wp.spin_limit = spin_limit;
   wp.nspan = sb.nspan; wp.span_b = sb.b; wp.span_phi = sb.phi;
   const int grid = p.N * p.HV * (states_only ? 2 * sb.nspan - 3 : sb.nspan);

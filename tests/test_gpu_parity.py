@@ -354,8 +354,8 @@ def test_segments_chosen_only_where_every_run_gets_an_sm():
 
 
 def test_bounded_wait_runs_out_and_reports_timeout():
-    """Every device-side wait is bounded.  The test hook launches the sequential kernel alone, waiting per chunk for
-    flags that nothing publishes, with a limit of a few thousand polls: the wait must run out, the status word must
+    """Every device-side wait is bounded.  The test hook launches the sequential kernel alone with the copies of its
+    operands withheld and a limit of a few thousand polls: the waits must run out, the status word must
     say HA_LA_ERR_TIMEOUT, the kernel must exit normally, and the library must work as before afterwards."""
     import torch
     import paper_2609_32114_b200 as ha
