@@ -1,11 +1,6 @@
 """Builds libha_la.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
 
-    python -m paper_2609_32114_b200.build [--force] [--verbose] [--profile]
-
---profile builds a second library, libha_la_prof.so, with -DHA_LA_PROFILE_PHASES: the tensor-core kernels then
-record clock64 / %globaltimer stamps at their phase boundaries (csrc/prof.cuh) and the library exports
-ha_la_debug_read_prof_walk to read them; `python -m paper_2609_32114_b200.prof_phases` prints them.
-The normal library contains none of this (the macros expand to nothing).
+    python -m paper_2609_32114_b200.build [--force] [--verbose]
 
 Objects are cached under paper_2609_32114_b200/build/ and rebuilt when their source, any
 header, or this script changes; translation units compile in parallel.
@@ -49,10 +44,9 @@ def _headers_mtime() -> float:
     return t
 
 
-def _compile(unit, verbose: bool, obj_dir: str = OBJ, more=()):
+def _compile(unit, verbose: bool):
     name, src, extra = unit
-    extra = list(extra) + list(more)
-    out = os.path.join(obj_dir, name + ".o")
+    out = os.path.join(OBJ, name + ".o")
     cmd = [_nvcc(), *ARCH, "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", CSRC, "-I", INCLUDE,
            *extra, "-c", os.path.join(CSRC, src), "-o", out]
     if verbose:
@@ -87,43 +81,31 @@ def build_torch_call(force: bool = False) -> str:
     return TORCH_CALL
 
 
-def build(force: bool = False, verbose: bool = False, extra_flags=(), lib_path: str = LIB, obj_dir: str = OBJ) -> str:
-    """Compile what is stale and link.  `extra_flags`, `lib_path`, `obj_dir` serve developer builds."""
-    os.makedirs(obj_dir, exist_ok=True)
+def build(force: bool = False, verbose: bool = False) -> str:
+    """Compile what is stale and link."""
+    os.makedirs(OBJ, exist_ok=True)
     hdr = _headers_mtime()
     todo = []
     for unit in UNITS:
-        out = os.path.join(obj_dir, unit[0] + ".o")
+        out = os.path.join(OBJ, unit[0] + ".o")
         src_t = os.path.getmtime(os.path.join(CSRC, unit[1]))
         if force or not os.path.exists(out) or os.path.getmtime(out) < max(src_t, hdr):
             todo.append(unit)
     if todo:
         with cf.ThreadPoolExecutor(max_workers=min(len(todo), os.cpu_count() or 4)) as ex:
-            for name, rc, log in ex.map(lambda u: _compile(u, verbose, obj_dir, extra_flags), todo):
+            for name, rc, log in ex.map(lambda u: _compile(u, verbose), todo):
                 if verbose or rc != 0:
                     sys.stderr.write(f"--- {name}\n{log}\n")
                 if rc != 0:
                     raise RuntimeError(f"nvcc failed on {name}")
-    objs = [os.path.join(obj_dir, u[0] + ".o") for u in UNITS]
-    if todo or not os.path.exists(lib_path) or os.path.getmtime(lib_path) < max(os.path.getmtime(o) for o in objs):
-        tmp = lib_path + f".tmp{os.getpid()}"
+    objs = [os.path.join(OBJ, u[0] + ".o") for u in UNITS]
+    if todo or not os.path.exists(LIB) or os.path.getmtime(LIB) < max(os.path.getmtime(o) for o in objs):
+        tmp = LIB + f".tmp{os.getpid()}"
         subprocess.check_call([_nvcc(), *ARCH, "-shared", "-o", tmp, *objs])
-        os.replace(tmp, lib_path)
+        os.replace(tmp, LIB)
     build_torch_call(force)
-    return lib_path
-
-
-PROF_LIB = os.path.join(PKG, "libha_la_prof.so")
-
-
-def build_profile(force: bool = False, verbose: bool = False) -> str:
-    """The instrumented developer build (see the module docstring)."""
-    return build(force=force, verbose=verbose, extra_flags=["-DHA_LA_PROFILE_PHASES"], lib_path=PROF_LIB,
-                 obj_dir=os.path.join(PKG, "build_prof"))
+    return LIB
 
 
 if __name__ == "__main__":
-    if "--profile" in sys.argv:
-        print(build_profile(force="--force" in sys.argv, verbose="--verbose" in sys.argv))
-    else:
-        print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))
+    print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))

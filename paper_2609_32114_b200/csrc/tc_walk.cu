@@ -31,13 +31,10 @@
 #include "tc_common.cuh"
 #include "tc_mma.cuh"
 #include "tc_ptx.cuh"
-#include "prof.cuh"
 
 namespace ha_la {
 
 using namespace ptx;
-
-HA_PROF_DECL(walk)
 
 namespace {
 
@@ -458,7 +455,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     }
     for (int c = 0; c < nsteps; ++c) {
       if (c == nsteps - kTailSteps) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-      HA_PROF(walk, 8 * c + 0);
       wait1(&full_sc[c & 1], c >> 1);
       // GDN: e^{G_t}[128], e^{G_L-G_t}[128]; KDA: e^{G_L} per key
       const float* sc = reinterpret_cast<const float*>(sm + Cfg::OFF_SC + (c & 1) * kStepScB);
@@ -467,7 +463,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         load_v(16 * g);
       }
       wait1(bar_x, c);
-      HA_PROF(walk, 8 * c + 1);
       tc_fence_after_sync();
       load_x(16 * g);
       if (KDA && OUT && c > 0) wait1(bar_o, c - 1);      // P U~ of the previous step has read its operand there
@@ -502,7 +497,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
           load_x(64 + 16 * g);
           if (!trans) load_v(64 + 16 * g);
         }
-        HA_PROF(walk, 8 * c + 2);
       }
       __syncwarp();
       if (!trans && lane == 0) mbar_arrive(empty_v);
@@ -518,7 +512,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
           for (int k = 0; k < 4; ++k) e[k] = *reinterpret_cast<const float4*>(sc + 128 + tk + 4 * k);
         }
         wait1(half ? bar_u1 : bar_u0, c);
-        HA_PROF(walk, 8 * c + 3);
         tc_fence_after_sync();
         uint32_t u[16], w[8];
         tmem_ld16(tq + Cfg::TM_U + tk, u);
@@ -547,7 +540,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
             named_arrive(BAR_U + half, kCompute + 32);
           }
         }
-        HA_PROF(walk, 8 * c + 4);
       }
 
       if (OUT) wait1(bar_y, c);
@@ -578,7 +570,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         named_arrive(BAR_UP, kCompute + 32);
       }
       wait1(bar_d2, c);
-      HA_PROF(walk, 8 * c + 5);
       tc_fence_after_sync();
       // ---- h^T <- decay h^T + D2
       {
@@ -603,7 +594,6 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       named_arrive(BAR_H, kCompute + 32);
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty_sc[c & 1]);
-      HA_PROF(walk, 8 * c + 6);
     }
 
     // where the end state goes: hT (from the last span), or the span's offset b_s / transition Phi_s
