@@ -68,7 +68,7 @@
  * Environment switches (test hooks, read by the host launch code; they change how the
  * work is launched, never the result): HA_LA_FORCE_SIMT=1 (read once) sends every shape
  * to the fp32 CUDA-core kernels; HA_LA_TC_SEGMENTS=1|2|4|8 fixes the number of runs a
- * sequence is cut into; HA_LA_TC_NV=32|64|128 and HA_LA_TC_OVERLAP=0|2 change only what
+ * sequence is cut into (see ha_la_prefill_num_runs); HA_LA_TC_NV=32|64|128 and HA_LA_TC_OVERLAP=0|2 change only what
  * ha_la_prefill_launch_plan answers.  Production callers leave them unset; a caller that sets one
  * does so before it asks for the workspace size (the size follows the plan, and a call whose
  * plan needs more than it was given returns HA_LA_ERR_WORKSPACE).
@@ -152,11 +152,17 @@ int ha_la_prefill_num_launches(const ha_la_prefill_args* args);
 int ha_la_prefill_launch_plan(const ha_la_prefill_args* args, int* slice_width, int* concurrent);
 
 /* Segments per sequence in the same cost model, or as forced by HA_LA_TC_SEGMENTS (host only; 0 if the shapes are
- * unsupported).  A call cuts its sequences by its own rule into runs that are walked at the same time -- the
- * Chunk-Seg-Seg mapping the paper describes for its FlashQLA baseline (Section "Head-Level Mapping with
- * Cross-Operator Fusion"): later runs are first walked from a zero state and from the identity, their true start
- * states follow from one affine fix-up per run, and then every run is walked from there.  A forced number above 1 is used as it is. */
+ * unsupported).  Kept for callers that read it: what a call does is ha_la_prefill_num_runs.  The workspace still has
+ * room for this many segments, which only a forced number of runs uses. */
 int ha_la_prefill_num_segments(const ha_la_prefill_args* args);
+
+/* Runs that ha_la_prefill cuts every sequence into for these shapes (host only; 1 = walked in order, 0 if unsupported).
+ * The runs are walked at the same time -- the Chunk-Seg-Seg mapping the paper describes for its FlashQLA baseline
+ * (Section "Head-Level Mapping with Cross-Operator Fusion"): later runs are first walked from a zero state and from
+ * the identity, their true start states follow from one affine fix-up per run, and then every run is walked from
+ * there.  HA_LA_TC_SEGMENTS fixes the number; one above the number of 64-token chunks of the longest sequence is
+ * ignored. */
+int ha_la_prefill_num_runs(const ha_la_prefill_args* args);
 
 /* Profiling aid (the paper's "Metrics" paragraph times kernels with device events): the same work
  * as ha_la_prefill, with a CUDA event recorded on `cuda_stream` before every kernel and after the

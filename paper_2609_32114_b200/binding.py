@@ -33,6 +33,7 @@ EXPORTS = (
     "ha_la_prefill_num_launches",
     "ha_la_prefill_launch_plan",
     "ha_la_prefill_num_segments",
+    "ha_la_prefill_num_runs",
     "ha_la_decode",
     "ha_la_debug_wait_timeout",
     "ha_la_status_string",
@@ -130,6 +131,8 @@ def load_library(path: Optional[str] = None):
     lib.ha_la_prefill_num_launches.restype = ctypes.c_int
     lib.ha_la_prefill_num_segments.argtypes = [A]
     lib.ha_la_prefill_num_segments.restype = ctypes.c_int
+    lib.ha_la_prefill_num_runs.argtypes = [A]
+    lib.ha_la_prefill_num_runs.restype = ctypes.c_int
     lib.ha_la_prefill_launch_plan.argtypes = [A, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]
     lib.ha_la_prefill_launch_plan.restype = ctypes.c_int
     lib.ha_la_decode.argtypes = [ctypes.POINTER(ha_la_decode_args), ctypes.c_void_p]
@@ -206,12 +209,18 @@ def ha_la_prefill_num_launches(args: ha_la_prefill_args) -> int:
 
 
 def ha_la_prefill_num_segments(args: ha_la_prefill_args) -> int:
-    """Segments a sequence's chunks are cut into (1 = walked strictly in order)."""
+    """Segments per sequence in the cost model of ha_la_prefill_launch_plan; what a call does is ha_la_prefill_num_runs."""
     return load_library().ha_la_prefill_num_segments(ctypes.byref(args))
 
 
+def ha_la_prefill_num_runs(args: ha_la_prefill_args) -> int:
+    """Runs a call cuts every sequence into, walked at the same time (1 = in order, 0 = unsupported)."""
+    return load_library().ha_la_prefill_num_runs(ctypes.byref(args))
+
+
 def ha_la_prefill_launch_plan(args: ha_la_prefill_args) -> Tuple[int, bool]:
-    """(slice width of the sequential kernel or 0 on the CUDA-core path, kernels side by side?)."""
+    """A cost model's answer for launches in chunks of 64 tokens (see include/ha_la.h): (slice width of the sequential
+    kernel or 0 on the CUDA-core path, kernels side by side?).  The kernels work in steps of 128 on whole heads."""
     nv, conc = ctypes.c_int(0), ctypes.c_int(0)
     rc = load_library().ha_la_prefill_launch_plan(ctypes.byref(args), ctypes.byref(nv), ctypes.byref(conc))
     if rc != HA_LA_OK:

@@ -62,7 +62,17 @@ int make_problem(const ha_la_prefill_args* a, Problem* p) {
   }
   p->max_seq_chunks = (p->max_len + p->step - 1) / p->step;
   if (!tc_supported(*p) && !simt_supported(*p)) return HA_LA_ERR_UNSUPPORTED;
+  p->planned_runs = p->runs = p->segments = 1;
+  if (use_tc(*p)) tc_plan(p);
   return HA_LA_OK;
+}
+
+size_t workspace_bytes(const Problem& p) {
+  return align_up(plan_bytes(p) + (use_tc(p) ? tc_workspace_bytes(p) : fp32_workspace_bytes(p)), 256);
+}
+
+bool workspace_ok(const ha_la_prefill_args* a, const Problem& p) {
+  return a->workspace && !((uintptr_t)a->workspace & 255) && a->workspace_bytes >= workspace_bytes(p);
 }
 
 }  // namespace
@@ -74,9 +84,7 @@ int ha_la_prefill_workspace_bytes(const ha_la_prefill_args* args, size_t* out_by
   Problem p;
   const int rc = make_problem(args, &p);
   if (rc != HA_LA_OK) return rc;
-  size_t bytes = plan_bytes(p);
-  bytes += use_tc(p) ? tc_workspace_bytes(p) : fp32_workspace_bytes(p);
-  *out_bytes = align_up(bytes, 256);
+  *out_bytes = workspace_bytes(p);
   return HA_LA_OK;
 }
 
@@ -92,13 +100,19 @@ static bool needs_plan(const ha_la_prefill_args* a) { return a->num_seqs > 0 || 
 int ha_la_prefill_num_launches(const ha_la_prefill_args* args) {
   Problem p;
   if (make_problem(args, &p) != HA_LA_OK) return 0;
-  return (needs_plan(args) ? 1 : 0) + (use_tc(p) ? tc_num_launches(p) : 2);
+  return (needs_plan(args) ? 1 : 0) + (p.runs > 1 ? 4 : 2);
 }
 
 int ha_la_prefill_num_segments(const ha_la_prefill_args* args) {
   Problem p;
   if (make_problem(args, &p) != HA_LA_OK) return 0;
-  return use_tc(p) ? tc_num_segments(p) : 1;
+  return p.segments;
+}
+
+int ha_la_prefill_num_runs(const ha_la_prefill_args* args) {
+  Problem p;
+  if (make_problem(args, &p) != HA_LA_OK) return 0;
+  return p.runs;
 }
 
 int ha_la_prefill_launch_plan(const ha_la_prefill_args* args, int* slice_width, int* concurrent) {
@@ -114,7 +128,7 @@ int ha_la_prefill_launch_plan(const ha_la_prefill_args* args, int* slice_width, 
 
 int ha_la_prefill(const ha_la_prefill_args* a, void* cuda_stream) {
   Problem p;
-  int rc = make_problem(a, &p);
+  const int rc = make_problem(a, &p);
   if (rc != HA_LA_OK) return rc;
   if (!a->q || !a->k || !a->v || !a->g || !a->beta || !a->o) return HA_LA_ERR_INVALID_ARG;
   const bool varlen = a->num_seqs > 0 || a->cu_seqlens;
@@ -126,10 +140,7 @@ int ha_la_prefill(const ha_la_prefill_args* a, void* cuda_stream) {
     return HA_LA_ERR_INVALID_ARG;
   if (a->variant == HA_LA_KDA && ((uintptr_t)a->g & 15)) return HA_LA_ERR_INVALID_ARG;   // fetched by bulk copies
 
-  size_t need = 0;
-  rc = ha_la_prefill_workspace_bytes(a, &need);
-  if (rc != HA_LA_OK) return rc;
-  if (!a->workspace || ((uintptr_t)a->workspace & 255) || a->workspace_bytes < need) return HA_LA_ERR_WORKSPACE;
+  if (!workspace_ok(a, p)) return HA_LA_ERR_WORKSPACE;
 
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   PlanView plan = plan_view(a->workspace, p);
@@ -177,15 +188,12 @@ int ha_la_prefill_timed(const ha_la_prefill_args* a, void* cuda_stream, int max_
 
 int ha_la_debug_wait_timeout(const ha_la_prefill_args* a, void* cuda_stream, unsigned int spin_limit) {
   Problem p;
-  int rc = make_problem(a, &p);
+  const int rc = make_problem(a, &p);
   if (rc != HA_LA_OK) return rc;
   if (!tc_supported(p) || a->cu_seqlens || a->num_seqs > 0) return HA_LA_ERR_UNSUPPORTED;
   if (!a->q || !a->k || !a->v || !a->g || !a->beta || !a->o || !a->status_word) return HA_LA_ERR_INVALID_ARG;
   if (spin_limit < 1 || spin_limit > (1u << 20)) return HA_LA_ERR_INVALID_ARG;
-  size_t need = 0;
-  rc = ha_la_prefill_workspace_bytes(a, &need);
-  if (rc != HA_LA_OK) return rc;
-  if (!a->workspace || ((uintptr_t)a->workspace & 255) || a->workspace_bytes < need) return HA_LA_ERR_WORKSPACE;
+  if (!workspace_ok(a, p)) return HA_LA_ERR_WORKSPACE;
   void* tc_ws = reinterpret_cast<char*>(a->workspace) + plan_bytes(p);
   return launch_tc_withheld(p, *a, tc_ws, spin_limit, reinterpret_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
              ? HA_LA_OK : HA_LA_ERR_CUDA;

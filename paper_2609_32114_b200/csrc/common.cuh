@@ -37,6 +37,10 @@ struct Problem {
   int max_seq_chunks;
   float scale;
   int varlen;       // packed batch (cu_seqlens) rather than equal-length rows
+  // tensor-core path, set once per call by tc_plan
+  int planned_runs; // runs a sequence is cut into by the rule (1: walked in order); sizes the workspace
+  int runs;         // ... by this call
+  int segments;     // the answer of ha_la_prefill_num_segments
 };
 
 inline __host__ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -73,9 +77,9 @@ cudaError_t launch_fp32(const Problem& p, const ha_la_prefill_args& a, PlanView 
 // Tensor-core (tcgen05) path: bf16, d_k = d_v = 128.
 bool tc_supported(const Problem& p);
 size_t tc_workspace_bytes(const Problem& p);
-int tc_num_launches(const Problem& p);
-int tc_num_segments(const Problem& p);                                      // segments per sequence launch_tc would use
-void tc_launch_plan(const Problem& p, int* slice_width, int* concurrent);   // what launch_tc would choose
+void tc_plan(Problem* p);                                                   // fills planned_runs, runs, segments
+void tc_launch_plan(const Problem& p, int* slice_width, int* concurrent);   // the answer of ha_la_prefill_launch_plan
+int sm_count();
 cudaError_t launch_tc(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* tc_ws,
                       cudaStream_t stream);
 cudaError_t launch_tc_withheld(const Problem& p, const ha_la_prefill_args& a, void* tc_ws, uint32_t spin_limit,

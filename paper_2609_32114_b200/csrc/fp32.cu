@@ -573,9 +573,9 @@ cudaError_t run(const Problem& p, const Fp32Params& fp, cudaStream_t stream) {
   // The narrowest slices that leave every CTA an SM: a chunk takes 2.2 us with 8 channels and 1.6 with 4 (d = 64); else 16
   // (fewer reads of the shared operands per channel).
   const long long heads = (long long)p.N * p.HV;
-  if (heads * (D / 4) <= 148)
+  if (heads * (D / 4) <= sm_count())
     return launch<fp32_walk_kernel<In, D, 4>>((unsigned)(heads * (D / 4)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
-  if (heads * (D / 8) <= 148)
+  if (heads * (D / 8) <= sm_count())
     return launch<fp32_walk_kernel<In, D, 8>>((unsigned)(heads * (D / 8)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
   return launch<fp32_walk_kernel<In, D, 16>>((unsigned)(heads * (D / 16)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
 }

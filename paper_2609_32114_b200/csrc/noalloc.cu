@@ -58,7 +58,7 @@ extern "C" int ha_la_prefill_noalloc(const ha_la_prefill_args* a, void* cuda_str
   if (rc != HA_LA_OK) return rc;
   const bool packed = a->num_seqs > 0 || a->cu_seqlens;
 
-  Problem p;
+  Problem p{};
   p.variant = a->variant; p.dtype = a->dtype;
   p.N = packed ? a->num_seqs : a->batch;
   p.T_total = a->batch * a->seqlen;

@@ -26,6 +26,16 @@ cudaError_t configure_tc_tp();
 cudaError_t configure_tc_walk(const Problem& p);
 cudaError_t configure_tc_kda();
 
+int sm_count() {
+  static int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 148;
+    return v;
+  }();
+  return n;
+}
+
 namespace {
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -55,16 +65,6 @@ bool make_map_tile(CUtensorMap* m, const void* base, int T, int H) {
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-int sm_count() {
-  static int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 148;
-    return v;
-  }();
-  return n;
 }
 
 constexpr int kMaxDevices = 64;
@@ -222,35 +222,30 @@ bool tc_supported(const Problem& p) {
   return p.dtype == HA_LA_BF16 && p.dk == 128 && p.dv == 128;
 }
 
-// Step records (and images), the scratch of the planned spans, and, when the planner below cuts the sequences into segments,
-// the segment scratch for that many.  (The call checks the caller's size against this same function, so an environment
-// switch that is changed between sizing and calling ends in HA_LA_ERR_WORKSPACE, not in an overrun.)
+void tc_plan(Problem* p) {
+  p->planned_runs = plan_spans(*p);
+  p->segments = plan_tc(*p).nseg;
+  const int forced = forced_segments();
+  p->runs = forced == 1 ? 1 : forced > 1 && p->segments > 1 ? p->segments : p->planned_runs;
+}
+
+// Step records (and images), the scratch of the planned runs, and, when the planner above answers with segments, scratch
+// for that many, which only runs that are forced use.  (The call checks the caller's size against this same function, so an
+// environment switch that is changed between sizing and calling ends in HA_LA_ERR_WORKSPACE, not in an overrun.)
 static size_t tc_base_bytes(const Problem& p) {
-  return tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA) + tc_span_bytes((size_t)p.N * p.HV, plan_spans(p));
+  return tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA) + tc_span_bytes((size_t)p.N * p.HV, p.planned_runs);
 }
 
 size_t tc_workspace_bytes(const Problem& p) {
-  return tc_base_bytes(p) + tc_seg_bytes((size_t)p.N * p.HV, plan_tc(p).nseg, (size_t)p.T_total, p.HV);
+  return tc_base_bytes(p) + tc_seg_bytes((size_t)p.N * p.HV, p.segments, (size_t)p.T_total, p.HV);
 }
 
-// HA_LA_TC_SEGMENTS forces the spans too (1: none); their scratch is then the segment scratch, which is larger.
 static SpanBuffers call_spans(const Problem& p, void* tc_ws) {
   uint8_t* b = reinterpret_cast<uint8_t*>(tc_ws);
   const size_t nj = (size_t)p.N * p.HV;
-  const int forced = forced_segments();
-  if (forced == 1) return tc_span_view(nullptr, nj, 1);
-  if (forced > 1) {
-    const int nseg = plan_tc(p).nseg;
-    if (nseg > 1) return tc_span_view(b + tc_base_bytes(p), nj, nseg);
-  }
-  return tc_span_view(b + tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA), nj, plan_spans(p));
+  if (p.runs > 1 && p.runs == p.segments) return tc_span_view(b + tc_base_bytes(p), nj, p.runs);   // (forced, or the same either way)
+  return tc_span_view(b + tc_ws_bytes_for((size_t)p.max_chunks * p.HV, p.variant == HA_LA_KDA), nj, p.runs);
 }
-
-int tc_num_launches(const Problem& p) {
-  return call_spans(p, nullptr).nspan > 1 ? 4 : 2;
-}
-
-int tc_num_segments(const Problem& p) { return plan_tc(p).nseg; }
 
 void tc_launch_plan(const Problem& p, int* slice_width, int* concurrent) {
   const TcPlan tp = plan_tc(p);

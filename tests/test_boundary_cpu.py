@@ -144,3 +144,26 @@ def test_workspace_follows_the_segment_plan(lib, monkeypatch):
     one = wb(long2)
     monkeypatch.delenv("HA_LA_TC_SEGMENTS")
     assert wb(long2) - one == 2 * n * 128 * 128 * 10 + 16384 * 2 * 128 * 2
+
+
+def test_number_of_runs(lib, monkeypatch):
+    """What a call really does to its sequences: few heads are cut into runs (four launches), a packed batch of long ones and
+    the fp32 path are not; the workspace holds two fp32 matrices per (sequence, V-head, run); a forced number is used."""
+    monkeypatch.delenv("HA_LA_TC_SEGMENTS", raising=False)
+    runs, launches, wb = ha.ha_la_prefill_num_runs, ha.ha_la_prefill_num_launches, ha.ha_la_prefill_workspace_bytes
+    layer, shard = _args(), _args(seqlen=16384, hk=2, hv=2)
+    packed = _args(seqlen=139389, num_seqs=8, max_seqlen=30933)
+    fp32 = _args(dtype="fp32", dk=64, dv=64, hk=1, hv=1, seqlen=256)
+    assert runs(layer) > 1 and runs(shard) > runs(layer) and runs(packed) == runs(fp32) == runs(_args(seqlen=128)) == 1
+    assert runs(_args(dk=96)) == 0
+    assert [launches(x) for x in (layer, shard, packed, fp32)] == [4, 4, 3, 2]
+    n = runs(layer)
+    assert wb(layer) > 16 * n * 2 * 65536
+    for forced in (1, 2, 4, 8):
+        monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(forced))
+        assert runs(layer) == runs(packed) == forced
+        assert launches(layer) == (2 if forced == 1 else 4)
+    short = _args(seqlen=448, hk=64, hv=64)                # seven chunks of 64: a forced eight is ignored
+    ignored = runs(short)
+    monkeypatch.delenv("HA_LA_TC_SEGMENTS")
+    assert ignored == runs(short) == 1
