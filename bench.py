@@ -371,6 +371,14 @@ def decode_bench(args, rank, local_rank, world):
         dist.destroy_process_group()
 
 
+def launch_mode_of(ha, args):
+    """What a call does to its sequences, in words (the library's own answer)."""
+    if ha.ha_la_prefill_path(args) != "tc":
+        return "fp32 kernels"
+    runs = ha.ha_la_prefill_num_runs(args)
+    return "one state-passing launch" if runs == 1 else f"sequences cut into {runs} runs, two state-passing launches"
+
+
 def measure(ha, helpers, w, inp, steps, warmup, dev, local_rank, dist, peaks, world, sample_clocks=True):
     """Device-timed steps of ha_la_prefill on workload `w`: `steps` timed calls after max(warmup, 3) untimed ones,
     between CUDA events on the launching stream, every step on a different resident input/output set."""
@@ -498,9 +506,7 @@ def measure(ha, helpers, w, inp, steps, warmup, dev, local_rank, dist, peaks, wo
     t_hbm = alg_bytes / (peaks["hbm_gbs"] * 1e9)
     t_flop = alg_flops / (peaks["bf16_tflops"] * 1e12)
     path_s = ms_per_step / 1e3
-    launches = ha.ha_la_prefill_num_launches(sets[0][0])
-    launch_mode = ("fp32 kernels" if ha.ha_la_prefill_path(sets[0][0]) != "tc" else
-                   "one state-passing launch" if launches == 2 else "sequences cut into runs, two state-passing launches")
+    launch_mode = launch_mode_of(ha, sets[0][0])
     roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": ncu_traffic(w.name, dom),
                 "alg_bytes": alg_bytes, "peak_source": peaks["source"],
@@ -508,8 +514,7 @@ def measure(ha, helpers, w, inp, steps, warmup, dev, local_rank, dist, peaks, wo
                 "per_kernel": {k: {"alg_bytes_it_touches": kernel_alg_bytes.get(k, 0.0),
                                    "achieved_gbs": kernel_alg_bytes.get(k, 0.0) / (v / 1e3) / 1e9 if v > 0 else None,
                                    "traffic": ncu_traffic(w.name, k)} for k, v in kernel_ms.items()},
-                # what the timed steps used (kernel_ms is always back to back, and then with the planner's
-                # back-to-back slice width, which may differ)
+                # what the timed steps used (kernel_ms: the same kernels, one at a time)
                 "launch_mode": launch_mode,
                 "path": {"bound": "hbm" if t_hbm >= t_flop else "tensor", "roofline_us": 1e6 * max(t_hbm, t_flop),
                          "measured_us": 1e6 * path_s, "frac": max(t_hbm, t_flop) / path_s,

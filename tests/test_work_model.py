@@ -39,3 +39,18 @@ def test_traffic_table_is_rebuilt_from_the_committed_summaries():
     assert stored == json.loads(json.dumps(ncu_summary.traffic()))
     chain = stored["gdn_layer_4k"]["tc_chain"]
     assert chain["dram_read"] > 0 and chain["source"].endswith(".md")
+
+
+def test_bench_names_the_launch_mode_of_every_workload():
+    """A packed batch has the plan kernel as a launch of its own, which must not pass for a second state-passing launch."""
+    import bench
+    import paper_2609_32114_b200 as ha
+
+    def mode(name, **kw):
+        w = synth.WORKLOADS[name]
+        return bench.launch_mode_of(ha, ha.make_args(**dict(dict(variant=w.variant, dtype=w.dtype, batch=1, hk=w.hk, hv=w.hv, dk=w.dk,
+                                                                 dv=w.dv), **kw)))
+
+    assert mode("gdn_fp32_small", seqlen=256) == "fp32 kernels"
+    assert mode("gdn_varlen", seqlen=139389, num_seqs=8, max_seqlen=30933) == "one state-passing launch"
+    assert mode("gdn_layer_4k", seqlen=4096).endswith("runs, two state-passing launches")
