@@ -159,17 +159,17 @@ def test_split_resume_and_in_place_state():
     assert helpers.rel_max_err(state.cpu().numpy()[0:1].reshape(h_orc.shape), h_orc) <= 2e-2
 
 
-@pytest.mark.parametrize("overlap", ["0", "2"])
+@pytest.mark.parametrize("runs", ["1", "2"])
 @pytest.mark.parametrize("variant", ["gdn", "kda"])
-def test_dependent_calls_queued_with_nothing_between_them(variant, overlap, monkeypatch):
+def test_dependent_calls_queued_with_nothing_between_them(variant, runs, monkeypatch):
     """A sequence prefilled piece by piece, the state handed on in place (h0 = hT = one buffer), every call
     prepared beforehand and then queued directly behind the previous one: the next call's first kernel is
-    launched and set up under the previous call's tail and must still see that call's state.  The whole
-    round is repeated so that the first piece follows the last piece of the round before."""
+    launched and set up under the previous call's tail and must still see that call's state, with sequences walked in
+    order and cut into runs.  The whole round is repeated so that the first piece follows the last piece of the round before."""
     import torch
     import paper_2609_32114_b200 as ha
 
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", overlap)
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", runs)
     base = W["gdn_layer_4k"] if variant == "gdn" else W["kda_8k"]
     w = synth.shrink(base, seq_lens=[2560], hk=2, hv=2, gate_shift=-3.0)      # slow decay: the state matters
     inp = synth.make_inputs(w, seed=131)
@@ -183,6 +183,7 @@ def test_dependent_calls_queued_with_nothing_between_them(variant, overlap, monk
         o_piece = torch.empty_like(cut(d["v"]))
         args, keep = ha.prepare_args(cut(d["q"]), cut(d["k"]), cut(d["v"]), cut(d["g"]), cut(d["beta"]),
                                      variant=variant, h0=state, hT=state, o=o_piece)
+        assert ha.ha_la_prefill_num_runs(args) == int(runs)
         calls.append((args, keep, a, b))
     stream = torch.cuda.current_stream().cuda_stream
     torch.cuda.synchronize()
@@ -199,23 +200,21 @@ def test_dependent_calls_queued_with_nothing_between_them(variant, overlap, monk
     assert helpers.rel_max_err(state.cpu().numpy().reshape(h_ref.shape), h_ref) <= 2e-2
 
 
-@pytest.mark.parametrize("shape", ["side_by_side", "back_to_back", "segments", "packed"])
+@pytest.mark.parametrize("shape", ["layer", "in_order", "two_heads", "packed"])
 def test_call_captured_in_a_cuda_graph(shape):
     """A call captured by stream capture and replayed on new contents of the same buffers: every replay must equal
-    an ordinary call on those contents.  (Side by side, the ready flags a replay leaves behind carry the very
-    epoch the next replay runs with: under capture the call clears them first.)"""
+    an ordinary call on those contents, with sequences cut into runs, walked in order and packed."""
     import torch
     import paper_2609_32114_b200 as ha
 
-    kw = {"side_by_side": dict(seq_lens=[2048], hk=16, hv=16), "back_to_back": dict(seq_lens=[1000], hk=4, hv=4),
-          "segments": dict(seq_lens=[8192], hk=2, hv=2), "packed": dict(seq_lens=[300, 0, 700, 64], hk=2, hv=4, varlen=True)}[shape]
+    kw = {"layer": dict(seq_lens=[2048], hk=16, hv=16), "in_order": dict(seq_lens=[1000], hk=4, hv=4),
+          "two_heads": dict(seq_lens=[8192], hk=2, hv=2), "packed": dict(seq_lens=[300, 0, 700, 64], hk=2, hv=4, varlen=True)}[shape]
     w = synth.shrink(W["gdn_varlen"] if shape == "packed" else W["gdn_layer_4k"], h0_std=0.02, **kw)
     dev = [helpers.to_device(synth.make_inputs(w, seed=s)) for s in (171, 172)]
     buf = {k: (v.clone() if hasattr(v, "clone") else v) for k, v in dev[0].items()}
     a, keep = ha.prepare_args(buf["q"], buf["k"], buf["v"], buf["g"], buf["beta"], variant=w.variant, h0=buf["h0"],
                               cu_seqlens=buf["cu_seqlens"], max_seqlen=buf["max_seqlen"])
-    nv, conc = ha.ha_la_prefill_launch_plan(a)
-    assert conc == (shape == "side_by_side") and (ha.ha_la_prefill_num_segments(a) > 1) == (shape == "segments")
+    assert (ha.ha_la_prefill_num_runs(a) > 1) == (shape in ("layer", "two_heads"))
     names = [k for k in ("q", "k", "v", "g", "beta", "h0") if buf[k] is not None]
     side = torch.cuda.Stream()
     ref = []
@@ -244,10 +243,10 @@ def test_call_captured_in_a_cuda_graph(shape):
 
 
 @pytest.mark.parametrize("seed", [21, 22, 23])
-def test_random_shapes_and_launch_modes(seed, monkeypatch):
-    """A seeded sweep over what the planner can be made to do: variant, packed or batched sequences with lengths
-    around the chunk boundaries (empty ones included), head counts and grouping, gate strength, initial state,
-    slice width, launch mode, segment count, output scale -- each case against the oracle."""
+def test_random_shapes_and_numbers_of_runs(seed, monkeypatch):
+    """A seeded sweep over variant, packed or batched sequences with lengths around the chunk boundaries (empty ones
+    included), head counts and grouping, gate strength, initial state, number of runs (the rule's and forced), output
+    scale -- each case against the oracle."""
     import random
 
     rng = random.Random(seed)
@@ -265,20 +264,17 @@ def test_random_shapes_and_launch_modes(seed, monkeypatch):
         base = W["gdn_varlen"] if variant == "gdn" else W["kda_8k"]
         w = synth.shrink(base, seq_lens=lens, hk=hk, hv=hv, gate_shift=rng.choice([-4.0, -2.0, 0.0, 2.0]),
                          h0_std=rng.choice([0.0, 0.02]), varlen=packed)
-        nv = rng.choice(["", "32", "64", "128"])
-        ov = rng.choice(["", "0", "2"])
-        sg = rng.choice(["", "", "2", "4", "8"]) if nv != "128" else ""
-        for key, val in (("HA_LA_TC_NV", nv), ("HA_LA_TC_OVERLAP", ov), ("HA_LA_TC_SEGMENTS", sg)):
-            if val:
-                monkeypatch.setenv(key, val)
-            else:
-                monkeypatch.delenv(key, raising=False)
+        runs = rng.choice(["", "1", "2", "4", "8"])
+        if runs:
+            monkeypatch.setenv("HA_LA_TC_SEGMENTS", runs)
+        else:
+            monkeypatch.delenv("HA_LA_TC_SEGMENTS", raising=False)
         inp = synth.make_inputs(w, seed=1000 * seed + it)
         try:
             helpers.check_parity(inp, scale=rng.choice([1.0, 0.5]))
         except AssertionError as e:
-            raise AssertionError(f"case {it}: {variant} lens={lens} hk={hk} hv={hv} packed={packed} nv={nv!r} "
-                                 f"overlap={ov!r} segments={sg!r}: {e}") from e
+            raise AssertionError(f"case {it}: {variant} lens={lens} hk={hk} hv={hv} packed={packed} "
+                                 f"runs={runs!r}: {e}") from e
 
 
 def test_run_to_run_determinism():
@@ -302,16 +298,15 @@ def test_bad_cu_seqlens_reports_device_check():
 
 
 @pytest.mark.parametrize("variant", ["gdn", "kda"])
-@pytest.mark.parametrize("nseg,nv", [(2, 32), (4, 32), (2, 64), (8, 64)])
-def test_segment_parallel_state_passing(variant, nseg, nv, monkeypatch):
-    """A sequence's chunks cut into segments that are walked at the same time (later segments from a zero state and
-    from the identity, then one affine fix-up per segment).  Slow decay and no decay at all keep the start state of
-    every segment in play -- a wrong start state shows there -- with an initial state, a ragged tail, segment
-    boundaries that do not divide the chunk count, and batched rows."""
+@pytest.mark.parametrize("nseg", [2, 4, 8])
+def test_segment_parallel_state_passing(variant, nseg, monkeypatch):
+    """A sequence cut into runs that are walked at the same time (later runs from a zero state and from the identity,
+    then one affine fix-up per run).  Slow decay and no decay at all keep the start state of every run in play -- a
+    wrong start state shows there -- with an initial state, a ragged tail, run boundaries that do not divide the
+    step count, and batched rows.  (More runs than the sequence has 64-token chunks are not forced.)"""
     import paper_2609_32114_b200 as ha
 
     monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(nseg))
-    monkeypatch.setenv("HA_LA_TC_NV", str(nv))
     base = W["gdn_layer_4k"] if variant == "gdn" else W["kda_8k"]
     for lens, shift in (([1100], -4.0), ([700, 700], None), ([130], 2.0)):
         w = synth.shrink(base, seq_lens=lens, hk=1, hv=2, gate_shift=shift or 0.0, h0_std=0.05)
@@ -319,18 +314,17 @@ def test_segment_parallel_state_passing(variant, nseg, nv, monkeypatch):
         if shift is None:
             inp["g"][:] = 0
         a = ha.make_args(variant=variant, dtype="bf16", batch=len(lens), seqlen=lens[0], hk=1, hv=2, dk=128, dv=128)
-        want = nseg if nseg <= (lens[0] + 63) // 64 else None
-        if want:
-            assert ha.ha_la_prefill_num_segments(a) == nseg
+        if nseg <= (lens[0] + 63) // 64:
+            assert ha.ha_la_prefill_num_runs(a) == nseg
         helpers.check_parity(inp)
 
 
 @pytest.mark.parametrize("variant", ["gdn", "kda"])
 @pytest.mark.parametrize("nseg", [2, 4])
 def test_segments_on_a_packed_batch(variant, nseg, monkeypatch):
-    """Packed batches are never cut into segments by the planner, but the kernels take them (HA_LA_TC_SEGMENTS
-    forces it): every sequence is cut into the same number of segments, so short and empty sequences end up with
-    empty segments, and there are more runs than SMs."""
+    """Packed batches of very different lengths are not cut into runs by the rule, but the kernels take them
+    (HA_LA_TC_SEGMENTS forces it): every sequence is cut into the same number of runs, so short and empty sequences
+    end up with empty runs."""
     monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(nseg))
     base = W["gdn_varlen"] if variant == "gdn" else W["kda_8k"]
     w = synth.shrink(base, seq_lens=[700, 0, 65, 1500, 130, 1], hk=2, hv=4, gate_shift=-3.0, h0_std=0.05, varlen=True)
@@ -342,8 +336,9 @@ def test_segments_on_a_packed_batch(variant, nseg, monkeypatch):
 
 
 def test_segments_chosen_only_where_every_run_gets_an_sm():
-    """Host side of the planner: the headline layer (16 heads) keeps one segment, a long sequence with two heads
-    is cut up, packed batches never are."""
+    """The cost model that ha_la_prefill_num_segments answers for (not what a call does: that is
+    ha_la_prefill_num_runs): the headline layer (16 heads) keeps one segment, a long sequence with two heads is cut
+    up, packed batches never are."""
     import paper_2609_32114_b200 as ha
 
     mk = lambda **kw: ha.make_args(**dict(dict(variant="gdn", dtype="bf16", batch=1, seqlen=4096, hk=16, hv=16,
@@ -384,24 +379,21 @@ def test_full_size_all_heads(name):
     print(name, res)
 
 
-@pytest.mark.parametrize("variant,nv,hv", [("gdn", 32, 16), ("gdn", 64, 16), ("kda", 64, 32), ("kda", 32, 16)])
-def test_consumed_images_dropped_from_l2(variant, nv, hv, monkeypatch):
-    """Side by side with operand images larger than L2, the chain kernel drops the images it has consumed
-    from L2 (a slice its own rows, the last slice of a head the shared ones, counted in the chunk's flag): every
-    head against the oracle, with four slices (32 channels) and two (64) per head, both variants; twice in a row
-    on one workspace, so that the second call finds the first call's counts in the flags."""
+@pytest.mark.parametrize("variant,hv,runs", [("gdn", 16, 1), ("gdn", 16, 0), ("kda", 32, 1), ("kda", 16, 0)])
+def test_operands_larger_than_l2(variant, hv, runs, monkeypatch):
+    """Inputs and operands that do not stay in L2, sequences walked in order (1) and cut by the rule (0): every head
+    against the oracle, twice in a row on one workspace."""
     import torch
     import paper_2609_32114_b200 as ha
 
-    monkeypatch.setenv("HA_LA_TC_NV", str(nv))
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", "2")
-    monkeypatch.setenv("HA_LA_TC_SEGMENTS", "1")
+    if runs:
+        monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
     base = W["gdn_layer_4k"] if variant == "gdn" else W["kda_8k"]
-    w = synth.shrink(base, seq_lens=[8192], hk=hv, hv=hv, h0_std=0.02)      # 128 chunks x hv heads x 64.8 KiB
-    inp = synth.make_inputs(w, seed=151 + nv)
+    w = synth.shrink(base, seq_lens=[8192], hk=hv, hv=hv, h0_std=0.02)      # 134 MB of q, k, v, o and more
+    inp = synth.make_inputs(w, seed=151 + hv)
     d = helpers.to_device(inp)
     a, keep = ha.prepare_args(d["q"], d["k"], d["v"], d["g"], d["beta"], variant=variant, h0=d["h0"])
-    assert ha.ha_la_prefill_launch_plan(a) == (nv, True)
+    assert (ha.ha_la_prefill_num_runs(a) == 1) == (runs == 1)
     stream = torch.cuda.current_stream().cuda_stream
     o_ref, h_ref = helpers.run_oracle(inp)
     for rep in range(2):
@@ -427,57 +419,53 @@ def test_tensors_beyond_two_gib():
 
 
 @pytest.mark.parametrize("variant", ["gdn", "kda"])
-@pytest.mark.parametrize("nv", [32, 64, 128])
-def test_tc_every_slice_width(nv, variant, monkeypatch):
-    """The tensor-core chain kernel at each value-slice width (normally chosen from the launch size): full
-    chunks (stored as tiles by the wider slices) and ragged last chunks (stored row by row) in one batch."""
+@pytest.mark.parametrize("runs", [1, 2, 8])
+def test_tc_full_and_ragged_steps_in_one_batch(runs, variant, monkeypatch):
+    """Full steps and ragged last steps in one packed batch, walked in order and in runs."""
     import paper_2609_32114_b200 as ha
 
-    monkeypatch.setenv("HA_LA_TC_NV", str(nv))
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
     base = W["gdn_varlen"] if variant == "gdn" else W["kda_8k"]
     w = synth.shrink(base, seq_lens=[130, 700, 64], hk=2, hv=4, gate_shift=-1.0, varlen=True)
-    inp = synth.make_inputs(w, seed=31 + nv)
-    a = ha.make_args(variant=variant, dtype="bf16", batch=1, seqlen=inp["T"], hk=2, hv=4, dk=128, dv=128, num_seqs=3)
-    assert ha.ha_la_prefill_path(a) == "tc"
+    inp = synth.make_inputs(w, seed=31 + runs)
+    a = ha.make_args(variant=variant, dtype="bf16", batch=1, seqlen=inp["T"], hk=2, hv=4, dk=128, dv=128, num_seqs=3, max_seqlen=700)
+    assert ha.ha_la_prefill_path(a) == "tc" and ha.ha_la_prefill_num_runs(a) == runs
     helpers.check_parity(inp)
 
 
-@pytest.mark.parametrize("case", ["gdn", "kda", "varlen", "gdn_nv64", "kda_nv64", "gdn_nv128", "kda_nv128"])
-def test_concurrent_prep_and_chain_mode(case, monkeypatch):
-    """Concurrent mode (chosen by the launch planner while the chain CTAs need at most half of the SMs; forced
-    here with HA_LA_TC_OVERLAP=2): the chain kernel runs next to the persistent prep kernel and takes each
-    chunk as soon as its flag is published.  HA_LA_TC_OVERLAP=0 forces the sequential mode.  Same results in
-    both, bit for bit, call after call."""
-    if case.startswith("gdn"):
+@pytest.mark.parametrize("runs", [1, 4])
+@pytest.mark.parametrize("case", ["gdn", "kda", "varlen"])
+def test_same_bits_call_after_call_whatever_the_answer_switches_say(case, runs, monkeypatch):
+    """The same call gives the same bits every time, and HA_LA_TC_NV and HA_LA_TC_OVERLAP, which change what
+    ha_la_prefill_launch_plan answers, change nothing in it."""
+    if case == "gdn":
         w = synth.shrink(W["gdn_layer_4k"], seq_lens=[2048], hk=4, hv=4)
-    elif case.startswith("kda"):
+    elif case == "kda":
         w = synth.shrink(W["kda_8k"], seq_lens=[1000], hk=2, hv=4)
     else:
         w = synth.shrink(W["gdn_varlen"], seq_lens=[700, 0, 65, 1500], hk=2, hv=2)
-    if case.endswith("nv64"):
-        monkeypatch.setenv("HA_LA_TC_NV", "64")
-    if case.endswith("nv128"):                           # the whole-head kernel (state in tensor memory)
-        monkeypatch.setenv("HA_LA_TC_NV", "128")
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
     inp = synth.make_inputs(w, seed=37)
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", "0")
-    o_seq, h_seq, st_seq = helpers.run_gpu(inp)
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", "2")
-    o_con, h_con, st_con = helpers.run_gpu(inp)
-    o_con2, h_con2, _ = helpers.run_gpu(inp)
-    assert st_seq == 0 and st_con == 0
-    np.testing.assert_array_equal(o_con, o_seq)
-    np.testing.assert_array_equal(h_con, h_seq)
-    np.testing.assert_array_equal(o_con2, o_seq)
+    o, h, status = helpers.run_gpu(inp)
+    assert status == 0
+    for nv, overlap in (("", ""), ("64", "2"), ("128", "0")):
+        if nv:
+            monkeypatch.setenv("HA_LA_TC_NV", nv)
+            monkeypatch.setenv("HA_LA_TC_OVERLAP", overlap)
+        o_again, h_again, _ = helpers.run_gpu(inp)
+        np.testing.assert_array_equal(o_again, o)
+        np.testing.assert_array_equal(h_again, h)
     helpers.check_parity(inp)
 
 
-def test_workspace_contents_do_not_matter(monkeypatch):
-    """The workspace is scratch: whatever it holds on entry (small integers, all ones, an earlier call's
-    flags) must not change the result -- in particular not pass for a 'chunk is ready' flag."""
+@pytest.mark.parametrize("runs", [1, 4])
+def test_workspace_contents_do_not_matter(runs, monkeypatch):
+    """The workspace is scratch: whatever it holds on entry (small integers, all ones, an earlier call's records and
+    states) must not change the result."""
     import torch
     import paper_2609_32114_b200 as ha
 
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", "2")          # concurrent mode whatever the planner would choose
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
     w = synth.shrink(W["gdn_layer_4k"], seq_lens=[1500], hk=2, hv=4)
     inp = synth.make_inputs(w, seed=41)
     d = helpers.to_device(inp)
@@ -501,18 +489,20 @@ def test_workspace_contents_do_not_matter(monkeypatch):
     assert torch.equal(o3, o0) and torch.equal(h3, h0)
 
 
-def test_back_to_back_calls_share_a_workspace(monkeypatch):
+def test_back_to_back_calls_share_a_workspace():
     """Many calls queued on one stream without synchronising in between, alternating between two problems
-    of different shape that share one workspace (so every call sees the other's leftovers and the
-    launch-mode switches between concurrent and sequential): results must equal the first call's."""
+    of different shape that share one workspace (so every call sees the other's leftovers, and calls in four
+    launches alternate with calls in three): results must equal the first call's."""
     import torch
     import paper_2609_32114_b200 as ha
 
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", "2")          # concurrent mode wherever the chain leaves SMs free
-    wa = synth.shrink(W["gdn_layer_4k"], seq_lens=[1024], hk=2, hv=2)           # few chains: concurrent mode
-    wb = synth.shrink(W["gdn_varlen"], seq_lens=[200, 0, 333, 64] * 10, hk=2, hv=4)   # 160 chains: sequential
+    wa = synth.shrink(W["gdn_layer_4k"], seq_lens=[2560], hk=2, hv=2)           # few heads: cut into runs
+    wb = synth.shrink(W["gdn_varlen"], seq_lens=[200, 0, 333, 64] * 10, hk=2, hv=4)   # 160 (sequence, head) pairs: packed, in order
     ia, ib = synth.make_inputs(wa, seed=43), synth.make_inputs(wb, seed=44)
     da, db = helpers.to_device(ia), helpers.to_device(ib)
+    launches = [ha.ha_la_prefill_num_launches(ha.make_args(variant="gdn", dtype="bf16", batch=1, seqlen=i["T"], hk=2, hv=hv, dk=128, dv=128,
+                                                           num_seqs=n, max_seqlen=333)) for i, hv, n in ((ia, 2, 0), (ib, 4, 40))]
+    assert launches == [4, 3]
 
     def call(d, w, ws):
         return ha.ha_la_prefill(d["q"], d["k"], d["v"], d["g"], d["beta"], variant=w.variant, h0=d["h0"],
@@ -540,13 +530,12 @@ def test_back_to_back_calls_share_a_workspace(monkeypatch):
     helpers.check_parity(ib)
 
 
-def test_two_streams_in_flight(monkeypatch):
-    """Calls on two streams at once, each with its own workspace: the prep and chain kernels of the two
-    calls compete for the SMs (together they want more than there are), nothing may deadlock or mix up."""
+def test_two_streams_in_flight():
+    """Calls on two streams at once, each with its own workspace: the kernels of the two calls (one of them cut into
+    runs) compete for the SMs (together they want more than there are), nothing may deadlock or mix up."""
     import torch
     import paper_2609_32114_b200 as ha
 
-    monkeypatch.setenv("HA_LA_TC_OVERLAP", "2")          # both calls in the concurrent mode
     w1 = synth.shrink(W["gdn_layer_4k"], seq_lens=[2048], hk=8, hv=8)
     w2 = synth.shrink(W["kda_8k"], seq_lens=[1024], hk=4, hv=8)
     i1, i2 = synth.make_inputs(w1, seed=51), synth.make_inputs(w2, seed=52)
@@ -584,7 +573,7 @@ def test_two_streams_in_flight(monkeypatch):
 
 @pytest.mark.parametrize("variant", ["gdn", "kda"])
 def test_many_sequences_more_ctas_than_sms(variant):
-    """A packed batch with many (sequence, V-head) chains of very different lengths: the chain kernel then
+    """A packed batch with many (sequence, V-head) pairs of very different lengths: the state-passing kernel then
     has more CTAs than the GPU has SMs and starts them longest sequence first."""
     rng = np.random.default_rng(5)
     lens = [int(x) for x in rng.integers(1, 900, size=90)]
@@ -599,7 +588,7 @@ def test_many_sequences_more_ctas_than_sms(variant):
 
 def test_more_sequences_than_the_ranking_limit():
     """4,500 short sequences (0..130 tokens) in one packed batch: beyond 4,096 sequences the plan kernel leaves
-    the launch order as given; the chain kernel then has thousands of CTAs, most of them with one or two chunks."""
+    the launch order as given; the state-passing kernel then has thousands of CTAs, most of them with one or two chunks."""
     rng = np.random.default_rng(11)
     lens = [int(x) for x in rng.integers(0, 131, size=4500)]
     w = synth.shrink(W["gdn_varlen"], seq_lens=lens, hk=1, hv=1, h0_std=0.02, varlen=True)
@@ -609,10 +598,10 @@ def test_more_sequences_than_the_ranking_limit():
     print(res)
 
 
-def test_randomized_shapes_widths_and_modes(monkeypatch):
+def test_randomized_shapes_and_runs(monkeypatch):
     """Thirty seeded random cases: both variants, one to five sequences with lengths around the chunk
     boundaries (empty ones included), grouped heads, three gate strengths, with and without an initial state,
-    every slice width of the chain kernel and every launch mode, against the oracle."""
+    walked in order, in runs and as the rule has it, against the oracle."""
     import random
 
     rng = random.Random(20260932114)
@@ -628,10 +617,9 @@ def test_randomized_shapes_widths_and_modes(monkeypatch):
         w = synth.shrink(base, seq_lens=lens, hk=hk, hv=hv, gate_shift=rng.choice([-2.0, 0.0, 2.0]),
                          h0_std=rng.choice([0.0, 0.02]), varlen=True)
         inp = synth.make_inputs(w, seed=1000 + it)
-        for var, val in (("HA_LA_TC_NV", rng.choice(["", "32", "64", "128"])),
-                         ("HA_LA_TC_OVERLAP", rng.choice(["", "0", "2"]))):
-            if val:
-                monkeypatch.setenv(var, val)
-            else:
-                monkeypatch.delenv(var, raising=False)
+        runs = rng.choice(["", "1", "2", "8"])
+        if runs:
+            monkeypatch.setenv("HA_LA_TC_SEGMENTS", runs)
+        else:
+            monkeypatch.delenv("HA_LA_TC_SEGMENTS", raising=False)
         helpers.check_parity(inp, scale=rng.choice([1.0, 0.5]))
