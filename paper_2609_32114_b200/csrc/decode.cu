@@ -11,8 +11,6 @@
 // (64 channels 80.6, 32 channels 81.5, 128 channels 84.1); 37 sequences x 32 heads: 30.7 -> 25.5 us.
 #include "common.cuh"
 
-#include <cuda_bf16.h>
-
 namespace ha_la {
 
 namespace {
@@ -24,20 +22,6 @@ struct DecodeParams {
   int HK, HV;
   float scale;
 };
-
-template <typename T> __device__ __forceinline__ float to_f32(T x);
-template <> __device__ __forceinline__ float to_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
-template <typename T> __device__ __forceinline__ T from_f32(float x);
-template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
-__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
-  const uint2 w = *reinterpret_cast<const uint2*>(p);
-  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
-                     __uint_as_float(w.y & 0xffff0000u));
-}
 
 constexpr int kCols = 64;                                // value channels per CTA
 constexpr int kThreads = 128;

@@ -27,13 +27,6 @@ using namespace ptx;
 
 namespace {
 
-template <typename T> __device__ __forceinline__ float to_f32(T x);
-template <> __device__ __forceinline__ float to_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
-template <typename T> __device__ __forceinline__ T from_f32(float x);
-template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
 constexpr int C = kChunk;
 constexpr int kNV = 16;                                  // value channels per slice of U in a record
 constexpr int LDP = C + 4;                               // row strides in floats: rows 16 bytes apart in the banks
@@ -65,13 +58,6 @@ struct Fp32Params {
 };
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-template <typename In> __device__ __forceinline__ float4 load4(const In* p);   // four consecutive inputs
-template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return ld4(p); }
-template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 w = *reinterpret_cast<const uint2*>(p);
-  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
-                     __uint_as_float(w.y & 0xffff0000u));
-}
 __device__ __forceinline__ float dot4(const float4& a, const float4& b, float c) {
   return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
 }
@@ -123,7 +109,7 @@ __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
 
   constexpr bool kLateV = KDA && D == 128;               // (its room holds the rescaled K rows first)
   auto v_row = [&](int i, int c) {
-    return i < L ? load4<In>(gv + ((size_t)(t0 + i) * p.HV + j) * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    return i < L ? load4(gv + ((size_t)(t0 + i) * p.HV + j) * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   // ---- load the chunk; rows >= L are no-op tokens (k = q = v = 0, beta = 0, g = 0)
 #pragma unroll
@@ -132,8 +118,8 @@ __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
     float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f), k4 = q4, g4 = q4;
     if (i < L) {
       const size_t off = ((size_t)(t0 + i) * p.HK + jq) * D + c;
-      q4 = load4<In>(gq + off);
-      k4 = load4<In>(gk + off);
+      q4 = load4(gq + off);
+      k4 = load4(gk + off);
       if (KDA) g4 = ld4(p.g + ((size_t)(t0 + i) * p.HV + j) * D + c);
     }
     *reinterpret_cast<float4*>(sQ + i * LD + c) = q4;
