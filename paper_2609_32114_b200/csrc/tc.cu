@@ -82,8 +82,9 @@ int forced_segments() {
 // products of 128^3 between them.  Costs measured on B200: 2.0 us per state-only step, 2.45 per step with outputs, 5 for
 // a CTA's start and end, 1.25 per product (5 when the products' 8 CTAs per pair do not all have an SM) and about 8 for
 // the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
-// within some 15 %.  And no launch beats HBM, at 6 TB/s, once its operands do not stay in L2: 8 sequences of 139 k tokens
-// in all were cut in two for a second launch of 470 us, 444 of them HBM's, after a first of 250; uncut they take 575.
+// within some 15 %.  And no launch beats HBM, at 6 TB/s, once its operands do not stay in L2: a packed batch of 8 sequences
+// with 136 k tokens cut in two took 220 + 15 us for the first launch and the products and 452 for the second, 444 of them
+// HBM's, against 570 us uncut (1160 against 1021 for the call).
 int plan_spans(const Problem& p) {
   const long long chains = (long long)p.N * p.HV;
   const int sms = sm_count(), longest = (p.max_len + kStep - 1) / kStep;
@@ -117,23 +118,12 @@ int plan_spans(const Problem& p) {
   return best_s;
 }
 
-// What ha_la_prefill_launch_plan and ha_la_prefill_num_segments answer, and what a forced HA_LA_TC_SEGMENTS must fit:
-// the choice for a launch in chunks of 64 tokens with a state-passing kernel of sliced heads.  The kernels above this
-// line's rule work in steps of 128 on whole heads; callers may have built on the answers, so they stay.
-// Slice width (value channels per chain CTA) and launch mode, from a cost model measured on B200.
-// Chain kernel: bound by the latency of its two MMA round trips per chunk, which grows with the slice width (about
-// 0.9 / 1.23 / 1.5 us per chunk at 32 / 64 / 128 channels; the last is a kernel of its own that keeps the whole head's
-// state in tensor memory) and does not depend on the number of CTAs.  Each CTA
-// needs an SM of its own, so the kernel's time is about  max(longest sequence, all sequences / SMs)  in chunk-times
-// when the lengths differ (more CTAs than SMs are started longest sequence first and pack well), and whole rounds
-// when they do not: with few chains the narrow slice wins, with many a wider one may.
-// Prep kernel: throughput-bound, about 3.45 (GDN) / 9.8 (KDA) SM-microseconds per (chunk, head), and never
-// faster than its rounds of one item per work group (3 per SM for GDN, 1 for KDA) at 9 / 10.5 us per item.
-// Back to back the two times add.  Concurrently (allowed while the chain's CTAs leave at least half of the SMs to
-// the prep kernel) the call takes the longer of the chain and of the prep kernel on the remaining SMs (plus some
-// interference), plus the wait for the first chunks; with several sequences the prep kernel works through them
-// one after the other, so the last sequence's chain starts only when most of the prep work is done.
-// Only bounds are known on the host: max_len for the longest sequence, max_chunks for the total.
+// What ha_la_prefill_launch_plan and ha_la_prefill_num_segments answer, and what a forced HA_LA_TC_SEGMENTS must fit.  No
+// launch follows it: it is the cost model of a pair of kernels in chunks of 64 tokens that stood before the step kernels, kept
+// because callers may have built on the answers and on the workspace size.  The pair was a chunk-local kernel, which ran at
+// 3.45 (GDN) / 9.8 (KDA) SM-microseconds per (chunk, head), never faster than its rounds of 9 / 10.5 us, and a state-passing
+// kernel of 0.9 / 1.23 / 1.5 us per chunk for slices of 32 / 64 / 128 value channels, a CTA and an SM each; it could run
+// beside the first one where it left that one half of the SMs, or cut a sequence into segments.
 struct TcPlan { int nv; bool concurrent; int nseg; };
 
 TcPlan plan_tc(const Problem& p) {
@@ -145,7 +135,7 @@ TcPlan plan_tc(const Problem& p) {
   const int widths[3] = {32, 64, 128};
   const double per_chunk_us[3] = {0.90, 1.23, 1.50};
   const bool kda = p.variant == HA_LA_KDA;
-  auto prep_time = [&](int on_sms) {                     // the prep kernel on `on_sms` SMs
+  auto prep_time = [&](int on_sms) {                     // the chunk-local kernel on `on_sms` SMs
     const double thru = items * (kda ? 9.8 : 3.45) / on_sms;
     const double groups = (double)on_sms * (kda ? 1 : 3);
     const double rounds = (double)(long long)((items + groups - 1) / groups) * (kda ? 10.5 : 9.0);
@@ -190,12 +180,8 @@ TcPlan plan_tc(const Problem& p) {
       if (overlapped < best) { best = overlapped; plan = TcPlan{widths[w], true, 1}; }
     }
   }
-  // Segment-parallel state passing (equal-length rows, sliced kernels, back to back with the prep kernel): a
-  // sequence's chain is cut into nseg segments that run at once; a later segment costs three times the columns of
-  // the first (its own from a zero state plus 128 transition columns), so it only pays while all those CTAs have an
-  // SM each, i.e. for few heads and long sequences.  Costs measured on B200: the chain's per-chunk times above,
-  // 7 us + 3.1 us per further segment for the start states (S - 1 products of 128^3 in turn) and 9 us + 15 ns per
-  // corrected chunk-head for the outputs.
+  // Segments: a later one cost three times the columns of the first, 3.1 us for its start state and 15 ns per chunk-head for
+  // the correction of its outputs, and they paid only while all CTAs had an SM each.
   const int forced_seg = forced_segments();
   if ((!p.varlen || forced_seg > 1) && forced_seg != 1 && longest >= 2) {
     for (int w = 0; w < 2; ++w) {                          // 32- and 64-channel slices

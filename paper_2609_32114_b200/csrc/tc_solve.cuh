@@ -1,5 +1,5 @@
 // The blocked inverse (I + A)^-1 of a unit lower triangular 128 x 128 matrix by eight warps, shared by the GDN and KDA
-// prep kernels (operator #3 of the paper's pipeline).  A is in shared memory: 16 x 16 blocks below the diagonal as fp16 B operands (16 bytes per lane, off_block
+// chunk-local kernels (operator #3 of the paper's pipeline).  A is in shared memory: 16 x 16 blocks below the diagonal as fp16 B operands (16 bytes per lane, off_block
 // order), the diagonal blocks in fp32.  T = (I + A)^-1 is kept as fp16 blocks of four row-major 8 x 8 matrices (128 bytes
 // each, tri_block order), which ldmatrix reads as any operand.
 #pragma once

@@ -2,9 +2,10 @@
 //   h_1 = b_0,   h_{s+1} = Phi_s h_s + b_s,   s = 1 .. nspan-2        (128 x 128 each, [key][value channel], fp32)
 // The columns (value channels) are independent: a CTA takes 16 of them, a warp 16 rows of every product.  What a product
 // costs is Phi_s on its way out of L2, 64 KiB per CTA, so that is copied in bulk one product ahead (operand fragments
-// read straight from global memory touch every line several times: 2.2 us per product instead of 0.9).  The product itself is 48 warp-level MMAs a warp on values split into two bf16 each (hi hi + hi lo +
-// lo hi, fp32 accumulation: 2^-16 of the factors).  The state's fragments go round the warps through 8 KiB of shared
-// memory, transposed in registers.  Fragment row r of a warp is key sigma(r), sigma(2 t + e) = 4 t + e, sigma(8 + 2 t + e)
+// read straight from global memory touch every line several times: 2.2 us per product).  The product itself is 48 warp-level
+// MMAs a warp on values split into two bf16 each (hi hi + hi lo + lo hi, fp32 accumulation: 2^-16 of the factors).  The
+// state's fragments go round the warps through 8 KiB of shared memory, transposed in registers.  Measured on B200: 1.1 us per
+// product with every CTA on an SM (four products 15 us by themselves, launch included, twenty 33).  Fragment row r of a warp is key sigma(r), sigma(2 t + e) = 4 t + e, sigma(8 + 2 t + e)
 // = 4 t + 2 + e: the four columns of Phi that a lane needs are then neighbours.
 #include "tc_common.cuh"
 #include "tc_mma.cuh"

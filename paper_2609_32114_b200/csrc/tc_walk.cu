@@ -5,13 +5,13 @@
 // tokens.  The state is kept TRANSPOSED: fp32 in registers, and as bf16 pairs in tensor memory (lane = value channel,
 // columns = key channels), where it is the A operand of the products; every other state-dependent operand is made there
 // too, so nothing that threads write goes through shared memory on its way to the tensor cores (no proxy fences), and
-// shared memory is left to the B operands, which arrive ready-made by bulk copy.  Per step (GDN; the prep kernel supplies
+// shared memory is left to the B operands, which arrive ready-made by bulk copy.  Per step (GDN; tc_tp.cu supplies
 // T diag(beta), P and the gate factors):
 //   X^T  = h^T K^T                          R^T = V^T - e^{G_j} X^T                 bf16 pairs
 //   U~^T = R^T (T diag(beta))^T                                                     bf16 pairs, plain and times e^{G_L-G_j}
 //   h^T <- e^{G_L} h^T + (U~ e^{G_L-G})^T K                                          op #5
 //   o^T  = scale [e^{G_i} (h^T Q^T) + U~^T P^T]   (old h; off the sequential path)   op #6
-// KDA: K e^G, Q e^G and K e^{G_L-G} come as images from the prep kernel, so no column factors are needed and the decay is
+// KDA: K e^G, Q e^G and K e^{G_L-G} come as images from tc_kda.cu, so no column factors are needed and the decay is
 // per key channel.
 //
 // What bounds a step: three products that wait for each other's epilogue (K = 128: eight instructions of 64 cycles, ~180
@@ -21,8 +21,9 @@
 // triangular: step ks of their products runs with N = 128 - 16 ks rows.  U and D2 run in token halves, so that an epilogue
 // starts when half of its input is final; Y goes behind X and P U~ behind D2, where the sequential path leaves the tensor
 // cores idle.
-// Measured on B200: 2.3 - 2.45 us per step of 128 tokens and head on one SM, 2.0 without outputs; the kernel before it, on
-// steps of 64, took 0.9 us per step on four SMs or 1.23 on two.  8 sequences of 136 k tokens, 16 heads: 700 -> 573 us.
+// Measured on B200: 2.3 - 2.45 us per step of 128 tokens and head on one SM, 2.6 where HBM is close (8 sequences of 136 k
+// tokens, 16 heads: 570 us for the 220 steps of the longest), 2.0 without outputs; the kernel before it, on steps of 64, took
+// 0.9 us per step on four SMs or 1.23 on two, and 700 us for that batch.
 //
 // Warp roles: sixteen compute warps (tensor-memory lanes 32 (w % 4).., group w / 4 of the columns), four output warps, two
 // producer warps, two warps that issue MMAs (the sequential path; the outputs).  Every wait is bounded.
@@ -230,7 +231,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       if (aborted()) break;
     }
   } else if (warp == W_P1) {
-    // ------------------------------------------------------------ producer of the prep kernel's records
+    // ------------------------------------------------------------ producer of the chunk-local kernel's records
     for (int c = 0; c < ncopied; ++c) {
       const uint8_t* rec = p.ws.rec + ((size_t)(slot0 + c) * p.HV + j) * kStepRecB;
       if (lane == 0) {
