@@ -454,8 +454,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
 #pragma unroll
       for (int i = 0; i < 8; ++i) vv[i >> 2][i & 3] = 0u;
     }
-    for (int c = 0; c < nsteps; ++c) {
-      if (c == nsteps - kTailSteps) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int c = 0, to_go = nsteps; to_go > 0; ++c, --to_go) {
+      if (to_go == kTailSteps) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       wait1(&full_sc[c & 1], c >> 1);
       // GDN: e^{G_t}[128], e^{G_L-G_t}[128]; KDA: e^{G_L} per key
       const float* sc = reinterpret_cast<const float*>(sm + Cfg::OFF_SC + (c & 1) * kStepScB);
