@@ -209,10 +209,11 @@ bool tc_supported(const Problem& p) {
 }
 
 void tc_plan(Problem* p) {
-  p->planned_runs = plan_spans(*p);
-  p->segments = plan_tc(*p).nseg;
   const int forced = forced_segments();
-  p->runs = forced == 1 ? 1 : forced > 1 && p->segments > 1 ? p->segments : p->planned_runs;
+  const bool fits = forced > 1 && forced <= (p->max_len + kChunk - 1) / kChunk;
+  p->planned_runs = plan_spans(*p);
+  p->segments = fits ? forced : plan_tc(*p).nseg;
+  p->runs = forced == 1 ? 1 : fits ? forced : p->planned_runs;
 }
 
 // Step records (and images), the scratch of the planned runs, and, when the planner above answers with segments, scratch

@@ -163,6 +163,9 @@ def test_number_of_runs(lib, monkeypatch):
         monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(forced))
         assert runs(layer) == runs(packed) == forced
         assert launches(layer) == (2 if forced == 1 else 4)
+        monkeypatch.setenv("HA_LA_TC_NV", "128")           # (changes what ha_la_prefill_launch_plan answers, no launch)
+        assert runs(layer) == forced
+        monkeypatch.delenv("HA_LA_TC_NV")
     short = _args(seqlen=448, hk=64, hv=64)                # seven chunks of 64: a forced eight is ignored
     ignored = runs(short)
     monkeypatch.delenv("HA_LA_TC_SEGMENTS")
