@@ -495,10 +495,10 @@ def measure(ha, helpers, w, inp, steps, warmup, dev, local_rank, dist, peaks, wo
                             f"{time.perf_counter() - t_load:.2f} s of the same steps")
     kernel_ms = {k: float(np.mean(v)) for k, v in kt.items()}
     dom = max(kernel_ms, key=kernel_ms.get)
-    # per-kernel attribution: the algorithmic bytes each kernel is the one to touch (the prep kernel reads q, k, v,
-    # g, beta; the chain kernel reads h0 and writes o and hT; the operand images between them are not algorithmic)
+    # per-kernel attribution: the algorithmic bytes each kernel is the first to touch (tc_prep, the chunk-local kernel, reads q, k,
+    # g, beta; tc_chain, the state-passing one, reads v and h0 and writes o and hT; the records between them are not algorithmic)
     e = 2 if w.dtype == "bf16" else 4
-    in_bytes = T * (2 * w.hk * w.dk * e + w.hv * w.dv * e + w.hv * 4 * (1 + (w.dk if w.variant == "kda" else 1)))
+    in_bytes = T * (2 * w.hk * w.dk * e + w.hv * 4 * (1 + (w.dk if w.variant == "kda" else 1)))
     kernel_alg_bytes = {"simt_prefill": alg_bytes, "tc_prep": in_bytes, "tc_chain": alg_bytes - in_bytes,
                         "tc_span": 0.0, "tc_span_fix": 0.0, "plan": 0.0}
     dom_s = kernel_ms[dom] / 1e3
