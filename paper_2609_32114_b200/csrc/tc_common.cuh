@@ -16,7 +16,6 @@ constexpr int kStep = 128;
 constexpr uint32_t kTriB = 18432, kStepScB = 1024;
 constexpr uint32_t kStepT = 0, kStepP = kTriB, kStepSc = 2 * kTriB, kStepRecB = 2 * kTriB + kStepScB;
 constexpr uint32_t kTileBytes = 32768;        // a 128-token, 128-feature bf16 tile, [kb][128 tok][64 feat], 128-byte swizzle
-constexpr __host__ __device__ int tri_block(int I, int J) { return I * (I + 1) / 2 + J; }
 constexpr __host__ __device__ uint32_t tri_slab(int J) { return 32u * (128 * J - 8 * J * (J - 1)); }   // byte offset of slab J
 constexpr __host__ __device__ uint32_t tri_row(int row, int J) { return tri_slab(J) + (row - 16 * J) * 32; }
 static_assert(tri_slab(8) == kTriB, "eight slabs");

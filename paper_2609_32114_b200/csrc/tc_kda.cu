@@ -44,7 +44,7 @@ constexpr int kKdaThreads = 512;                           // eight scaling warp
 constexpr uint32_t OFF_K = 0, OFF_Q = kTileBytes, OFF_K1 = 2 * kTileBytes, kBufBytes = 3 * kTileBytes;
 constexpr uint32_t OFF_A = 2 * kBufBytes;                  // fp16 A below the diagonal blocks: 28 blocks, operand order
 constexpr uint32_t OFF_D = OFF_A + 28 * 512;               // fp32 diagonal blocks of A
-constexpr uint32_t OFF_TOT = OFF_D + 8 * 16 * LDD * 4;     // float [8][128]: log2 decay of each block
+constexpr uint32_t OFF_TOT = OFF_D + (kDiagBytes + 127) / 128 * 128;     // float [8][128]: log2 decay of each block
 constexpr uint32_t OFF_RHO = OFF_TOT + 4096;               // per buffer: int16 [9][rho_slot(channel pair)][2], rho_J
 constexpr uint32_t OFF_BETA = OFF_RHO + 2 * 9 * 256;       // per buffer: float [128]
 constexpr uint32_t OFF_FALL = OFF_BETA + 2 * 512;          // per buffer: int [8][2] (channel halves), block needs the evaluation entry by entry
@@ -116,7 +116,7 @@ __device__ __noinline__ void slow_diagonal(const __nv_bfloat16* k, const __nv_bf
         b += __shfl_xor_sync(0xffffffffu, b, o);
       }
       if (lane == 0) {
-        sd[i * LDD + jj] = jj < i ? a * sBeta[ti] : 0.f;
+        sd[diag_index(i, jj)] = jj < i ? a * sBeta[ti] : 0.f;
         const int t = (jj & 7) >> 1;                     // (store_tri_block's place for column jj)
         *reinterpret_cast<__nv_bfloat16*>(dst + tri_row(ti, I) + (((t >> 1) ^ ((i & 7) >> 2)) << 4) + (t & 1) * 8 + (jj >> 3) * 4 + (jj & 1) * 2) =
             __float2bfloat16_rn(scale * b);
@@ -345,7 +345,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             }
           }
           if (J == I) {
-            float* sd = sD + I * 16 * LDD;
+            float* sd = sD + I * kDiagStride;
             if (fall[2 * I] | fall[2 * I + 1]) {
               const size_t jq = gm.j / R;
               slow_diagonal(p.k + ((size_t)gm.tok0 * p.HK + jq) * 128, p.q + ((size_t)gm.tok0 * p.HK + jq) * 128, (size_t)p.HK * 128,
@@ -354,8 +354,8 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             }
 #pragma unroll
             for (int n = 0; n < 2; ++n) {                // (the substitution reads the strictly lower entries only)
-              *reinterpret_cast<float2*>(sd + g8 * LDD + 8 * n + t2) = make_float2(b0 * a[n][0], b0 * a[n][1]);
-              *reinterpret_cast<float2*>(sd + (g8 + 8) * LDD + 8 * n + t2) = make_float2(b1 * a[n][2], b1 * a[n][3]);
+              *reinterpret_cast<float2*>(sd + diag_index(g8, 8 * n + t2)) = make_float2(b0 * a[n][0], b0 * a[n][1]);
+              *reinterpret_cast<float2*>(sd + diag_index(g8 + 8, 8 * n + t2)) = make_float2(b1 * a[n][2], b1 * a[n][3]);
 #pragma unroll
               for (int e = 0; e < 4; ++e)
                 if (8 * n + t2 + (e & 1) > g8 + (e >> 1) * 8) pq[n][e] = 0.f;
@@ -367,7 +367,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
           }
           const uint32_t f[4] = {pack_bf16(p.scale * pq[0][0], p.scale * pq[0][1]), pack_bf16(p.scale * pq[1][0], p.scale * pq[1][1]),
                                  pack_bf16(p.scale * pq[0][2], p.scale * pq[0][3]), pack_bf16(p.scale * pq[1][2], p.scale * pq[1][3])};
-          store_tri_block(rec + kStepP, I, J, lane, f);
+          store_tri_block(rec + kStepP + tri_offset(I, J) + tri_lane(lane), f);
         }
       }
       sync_half(6);
@@ -379,7 +379,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         }
       }
       const bool bad = solve_and_emit(rec + kStepT, sbuf + OFF_K1, sA, sD, smem_u32(sD), sBeta, warp, lane,
-                                      [&]() { sync_half(6); }, [](int) {});
+                                      [&]() { sync_half(6); }, []() {});
       if (bad) report_status(p.status, HA_LA_ERR_DEVICE_CHECK);
       arrive(3 + b);
       item += stride;

@@ -96,3 +96,34 @@ def test_packed_batch_without_a_token(variant, dtype, d, seqs):
         assert ha.ha_la_prefill_raw(a, torch.cuda.current_stream().cuda_stream) == 0
         torch.cuda.synchronize()
         assert int(status.item()) == 0 and torch.equal(hT, torch.zeros_like(h0) if start is None else start)
+
+
+@pytest.mark.parametrize("hk,hv,lens", [(32, 32, [4500]), (16, 32, [4097]), (3, 9, [9000, 5, 4000])])
+def test_gdn_units_of_all_groups_in_turn(hk, hv, lens):
+    """Six to eight units (a step of a V-head) for every CTA of the chunk-local kernel: each of its three groups takes several, with
+    both stages of tiles and both halves of tensor memory under each, alone or as one of several V-heads of a q/k head."""
+    helpers.check_parity(_inputs("gdn", lens, len(lens) > 1, hk, hv, 367, gate_shift=2.0), pairs=[(0, 0), (0, hv // 2), (len(lens) - 1, hv - 1)])
+
+
+@pytest.mark.parametrize("log_gate", [-3.0, -9.0, -90.0, -500.0])
+def test_gdn_strong_decay(log_gate):
+    """Decays between blocks of 16 tokens from moderate to far below the smallest fp32 number, at and around their edges."""
+    inp = _inputs("gdn", [300], False, 1, 2, 373)
+    for tok in (5, 15, 16, 37, 70, 71, 112, 131, 200):
+        inp["g"][tok] = log_gate
+    inp["g"][140:190] = log_gate / 8
+    helpers.check_parity(inp)
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("first,length", [(0, 16), (16, 40), (64, 96), (112, 128), (128, 160)])
+def test_overflow_in_any_block_is_reported(variant, first, length):
+    """Sixteen strongly correlated keys far outside the stable range, in one block of the solve: whichever it is, also where the
+    sequence ends behind it, the status word says so."""
+    import numpy as np
+
+    inp = _inputs(variant, [length], False, 1, 1, 379, gate_shift=-6.0)
+    inp["g"][:] = 0.0
+    inp["k"][first:first + 16] = synth.round_to_bf16((60.0 * inp["k"][first] + 0.0 * inp["k"][first:first + 16]).astype(np.float32))
+    inp["beta"][first:first + 16] = 1.0
+    assert helpers.run_gpu(inp)[2] == 6
