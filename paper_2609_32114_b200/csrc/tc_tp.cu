@@ -131,7 +131,7 @@ tc_tp_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
   };
   if (grp == kGroups) {
     // ------------------------------------------------------------ tiles and products (one thread)
-    if (lane == 0) {
+    if (elect_one()) {
       auto issue_tiles = [&](const Geom& g, int st) {
         uint8_t* t = smem_raw + st * kStageB;
         mbar_expect_tx(&full[st], kStageB);

@@ -256,15 +256,12 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       if (aborted()) break;
     }
   } else if (warp >= W_MMA) {
-    // ------------------------------------------------------------ MMA issue (lane 0 issues; the warp keeps the barriers)
-    // One warp issues the products of the sequential path, another those of the outputs: an instruction is accepted when
-    // the one a few places before it has run, so an issuing thread is held up by its own products.  The tensor cores work
+    // ------------------------------------------------------------ MMA issue (one thread issues; the warp keeps the barriers)
+    // One warp issues the products of the sequential path, another those of the outputs.  The tensor cores work
     // in order of issue, so the second warp goes when the first one tells it to: Y behind X, under X's epilogue, and P U~
-    // behind D2, under the epilogue of the state.  Descriptors advance by constants: their arithmetic takes the thread as
-    // long as an instruction of the MMA itself.
+    // behind D2, under the epilogue of the state.  Descriptors advance by constants.
     constexpr uint32_t id_kk = idesc_bf16(128, 128, false, false);   // B K-major: X, Y (rows = tokens)
     constexpr uint32_t id_km = idesc_bf16(128, 128, false, true);    // B MN-major: D2 (rows = the K index, tokens)
-    const bool lead = lane == 0;
     auto tile_product = [&](uint32_t d, uint64_t b) {    // K-major B tile, 128 rows: 16 features per instruction
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks)
@@ -286,40 +283,42 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         const int st = KDA ? 0 : (c & 1);
         const uint64_t dK = dK0 + st * (kTileBytes >> 4);
         const uint64_t dKm = dKm0 + (KDA ? 1 : st) * (kTileBytes >> 4);
-        if (lead) wait1(&full_k[st], KDA ? c : (c >> 1));
+        if (elect_one()) wait1(&full_k[st], KDA ? c : (c >> 1));
+        __syncwarp();
         named_sync(BAR_H, kCompute + 32);                // h operand of the previous step
-        if (lead) {
+        if (elect_one()) {
           tc_fence_after_sync();
           tile_product(Cfg::TM_X, dK);
           umma_commit(bar_x);
         }
         __syncwarp();
         if (OUT) named_arrive(BAR_GY, 64);
-        if (lead) {
+        if (elect_one()) {
           wait1(full_t, c);
           if (OUT && c > 0) wait1(bar_o, c - 1);         // (its operand lies in U's columns)
         }
 #pragma unroll
         for (int half = 0; half < 2; ++half) {           // (tokens 0 .. 63 of U are final after the first four k-steps)
           named_sync(BAR_R + half, kCompute + 32);
-          if (lead) {
+          if (elect_one()) {
             tc_fence_after_sync();
             tri_half(half, Cfg::TM_U, Cfg::TM_R, 8, dT, 0u);
             umma_commit(half ? bar_u1 : bar_u0);
           }
         }
-        if (KDA && lead) wait1(&full_k[1], c);
+        if (KDA && elect_one()) wait1(&full_k[1], c);
+        __syncwarp();
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
           named_sync(BAR_U + half, kCompute + 32);
-          if (lead) {
+          if (elect_one()) {
             tc_fence_after_sync();
 #pragma unroll
             for (int ks = 4 * half; ks < 4 * half + 4; ++ks)   // K index = tokens: 16 rows of 128 bytes per step
               umma_ts(Cfg::TM_X, Cfg::TM_R + 8 * ks, dKm + ks * (2048u >> 4), id_km, ks > 0);
           }
         }
-        if (lead) {
+        if (elect_one()) {
           umma_commit(bar_d2);
           if (!KDA) umma_commit(&empty_k[st]);
         }
@@ -331,12 +330,12 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       const uint64_t dQ = smem_desc(smem_u32(sm + Cfg::OFF_Q), 16, 1024, kSwizzle128B);
       const uint64_t dP = smem_desc(smem_u32(sm + Cfg::OFF_P), 16, 256, kSwizzle32B);
       for (int c = 0; c < nsteps; ++c) {
-        if (lead) {
+        if (elect_one()) {
           wait1(full_q, c);
           if (c > 0) wait1(out_free, c - 1);
         }
         named_sync(BAR_GY, 64);
-        if (lead) {
+        if (elect_one()) {
           tc_fence_after_sync();
           tile_product(Cfg::TM_Y, dQ);
           umma_commit(bar_y);
@@ -344,7 +343,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         }
         if (!KDA) named_sync(BAR_UP, kCompute + 32);
         named_sync(BAR_GP, 64);
-        if (lead) {
+        if (elect_one()) {
           tc_fence_after_sync();
           tri_half(0, Cfg::TM_Y, KDA ? Cfg::TM_R : Cfg::TM_UP, KDA ? 8 : 16, dP, 1u);
           tri_half(1, Cfg::TM_Y, KDA ? Cfg::TM_R : Cfg::TM_UP, KDA ? 8 : 16, dP, 1u);
