@@ -14,16 +14,15 @@
 // KDA: K e^G, Q e^G and K e^{G_L-G} come as images from tc_kda.cu, so no column factors are needed and the decay is
 // per key channel.
 //
-// What bounds a step: three products that wait for each other's epilogue (K = 128: eight instructions of 64 cycles, ~180
-// cycles to a visible result, ~250 of tensor-memory traffic and arithmetic by the compute warps), with the tensor cores
-// (2.3 k cycles for all five products) and shared memory (133 KiB in, 132 KiB of B operands, 96 KiB of V and o tiles: 2.9 k
-// at 128 bytes per cycle) close behind; on large calls HBM (165 KiB per step and head, KDA 197).  T and P are lower
-// triangular: step ks of their products runs with N = 128 - 16 ks rows.  U and D2 run in token halves, so that an epilogue
+// What bounds a step: the serial path of three products and their epilogues (a product: N / 2 cycles per instruction of 16 deep,
+// ~180 cycles to a visible result; an epilogue of the compute warps 350 - 900 cycles of tensor-memory round trips), with outputs
+// the compute warps themselves (2.5 k of 3.7 k cycles), and on large calls HBM (165 KiB per step and head, KDA 197).  T and P are
+// lower triangular: step ks of their products runs with N = 128 - 16 ks rows.  U and D2 run in token halves, so that an epilogue
 // starts when half of its input is final; Y goes behind X and P U~ behind D2, where the sequential path leaves the tensor
 // cores idle.
-// Measured on B200: 2.3 - 2.45 us per step of 128 tokens and head on one SM, 2.6 where HBM is close (8 sequences of 136 k
-// tokens, 16 heads: 570 us for the 220 steps of the longest), 2.0 without outputs; the kernel before it, on steps of 64, took
-// 0.9 us per step on four SMs or 1.23 on two, and 700 us for that batch.
+// Measured on B200: 2.0 us per step of 128 tokens and head with outputs and 1.5 without while the operands come out of L2, 2.35 and
+// 1.75 out of HBM with most SMs at work.  Issue under elect.sync and the operand slots as they are, from 2.45 / 2.0:
+// 32 heads, T = 16384 states only 88 -> 76 us, with outputs 115 -> 107; 8 sequences of 136 k tokens, 16 heads 571 -> 549 (HBM 440).
 //
 // Warp roles: sixteen compute warps (tensor-memory lanes 32 (w % 4).., group w / 4 of the columns), four output warps, two
 // producer warps, two warps that issue MMAs (the sequential path; the outputs).  Every wait is bounded.
@@ -42,16 +41,22 @@ namespace {
 constexpr int kCompute = 512;                              // compute threads: four warps for each of four column groups
 constexpr int walk_threads(bool out) { return kCompute + 32 * (out ? 8 : 3); }
 
+// Shared memory: 32-KiB tiles, then the triangular operands.  The slots go where a copy would otherwise start too late: out of HBM
+// and behind the other copies an operand takes up to 3.8 k cycles.
+template <bool KDA, bool OUT>
 struct WalkCfg {
-  static constexpr uint32_t OFF_K = 0;                     // GDN: two K tiles (steps alternate); KDA: K e^G, K e^{G_L-G}
-  static constexpr uint32_t OFF_Q = 65536;                 // Q (KDA: Q e^G)
-  static constexpr uint32_t OFF_V = 98304;                 // V tile, [2][128 tok][64 ch]
-  static constexpr uint32_t OFF_T = 131072;
-  static constexpr uint32_t OFF_P = OFF_T + kTriB;
-  static constexpr uint32_t OFF_OUT = OFF_P + kTriB;       // output staging: [4 warps][128 tok][32 ch]
-  static constexpr uint32_t OFF_SC = OFF_OUT + 32768;      // two sets of gate factors
+  static constexpr int kNK = OUT ? (KDA ? 1 : 2) : (KDA ? 2 : 3);   // slots of K (KDA: of K e^G); step c has slot c % kNK
+  static constexpr int kND = KDA ? (OUT ? 1 : 2) : 0;      // ... of KDA's K e^{G_L-G}
+  static constexpr int kNV = 2;                            // ... of V, [2][128 tok][64 ch]
+  static constexpr int kNT = KDA || OUT ? 1 : 2;           // ... of T diag(beta)
+  static constexpr uint32_t OFF_K = 0, OFF_D = kNK * kTileBytes, OFF_Q = OFF_D + kND * kTileBytes;   // Q (KDA: Q e^G)
+  static constexpr uint32_t OFF_V = OFF_Q + (OUT ? kTileBytes : 0), OFF_T = OFF_V + kNV * kTileBytes;
+  static constexpr uint32_t OFF_P = OFF_T + kNT * kTriB;
+  static constexpr uint32_t OFF_OUT = OFF_P + (OUT ? kTriB : 0);   // output staging: [4 warps][64 tok][32 ch]
+  static constexpr uint32_t OFF_SC = OFF_OUT + (OUT ? 16384 : 0);  // two sets of gate factors
   static constexpr uint32_t OFF_BAR = OFF_SC + 2 * kStepScB;
-  static constexpr uint32_t kSmem = OFF_BAR + 20 * 8 + 16;
+  static constexpr int kBars = 27;
+  static constexpr uint32_t kSmem = OFF_BAR + kBars * 8 + 16;
   static_assert(kSmem <= 227 * 1024, "shared memory budget");
   // tensor-memory columns (all 512 are allocated, so the base is column 0): X, then D2 | U, then (GDN) plain U~ as operand | Y, then o | h operand | R, then U~ operand
   static constexpr uint32_t TM_X = 0, TM_U = 128, TM_UP = 128, TM_Y = 256, TM_H = 384, TM_R = 448;
@@ -109,26 +114,28 @@ template <bool KDA, bool OUT>
 __global__ void __launch_bounds__(walk_threads(OUT), 1)
 tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
                const __grid_constant__ CUtensorMap map_v, WalkParams p) {
-  using Cfg = WalkCfg;
+  using Cfg = WalkCfg<KDA, OUT>;
+  constexpr int NK = Cfg::kNK, ND = Cfg::kND, NV = Cfg::kNV, NT = Cfg::kNT;
   extern __shared__ __align__(1024) uint8_t sm[];       // no static shared memory in this kernel: 1024-aligned
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + Cfg::OFF_BAR);
-  uint64_t* full_k = bar;            // [2] operand tiles of X and D2 (GDN: one per step, two slots; KDA: one each)
-  uint64_t* empty_k = bar + 2;       // [2] (GDN) D2 of the slot's step complete
-  uint64_t* full_q = bar + 4;
-  uint64_t* bar_y = bar + 5;         // Y complete (Q and the old h operand have been read)
-  uint64_t* full_v = bar + 6;
-  uint64_t* empty_v = bar + 7;       // V read by the compute warps
-  uint64_t* full_t = bar + 8;        // (T is free again when U is complete, P when the step's output product is)
-  uint64_t* full_p = bar + 9;
-  uint64_t* full_sc = bar + 10;      // [2]
-  uint64_t* bar_x = bar + 12;
-  uint64_t* bar_u0 = bar + 13;       // U complete for the first 64 tokens
-  uint64_t* bar_d2 = bar + 14;
-  uint64_t* bar_o = bar + 15;        // o complete in tensor memory
-  uint64_t* out_free = bar + 16;     // ... and read by the output warps
-  uint64_t* empty_sc = bar + 17;     // [2] gate factors read by everyone
-  uint64_t* bar_u1 = bar + 19;       // ... for the others
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 20);
+  uint64_t* full_k = bar;            // [NK] K tile (KDA: K e^G)
+  uint64_t* empty_k = bar + 3;       // [NK] D2 of the slot's step complete (its T diag(beta) has been read as well)
+  uint64_t* full_d = bar + 6;        // [ND] (KDA) K e^{G_L-G}
+  uint64_t* full_q = bar + 8;
+  uint64_t* bar_y = bar + 9;         // Y complete (Q and the old h operand have been read)
+  uint64_t* full_v = bar + 10;       // [NV]
+  uint64_t* empty_v = bar + 12;      // [NV] V read by the compute warps
+  uint64_t* full_t = bar + 14;       // [NT]
+  uint64_t* full_p = bar + 16;       // (P is free again when the step's output product is complete)
+  uint64_t* full_sc = bar + 17;      // [2]
+  uint64_t* empty_sc = bar + 19;     // [2] gate factors read by everyone
+  uint64_t* bar_x = bar + 21;
+  uint64_t* bar_u0 = bar + 22;       // U complete for the first 64 tokens
+  uint64_t* bar_u1 = bar + 23;       // ... for the others
+  uint64_t* bar_d2 = bar + 24;
+  uint64_t* bar_o = bar + 25;        // o complete in tensor memory
+  uint64_t* out_free = bar + 26;     // ... and read by the output warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + Cfg::kBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   constexpr int W_OUT = kCompute / 32, W_P0 = W_OUT + (OUT ? 4 : 0), W_P1 = W_P0 + 1, W_MMA = W_P1 + 1;
@@ -152,9 +159,10 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   take_span();
 
   if (tid == 0) {
-    for (int i = 0; i < 20; ++i) {
+    for (int i = 0; i < Cfg::kBars; ++i) {
       const uint64_t* b = bar + i;
-      mbar_init(&bar[i], b == empty_v ? kCompute / 32 : b == out_free ? 4 : b == empty_sc || b == empty_sc + 1 ? kCompute / 32 : 1);
+      const bool by_compute = b == empty_v || b == empty_v + 1 || b == empty_sc || b == empty_sc + 1;
+      mbar_init(&bar[i], by_compute ? kCompute / 32 : b == out_free ? 4 : 1);
     }
     *abort_flag = 0;
     mbar_fence_init();
@@ -187,29 +195,26 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
 
   if (warp == W_P0) {
     // ------------------------------------------------------------ producer of the tiles: X / D2 operands, Q, V
+    int st = 0;                                          // c % NK
+    uint32_t ph = 0;                                     // (c / NK) & 1
     for (int c = 0; c < ncopied; ++c) {
       if (lane == 0) {
         const int t0 = tok0 + c * kStep;
         const uint8_t* img = KDA ? p.ws.img + ((size_t)(slot0 + c) * p.HV + j) * 3 * kTileBytes : nullptr;
-        if constexpr (KDA) {
-          if (c > 0) wait1(bar_x, c - 1);
-          if (!*abort_flag) {
-            mbar_expect_tx(&full_k[0], kTileBytes);
-            bulk_load(sm + Cfg::OFF_K, img, kTileBytes, &full_k[0]);
-          }
-        } else {
-          const int st = c & 1;
-          if (c > 1) wait1(&empty_k[st], (c >> 1) - 1);
-          if (!*abort_flag) {
-            mbar_expect_tx(&full_k[st], kTileBytes);
-            tma_load_4d(sm + Cfg::OFF_K + st * kTileBytes, &map_k, &full_k[st], 0, jq, t0, 0);
-          }
+        if (c >= NK) {
+          if constexpr (KDA && NK == 1) wait1(bar_x, c - 1);             // (X has read it: earlier than D2)
+          else wait1(&empty_k[st], ph ^ 1);
+        }
+        if (!*abort_flag) {
+          mbar_expect_tx(&full_k[st], kTileBytes);
+          if constexpr (KDA) bulk_load(sm + Cfg::OFF_K + st * kTileBytes, img, kTileBytes, &full_k[st]);
+          else tma_load_4d(sm + Cfg::OFF_K + st * kTileBytes, &map_k, &full_k[st], 0, jq, t0, 0);
         }
         if (!trans) {                                    // (transition: V = 0)
-          if (c > 0) wait1(empty_v, c - 1);
+          if (c >= NV) wait1(&empty_v[c & 1], (c >> 1) - 1);
           if (!*abort_flag) {
-            mbar_expect_tx(full_v, kTileBytes);
-            tma_load_4d(sm + Cfg::OFF_V, &map_v, full_v, 0, j, t0, 0);
+            mbar_expect_tx(&full_v[c & 1], kTileBytes);
+            tma_load_4d(sm + Cfg::OFF_V + (c & 1) * kTileBytes, &map_v, &full_v[c & 1], 0, j, t0, 0);
           }
         }
         if constexpr (OUT) {
@@ -221,17 +226,21 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
           }
         }
         if constexpr (KDA) {
-          if (c > 0) wait1(bar_d2, c - 1);
+          const int ds = ND == 2 ? st : 0;
+          if (ND == 1 && c > 0) wait1(&empty_k[0], c - 1);               // (two slots: waited for above)
           if (!*abort_flag) {
-            mbar_expect_tx(&full_k[1], kTileBytes);
-            bulk_load(sm + Cfg::OFF_K + kTileBytes, img + 2 * kTileBytes, kTileBytes, &full_k[1]);
+            mbar_expect_tx(&full_d[ds], kTileBytes);
+            bulk_load(sm + Cfg::OFF_D + ds * kTileBytes, img + 2 * kTileBytes, kTileBytes, &full_d[ds]);
           }
         }
       }
+      if (++st == NK) { st = 0; ph ^= 1; }
       if (aborted()) break;
     }
   } else if (warp == W_P1) {
     // ------------------------------------------------------------ producer of the chunk-local kernel's records
+    int s2 = 0;                                          // (c - 2) % NK
+    uint32_t ph2 = 0;                                    // ((c - 2) / NK) & 1
     for (int c = 0; c < ncopied; ++c) {
       const uint8_t* rec = p.ws.rec + ((size_t)(slot0 + c) * p.HV + j) * kStepRecB;
       if (lane == 0) {
@@ -240,10 +249,12 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
           mbar_expect_tx(&full_sc[c & 1], kStepScB);
           bulk_load(sm + Cfg::OFF_SC + (c & 1) * kStepScB, rec + kStepSc, kStepScB, &full_sc[c & 1]);
         }
-        if (c > 0) wait1(bar_u1, c - 1);
+        const int ts = NT == 2 ? c & 1 : 0;
+        if (NT == 1 && c > 0) wait1(bar_u1, c - 1);
+        if (NT == 2 && c > 1) wait1(&empty_k[s2], ph2);  // (that slot's next step comes after this one: no phase is missed)
         if (!*abort_flag) {
-          mbar_expect_tx(full_t, kTriB);
-          bulk_load(sm + Cfg::OFF_T, rec + kStepT, kTriB, full_t);
+          mbar_expect_tx(&full_t[ts], kTriB);
+          bulk_load(sm + Cfg::OFF_T + ts * kTriB, rec + kStepT, kTriB, &full_t[ts]);
         }
         if constexpr (OUT) {
           if (c > 0) wait1(bar_o, c - 1);
@@ -253,6 +264,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
           }
         }
       }
+      if (c > 1 && ++s2 == NK) { s2 = 0; ph2 ^= 1; }
       if (aborted()) break;
     }
   } else if (warp >= W_MMA) {
@@ -277,13 +289,16 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     };
     if (warp == W_MMA) {
       const uint64_t dK0 = smem_desc(smem_u32(sm + Cfg::OFF_K), 16, 1024, kSwizzle128B);
-      const uint64_t dKm0 = smem_desc(smem_u32(sm + Cfg::OFF_K), 16384, 1024, kSwizzle128B);
-      const uint64_t dT = smem_desc(smem_u32(sm + Cfg::OFF_T), 16, 256, kSwizzle32B);
+      const uint64_t dD0 = smem_desc(smem_u32(sm + (KDA ? Cfg::OFF_D : Cfg::OFF_K)), 16384, 1024, kSwizzle128B);
+      const uint64_t dT0 = smem_desc(smem_u32(sm + Cfg::OFF_T), 16, 256, kSwizzle32B);
+      int st = 0;                                        // c % NK
+      uint32_t ph = 0;                                   // (c / NK) & 1
       for (int c = 0; c < nsteps; ++c) {
-        const int st = KDA ? 0 : (c & 1);
+        const int ts = NT == 2 ? c & 1 : 0;
         const uint64_t dK = dK0 + st * (kTileBytes >> 4);
-        const uint64_t dKm = dKm0 + (KDA ? 1 : st) * (kTileBytes >> 4);
-        if (elect_one()) wait1(&full_k[st], KDA ? c : (c >> 1));
+        const uint64_t dD = dD0 + (ND == 1 ? 0 : st) * (kTileBytes >> 4);
+        const uint64_t dT = dT0 + ts * (kTriB >> 4);
+        if (elect_one()) wait1(&full_k[st], ph);
         __syncwarp();
         named_sync(BAR_H, kCompute + 32);                // h operand of the previous step
         if (elect_one()) {
@@ -294,7 +309,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         __syncwarp();
         if (OUT) named_arrive(BAR_GY, 64);
         if (elect_one()) {
-          wait1(full_t, c);
+          wait1(&full_t[ts], NT == 2 ? c >> 1 : c);
           if (OUT && c > 0) wait1(bar_o, c - 1);         // (its operand lies in U's columns)
         }
 #pragma unroll
@@ -306,7 +321,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
             umma_commit(half ? bar_u1 : bar_u0);
           }
         }
-        if (KDA && elect_one()) wait1(&full_k[1], c);
+        if (KDA && elect_one()) wait1(&full_d[ND == 2 ? st : 0], ND == 2 ? ph : c);
         __syncwarp();
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -315,13 +330,14 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
             tc_fence_after_sync();
 #pragma unroll
             for (int ks = 4 * half; ks < 4 * half + 4; ++ks)   // K index = tokens: 16 rows of 128 bytes per step
-              umma_ts(Cfg::TM_X, Cfg::TM_R + 8 * ks, dKm + ks * (2048u >> 4), id_km, ks > 0);
+              umma_ts(Cfg::TM_X, Cfg::TM_R + 8 * ks, dD + ks * (2048u >> 4), id_km, ks > 0);
           }
         }
         if (elect_one()) {
           umma_commit(bar_d2);
-          if (!KDA) umma_commit(&empty_k[st]);
+          umma_commit(&empty_k[st]);
         }
+        if (++st == NK) { st = 0; ph ^= 1; }
         __syncwarp();
         if (OUT) named_arrive(BAR_GP, 64);
       }
@@ -357,7 +373,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       const int q = warp - W_OUT;
       const int lm = lane >> 3, lr = lane & 7;
       const uint32_t ty = tmem + Cfg::TM_Y + (static_cast<uint32_t>(q * 32) << 16);
-      const uint32_t tile = smem_u32(sm + Cfg::OFF_OUT) + q * 8192;       // [128 tok][32 ch], 64-byte rows
+      const uint32_t tile = smem_u32(sm + Cfg::OFF_OUT) + q * 4096;       // [64 tok][32 ch], 64-byte rows
       const uint32_t tile0[2] = {tile + sw64_offset((lm >> 1) * 8 + lr, lm & 1), tile + sw64_offset((lm >> 1) * 8 + lr, 2 + (lm & 1))};
       __nv_bfloat16* obase = reinterpret_cast<__nv_bfloat16*>(p.o) + (size_t)j * 128 + q * 32;
       for (int c = 0; c < nsteps; ++c) {
@@ -368,6 +384,31 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
 #pragma unroll
           for (int hl = 0; hl < 2; ++hl) tmem_ld_16x256b_x4(ty + (static_cast<uint32_t>(16 * hl) << 16) + 32 * tb, r[tb & 1][hl]);
         };
+        // 32 tokens x 16 channels, packed: [m] is 16 tokens
+        auto pack_o = [&](int tb, int hl, uint32_t (&w)[2][4]) {
+#pragma unroll
+          for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) w[m][x] = pack_bf16(as_f2(r[tb & 1][hl][8 * m + 2 * x], r[tb & 1][hl][8 * m + 2 * x + 1]));
+        };
+        auto stage = [&](int tb, int hl, const uint32_t (&w)[2][4]) {     // transposed on the way
+#pragma unroll
+          for (int m = 0; m < 2; ++m) stsm4t(tile0[hl] + (32 * (tb & 1) + 16 * m) * 64, w[m]);
+        };
+        const int left = len - c * kStep;
+        __nv_bfloat16* orow = obase + (size_t)(tok0 + c * kStep) * p.HV * 128 + (lane & 3) * 8;
+        auto send = [&](int half) {
+          __syncwarp();
+#pragma unroll 4
+          for (int it = 0; it < 8; ++it) {
+            const int t = it * 8 + (lane >> 2);
+            uint32_t w[4];
+            lds4(w, tile + sw64_offset(t, lane & 3));
+            if (64 * half + t < left) *reinterpret_cast<uint4*>(orow + (size_t)(64 * half + t) * p.HV * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+          __syncwarp();
+        };
+        uint32_t later[2][2][2][4];                      // the second 64 tokens, out of tensor memory before the first are sent
         load_o(0);
 #pragma unroll
         for (int tb = 0; tb < 4; ++tb) {
@@ -379,26 +420,22 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
             if (lane == 0) mbar_arrive(out_free);        // (the next Y may go there)
           }
 #pragma unroll
-          for (int hl = 0; hl < 2; ++hl)
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {                // 16 tokens x 16 channels, transposed on the way
-              uint32_t w[4];
-#pragma unroll
-              for (int x = 0; x < 4; ++x) w[x] = pack_bf16(as_f2(r[tb & 1][hl][8 * m + 2 * x], r[tb & 1][hl][8 * m + 2 * x + 1]));
-              stsm4t(tile0[hl] + (32 * tb + 16 * m) * 64, w);
+          for (int hl = 0; hl < 2; ++hl) {
+            if (tb < 2) {
+              uint32_t w[2][4];
+              pack_o(tb, hl, w);
+              stage(tb, hl, w);
+            } else {
+              pack_o(tb, hl, later[tb - 2][hl]);
             }
+          }
         }
-        __syncwarp();
-        const int left = len - c * kStep;
-        __nv_bfloat16* orow = obase + (size_t)(tok0 + c * kStep) * p.HV * 128 + (lane & 3) * 8;
-#pragma unroll 4
-        for (int it = 0; it < 16; ++it) {
-          const int t = it * 8 + (lane >> 2);
-          uint32_t w[4];
-          lds4(w, tile + sw64_offset(t, lane & 3));
-          if (t < left) *reinterpret_cast<uint4*>(orow + (size_t)t * p.HV * 128) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-        __syncwarp();
+        send(0);
+#pragma unroll
+        for (int tb = 2; tb < 4; ++tb)
+#pragma unroll
+          for (int hl = 0; hl < 2; ++hl) stage(tb, hl, later[tb - 2][hl]);
+        send(1);
       }
     }
   } else {
@@ -438,7 +475,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     named_arrive(BAR_H, kCompute + 32);
 
     const uint32_t hi = 16u << 16;                       // sixteen lanes further
-    const uint32_t va0 = smem_u32(sm + Cfg::OFF_V) + ((4 * q) >> 3) * 16384;
+    uint32_t va0 = smem_u32(sm + Cfg::OFF_V) + ((4 * q) >> 3) * 16384;    // (of the step's slot)
     uint32_t vv[2][4], x[2][8];
     auto load_v = [&](int tk) {                          // V^T of 16 tokens, 2 x 16 channels (transposed by ldmatrix)
 #pragma unroll
@@ -459,7 +496,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       // GDN: e^{G_t}[128], e^{G_L-G_t}[128]; KDA: e^{G_L} per key
       const float* sc = reinterpret_cast<const float*>(sm + Cfg::OFF_SC + (c & 1) * kStepScB);
       if (!trans) {
-        wait1(full_v, c);
+        wait1(&full_v[c & 1], c >> 1);
         load_v(16 * g);
       }
       wait1(bar_x, c);
@@ -499,7 +536,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         }
       }
       __syncwarp();
-      if (!trans && lane == 0) mbar_arrive(empty_v);
+      if (!trans && lane == 0) mbar_arrive(&empty_v[c & 1]);
+      va0 += (c & 1) ? -(int)kTileBytes : (int)kTileBytes;
 
       // ---- U~^T as operands.  GDN: times e^{G_L-G_t} for the state update, and plain for the outputs, over columns of U
       // that this warp has read already (columns in step_pos order).  KDA: the latter for both.
@@ -620,7 +658,7 @@ template <bool KDA, bool OUT>
 cudaError_t run_walk(const WalkParams* wp, const CUtensorMap* mk, const CUtensorMap* mq, const CUtensorMap* mv, int grid,
                      bool dependent, cudaStream_t stream) {
   auto kern = tc_walk_kernel<KDA, OUT>;
-  constexpr int smem = WalkCfg::kSmem;
+  constexpr int smem = WalkCfg<KDA, OUT>::kSmem;
   if (!wp) {                                             // configure only (this also loads the kernel)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
