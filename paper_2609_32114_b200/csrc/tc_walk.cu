@@ -55,7 +55,7 @@ struct WalkCfg {
   static constexpr uint32_t OFF_OUT = OFF_P + (OUT ? kTriB : 0);   // output staging: [4 warps][64 tok][32 ch]
   static constexpr uint32_t OFF_SC = OFF_OUT + (OUT ? 16384 : 0);  // two sets of gate factors
   static constexpr uint32_t OFF_BAR = OFF_SC + 2 * kStepScB;
-  static constexpr int kBars = 27;
+  static constexpr int kBars = 28;
   static constexpr uint32_t kSmem = OFF_BAR + kBars * 8 + 16;
   static_assert(kSmem <= 227 * 1024, "shared memory budget");
   // tensor-memory columns (all 512 are allocated, so the base is column 0): X, then D2 | U, then (GDN) plain U~ as operand | Y, then o | h operand | R, then U~ operand
@@ -129,7 +129,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   uint64_t* full_p = bar + 16;       // (P is free again when the step's output product is complete)
   uint64_t* full_sc = bar + 17;      // [2]
   uint64_t* empty_sc = bar + 19;     // [2] gate factors read by everyone
-  uint64_t* bar_x = bar + 21;
+  uint64_t* bar_x0 = bar + 21;       // X complete for the first 64 tokens
+  uint64_t* bar_x = bar + 27;        // ... for the others
   uint64_t* bar_u0 = bar + 22;       // U complete for the first 64 tokens
   uint64_t* bar_u1 = bar + 23;       // ... for the others
   uint64_t* bar_d2 = bar + 24;
@@ -273,11 +274,12 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     // in order of issue, so the second warp goes when the first one tells it to: Y behind X, under X's epilogue, and P U~
     // behind D2, under the epilogue of the state.  Descriptors advance by constants.
     constexpr uint32_t id_kk = idesc_bf16(128, 128, false, false);   // B K-major: X, Y (rows = tokens)
+    constexpr uint32_t id_half = idesc_bf16(128, 64, false, false);
     constexpr uint32_t id_km = idesc_bf16(128, 128, false, true);    // B MN-major: D2 (rows = the K index, tokens)
-    auto tile_product = [&](uint32_t d, uint64_t b) {    // K-major B tile, 128 rows: 16 features per instruction
+    auto tile_product = [&](uint32_t d, uint64_t b, uint32_t id) {   // rows (tokens) of a K-major B tile, 16 features per instruction
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks)
-        umma_ts(d, Cfg::TM_H + 8 * ks, b + ((uint32_t)((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), id_kk, ks > 0);
+        umma_ts(d, Cfg::TM_H + 8 * ks, b + ((uint32_t)((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), id, ks > 0);
     };
     // A [128 x 128] (triangular operand)^T, k-steps 4 half ..: slab ks is the operand of the result's columns 16 ks ..
     auto tri_half = [&](int half, uint32_t d, uint32_t a, uint32_t astep, uint64_t tri, uint32_t acc) {
@@ -303,7 +305,9 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         named_sync(BAR_H, kCompute + 32);                // h operand of the previous step
         if (elect_one()) {
           tc_fence_after_sync();
-          tile_product(Cfg::TM_X, dK);
+          tile_product(Cfg::TM_X, dK, id_half);
+          umma_commit(bar_x0);
+          tile_product(Cfg::TM_X + 64, dK + (64 * 128 >> 4), id_half);
           umma_commit(bar_x);
         }
         __syncwarp();
@@ -353,7 +357,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         named_sync(BAR_GY, 64);
         if (elect_one()) {
           tc_fence_after_sync();
-          tile_product(Cfg::TM_Y, dQ);
+          tile_product(Cfg::TM_Y, dQ, id_kk);
           umma_commit(bar_y);
           wait1(full_p, c);
         }
@@ -499,7 +503,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         wait1(&full_v[c & 1], c >> 1);
         load_v(16 * g);
       }
-      wait1(bar_x, c);
+      wait1(bar_x0, c);
       tc_fence_after_sync();
       load_x(16 * g);
       if (KDA && OUT && c > 0) wait1(bar_o, c - 1);      // P U~ of the previous step has read its operand there
@@ -531,6 +535,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         tc_fence_before_sync();
         named_arrive(BAR_R + half, kCompute + 32);
         if (half == 0) {
+          wait1(bar_x, c);
+          tc_fence_after_sync();
           load_x(64 + 16 * g);
           if (!trans) load_v(64 + 16 * g);
         }
