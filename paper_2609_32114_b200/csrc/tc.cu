@@ -79,7 +79,8 @@ int forced_segments() {
 
 // Spans per sequence of the step path (tc_walk.cu): with few (sequence, head) pairs a sequence is cut into S runs that
 // are walked at the same time, in two launches, 2 S - 3 state-only runs and then S runs with outputs, with S - 2
-// products of 128^3 between them.  Costs measured on B200: 2.0 us per state-only step, 2.45 per step with outputs, 5 for
+// products of 128^3 between them.  Costs measured on B200 with the step kernels as first built: 2.0 us per state-only step, 2.45 per step
+// with outputs (1.65 and 2.25 now: another S, mostly by one, in a call of twenty, and no other times where that was measured), 5 for
 // a CTA's start and end, 1.25 per product (5 when the products' 8 CTAs per pair do not all have an SM) and about 8 for
 // the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
 // within some 15 %.  And no launch beats HBM, at 6 TB/s, once its operands do not stay in L2: a packed batch of 8 sequences

@@ -20,7 +20,7 @@
 // block packed to 16 bits is at once the operand of the solve's warp-level products and four 128-byte rows of an 8 x 8
 // core of the result operand, so results go from registers to global memory as whole 128-byte lines without staging.
 //
-// The solve: the 16 x 16 diagonal blocks by one warp each (8 x 8 halves by forward substitution in fp32, joined by a
+// The solve: the 16 x 16 diagonal blocks, two by one warp (8 x 8 halves by forward substitution in fp32, joined by a
 // product), then three levels of joining, T_lo = -T_hi (A_lo T_lo'), evaluated transposed so that the accumulators of
 // the first product are the A operand of the second.  A and T are held as fp16 there (T is rounded to bf16 for the next
 // operator anyway); this assumes the delta rule's usual normalisation (beta |k|^2 of order one), far inside the fp16
