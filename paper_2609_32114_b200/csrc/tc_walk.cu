@@ -199,7 +199,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     int st = 0;                                          // c % NK
     uint32_t ph = 0;                                     // (c / NK) & 1
     for (int c = 0; c < ncopied; ++c) {
-      if (lane == 0) {
+      if (elect_one()) {
         const int t0 = tok0 + c * kStep;
         const uint8_t* img = KDA ? p.ws.img + ((size_t)(slot0 + c) * p.HV + j) * 3 * kTileBytes : nullptr;
         if (c >= NK) {
@@ -244,7 +244,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     uint32_t ph2 = 0;                                    // ((c - 2) / NK) & 1
     for (int c = 0; c < ncopied; ++c) {
       const uint8_t* rec = p.ws.rec + ((size_t)(slot0 + c) * p.HV + j) * kStepRecB;
-      if (lane == 0) {
+      if (elect_one()) {
         if (c > 1) wait1(&empty_sc[c & 1], (c >> 1) - 1);
         if (!*abort_flag) {
           mbar_expect_tx(&full_sc[c & 1], kStepScB);
