@@ -16,7 +16,7 @@ using namespace ptx;
 
 namespace {
 
-constexpr int kFixCols = 16;
+constexpr int kFixCols = 16, kManySpans = 12;
 
 __device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
   hi = pack_bf16(x, y);
@@ -27,6 +27,12 @@ __device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint3
 constexpr uint32_t kPhiBytes = 65536;
 constexpr uint32_t OFF_FRAG = 2 * kPhiBytes, OFF_FBAR = OFF_FRAG + 2 * 8 * 2 * 32 * 16, kSpanSmem = OFF_FBAR + 32;
 
+// Two instances.  With MANY the copies are issued under elect.sync, which gives a kernel of 79 registers instead of 66 whose products
+// are 0.2 us shorter and whose start is 3 us longer.  Calls measured with either, MANY second, GDN unless said: 2 heads, T = 6000, 12
+// spans 43.1 -> 42.1 us; 4 heads, T = 8192, 16 spans 54.3 -> 53.5; T = 16384, 19 spans 74.4 -> 72.7 (KDA, T = 12000 89.6 -> 88.0); 2 heads,
+// T = 16384, 22 spans 68.4 -> 66.4; T = 32768, 32 spans 94.8 -> 91.5; but 8 heads, T = 12000, 10 spans 78.7 -> 79.6; 16 heads, T = 4096,
+// 6 spans 55.9 -> 59.0; and packed batches, whose lengths come from a table, are longer with it at any number (14 spans 142 -> 148).
+template <bool MANY>
 __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row, int HV, const int32_t* seq_len, int32_t* status) {
   extern __shared__ __align__(128) uint8_t sm[];
   uint4 (*frag)[8][2][32] = reinterpret_cast<uint4(*)[8][2][32]>(sm + OFF_FRAG);   // [s & 1][k-step][n-tile][lane]: hi b0, b1, lo b0, b1
@@ -60,7 +66,8 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
     for (int i = 0; i < 4; ++i)
       bulk_load(sm + (s & 1) * kPhiBytes + i * 16384, phi + (size_t)s * stride + i * 4096, 16384, &full[s & 1]);
   };
-  if (threadIdx.x == 0) {
+  auto issuing = [&]() { return MANY ? warp == 0 && elect_one() : threadIdx.x == 0; };
+  if (issuing()) {
     fetch(1);
     fetch(2);
   }
@@ -86,7 +93,7 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
     }
     __syncthreads();                                     // (and everyone is done with the product before)
     if (s + 1 == sb.nspan) break;
-    if (s > 1 && threadIdx.x == 0) fetch(s + 1);
+    if (s > 1 && issuing()) fetch(s + 1);
     mbar_wait(&full[s & 1], ((s - 1) >> 1) & 1, abort_flag);
     if (s * spspan >= nst) continue;                     // (the same for every thread of the CTA)
     // Rows lie 512 bytes apart, so lanes of an odd row take the other k-step of a pair first: other banks.
@@ -139,7 +146,8 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
 }  // namespace
 
 cudaError_t configure_span_fix() {
-  return cudaFuncSetAttribute(span_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmem);
+  cudaError_t e = cudaFuncSetAttribute(span_fix_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmem);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(span_fix_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmem);
 }
 
 cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& sb, int32_t* status, cudaStream_t stream) {
@@ -154,7 +162,8 @@ cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = g_timer ? 0 : 1;                        // (per-kernel timing wants one kernel at a time)
-  return cudaLaunchKernelEx(&cfg, span_fix_kernel, sb, p.T_row, p.HV, (const int32_t*)plan.seq_len, status);
+  auto kern = !plan.seq_len && sb.nspan >= kManySpans ? span_fix_kernel<true> : span_fix_kernel<false>;
+  return cudaLaunchKernelEx(&cfg, kern, sb, p.T_row, p.HV, (const int32_t*)plan.seq_len, status);
 }
 
 }  // namespace ha_la

@@ -127,3 +127,14 @@ def test_overflow_in_any_block_is_reported(variant, first, length):
     inp["k"][first:first + 16] = synth.round_to_bf16((60.0 * inp["k"][first] + 0.0 * inp["k"][first:first + 16]).astype(np.float32))
     inp["beta"][first:first + 16] = 1.0
     assert helpers.run_gpu(inp)[2] == 6
+
+
+@pytest.mark.parametrize("variant,tokens", [("gdn", 6000), ("gdn", 6016), ("kda", 8200)])
+def test_many_runs(variant, tokens):
+    """Sequences that the rule cuts into twelve runs and more, whose start states another instance makes; the last run full or ragged."""
+    import paper_2609_32114_b200 as ha
+
+    inp = _inputs(variant, [tokens], False, 1, 2, 383, gate_shift=5.0)
+    a = ha.make_args(variant=variant, dtype="bf16", batch=1, seqlen=tokens, hk=1, hv=2, dk=128, dv=128)
+    assert ha.ha_la_prefill_num_runs(a) >= 12
+    helpers.check_parity(inp)
