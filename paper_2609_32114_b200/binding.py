@@ -261,6 +261,12 @@ def ha_la_prefill_timed(args: ha_la_prefill_args, stream: int = 0):
     return [(names[i].decode(), float(ms[i])) for i in range(n.value)]
 
 
+def _aligned_part(address, nbytes):
+    """What of a buffer starts on a 256-byte boundary: (address, bytes).  Nothing of one that ends before its first."""
+    start = (address + 255) // 256 * 256
+    return start, max(0, nbytes - (start - address))
+
+
 def prepare_args(q, k, v, g, beta, *, variant="gdn", h0=None, cu_seqlens=None, max_seqlen=0, scale=1.0,
                  o=None, hT=None, want_hT=True, workspace=None, status_word=None):
     """Marshal torch CUDA tensors into ha_la_prefill_args (allocating o / hT / workspace / status word
@@ -297,9 +303,7 @@ def prepare_args(q, k, v, g, beta, *, variant="gdn", h0=None, cu_seqlens=None, m
     need = ha_la_prefill_workspace_bytes(args)
     if workspace is None:
         workspace = torch.empty(need + 256, dtype=torch.uint8, device=q.device)
-    wp = (workspace.data_ptr() + 255) // 256 * 256
-    args.workspace = wp
-    args.workspace_bytes = workspace.numel() - (wp - workspace.data_ptr())
+    args.workspace, args.workspace_bytes = _aligned_part(workspace.data_ptr(), workspace.numel())
     keep = dict(q=q, k=k, v=v, g=g, beta=beta, h0=h0, cu_seqlens=cu_seqlens, o=o, hT=hT, workspace=workspace,
                 status_word=status_word)
     return args, keep

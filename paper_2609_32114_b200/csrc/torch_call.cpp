@@ -139,7 +139,8 @@ PyObject* prefill_call(PyObject* const* a, Py_ssize_t n) {
   d.o = ptr(o); d.hT = (float*)ptr(hT); d.status_word = (int32_t*)ptr(sw);
   const uintptr_t base = (uintptr_t)ws->data_ptr(), al = (base + 255) / 256 * 256;
   d.workspace = (void*)al;
-  d.workspace_bytes = (size_t)(ws->numel() - (int64_t)(al - base));
+  const int64_t pad = (int64_t)(al - base);
+  d.workspace_bytes = ws->numel() > pad ? (size_t)(ws->numel() - pad) : 0;   // (a buffer may end before its first aligned byte)
   void* stream = stream_of(a[8], *q);
   if (PyErr_Occurred()) return nullptr;
   Py_BEGIN_ALLOW_THREADS
