@@ -267,6 +267,31 @@ def _aligned_part(address, nbytes):
     return start, max(0, nbytes - (start - address))
 
 
+def _reachable(t, q):
+    return t.device == q.device or (t.device.type == "cpu" and t.is_pinned())
+
+
+def _check_inputs(q, k, v, g, beta, kda, one_row):
+    """q [rows.., HK, dk] sets the sizes of k, v [rows.., HV, dv], g [rows.., HV] (KDA: and dk) and beta [rows.., HV].  The others
+    may have more rows than q where they lie one behind the other (`one_row`: of tokens, in a batch of one)."""
+    lead, (hk, dk), (hv, dv) = tuple(q.shape[:-2]), q.shape[-2:], v.shape[-2:]
+    for name, t, last in (("k", k, (hk, dk)), ("v", v, (hv, dv)), ("g", g, (hv, dk) if kda else (hv,)), ("beta", beta, (hv,))):
+        rows, heads = tuple(t.shape[:len(lead)]), tuple(t.shape[len(lead):])
+        if not (_reachable(t, q) and heads == last and len(rows) == len(lead) and rows[0] >= lead[0] and
+                (rows[1:] == lead[1:] or (one_row and rows[1:] > lead[1:]))):
+            raise ValueError(f"{name}: {tuple(t.shape)} on {t.device} does not go with q {tuple(q.shape)} on {q.device} and {hv} V-heads")
+
+
+def _check_room(name, t, q, dtype, n):
+    """A tensor (or None) that the kernels take by its address: contiguous, `n` elements of `dtype` (None: `n` bytes)."""
+    if t is None:
+        return
+    have = t.numel() * (t.element_size() if dtype is None else 1)
+    if not (_reachable(t, q) and t.is_contiguous() and (dtype is None or t.dtype == dtype) and have >= n):
+        raise ValueError(f"{name}: {t.dtype} {tuple(t.shape)}, strides {tuple(t.stride())}, on {t.device}; wanted are {n} "
+                         f"{'bytes' if dtype is None else dtype}, contiguous, on {q.device}")
+
+
 def prepare_args(q, k, v, g, beta, *, variant="gdn", h0=None, cu_seqlens=None, max_seqlen=0, scale=1.0,
                  o=None, hT=None, want_hT=True, workspace=None, status_word=None):
     """Marshal torch CUDA tensors into ha_la_prefill_args (allocating o / hT / workspace / status word
@@ -289,6 +314,11 @@ def prepare_args(q, k, v, g, beta, *, variant="gdn", h0=None, cu_seqlens=None, m
     N = (cu_seqlens.numel() - 1) if packed else B
     if packed:
         assert cu_seqlens.dtype == torch.int32 and cu_seqlens.is_cuda and B == 1
+    _check_inputs(q, k, v, g, beta, variant in ("kda", HA_LA_KDA), B == 1)
+    state = N * HV * dk * dv
+    for name, t, dt, n in (("h0", h0, torch.float32, state), ("hT", hT, torch.float32, state), ("o", o, q.dtype, B * T * HV * dv),
+                           ("cu_seqlens", cu_seqlens, torch.int32, 0), ("workspace", workspace, None, 0), ("status_word", status_word, None, 4)):
+        _check_room(name, t, q, dt, n)
     if o is None:
         o = torch.empty_like(v)
     if hT is None and want_hT:
@@ -352,8 +382,17 @@ def prepare_decode_args(q, k, v, g, beta, state, *, variant="gdn", scale=1.0, o=
     `state_out` (default: in place into `state`; allocated when `state` is None)."""
     import torch
 
+    if not q.is_cuda:
+        raise ValueError("ha_la_decode needs CUDA tensors (there is no CPU path)")
     N, HK, d = q.shape
     HV = v.shape[1]
+    if q.dtype not in (torch.bfloat16, torch.float32):
+        raise ValueError(f"q: {q.dtype}")
+    _check_inputs(q, k, v, g, beta, variant != "gdn", False)
+    for name, t, dt, n in (("q", q, q.dtype, 0), ("k", k, q.dtype, 0), ("v", v, q.dtype, 0), ("g", g, torch.float32, 0),
+                           ("beta", beta, torch.float32, 0), ("state", state, torch.float32, N * HV * d * v.shape[2]),
+                           ("state_out", state_out, torch.float32, N * HV * d * v.shape[2]), ("o", o, q.dtype, N * HV * v.shape[2])):
+        _check_room(name, t, q, dt, n)
     if o is None:
         o = torch.empty_like(v)
     if state_out is None:

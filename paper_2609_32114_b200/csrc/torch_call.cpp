@@ -1,8 +1,8 @@
 // The two torch entry points of binding.py (ha_la_prefill, ha_la_decode) as one native call each: tensors are unpacked,
 // checked, missing outputs allocated and the C struct filled here instead of in Python (one decoding step cost its caller
 // 12 us of interpreter and ctypes time around a 3 us kernel).  Nothing is computed here.  A call that is not entirely
-// ordinary -- a tensor of another type or layout, the batch dimension left out -- returns None, and binding.py takes it
-// through its own marshalling, which also words the errors.
+// ordinary -- a tensor of another type, layout, size or device, the batch dimension left out -- returns None, and binding.py
+// takes it through its own marshalling, which also words the errors.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -29,11 +29,25 @@ bool unpack(PyObject* o, const at::Tensor** t) {
 bool plain(const at::Tensor* t, at::ScalarType type, int64_t dim) {
   return t && t->is_cuda() && t->scalar_type() == type && t->dim() == dim && t->is_contiguous();
 }
+// q [rows.., HK, dk] sets the sizes of k, v [rows.., HV, dv], g [rows.., HV] (KDA: and dk) and beta [rows.., HV].  The others may
+// have more rows than q where they lie one behind the other.
 bool inputs(const at::Tensor* q, const at::Tensor* k, const at::Tensor* v, const at::Tensor* g, const at::Tensor* beta,
             int64_t dim, bool kda) {
   if (!q || !(q->scalar_type() == at::kBFloat16 || q->scalar_type() == at::kFloat)) return false;
-  return plain(q, q->scalar_type(), dim) && plain(k, q->scalar_type(), dim) && plain(v, q->scalar_type(), dim) &&
-         plain(g, at::kFloat, kda ? dim : dim - 1) && plain(beta, at::kFloat, dim - 1);
+  if (!plain(q, q->scalar_type(), dim) || !plain(k, q->scalar_type(), dim) || !plain(v, q->scalar_type(), dim) ||
+      !plain(g, at::kFloat, kda ? dim : dim - 1) || !plain(beta, at::kFloat, dim - 1))
+    return false;
+  const int64_t h = dim - 2, HV = v->size(h);            // (dimension of the heads)
+  for (const at::Tensor* t : {k, v, g, beta}) {
+    if (t->get_device() != q->get_device() || t->size(0) < q->size(0)) return false;
+    if (h == 2 && !(t->size(1) == q->size(1) || (q->size(0) == 1 && t->size(1) > q->size(1)))) return false;
+  }
+  return k->size(h) == q->size(h) && k->size(h + 1) == q->size(h + 1) && g->size(h) == HV && beta->size(h) == HV &&
+         (!kda || g->size(h + 1) == q->size(h + 1));
+}
+// an optional tensor with room for n elements that the kernels can take by its address
+bool room(const at::Tensor* t, const at::Tensor& q, at::ScalarType type, int64_t n) {
+  return !t || (t->is_cuda() && t->get_device() == q.get_device() && t->scalar_type() == type && t->is_contiguous() && t->numel() >= n);
 }
 void* ptr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
 
@@ -59,6 +73,10 @@ PyObject* decode_call(PyObject* const* a, Py_ssize_t n) {
   const bool kda = a[7] == Py_True;
   if (!unpack(a[0], &q) || !unpack(a[1], &k) || !unpack(a[2], &v) || !unpack(a[3], &g) || !unpack(a[4], &beta) ||
       !unpack(a[5], &st) || !unpack(a[9], &o) || !unpack(a[10], &so) || !inputs(q, k, v, g, beta, 3, kda))
+    Py_RETURN_NONE;
+  const int64_t state = q->size(0) * v->size(1) * q->size(2) * v->size(2);
+  if (!room(st, *q, at::kFloat, state) || !room(so, *q, at::kFloat, state) ||
+      !room(o, *q, q->scalar_type(), q->size(0) * v->size(1) * v->size(2)))
     Py_RETURN_NONE;
   ha_la_decode_args d{};
   d.variant = kda;
@@ -105,8 +123,12 @@ PyObject* prefill_call(PyObject* const* a, Py_ssize_t n) {
       !unpack(a[5], &h0) || !unpack(a[6], &cu) || !unpack(a[11], &o) || !unpack(a[12], &hT) || !unpack(a[14], &ws) ||
       !unpack(a[15], &sw) || !inputs(q, k, v, g, beta, 4, kda))
     Py_RETURN_NONE;
-  if (cu && (!plain(cu, at::kInt, 1) || q->size(0) != 1)) Py_RETURN_NONE;
-  if (ws && !plain(ws, at::kByte, 1)) Py_RETURN_NONE;
+  if (cu && (!plain(cu, at::kInt, 1) || cu->get_device() != q->get_device() || q->size(0) != 1)) Py_RETURN_NONE;
+  if (ws && (!plain(ws, at::kByte, 1) || ws->get_device() != q->get_device())) Py_RETURN_NONE;
+  const int64_t N = cu ? cu->numel() - 1 : q->size(0), state = N * v->size(2) * q->size(3) * v->size(3);
+  if (!room(h0, *q, at::kFloat, state) || !room(hT, *q, at::kFloat, state) ||
+      !room(o, *q, q->scalar_type(), q->size(0) * q->size(1) * v->size(2) * v->size(3)) || !room(sw, *q, at::kInt, 1))
+    Py_RETURN_NONE;
   ha_la_prefill_args d{};
   d.variant = kda;
   d.dtype = q->scalar_type() == at::kFloat;
@@ -118,10 +140,9 @@ PyObject* prefill_call(PyObject* const* a, Py_ssize_t n) {
   d.d_v = (int32_t)v->size(3);
   d.chunk = 64;
   d.scale = (float)PyFloat_AsDouble(a[10]);
-  d.num_seqs = cu ? (int32_t)(cu->numel() - 1) : 0;
+  d.num_seqs = cu ? (int32_t)N : 0;
   d.max_seqlen = (int32_t)PyLong_AsLong(a[7]);
   if (PyErr_Occurred()) return nullptr;
-  const int64_t N = cu ? cu->numel() - 1 : q->size(0);
   d.q = ptr(q); d.k = ptr(k); d.v = ptr(v);
   d.g = (const float*)ptr(g); d.beta = (const float*)ptr(beta);
   d.h0 = (const float*)ptr(h0); d.cu_seqlens = (const int32_t*)ptr(cu);
