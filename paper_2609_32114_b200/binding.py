@@ -349,6 +349,25 @@ def _prefill_call(q, k, v, g, beta, stream, *, variant="gdn", h0=None, cu_seqlen
             status_word)
 
 
+def _marshal_on(stream, prepare, q, *rest, **kw):
+    """prepare(q, *rest, **kw) for a call on `stream` (a cudaStream_t, None: torch's current one): what it allocates and fills is
+    that stream's, and recorded on the current one (see CallStream in csrc/torch_call.cpp).  Returns (args, tensors, stream)."""
+    import torch
+
+    if stream is None:
+        return *prepare(q, *rest, **kw), torch.cuda.current_stream(q.device).cuda_stream
+    current = torch.cuda.current_stream(q.device if q.is_cuda else None)
+    if current.cuda_stream == stream or not q.is_cuda:     # (prepare refuses the latter)
+        return *prepare(q, *rest, **kw), stream
+    with torch.cuda.stream(torch.cuda.ExternalStream(stream, device=q.device)):
+        args, keep = prepare(q, *rest, **kw)
+    for name in ("o", "hT", "workspace", "status_word", "state_out"):
+        t = keep.get(name)
+        if t is not None and kw.get(name) is None and all(t is not x for x in rest):
+            t.record_stream(current)
+    return args, keep, stream
+
+
 def ha_la_prefill(q, k, v, g, beta, *, stream=None, **kw):
     """Prefill on torch CUDA tensors: prepare_args + the C call on torch's current stream.
 
@@ -363,12 +382,8 @@ def ha_la_prefill(q, k, v, g, beta, *, stream=None, **kw):
     if r is not None:
         raise HaLaError(r, "ha_la_prefill")
     # not an entirely ordinary call: marshalled here
-    import torch
-
     squeeze = q.dim() == 3
-    args, keep = prepare_args(q, k, v, g, beta, **kw)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
+    args, keep, stream = _marshal_on(stream, prepare_args, q, k, v, g, beta, **kw)
     rc = ha_la_prefill_raw(args, stream)
     if rc != HA_LA_OK:
         raise HaLaError(rc, "ha_la_prefill")
@@ -419,13 +434,8 @@ def ha_la_decode(q, k, v, g, beta, state, *, stream=None, variant="gdn", scale=1
     if r is not None:
         raise HaLaError(r, "ha_la_decode")
     # not an entirely ordinary call: marshalled here
-    import torch
-
     kw = dict(variant=variant, scale=scale, o=o, state_out=state_out)
-
-    args, keep = prepare_decode_args(q, k, v, g, beta, state, **kw)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
+    args, keep, stream = _marshal_on(stream, prepare_decode_args, q, k, v, g, beta, state, **kw)
     rc = ha_la_decode_raw(args, stream)
     if rc != HA_LA_OK:
         raise HaLaError(rc, "ha_la_decode")

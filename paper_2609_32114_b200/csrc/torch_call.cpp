@@ -6,9 +6,12 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+
+#include <optional>
 
 #include "ha_la.h"
 
@@ -51,10 +54,33 @@ bool room(const at::Tensor* t, const at::Tensor& q, at::ScalarType type, int64_t
 }
 void* ptr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
 
-void* stream_of(PyObject* stream, const at::Tensor& q) {
-  if (stream == Py_None) return at::cuda::getCurrentCUDAStream(q.get_device()).stream();
-  return PyLong_AsVoidPtr(stream);
-}
+// The stream of a call.  Where the caller names another than torch's current one, that is the current one while this lives:
+// tensors that the call allocates and fills come from that stream's pool and are filled in its order, and nothing that is
+// queued on the current stream can still be using (or clear, in the status word's case) what the kernels write.  The caller
+// reads them on the current stream once it has waited, so they are recorded there too and not reused before that is over.
+struct CallStream {
+  void* handle = nullptr;
+  std::optional<c10::cuda::CUDAStream> current;          // (set: another stream's call)
+  std::optional<c10::cuda::CUDAStreamGuard> guard;
+  bool set(PyObject* stream, const at::Tensor& q) {      // false: Python error
+    if (stream == Py_None) {
+      handle = at::cuda::getCurrentCUDAStream(q.get_device()).stream();
+      return true;
+    }
+    handle = PyLong_AsVoidPtr(stream);
+    return !PyErr_Occurred();
+  }
+  void will_allocate(PyObject* stream, const at::Tensor& q) {
+    if (stream == Py_None || current) return;
+    const c10::cuda::CUDAStream c = c10::cuda::getCurrentCUDAStream(q.get_device());
+    if (c.stream() == handle) return;
+    current = c;
+    guard.emplace(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(handle), q.get_device()));
+  }
+  void allocated(const at::Tensor& t) const {
+    if (current) t.record_stream(current->unwrap());
+  }
+};
 
 // (prefill, workspace bytes, decode): the library's entry points, as addresses
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -88,20 +114,21 @@ PyObject* decode_call(PyObject* const* a, Py_ssize_t n) {
   d.d_v = (int32_t)v->size(2);
   d.scale = (float)PyFloat_AsDouble(a[8]);
   if (PyErr_Occurred()) return nullptr;
+  CallStream on;
+  if (!on.set(a[6], *q)) return nullptr;
   at::Tensor o_new, s_new;
-  if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
+  if (!o || (!so && !st)) on.will_allocate(a[6], *q);
+  if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; on.allocated(o_new); }
   if (!so) {
     if (st) so = st;
-    else { s_new = at::empty({d.num_seqs, d.num_v_heads, d.d_k, d.d_k}, g->options()); so = &s_new; }
+    else { s_new = at::empty({d.num_seqs, d.num_v_heads, d.d_k, d.d_k}, g->options()); so = &s_new; on.allocated(s_new); }
   }
   d.q = ptr(q); d.k = ptr(k); d.v = ptr(v);
   d.g = (const float*)ptr(g); d.beta = (const float*)ptr(beta);
   d.h_in = (const float*)ptr(st); d.h_out = (float*)ptr(so); d.o = ptr(o);
-  void* stream = stream_of(a[6], *q);
-  if (PyErr_Occurred()) return nullptr;
   int rc;
   Py_BEGIN_ALLOW_THREADS
-  rc = g_decode(&d, stream);
+  rc = g_decode(&d, on.handle);
   Py_END_ALLOW_THREADS
   if (rc != HA_LA_OK) return PyLong_FromLong(rc);
   PyObject* po = o == &o_new ? THPVariable_Wrap(o_new) : Py_NewRef(a[9]);
@@ -153,19 +180,20 @@ PyObject* prefill_call(PyObject* const* a, Py_ssize_t n) {
   // (asked for its truth value only where the call has to know: when it brings no hT)
   const int want_hT = hT ? 0 : PyObject_IsTrue(a[13]);
   if (want_hT < 0) return nullptr;
-  if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; }
-  if (!hT && want_hT) { h_new = at::empty({N, v->size(2), q->size(3), v->size(3)}, g->options()); hT = &h_new; }
-  if (!ws) { w_new = at::empty({(int64_t)need + 256}, g->options().dtype(at::kByte)); ws = &w_new; }
-  if (!sw) { s_new = at::zeros({1}, g->options().dtype(at::kInt)); sw = &s_new; }
+  CallStream on;
+  if (!on.set(a[8], *q)) return nullptr;
+  if (!o || (!hT && want_hT) || !ws || !sw) on.will_allocate(a[8], *q);
+  if (!o) { o_new = at::empty(v->sizes(), v->options()); o = &o_new; on.allocated(o_new); }
+  if (!hT && want_hT) { h_new = at::empty({N, v->size(2), q->size(3), v->size(3)}, g->options()); hT = &h_new; on.allocated(h_new); }
+  if (!ws) { w_new = at::empty({(int64_t)need + 256}, g->options().dtype(at::kByte)); ws = &w_new; on.allocated(w_new); }
+  if (!sw) { s_new = at::zeros({1}, g->options().dtype(at::kInt)); sw = &s_new; on.allocated(s_new); }
   d.o = ptr(o); d.hT = (float*)ptr(hT); d.status_word = (int32_t*)ptr(sw);
   const uintptr_t base = (uintptr_t)ws->data_ptr(), al = (base + 255) / 256 * 256;
   d.workspace = (void*)al;
   const int64_t pad = (int64_t)(al - base);
   d.workspace_bytes = ws->numel() > pad ? (size_t)(ws->numel() - pad) : 0;   // (a buffer may end before its first aligned byte)
-  void* stream = stream_of(a[8], *q);
-  if (PyErr_Occurred()) return nullptr;
   Py_BEGIN_ALLOW_THREADS
-  rc = g_prefill(&d, stream);
+  rc = g_prefill(&d, on.handle);
   Py_END_ALLOW_THREADS
   if (rc != HA_LA_OK) return PyLong_FromLong(rc);
   PyObject* r = PyTuple_New(4);
