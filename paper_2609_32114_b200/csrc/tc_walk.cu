@@ -269,7 +269,8 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       if (aborted()) break;
     }
   } else if (warp >= W_MMA) {
-    // ------------------------------------------------------------ MMA issue (one thread issues; the warp keeps the barriers)
+    // ------------------------------------------------------------ MMA issue (one thread issues; the warp waits and keeps the barriers:
+    // bar.sync, bar.arrive and elect.sync are for converged warps.  Waits by the elected thread and __syncwarp: 1.5 % more per step)
     // One warp issues the products of the sequential path, another those of the outputs.  The tensor cores work
     // in order of issue, so the second warp goes when the first one tells it to: Y behind X, under X's epilogue, and P U~
     // behind D2, under the epilogue of the state.  Descriptors advance by constants.
@@ -300,7 +301,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         const uint64_t dK = dK0 + st * (kTileBytes >> 4);
         const uint64_t dD = dD0 + (ND == 1 ? 0 : st) * (kTileBytes >> 4);
         const uint64_t dT = dT0 + ts * (kTriB >> 4);
-        if (elect_one()) wait1(&full_k[st], ph);
+        wait1(&full_k[st], ph);
         __syncwarp();
         named_sync(BAR_H, kCompute + 32);                // h operand of the previous step
         if (elect_one()) {
@@ -312,10 +313,9 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
         }
         __syncwarp();
         if (OUT) named_arrive(BAR_GY, 64);
-        if (elect_one()) {
-          wait1(&full_t[ts], NT == 2 ? c >> 1 : c);
-          if (OUT && c > 0) wait1(bar_o, c - 1);         // (its operand lies in U's columns)
-        }
+        wait1(&full_t[ts], NT == 2 ? c >> 1 : c);
+        if (OUT && c > 0) wait1(bar_o, c - 1);         // (its operand lies in U's columns)
+        __syncwarp();
 #pragma unroll
         for (int half = 0; half < 2; ++half) {           // (tokens 0 .. 63 of U are final after the first four k-steps)
           named_sync(BAR_R + half, kCompute + 32);
@@ -324,8 +324,9 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
             tri_half(half, Cfg::TM_U, Cfg::TM_R, 8, dT, 0u);
             umma_commit(half ? bar_u1 : bar_u0);
           }
+          __syncwarp();
         }
-        if (KDA && elect_one()) wait1(&full_d[ND == 2 ? st : 0], ND == 2 ? ph : c);
+        if (KDA) wait1(&full_d[ND == 2 ? st : 0], ND == 2 ? ph : c);
         __syncwarp();
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -335,14 +336,14 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
 #pragma unroll
             for (int ks = 4 * half; ks < 4 * half + 4; ++ks)   // K index = tokens: 16 rows of 128 bytes per step
               umma_ts(Cfg::TM_X, Cfg::TM_R + 8 * ks, dD + ks * (2048u >> 4), id_km, ks > 0);
+            if (half) {
+              umma_commit(bar_d2);
+              umma_commit(&empty_k[st]);
+            }
           }
-        }
-        if (elect_one()) {
-          umma_commit(bar_d2);
-          umma_commit(&empty_k[st]);
+          __syncwarp();
         }
         if (++st == NK) { st = 0; ph ^= 1; }
-        __syncwarp();
         if (OUT) named_arrive(BAR_GP, 64);
       }
       named_sync(BAR_H, kCompute + 32);                  // pairs with the compute warps' last arrival
@@ -350,17 +351,18 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
       const uint64_t dQ = smem_desc(smem_u32(sm + Cfg::OFF_Q), 16, 1024, kSwizzle128B);
       const uint64_t dP = smem_desc(smem_u32(sm + Cfg::OFF_P), 16, 256, kSwizzle32B);
       for (int c = 0; c < nsteps; ++c) {
-        if (elect_one()) {
-          wait1(full_q, c);
-          if (c > 0) wait1(out_free, c - 1);
-        }
+        wait1(full_q, c);
+        if (c > 0) wait1(out_free, c - 1);
+        __syncwarp();
         named_sync(BAR_GY, 64);
         if (elect_one()) {
           tc_fence_after_sync();
           tile_product(Cfg::TM_Y, dQ, id_kk);
           umma_commit(bar_y);
-          wait1(full_p, c);
         }
+        __syncwarp();
+        wait1(full_p, c);
+        __syncwarp();
         if (!KDA) named_sync(BAR_UP, kCompute + 32);
         named_sync(BAR_GP, 64);
         if (elect_one()) {
@@ -369,6 +371,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
           tri_half(1, Cfg::TM_Y, KDA ? Cfg::TM_R : Cfg::TM_UP, KDA ? 8 : 16, dP, 1u);
           umma_commit(bar_o);
         }
+        __syncwarp();
       }
     }
   } else if (warp >= W_OUT) {
