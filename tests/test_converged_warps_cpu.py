@@ -24,12 +24,24 @@ def _statement_end(src, i):
     raise ValueError("unbalanced")
 
 
+def _block_end(src, i):
+    """The end of the block that src[i:] is in."""
+    depth = 0
+    for j in range(i, len(src)):
+        depth += {"{": 1, "}": -1}.get(src[j], 0)
+        if depth < 0:
+            return j
+    return len(src)
+
+
 def loose_ends(src):
-    """What follows elected blocks without a __syncwarp (or the warp-wide vote in aborted()) between."""
+    """What follows elected blocks, in the block that they are in (which may be a loop's), without a __syncwarp (or the warp-wide vote in
+    aborted()) between."""
     src = re.sub(r"//[^\n]*", "", src)
     bad = []
     for m in re.finditer(r"\bif \((?:\w+ && )?elect_one\(\)\)", src):
-        nxt = NEXT.search(src, _statement_end(src, m.end()))
+        end = _statement_end(src, m.end())
+        nxt = NEXT.search(src, end, _block_end(src, end))
         if nxt is None or nxt.group() not in ("__syncwarp", "aborted()"):
             bad.append((src.count("\n", 0, m.start()) + 1, nxt and nxt.group()))
     return bad
@@ -46,7 +58,7 @@ def test_the_elected_blocks_are_found():
 
 
 @pytest.mark.parametrize("src", ["if (elect_one()) { wait1(a, c); } named_sync(1, 64);", "if (KDA && elect_one()) wait1(a, c);\n named_arrive(1, 64);",
-                                 "if (elect_one()) {\n for (;;) { x(); }\n }\n if (elect_one()) y(); __syncwarp();", "if (elect_one()) z(); }"])
+                                 "if (elect_one()) {\n for (;;) { x(); }\n }\n if (elect_one()) y(); __syncwarp();", "{ if (elect_one()) z(); } __syncwarp();"])
 def test_planted(src):
     assert len(loose_ends(src)) == 1
 
@@ -55,7 +67,7 @@ def loose_waits(src):
     """Polling waits of the two issuing warps, which the threads of a warp may leave one by one."""
     src = re.sub(r"//[^\n]*", "", src)
     src = src[src.index("if (warp == W_MMA) {"):src.index("warp >= W_OUT")]
-    nxt = [NEXT.search(src, m.end()) for m in re.finditer(r"wait1\(", src)]
+    nxt = [NEXT.search(src, m.end(), _block_end(src, m.end())) for m in re.finditer(r"wait1\(", src)]
     assert len(nxt) >= 7
     return [n and n.group() for n in nxt if n is None or n.group() != "__syncwarp"]
 
@@ -64,7 +76,7 @@ def test_the_issuing_warps_wait_together():
     assert loose_waits(open(os.path.join(CSRC, "tc_walk.cu")).read()) == []
 
 
-@pytest.mark.parametrize("behind,find", [("umma_commit(bar_x);", loose_ends), ("umma_commit(half ? bar_u1 : bar_u0);", loose_ends), ("wait1(&full_k[st], ph);", loose_waits),
+@pytest.mark.parametrize("behind,find", [("umma_commit(bar_x);", loose_ends), ("umma_commit(half ? bar_u1 : bar_u0);", loose_ends), ("umma_commit(bar_o);", loose_ends), ("wait1(&full_k[st], ph);", loose_waits),
                                          ("wait1(full_p, c);", loose_waits)])
 def test_planted_in_the_kernel(behind, find):
     src = open(os.path.join(CSRC, "tc_walk.cu")).read()
