@@ -73,10 +73,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
-// For a CTA in which a wait ran out: gives its copies that may still be in flight time to land (64 us and more), so that
-// they do not end in the shared memory of whatever runs on this SM next.
+__device__ __forceinline__ uint64_t global_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+
+// For a CTA in which a wait ran out: gives its copies that may still be in flight 64 us to land, so that they do not end in the
+// shared memory of whatever runs on this SM next.  By the clock (and a count, should that stand still): nanosleep's time is an
+// upper bound only, it may return at once.
 __device__ __forceinline__ void settle_copies() {
-  for (int i = 0; i < 64; ++i) __nanosleep(1000);
+  const uint64_t t0 = global_ns();
+  for (int i = 0; i < 65536 && global_ns() - t0 < 64000; ++i) __nanosleep(1000);
 }
 
 // ---------------------------------------------------------------- proxies and fences

@@ -44,3 +44,10 @@ def test_a_kernel_that_gave_up_waiting_lets_its_copies_land():
             assert src[m.end():].split("}")[0].strip() == "settle_copies();", os.path.basename(f)
             found += 1
     assert found == 5                                      # every kernel that copies in bulk
+
+
+def test_that_pause_is_by_the_clock():
+    """nanosleep may return at once, so the pause has to be measured, and bounded should the clock stand still."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "tc_ptx.cuh")).read())
+    body = src[src.index("void settle_copies()"):].split("\n}")[0]
+    assert "%globaltimer" in src and re.search(r"for \(int i = 0; i < \d+ && global_ns\(\) - t0 < \d+;", body)
