@@ -40,10 +40,10 @@ using namespace solve;
 namespace {
 
 constexpr int kKdaThreads = 512;                           // eight scaling warps, eight solving warps
-// per buffer (items alternate): K then K 2^{G-rho} in place | Q likewise | K 2^{rho-G}, then T (fp16 blocks)
+// per buffer (items alternate): K then K 2^{G-rho} in place | Q likewise | K 2^{rho-G}, then, once contracted, T (fp16 blocks)
 constexpr uint32_t OFF_K = 0, OFF_Q = kTileBytes, OFF_K1 = 2 * kTileBytes, kBufBytes = 3 * kTileBytes;
 constexpr uint32_t OFF_A = 2 * kBufBytes;                  // fp16 A below the diagonal blocks: 28 blocks, operand order
-constexpr uint32_t OFF_D = OFF_A + 28 * 512;               // fp32 diagonal blocks of A
+constexpr uint32_t OFF_D = OFF_A + kABlocks * 512;         // fp32 diagonal blocks of A, then the solve's last intermediate
 constexpr uint32_t OFF_TOT = OFF_D + (kDiagBytes + 127) / 128 * 128;     // float [8][128]: log2 decay of each block
 constexpr uint32_t OFF_RHO = OFF_TOT + 4096;               // per buffer: int16 [9][rho_slot(channel pair)][2], rho_J
 constexpr uint32_t OFF_BETA = OFF_RHO + 2 * 9 * 256;       // per buffer: float [128]
@@ -51,6 +51,7 @@ constexpr uint32_t OFF_FALL = OFF_BETA + 2 * 512;          // per buffer: int [8
 constexpr uint32_t OFF_BAR = OFF_FALL + 2 * 64;
 constexpr uint32_t kKdaSmem = OFF_BAR + 32;
 static_assert(kKdaSmem <= 227 * 1024, "shared memory budget");
+static_assert(kXBlocks * 512 <= OFF_TOT - OFF_D && kTBlocks * 512 <= kTileBytes, "what lies over what (OFF_TOT is the next item's already)");
 constexpr float kMaxUp = 100.f;
 
 struct KdaParams {
