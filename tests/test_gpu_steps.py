@@ -80,22 +80,25 @@ def test_packed_batch_without_a_token(variant, dtype, d, seqs):
     import torch
     import paper_2609_32114_b200 as ha
 
-    any_ = torch.zeros(4096, device="cuda")                # in the place of q, k, v, g, beta, o: no token of them is touched
+    any_ = torch.rand(4096, device="cuda") + 1.0           # in the place of q, k, v, g, beta, o: no token of them is touched
     cu = torch.zeros(seqs + 1, dtype=torch.int32, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    h0 = torch.randn(seqs, 3, d, d, device="cuda")
+    h0 = torch.randn(4, 3, d, d, device="cuda")[:seqs]     # (room behind the states, the workspace and any_ for the numbers below)
     p = any_.data_ptr()
     for start in (h0, None):
-        hT = torch.full_like(h0, float("nan"))
+        hT_all = torch.full((4, 3, d, d), float("nan"), device="cuda")
+        hT = hT_all[:seqs]
         a = ha.make_args(variant=variant, dtype=dtype, batch=1, seqlen=0, hk=1, hv=3, dk=d, dv=d, num_seqs=seqs, q=p, k=p, v=p, g=p,
                          beta=p, o=p, h0=0 if start is None else start.data_ptr(), cu_seqlens=cu.data_ptr(), hT=hT.data_ptr(),
                          status_word=status.data_ptr())
         need = ha.ha_la_prefill_workspace_bytes(a)
-        ws = torch.full((need + 256,), 0x7f, dtype=torch.uint8, device="cuda")    # lengths of two thousand million, if they were read
+        # were the tables read before they are written: sequence, token, length and slot one, which shows as a wrong state
+        ws = torch.ones((need + (4 << 20)) // 4, dtype=torch.int32, device="cuda")
         a.workspace, a.workspace_bytes = (ws.data_ptr() + 255) // 256 * 256, need
         assert ha.ha_la_prefill_raw(a, torch.cuda.current_stream().cuda_stream) == 0
         torch.cuda.synchronize()
         assert int(status.item()) == 0 and torch.equal(hT, torch.zeros_like(h0) if start is None else start)
+        assert bool(hT_all[seqs:].isnan().all())
 
 
 @pytest.mark.parametrize("hk,hv,lens", [(32, 32, [4500]), (16, 32, [4097]), (3, 9, [9000, 5, 4000])])
@@ -138,3 +141,43 @@ def test_many_runs(variant, tokens):
     a = ha.make_args(variant=variant, dtype="bf16", batch=1, seqlen=tokens, hk=1, hv=2, dk=128, dv=128)
     assert ha.ha_la_prefill_num_runs(a) >= 12
     helpers.check_parity(inp)
+
+
+def _four_alike(variant, length, where, size):
+    """One head of `length` tokens, no decay, beta = 0 but for the tokens `where`, whose keys are alike with |k|^2 = size: the
+    inverse has size (size - 1)^n between tokens n + 1 apart in that list, the identity elsewhere."""
+    import numpy as np
+
+    inp = _inputs(variant, [length], False, 1, 1, 389, gate_shift=-6.0)
+    inp["g"][:] = 0.0
+    inp["beta"][:] = 0.0
+    inp["beta"][list(where)] = 1.0
+    key = np.zeros(128, np.float32)
+    key[::8] = (size / 16) ** 0.5
+    inp["k"][:, :, ::8] = 0.0                              # (all others at right angles to them)
+    inp["k"][list(where)] = synth.round_to_bf16(key)
+    return inp
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("level", ["diagonal", "1", "2", "3", "A"])
+def test_overflow_is_reported_from_every_block(variant, level):
+    """The one value that leaves the fp16 range in a block of the inverse on the diagonal, next to it (level 1), two blocks from it
+    (level 2), of A T between the halves (level 3), or of A itself, everything else far inside: reported whichever block it is, to
+    the end of a step and where the sequence ends behind it.  With smaller keys nothing is."""
+    first = lambda b: 16 * b
+    if level == "diagonal":
+        at = [(first(b), first(b) + 5, first(b) + 9, first(b) + 15) for b in range(8)]
+    elif level == "1":
+        at = [(first(b) + 2, first(b) + 9, first(b + 1) + 3, first(b + 1) + 12) for b in (0, 2, 4, 6)]
+    elif level == "2":
+        at = [(first(J) + 1, first(J) + 8, first(I) + 4, first(I) + 13) for h in (0, 4) for I in (h + 2, h + 3) for J in (h, h + 1)]
+    elif level == "3":
+        at = [(first(J) + 1, first(J) + 6, first(J) + 15, first(I) + 7) for I in range(4, 8) for J in range(4)]
+    else:
+        at = [(first(J) + 3, first(I) + 10) for I in range(8) for J in range(I)]
+    big, small = (90000.0, 40000.0) if level == "A" else (50.0, 25.0)   # 50 49^2 = 120050 > 65504 > 25 24^2
+    for where in at:
+        for length in {where[-1] + 1, 128, 150}:
+            assert helpers.run_gpu(_four_alike(variant, length, where, big))[2] == 6, (where, length)
+            assert helpers.run_gpu(_four_alike(variant, length, where, small))[2] == 0, (where, length)
