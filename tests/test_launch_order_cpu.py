@@ -36,6 +36,32 @@ def test_nothing_is_read_before_the_wait(file, kernel, body):
     assert re.findall(TABLES, before) == [] and re.findall(INPUTS, before) == [], f"{kernel} in {file}"
 
 
+# ... and by way of copies, helpers, casts and pointers made from a parameter
+ACCESS = (r"\b(?:bulk_load|tma_load_4d|prefetch_l2|__ldcs|__ldg|__ldcg|__stcs|load4|ld4|load_tile|load_gates|issue_tiles|fetch|atomic\w+)\s*\("
+          r"|reinterpret_cast<[^>]*\*>\(p\.\w+[^)]*\)\s*\[|(?<=[=(,?:])\s*\*\s*\(?(?:p|sb)\.|(?<![\w.])(?:src|dst|phi|rec|img|gp|my_len)\s*\[")
+
+
+def accesses(before):
+    """Accesses in the code that runs ahead of the wait: all but the bodies of lambdas, which are called later or found by name."""
+    flat = re.sub(r"auto \w+ = \[&\]\([^)]*\) \{(?:[^{}]|\{[^{}]*\})*\};", "", before)
+    return re.findall(ACCESS, flat)
+
+
+@pytest.mark.parametrize("file,kernel,body", list(_kernels()), ids=lambda x: x if isinstance(x, str) and len(x) < 30 else "")
+def test_no_copy_or_pointer_is_followed_before_the_wait(file, kernel, body):
+    assert accesses(body[body.index("{"):body.index("griddepcontrol.wait")]) == [], f"{kernel} in {file}"
+
+
+@pytest.mark.parametrize("early", ["bulk_load(sm, rec + kStepT, kTriB, &full[0]);", "tma_load_4d(sm, &map_k, &full[0], 0, j, t0, 0);", "fetch(1);",
+                                   "load_tile(b, h);", "const float x = src[lane];", "vv = load4(reinterpret_cast<const In*>(p.v) + nj);",
+                                   "len = *(p.seq_len + n);", "len = *p.seq_len;", "sk[0] = to_f32(reinterpret_cast<const In*>(p.k)[qk]);",
+                                   "h = __ldcs(reinterpret_cast<const float4*>(p.h_in + base));", "issue_tiles(gm, 0);", "q = ld4(p.g + off);"])
+def test_planted_access_before_the_wait(early):
+    for _, kernel, body in _kernels():
+        at = body.index("asm volatile(\"griddepcontrol.wait")
+        assert accesses(body[body.index("{"):at] + early), kernel
+
+
 def test_a_kernel_that_gave_up_waiting_lets_its_copies_land():
     found = 0
     for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
