@@ -4,8 +4,8 @@
 // costs is Phi_s on its way out of L2, 64 KiB per CTA, so that is copied in bulk one product ahead (operand fragments
 // read straight from global memory touch every line several times: 2.2 us per product).  The product itself is 48 warp-level
 // MMAs a warp on values split into two bf16 each (hi hi + hi lo + lo hi, fp32 accumulation: 2^-16 of the factors).  The
-// state's fragments go round the warps through 8 KiB of shared memory, transposed in registers.  Measured on B200: 1.1 us per
-// product with every CTA on an SM (four products 15 us by themselves, launch included, twenty 33).  Fragment row r of a warp is key sigma(r), sigma(2 t + e) = 4 t + e, sigma(8 + 2 t + e)
+// state's fragments go round the warps through 8 KiB of shared memory, transposed in registers.  What bounds it is the chain: about
+// 1 us per product with every CTA on an SM.  Fragment row r of a warp is key sigma(r), sigma(2 t + e) = 4 t + e, sigma(8 + 2 t + e)
 // = 4 t + 2 + e: the four columns of Phi that a lane needs are then neighbours.
 #include "tc_common.cuh"
 #include "tc_mma.cuh"
@@ -16,7 +16,7 @@ using namespace ptx;
 
 namespace {
 
-constexpr int kFixCols = 16, kManySpans = 12;
+constexpr int kFixCols = 16, kFewPairs = 4;
 
 __device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
   hi = pack_bf16(x, y);
@@ -27,12 +27,14 @@ __device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint3
 constexpr uint32_t kPhiBytes = 65536;
 constexpr uint32_t OFF_FRAG = 2 * kPhiBytes, OFF_FBAR = OFF_FRAG + 2 * 8 * 2 * 32 * 16, kSpanSmem = OFF_FBAR + 32;
 
-// Two instances.  With MANY the copies are issued under elect.sync, which gives a kernel of 79 registers instead of 66 whose products
-// are 0.2 us shorter and whose start is 3 us longer.  Calls measured with either, MANY second, GDN unless said: 2 heads, T = 6000, 12
-// spans 43.1 -> 42.1 us; 4 heads, T = 8192, 16 spans 54.3 -> 53.5; T = 16384, 19 spans 74.4 -> 72.7 (KDA, T = 12000 89.6 -> 88.0); 2 heads,
-// T = 16384, 22 spans 68.4 -> 66.4; T = 32768, 32 spans 94.8 -> 91.5; but 8 heads, T = 12000, 10 spans 78.7 -> 79.6; 16 heads, T = 4096,
-// 6 spans 55.9 -> 59.0; and packed batches, whose lengths come from a table, are longer with it at any number (14 spans 142 -> 148).
-template <bool MANY>
+// Two instances that differ in who issues the copies, a thread elected by elect.sync or thread 0, and for that in the code that the
+// compiler makes of the whole kernel (79 registers against 66).  Which is faster goes by the number of CTAs.  Calls, thread 0's first: up to
+// four (sequence, V-head) pairs, 32 CTAs, gain at any number of runs and packed or not (1 head, T = 12000, 19 runs 55.7 -> 53.2 us; 2 heads,
+// T = 3000, 8 runs 34.0 -> 33.3, T = 16000, 21 runs 65.9 -> 63.6; 4 heads, T = 3000 35.1 -> 34.7, T = 24000, 19 runs 90.1 -> 88.0; two sequences
+// of 11 k tokens, 2 heads 68.9 -> 67.7); five and six pairs are within 1 % either way; more lose (7 heads, T = 3000 38.3 -> 39.2; 8 heads, T = 6000
+// 52.5 -> 54.4; four rows of 4000, 2 heads 43.7 -> 46.1; 16 heads, T = 4096 55.9 -> 59.0).  The reason is not known: measure again after
+// an edit of this kernel or with another compiler.
+template <bool ELECT>
 __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row, int HV, const int32_t* seq_len, int32_t* status) {
   extern __shared__ __align__(128) uint8_t sm[];
   uint4 (*frag)[8][2][32] = reinterpret_cast<uint4(*)[8][2][32]>(sm + OFF_FRAG);   // [s & 1][k-step][n-tile][lane]: hi b0, b1, lo b0, b1
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
     for (int i = 0; i < 4; ++i)
       bulk_load(sm + (s & 1) * kPhiBytes + i * 16384, phi + (size_t)s * stride + i * 4096, 16384, &full[s & 1]);
   };
-  auto issuing = [&]() { return MANY ? warp == 0 && elect_one() : threadIdx.x == 0; };
+  auto issuing = [&]() { return ELECT ? warp == 0 && elect_one() : threadIdx.x == 0; };
   if (issuing()) {
     fetch(1);
     fetch(2);
@@ -162,7 +164,7 @@ cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = g_timer ? 0 : 1;                        // (per-kernel timing wants one kernel at a time)
-  auto kern = !plan.seq_len && sb.nspan >= kManySpans ? span_fix_kernel<true> : span_fix_kernel<false>;
+  auto kern = p.N * p.HV <= kFewPairs ? span_fix_kernel<true> : span_fix_kernel<false>;
   return cudaLaunchKernelEx(&cfg, kern, sb, p.T_row, p.HV, (const int32_t*)plan.seq_len, status);
 }
 

@@ -134,7 +134,7 @@ def test_overflow_in_any_block_is_reported(variant, first, length):
 
 @pytest.mark.parametrize("variant,tokens", [("gdn", 6000), ("gdn", 6016), ("kda", 8200)])
 def test_many_runs(variant, tokens):
-    """Sequences that the rule cuts into twelve runs and more, whose start states another instance makes; the last run full or ragged."""
+    """Sequences that the rule cuts into twelve runs and more; the last run full or ragged."""
     import paper_2609_32114_b200 as ha
 
     inp = _inputs(variant, [tokens], False, 1, 2, 383, gate_shift=5.0)
@@ -181,3 +181,12 @@ def test_overflow_is_reported_from_every_block(variant, level):
         for length in {where[-1] + 1, 128, 150}:
             assert helpers.run_gpu(_four_alike(variant, length, where, big))[2] == 6, (where, length)
             assert helpers.run_gpu(_four_alike(variant, length, where, small))[2] == 0, (where, length)
+
+
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("hv,lens", [(4, [1100]), (5, [1100]), (1, [900, 0, 130, 1]), (1, [900, 0, 130, 1, 513]), (2, [900, 600])])
+@pytest.mark.parametrize("runs", [2, 8])
+def test_start_states_on_both_sides_of_four_pairs(variant, hv, lens, runs, monkeypatch):
+    """Four (sequence, V-head) pairs and fewer have their start states from another instance than five and more."""
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
+    helpers.check_parity(_inputs(variant, lens, len(lens) > 1, 1, hv, 397, gate_shift=4.0))
