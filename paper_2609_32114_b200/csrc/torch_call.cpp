@@ -40,17 +40,21 @@ bool inputs(const at::Tensor* q, const at::Tensor* k, const at::Tensor* v, const
   if (!plain(q, q->scalar_type(), dim) || !plain(k, q->scalar_type(), dim) || !plain(v, q->scalar_type(), dim) ||
       !plain(g, at::kFloat, kda ? dim : dim - 1) || !plain(beta, at::kFloat, dim - 1))
     return false;
-  const int64_t h = dim - 2, HV = v->size(h);            // (dimension of the heads)
-  for (const at::Tensor* t : {k, v, g, beta}) {
-    if (t->get_device() != q->get_device() || t->size(0) < q->size(0)) return false;
-    if (h == 2 && !(t->size(1) == q->size(1) || (q->size(0) == 1 && t->size(1) > q->size(1)))) return false;
+  // (as arrays: a tensor's size(i) is a call and a range check each)
+  const int64_t *qs = q->sizes().data(), *ks = k->sizes().data(), *vs = v->sizes().data(), *gs = g->sizes().data(), *bs = beta->sizes().data();
+  const int h = (int)dim - 2;                            // (dimension of the heads)
+  const auto device = q->device();
+  for (const at::Tensor* t : {k, v, g, beta})
+    if (t->device() != device) return false;
+  for (const int64_t* ts : {ks, vs, gs, bs}) {
+    if (ts[0] < qs[0]) return false;
+    if (h == 2 && !(ts[1] == qs[1] || (qs[0] == 1 && ts[1] > qs[1]))) return false;
   }
-  return k->size(h) == q->size(h) && k->size(h + 1) == q->size(h + 1) && g->size(h) == HV && beta->size(h) == HV &&
-         (!kda || g->size(h + 1) == q->size(h + 1));
+  return ks[h] == qs[h] && ks[h + 1] == qs[h + 1] && gs[h] == vs[h] && bs[h] == vs[h] && (!kda || gs[h + 1] == qs[h + 1]);
 }
 // an optional tensor with room for n elements that the kernels can take by its address
 bool room(const at::Tensor* t, const at::Tensor& q, at::ScalarType type, int64_t n) {
-  return !t || (t->is_cuda() && t->get_device() == q.get_device() && t->scalar_type() == type && t->is_contiguous() && t->numel() >= n);
+  return !t || (t->device() == q.device() && t->scalar_type() == type && t->is_contiguous() && t->numel() >= n);
 }
 void* ptr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
 
@@ -150,8 +154,8 @@ PyObject* prefill_call(PyObject* const* a, Py_ssize_t n) {
       !unpack(a[5], &h0) || !unpack(a[6], &cu) || !unpack(a[11], &o) || !unpack(a[12], &hT) || !unpack(a[14], &ws) ||
       !unpack(a[15], &sw) || !inputs(q, k, v, g, beta, 4, kda))
     Py_RETURN_NONE;
-  if (cu && (!plain(cu, at::kInt, 1) || cu->get_device() != q->get_device() || q->size(0) != 1)) Py_RETURN_NONE;
-  if (ws && (!plain(ws, at::kByte, 1) || ws->get_device() != q->get_device())) Py_RETURN_NONE;
+  if (cu && (!plain(cu, at::kInt, 1) || cu->device() != q->device() || q->size(0) != 1)) Py_RETURN_NONE;
+  if (ws && (!plain(ws, at::kByte, 1) || ws->device() != q->device())) Py_RETURN_NONE;
   const int64_t N = cu ? cu->numel() - 1 : q->size(0), state = N * v->size(2) * q->size(3) * v->size(3);
   if (!room(h0, *q, at::kFloat, state) || !room(hT, *q, at::kFloat, state) ||
       !room(o, *q, q->scalar_type(), q->size(0) * q->size(1) * v->size(2) * v->size(3)) || !room(sw, *q, at::kInt, 1))
