@@ -36,6 +36,7 @@ KEYS = [
     ("smsp__inst_executed.sum", "warp instructions"),
     ("sm__cycles_active.avg", "SM active cycles (avg)"),
     ("l1tex__data_bank_conflicts_pipe_lsu_mem_shared.sum", "shared-memory bank conflicts"),
+    ("l1tex__data_pipe_lsu_wavefronts.avg.pct_of_peak_sustained_elapsed", "LSU data pipe (% of peak)"),
 ]
 
 
@@ -45,7 +46,7 @@ def report(rep: str, workload: str, title: str, cmd: str) -> str:
     hdr, units = rows[0], rows[1]
     stall = [h for h in hdr if "issue_stalled" in h and "per_issue_active" in h and "not_issued" not in h]
     out = [f"# {title}", "", f"workload: {workload}", "",
-           "Command (runs committed files only; on a B200 through the pool's runner):", "", f"    {cmd}", ""]
+           "Command (committed files only, on a B200):", "", f"    {cmd}", ""]
     for r in rows[2:]:
         out.append(f"## {r[hdr.index('Kernel Name')]}")
         for k, label in KEYS:
