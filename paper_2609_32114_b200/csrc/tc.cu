@@ -79,10 +79,11 @@ int forced_segments() {
 
 // Spans per sequence of the step path (tc_walk.cu): with few (sequence, head) pairs a sequence is cut into S runs that
 // are walked at the same time, in two launches, 2 S - 3 state-only runs and then S runs with outputs, with S - 2
-// products of 128^3 between them.  Costs measured on B200 with the step kernels as first built: 2.0 us per state-only step, 2.45 per step
-// with outputs (1.65 and 2.25 now: another S, mostly by one, in a call of twenty, and no other times where that was measured), 5 for
+// products of 128^3 between them.  The rule's costs: 2.0 us per state-only step, 2.45 per step with outputs, 5 for
 // a CTA's start and end, 1.25 per product (5 when the products' 8 CTAs per pair do not all have an SM) and about 8 for
-// the two further launches.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
+// the two further launches.  The steps take less now (tc_walk.cu), but with 1.65 and 2.25 here the choice gets no better: it
+// changes in 5 % of calls, and 44 of those timed both ways went from 13 % longer (one row of 1300 tokens, 4 heads, in order instead of 6
+// runs 28.8 -> 32.6 us) to 7 % shorter (three sequences of 3 k tokens, 4 heads, 13 runs -> 9 68.4 -> 63.4), 0.1 % longer on average.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
 // within some 15 %.  And no launch beats HBM, at 6 TB/s, once its operands do not stay in L2: a packed batch of 8 sequences
 // with 136 k tokens cut in two took 220 + 15 us for the first launch and the products and 452 for the second, 444 of them
 // HBM's, against 570 us uncut (1160 against 1021 for the call).

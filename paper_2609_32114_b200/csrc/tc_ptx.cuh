@@ -13,10 +13,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// One thread of a converged warp.  Code that issues tcgen05.mma is to stand under `if (elect_one())`, not under a test of the lane: the
-// compiler then knows that a single thread is active and keeps the operands in uniform registers.  Measured on B200, 32
-// products with A in tensor memory: 53 cycles each to issue behind `lane == 0`, whatever N; 10 behind this, so that the
-// tensor cores' own N / 2 cycles are what counts.
+// One thread of a converged warp.  Code that issues tcgen05.mma is to stand under `if (elect_one())`, not under a test of the lane.
+// Measured on B200, 32 products with A in tensor memory: 53 cycles each to issue behind `lane == 0`, whatever N; 10 behind
+// this (the compiler can tell that a single thread is active, presumably), so that the tensor cores' own N / 2 cycles are what counts.
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred = 0;
   asm volatile("{\n\t.reg .b32 x;\n\t.reg .pred p;\n\telect.sync x|p, 0xffffffff;\n\t@p mov.s32 %0, 1;\n\t}" : "+r"(pred));

@@ -26,13 +26,12 @@
 // operator anyway); this assumes the delta rule's usual normalisation (beta |k|^2 of order one), far inside the fp16
 // range, and a result outside it is reported.
 //
-// What bounds it: with a q/k head per V-head and long calls HBM, 101 KiB a unit (8 sequences of 136 k tokens, 16 heads: 283 us, 93 % of
-// the measured copy rate); with tiles out of L2, and in short calls, the shared-memory accesses and dependent phases of the
-// solve and the masks.  Two things counted: instructions (index arithmetic and register moves were a third of 10.2 k
-// warp instructions per unit; three groups instead of two alone took 388 us to 342) and the serial chain of a unit (masks
-// 2.4 -> 2.0 k cycles, solve 6.6 -> 2.8 k, by themselves on an SM).  Measured on B200, this kernel alone, two groups before ->
-// now: 16 heads, T = 333 14.5 -> 13.0 us (launch included), T = 4096 26.6 -> 22.9; 32 heads on 16 q/k heads, T = 16384 93 -> 79;
-// 32 heads, T = 8192 65 -> 54; the 136 k tokens 388 -> 283.
+// What bounds it: with a q/k head per V-head and long calls HBM, 101 KiB a unit (8 sequences of 136 k tokens, 16 heads, 17 k units:
+// 278 us, 98 % of the measured copy rate); with tiles out of L2, and in short calls, the shared-memory accesses and dependent
+// phases of the solve and the masks: 8.5 k warp instructions and 4.8 k SM-cycles a unit with two V-heads per q/k head, the LSU
+// data pipe 51 % busy.  This kernel by itself on B200, launch included: 16 heads, T = 333 13.6 us, T = 4096 23; 32 heads,
+// T = 16384 86, on 16 q/k heads 80, on 8 77.  (Two groups that shared a unit's loads and products among V-heads: 14.5, 27,
+// -, 93 and, on the 136 k tokens, 388.)
 //
 // Tokens past the end of a sequence are made no-ops by beta = 0 and g = 0; whatever the TMA box read for them (the
 // next sequence's rows, or zero fill past the end of the tensor) is multiplied by exact zeros.  This relies on the

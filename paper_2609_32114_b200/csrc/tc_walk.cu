@@ -20,9 +20,8 @@
 // lower triangular: step ks of their products runs with N = 128 - 16 ks rows.  U and D2 run in token halves, so that an epilogue
 // starts when half of its input is final; Y goes behind X and P U~ behind D2, where the sequential path leaves the tensor
 // cores idle.
-// Measured on B200: 2.0 us per step of 128 tokens and head with outputs and 1.5 without while the operands come out of L2, 2.35 and
-// 1.75 out of HBM with most SMs at work.  Issue under elect.sync and the operand slots as they are, from 2.45 / 2.0:
-// 32 heads, T = 16384 states only 88 -> 76 us, with outputs 115 -> 107; 8 sequences of 136 k tokens, 16 heads 571 -> 549 (HBM 440).
+// Measured on B200, a launch by itself: 2.2 us per step of 128 tokens with outputs and 1.4 without (between 6 and 43 steps, most SMs
+// at work) and 11 for its start and end; 8 sequences of 136 k tokens, 16 heads 537 us, 5.4 TB/s.
 //
 // Warp roles: sixteen compute warps (tensor-memory lanes 32 (w % 4).., group w / 4 of the columns), four output warps, two
 // producer warps, two warps that issue MMAs (the sequential path; the outputs).  Every wait is bounded.
