@@ -11,6 +11,7 @@ FAKE = """
 import sys, torch
 import paper_2609_32114_b200 as ha
 from torch._subclasses.fake_tensor import FakeTensorMode
+ha.binding._torch_call()     # (a missing extension is not what this is about)
 with FakeTensorMode():
     e = lambda *s: torch.empty(*s, dtype=torch.bfloat16, device="cuda")
     f = lambda *s: torch.empty(*s, dtype=torch.float32, device="cuda")
