@@ -80,7 +80,7 @@ int forced_segments() {
 // Spans per sequence of the step path (tc_walk.cu): with few (sequence, head) pairs a sequence is cut into S runs that
 // are walked at the same time, in two launches, 2 S - 3 state-only runs and then S runs with outputs, with S - 2
 // products of 128^3 between them.  The rule's costs: 2.0 us per state-only step, 2.45 per step with outputs, 5 for
-// a CTA's start and end, 1.25 per product (5 when the products' 8 CTAs per pair do not all have an SM) and about 8 for
+// a CTA's start and end, 1.25 per product (0.75 where the products' CTAs take 8 columns, 5 where CTAs of 16 do not all have an SM: tc_span.cu) and about 8 for
 // the two further launches.  The steps take less now (tc_walk.cu), but with 1.65 and 2.25 here the choice gets no better: it
 // changes in 5 % of calls, and 44 of those timed both ways went from 13 % longer (one row of 1300 tokens, 4 heads, in order instead of 6
 // runs 28.8 -> 32.6 us) to 7 % shorter (three sequences of 3 k tokens, 4 heads, 13 runs -> 9 68.4 -> 63.4), 0.1 % longer on average.  A CTA fills an SM: equal lengths go in whole rounds, others pack (the longest first) to
@@ -114,7 +114,7 @@ int plan_spans(const Problem& p) {
   int best_s = 1;
   double best = launch_us(1, 1, true);
   for (int S = 2; S <= 32 && S <= longest; ++S) {
-    const double t = launch_us(2 * S - 3, S, false) + launch_us(S, S, true) + (8 * chains <= sms ? 1.25 : 5.0) * (S - 2) + 8.0;
+    const double t = launch_us(2 * S - 3, S, false) + launch_us(S, S, true) + (16 * chains <= sms ? 0.75 : 8 * chains <= sms ? 1.25 : 5.0) * (S - 2) + 8.0;
     if (t < best) { best = t; best_s = S; }
   }
   return best_s;

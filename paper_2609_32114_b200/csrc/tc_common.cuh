@@ -44,9 +44,17 @@ inline __host__ size_t tc_seg_bytes(size_t nj, int nseg, size_t rows, int HV) {
   return nj * nseg * 128 * 128 * (4 + 4 + 2) + align_up(rows * HV * 128 * 2, 1024);
 }
 
+// A transition Phi_s as operand fragments of warp-level products, 64 KiB of words: per 16 output keys w and 16 input keys ks, first
+// the high, then (128 words on) the low bf16 parts, 4 words a lane.  Fragment row (and k index) f of a block of 16 is key sigma(f),
+// sigma(2 t + e) = 4 t + e, sigma(8 + 2 t + e) = 4 t + 2 + e.  The word of output key 16 w + r and input keys v, v + 1 (v even; an odd
+// one gives the same word); rows r and r + 2 (r % 4 < 2) are neighbours.
+constexpr __host__ __device__ int phi_word(int w, int r, int v) {
+  return ((w * 8 + (v >> 4)) * 2 * 32 + (2 * (r >> 2) + (r & 1)) * 4 + ((v & 15) >> 2)) * 4 + ((v >> 1) & 1) * 2 + ((r >> 1) & 1);
+}
+
 // Scratch of a call whose sequences are cut into spans: per (sequence, V-head) and span the offset b_s, which the span's
-// true start state h_s replaces, and the transition Phi_s (fp32 128 x 128 each, [key][value channel]; span 0 has none: its
-// place keeps h0 in a call that works in place).
+// true start state h_s replaces (fp32 128 x 128, [key][value channel]), and the transition Phi_s (in phi_word order; span 0 has
+// none: its place keeps h0 in a call that works in place).
 struct SpanBuffers {
   int nspan;            // 1: off
   float* b;

@@ -1,12 +1,13 @@
 // Start states of the spans of a sequence that is cut into runs walked at the same time (tc_walk.cu):
 //   h_1 = b_0,   h_{s+1} = Phi_s h_s + b_s,   s = 1 .. nspan-2        (128 x 128 each, [key][value channel], fp32)
-// The columns (value channels) are independent: a CTA takes 16 of them, a warp 16 rows of every product.  What a product
-// costs is Phi_s on its way out of L2, 64 KiB per CTA, so that is copied in bulk one product ahead (operand fragments
-// read straight from global memory touch every line several times: 2.2 us per product).  The product itself is 48 warp-level
-// MMAs a warp on values split into two bf16 each (hi hi + hi lo + lo hi, fp32 accumulation: 2^-16 of the factors).  The
-// state's fragments go round the warps through 8 KiB of shared memory, transposed in registers.  What bounds it is the chain:
-// 1.2 us per product with every CTA on an SM (2 heads, ten products 18.4 us by themselves, twenty 30.8).  Fragment row r of a warp is key sigma(r), sigma(2 t + e) = 4 t + e, sigma(8 + 2 t + e)
-// = 4 t + 2 + e: the four columns of Phi that a lane needs are then neighbours.
+// The columns (value channels) are independent: a CTA takes 8 NT of them, a warp 16 rows of a product.  A product is warp-level MMAs on
+// values split into two bf16 each (hi hi + hi lo + lo hi, fp32 accumulation: 2^-16 of the factors), Phi_s copied in bulk ahead of it.  The
+// state's fragments go round the warps through shared memory, transposed by stmatrix.
+// What bounds it is the chain of products, and in a product the warp-level MMAs (24 NT a warp; a scheduler takes 14 - 16 cycles for each).
+// So few columns to a CTA while every CTA has an SM, and everything else kept out of the chain: Phi_s comes split and in fragment
+// order from the walk (phi_word), two groups of warps take the products in turn, one reading Phi_{s+1} into its registers under the other's product, and
+// b_s is fetched two products ahead (its latency alone was half of a product's time).  Per product, on B200: 8 columns 0.72 us, 16 columns 1.1; 16 columns by one group that
+// split Phi_s itself 1.2.  Calls: 2 heads, T = 16384, 22 runs 65.5 -> 55.6 us; 16 heads, T = 4096, 6 runs 55.9 -> 55.5.
 #include "tc_common.cuh"
 #include "tc_mma.cuh"
 
@@ -16,41 +17,26 @@ using namespace ptx;
 
 namespace {
 
-constexpr int kFixCols = 16, kFewPairs = 4;
-
-__device__ __forceinline__ void split_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
-  hi = pack_bf16(x, y);
-  const float2 h = unpack_bf16(hi);
-  lo = pack_bf16(x - h.x, y - h.y);
-}
-
 constexpr uint32_t kPhiBytes = 65536;
-constexpr uint32_t OFF_FRAG = 2 * kPhiBytes, OFF_FBAR = OFF_FRAG + 2 * 8 * 2 * 32 * 16, kSpanSmem = OFF_FBAR + 32;
+template <int NT> constexpr uint32_t kFragBytes = 2 * 8 * NT * 512;     // [set][k-step][n-tile]: hi, lo
+template <int NT, int BUFS> constexpr uint32_t kSpanSmem = BUFS * kPhiBytes + kFragBytes<NT> + BUFS * 8 + 8;
 
-// Two instances that differ in who issues the copies, a thread elected by elect.sync or thread 0, and for that in the code that the
-// compiler makes of the whole kernel (79 registers against 66).  Which is faster goes by the number of CTAs.  Calls, thread 0's first: up to
-// four (sequence, V-head) pairs, 32 CTAs, gain at any number of runs and packed or not (1 head, T = 12000, 19 runs 55.7 -> 53.2 us; 2 heads,
-// T = 3000, 8 runs 34.0 -> 33.3, T = 16000, 21 runs 65.9 -> 63.6; 4 heads, T = 3000 35.1 -> 34.7, T = 24000, 19 runs 90.1 -> 88.0; two sequences
-// of 11 k tokens, 2 heads 68.9 -> 67.7); five and six pairs are within 1 % either way; more lose (7 heads, T = 3000 38.3 -> 39.2; 8 heads, T = 6000
-// 52.5 -> 54.4; four rows of 4000, 2 heads 43.7 -> 46.1; 16 heads, T = 4096 55.9 -> 59.0).  The reason is not known: measure again after
-// an edit of this kernel or with another compiler.
-template <bool ELECT>
-__global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row, int HV, const int32_t* seq_len, int32_t* status) {
+// 8 NT columns.  Two groups of eight warps take the products in turn (TURNS), so that one reads Phi_{s+1} into its registers under the
+// other's product; or a single group.  BUFS: matrices in shared memory.
+template <int NT, bool TURNS, int BUFS>
+__global__ void __launch_bounds__(TURNS ? 512 : 256, 1) span_fix_kernel(SpanBuffers sb, int T_row, int HV, const int32_t* seq_len, int32_t* status) {
   extern __shared__ __align__(128) uint8_t sm[];
-  uint4 (*frag)[8][2][32] = reinterpret_cast<uint4(*)[8][2][32]>(sm + OFF_FRAG);   // [s & 1][k-step][n-tile][lane]: hi b0, b1, lo b0, b1
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + OFF_FBAR);                     // [2]
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 2);
-  const int nj = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + BUFS * kPhiBytes + kFragBytes<NT>);              // [BUFS]
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(full + BUFS);
+  const int nj = blockIdx.x, grp = threadIdx.x >> 8, warp = (threadIdx.x >> 5) & 7, lane = threadIdx.x & 31;
   const int g8 = lane >> 2, t = lane & 3;
   const int r0 = 16 * warp + 4 * (g8 >> 1) + (g8 & 1);   // sigma(g8); sigma(g8 + 8) is two further
   const size_t stride = 128 * 128;
   const float* phi = sb.phi + (size_t)nj * sb.nspan * stride;
-  const size_t tile = (size_t)nj * sb.nspan * stride + (size_t)r0 * 128 + blockIdx.y * kFixCols + 2 * t;
-  float* b = sb.b + tile;                                // h_s replaces b_s: the same thread reads the one and writes the other
+  float* b = sb.b + (size_t)nj * sb.nspan * stride + (size_t)r0 * 128 + blockIdx.y * 8 * NT + 2 * t;
   const int32_t* my_len = seq_len ? seq_len + nj / HV : nullptr;
   if (threadIdx.x == 0) {
-    mbar_init(&full[0], 1);
-    mbar_init(&full[1], 1);
+    for (int i = 0; i < BUFS; ++i) mbar_init(&full[i], 1);
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -61,83 +47,107 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
   const int len = my_len ? *my_len : T_row;              // (another kernel's table: read behind the wait)
   const int nst = (len + kStep - 1) / kStep;
   const int spspan = (nst + sb.nspan - 1) / sb.nspan;
+  const int last = nst > 0 ? min(sb.nspan - 2, (nst - 1) / spspan) : 0;   // products 1 .. last
   auto fetch = [&](int s) {                              // one thread
-    if (s + 1 >= sb.nspan) return;
-    mbar_expect_tx(&full[s & 1], kPhiBytes);
+    if (s > last) return;
+    const int f = s % BUFS;
+    mbar_expect_tx(&full[f], kPhiBytes);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      bulk_load(sm + (s & 1) * kPhiBytes + i * 16384, phi + (size_t)s * stride + i * 4096, 16384, &full[s & 1]);
+    for (int i = 0; i < 2; ++i)
+      bulk_load(sm + f * kPhiBytes + i * 32768, phi + (size_t)s * stride + i * 8192, 32768, &full[f]);
   };
-  auto issuing = [&]() { return ELECT ? warp == 0 && elect_one() : threadIdx.x == 0; };
-  if (issuing()) {
-    fetch(1);
-    fetch(2);
+  if (threadIdx.x == 0)
+    for (int s = 1; s <= BUFS; ++s) fetch(s);
+  struct Tile { float2 x[NT][2]; };                      // [n-tile][sigma(g8), sigma(g8 + 8)]
+  auto load_tile = [&](int s) {
+    Tile d;
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) d.x[n][e] = *reinterpret_cast<const float2*>(b + (size_t)s * stride + e * 2 * 128 + 8 * n);
+    return d;
+  };
+  auto save = [&](const Tile& d, int s) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) *reinterpret_cast<float2*>(b + (size_t)s * stride + e * 2 * 128 + 8 * n) = d.x[n][e];
+  };
+  const uint32_t frag = smem_u32(sm + BUFS * kPhiBytes) + lane * 16;
+  auto put = [&](const Tile& d, int s) {                 // as operand of product s
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      uint32_t w[4];
+      split_bf16(d.x[n][0].x, d.x[n][0].y, w[0], w[2]);
+      split_bf16(d.x[n][1].x, d.x[n][1].y, w[1], w[3]);
+      stsm4t(frag + (((s & 1) * 8 + warp) * NT + n) * 512, w);
+    }
+  };
+  uint32_t hi[8][4], lo[8][4];                           // this warp's rows of Phi_s
+  auto take = [&](int s) {
+    const int f = s % BUFS, ph = (s - 1) / BUFS & 1;
+    if (!mbar_test_wait(&full[f], ph)) mbar_wait(&full[f], ph, abort_flag);
+    const uint32_t sp = smem_u32(sm) + f * kPhiBytes + warp * 8192 + lane * 16;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      lds4(hi[k], sp + k * 1024);
+      lds4(lo[k], sp + k * 1024 + 512);
+    }
+  };
+  // Product s is group s % 2's, which holds h_s behind it as h_{s+1}.  Where b_s was, h_s goes, but only when product s has read that:
+  // behind the barrier ahead of product s + 1.
+  const int step = TURNS ? 2 : 1, first = TURNS && grp == 0 ? 2 : 1;
+  Tile h, o;                                             // h_s; b_s of the product to come
+  if (first <= last) {
+    o = load_tile(first);
+    take(first);
   }
-  float2 h[2][2], o[2][2];                               // h_s and b_s: [n-tile][sigma(g8), sigma(g8 + 8)]
-  auto load_tile = [&](const float* src, float2 (&d)[2][2]) {
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) d[n][e] = *reinterpret_cast<const float2*>(src + e * 2 * 128 + 8 * n);
-  };
-  load_tile(b, h);
-  for (int s = 1; s < sb.nspan; ++s) {
-    if (s + 1 < sb.nspan) load_tile(b + (size_t)s * stride, o);
-#pragma unroll
-    for (int n = 0; n < 2; ++n) {
-#pragma unroll
-      for (int e = 0; e < 2; ++e) *reinterpret_cast<float2*>(b + (size_t)s * stride + e * 2 * 128 + 8 * n) = h[n][e];
-      uint4 w;
-      split_bf16(h[n][0].x, h[n][0].y, w.x, w.z);
-      split_bf16(h[n][1].x, h[n][1].y, w.y, w.w);
-      w.x = transpose8x8(w.x); w.y = transpose8x8(w.y); w.z = transpose8x8(w.z); w.w = transpose8x8(w.w);
-      frag[s & 1][warp][n][lane] = w;
+  if (first == 1) {
+    h = load_tile(0);
+    if (last > 0) {
+      put(h, 1);
+      save(h, 1);                                        // (this thread has read b_1)
     }
-    __syncthreads();                                     // (and everyone is done with the product before)
-    if (s + 1 == sb.nspan) break;
-    if (s > 1 && issuing()) fetch(s + 1);
-    mbar_wait(&full[s & 1], ((s - 1) >> 1) & 1, abort_flag);
-    if (s * spspan >= nst) continue;                     // (the same for every thread of the CTA)
-    // Rows lie 512 bytes apart, so lanes of an odd row take the other k-step of a pair first: other banks.
-    const float* sp = reinterpret_cast<const float*>(sm + (s & 1) * kPhiBytes) + r0 * 128 + 4 * t;
-    const bool odd = g8 & 1;
-    float c[2][3][4] = {};
+  }
+  for (int s = first; s <= last; s += step) {
+    if (!TURNS) __syncthreads();
+    else if (s == 1) asm volatile("bar.sync 3, 256;" ::: "memory");
+    else if (grp == 0) asm volatile("bar.sync 1, 512;" ::: "memory");
+    else asm volatile("bar.sync 2, 512;" ::: "memory");
+    if ((threadIdx.x & 255) == 0) fetch(s + BUFS);        // (Phi_s is in registers)
+    if (s > first) save(h, TURNS ? s - 1 : s);
+    float c[NT][3][4] = {};
 #pragma unroll
-    for (int k = 0; k < 8; k += 2) {
-      float4 x[2], y[2];
+    for (int k = 0; k < 8; ++k)
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int o16 = 16 * k + 16 * (odd ? i ^ 1 : i);
-        x[i] = *reinterpret_cast<const float4*>(sp + o16);
-        y[i] = *reinterpret_cast<const float4*>(sp + 2 * 128 + o16);
-      }
-      if (odd) {
-        const float4 tx = x[0], ty = y[0];
-        x[0] = x[1]; x[1] = tx;
-        y[0] = y[1]; y[1] = ty;
+      for (int n = 0; n < NT; ++n) {
+        uint32_t w[4];
+        ldsm4(w, frag + (((s & 1) * 8 + k) * NT + n) * 512);
+        mma_bf16(c[n][0], hi[k], w[0], w[1]);
+        mma_bf16(c[n][1], hi[k], w[2], w[3]);
+        mma_bf16(c[n][2], lo[k], w[0], w[1]);
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        uint32_t hi[4], lo[4];
-        split_bf16(x[i].x, x[i].y, hi[0], lo[0]);
-        split_bf16(y[i].x, y[i].y, hi[1], lo[1]);
-        split_bf16(x[i].z, x[i].w, hi[2], lo[2]);
-        split_bf16(y[i].z, y[i].w, hi[3], lo[3]);
-#pragma unroll
-        for (int n = 0; n < 2; ++n) {
-          const uint4 w = frag[s & 1][k + i][n][lane];
-          mma_bf16(c[n][0], hi, w.x, w.y);
-          mma_bf16(c[n][1], hi, w.z, w.w);
-          mma_bf16(c[n][2], lo, w.x, w.y);
-        }
-      }
-    }
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
+    for (int n = 0; n < NT; ++n)
 #pragma unroll
       for (int e = 0; e < 2; ++e)
-        h[n][e] = make_float2(o[n][e].x + (c[n][0][2 * e] + (c[n][1][2 * e] + c[n][2][2 * e])),
-                              o[n][e].y + (c[n][0][2 * e + 1] + (c[n][1][2 * e + 1] + c[n][2][2 * e + 1])));
+        h.x[n][e] = make_float2(o.x[n][e].x + (c[n][0][2 * e] + (c[n][1][2 * e] + c[n][2][2 * e])),
+                                o.x[n][e].y + (c[n][0][2 * e + 1] + (c[n][1][2 * e + 1] + c[n][2][2 * e + 1])));
+    if (s < last) {
+      put(h, s + 1);
+      if (TURNS && grp == 0) asm volatile("bar.arrive 2, 512;" ::: "memory");
+      else if (TURNS) asm volatile("bar.arrive 1, 512;" ::: "memory");
+    }
+    if (s + step <= last) {
+      o = load_tile(s + step);
+      take(s + step);
+    }
+  }
+  __syncthreads();
+  if (!TURNS || grp == (last > 0 ? last & 1 : 1)) {      // the state behind the last product, also that of empty spans
+    for (int s = last + 1; s < sb.nspan; ++s) save(h, s);
+  } else if (last > 1) {
+    save(h, last);
   }
   if (threadIdx.x == 0 && *abort_flag) {
     report_status(status, HA_LA_ERR_TIMEOUT);
@@ -145,27 +155,41 @@ __global__ void __launch_bounds__(256) span_fix_kernel(SpanBuffers sb, int T_row
   }
 }
 
+struct Instance {
+  void (*kern)(SpanBuffers, int, int, const int32_t*, int32_t*);
+  int cols, threads;
+  uint32_t smem;
+};
+template <int NT, bool TURNS, int BUFS> constexpr Instance kInstance{span_fix_kernel<NT, TURNS, BUFS>, 8 * NT, TURNS ? 512 : 256, kSpanSmem<NT, BUFS>};
+
 }  // namespace
 
 cudaError_t configure_span_fix() {
-  cudaError_t e = cudaFuncSetAttribute(span_fix_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmem);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(span_fix_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanSmem);
+  for (const Instance& i : {kInstance<1, true, 3>, kInstance<2, true, 3>, kInstance<2, false, 2>}) {
+    static_assert(kSpanSmem<2, 3> <= 227 * 1024, "shared memory budget");
+    const cudaError_t e = cudaFuncSetAttribute(i.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)i.smem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_span_fix(const Problem& p, PlanView plan, const SpanBuffers& sb, int32_t* status, cudaStream_t stream) {
   timer_mark(stream, "tc_span_fix");
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.N * p.HV), 128 / kFixCols);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = kSpanSmem;
+  // As few columns to a CTA as leave every CTA an SM.  More CTAs than SMs: a group of warps alone (two rounds of those CTAs with one product, 32 heads:
+  // 245.6 us for a call, 246.0 with two groups, 249.9 with two such CTAs to an SM).
+  const int pairs = p.N * p.HV, sms = sm_count();
+  const Instance i = pairs * 16 <= sms ? kInstance<1, true, 3> : pairs * 8 <= sms ? kInstance<2, true, 3> : kInstance<2, false, 2>;
+  cfg.gridDim = dim3((unsigned)pairs, (unsigned)(128 / i.cols));
+  cfg.blockDim = dim3(i.threads);
+  cfg.dynamicSmemBytes = i.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = g_timer ? 0 : 1;                        // (per-kernel timing wants one kernel at a time)
-  auto kern = p.N * p.HV <= kFewPairs ? span_fix_kernel<true> : span_fix_kernel<false>;
-  return cudaLaunchKernelEx(&cfg, kern, sb, p.T_row, p.HV, (const int32_t*)plan.seq_len, status);
+  return cudaLaunchKernelEx(&cfg, i.kern, sb, p.T_row, p.HV, (const int32_t*)plan.seq_len, status);
 }
 
 }  // namespace ha_la

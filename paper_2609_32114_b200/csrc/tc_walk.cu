@@ -646,7 +646,27 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
     float* dst = nullptr;
     if (!OUT) dst = (trans ? p.span_phi : p.span_b) + (((size_t)n * p.HV + j) * p.nspan + span) * 16384;
     else if (p.hT && span == p.nspan - 1) dst = p.hT + ((size_t)n * p.HV + j) * 16384;
-    if (dst) {
+    if (!OUT && trans) {
+      // Phi_s as the start states' products take it (phi_word): split into two bf16, the halves of a pair of neighbouring columns v
+      // from neighbouring lanes.  An even lane writes the first 16 of this thread's rows, an odd one the others.
+      uint32_t* word = reinterpret_cast<uint32_t*>(dst) + phi_word(2 * g + (lane & 1), 0, v);
+      const bool odd = lane & 1;
+      float x[16], y[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const float got = __shfl_xor_sync(0xffffffffu, odd ? h[k] : h[16 + k], 1);
+        x[k] = odd ? got : h[k];
+        y[k] = odd ? h[16 + k] : got;
+      }
+#pragma unroll
+      for (int k = 0; k < 16; k += (k & 1) ? 3 : 1) {    // rows k and k + 2 are neighbours there
+        uint2 hi, lo;
+        split_bf16(x[k], y[k], hi.x, lo.x);
+        split_bf16(x[k + 2], y[k + 2], hi.y, lo.y);
+        *reinterpret_cast<uint2*>(word + phi_word(0, k, 0)) = hi;
+        *reinterpret_cast<uint2*>(word + phi_word(0, k, 0) + 128) = lo;
+      }
+    } else if (dst) {
 #pragma unroll
       for (int k = 0; k < 32; ++k) dst[(size_t)(32 * g + k) * 128 + v] = h[k];
     }

@@ -190,3 +190,13 @@ def test_start_states_on_both_sides_of_four_pairs(variant, hv, lens, runs, monke
     """Four (sequence, V-head) pairs and fewer have their start states from another instance than five and more."""
     monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
     helpers.check_parity(_inputs(variant, lens, len(lens) > 1, 1, hv, 397, gate_shift=4.0))
+
+
+@pytest.mark.parametrize("pairs", [9, 10, 18, 19])
+@pytest.mark.parametrize("runs", [2, 4, 8])
+def test_start_states_of_every_instance(pairs, runs, monkeypatch):
+    """Both sides of the numbers of pairs where the start states' CTAs change (148 SMs: 8 columns up to 9 pairs, 16 up to 18, one group of
+    warps beyond), without a product and with two and six of them, the last runs of the shorter sequence empty."""
+    monkeypatch.setenv("HA_LA_TC_SEGMENTS", str(runs))
+    lens = [1100] if pairs % 2 else [1100, 390]
+    helpers.check_parity(_inputs("gdn", lens, len(lens) > 1, 1, pairs // len(lens), 401, gate_shift=4.0))
