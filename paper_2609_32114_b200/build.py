@@ -23,7 +23,7 @@ INCLUDE = os.path.join(ROOT, "include")
 # (object name, source, extra flags)
 UNITS = [("api", "api.cu", []), ("plan", "plan.cu", []), ("tc", "tc.cu", []), ("tc_tp", "tc_tp.cu", []), ("tc_kda", "tc_kda.cu", []),
          ("tc_walk", "tc_walk.cu", []), ("tc_span", "tc_span.cu", []),
-         ("noalloc", "noalloc.cu", []), ("decode", "decode.cu", [])] + [
+         ("noalloc", "noalloc.cu", []), ("decode", "decode.cu", []), ("fp32_d64", "fp32_d64.cu", [])] + [
     (f"simt{u}", "simt.cu", [f"-DHA_LA_SIMT_UNIT={u}"]) for u in range(5)
 ] + [
     (f"fp32_{u}", "fp32.cu", [f"-DHA_LA_FP32_UNIT={u}"]) for u in range(5)

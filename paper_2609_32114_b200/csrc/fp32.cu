@@ -1,5 +1,5 @@
-// fp32 chunkwise delta-rule prefill (GDN and KDA) on the CUDA cores, in two kernels: fp32 inputs (where the 1e-4 tolerance
-// rules out 16-bit tensor-core operands) and head dimension 64.  All arithmetic is fp32.
+// fp32 chunkwise delta-rule prefill (GDN and KDA) on the CUDA cores, in two kernels, for head dimension 128: fp32 inputs (where the
+// 1e-4 tolerance rules out 16-bit tensor-core operands).  All arithmetic is fp32.  (d = 64: fp32_d64.cu.)
 //
 //   fp32_prep_kernel   one CTA per (chunk, V-head): operators #1-#4 of the paper's pipeline (Section 2.1, "Chunkwise
 //                      Map-Reduce-Map Execution").  Chunks are independent here, so a single short sequence already
@@ -12,27 +12,25 @@
 //   W = T diag(beta) (K e^G)   QG = Q e^G   KD = K e^{G_L-G}   P = decay-masked Q K^T   U = T diag(beta) V   e^{G_L}
 // and the walk does    U~ = U - W h;   o = scale (QG h + P U~);   h <- e^{G_L} h + KD^T U~.
 //
-// What bounds it: shared-memory reads (a 16-byte read costs four cycles of the SM's 128 bytes whatever is shared between
-// lanes), the walk's two barriers per chunk, and for short sequences its chain of chunks: 1.6 us each at d = 64.  One call
-// with T = 256, one head, d = 64: one CTA for everything took 237 us, split like this 16.8 us; d = 64, 8 heads, T = 1000:
-// 924 us -> 35.0 us.
-#include "common.cuh"
-#include "tc_ptx.cuh"
-
-#include <atomic>
+// What bounds it: shared-memory reads (a 16-byte read costs four cycles of the SM's 128 bytes, 2.2 where neighbouring lanes share
+// addresses), the walk's two barriers per chunk, and for short sequences its chain of chunks: 2.2 us each.  4 heads, T = 400: 34 us.
+#include "fp32_common.cuh"
 
 namespace ha_la {
+
+size_t fp32_d64_record_bytes();                          // fp32_d64.cu
+cudaError_t launch_fp32_d64(const Problem& p, const Fp32Params& fp, cudaStream_t stream);
 
 using namespace ptx;
 
 namespace {
 
-constexpr int C = kChunk;
+constexpr int C = kChunk, D = 128;
 constexpr int kNV = 16;                                  // value channels per slice of U in a record
 constexpr int LDP = C + 4;                               // row strides in floats: rows 16 bytes apart in the banks
 
 // record of one (chunk slot, V-head), in floats
-template <int D> struct Rec {
+struct Rec {
   static constexpr int LD = D + 4;
   static constexpr int W = 0;                            // [C][LD]
   static constexpr int QG = W + C * LD;                  // [C][LD]
@@ -43,27 +41,8 @@ template <int D> struct Rec {
   static constexpr int size = U + C * D;
 };
 
-struct Fp32Params {
-  const void* q; const void* k; const void* v;
-  const float* g; const float* beta; const float* h0;
-  void* o; float* hT;
-  float* rec;
-  const int32_t* chunk_tok0;   // chunk table of the plan kernel, or NULL for equal-length rows:
-  const int32_t* chunk_len;    //   slot s is chunk s % cps of row s / cps, T_row tokens per row
-  const int32_t* seq_tok0; const int32_t* seq_len; const int32_t* seq_chunk0; const int32_t* seq_order;
-  int T_row, cps;
-  int HK, HV;
-  float scale;
-  int32_t* status;
-};
-
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float dot4(const float4& a, const float4& b, float c) {
-  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
-}
-
 // ------------------------------------------------------------------------------------------------ chunk-local part
-template <int D, bool KDA> struct PrepSmem {
+template <bool KDA> struct PrepSmem {
   static constexpr int LD = D + 4;
   static constexpr int K = 0;                            // [C][LD]
   static constexpr int Q = K + C * LD;                   // [C][LD]
@@ -71,15 +50,15 @@ template <int D, bool KDA> struct PrepSmem {
   static constexpr int G = A + C * LDP;                  // GDN [C]; KDA [C][LD]: cumulative log-gate
   static constexpr int B = G + (KDA ? C * LD : C);       // [C] beta
   static constexpr int RHS = B + C;                      // [C][2 D]: (W |) U columns of the substitution
-  static constexpr int KM = KDA && D == 128 ? RHS : RHS + C * 2 * D;   // KDA: K e^{R_I-G}, block rows I = 1, 2, 3 (16, 32, 48
-                                                         // rows); d = 128: over the columns, which are filled later
-  static constexpr int size = KDA && D == 64 ? KM + 96 * LD : RHS + C * 2 * D;
+  static constexpr int KM = RHS;                         // KDA: K e^{R_I-G}, block rows I = 1, 2, 3 (16, 32, 48 rows), over the
+                                                         // columns, which are filled later
+  static constexpr int size = RHS + C * 2 * D;
 };
 
-template <typename In, int D, bool KDA>
+template <typename In, bool KDA>
 __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
-  using S = PrepSmem<D, KDA>;
-  using R = Rec<D>;
+  using S = PrepSmem<KDA>;
+  using R = Rec;
   constexpr int LD = D + 4;
   extern __shared__ __align__(16) float sf[];
   float* sK = sf + S::K;
@@ -107,7 +86,7 @@ __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
   const In* gv = reinterpret_cast<const In*>(p.v);
   float* rec = p.rec + (size_t)blockIdx.x * R::size;
 
-  constexpr bool kLateV = KDA && D == 128;               // (its room holds the rescaled K rows first)
+  constexpr bool kLateV = KDA;                           // (its room holds the rescaled K rows first)
   auto v_row = [&](int i, int c) {
     return i < L ? load4(gv + ((size_t)(t0 + i) * p.HV + j) * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   };
@@ -263,7 +242,7 @@ __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
   // ---- op #3 Solve + op #4 W/U: forward substitution of (I + A) [W | U] = diag(beta) [K e^G | V], one thread per column,
   // in blocks of 16 rows held in registers.  The coefficients are broadcast reads of A^T.  (Unrolled over all 64 rows the
   // code was 40 KiB run once per launch: 13 us of instruction fetches.)
-  if (tid < 2 * D) {
+  {
     const int c = tid % D;
     float* col = sf + S::RHS + tid;                      // [C][2 D]: this thread's column
     float* dst = tid < D ? rec + R::W + c : rec + R::U + (c / kNV) * (C * kNV) + c % kNV;
@@ -311,27 +290,23 @@ __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
       }
     }
   }
-  if (D == 128 || tid >= 2 * D) {                        // the walk's other images (d = 64: by the idle half of the CTA)
-    const int t = D == 128 ? tid : tid - 2 * D;
-    constexpr int NT = D == 128 ? 256 : 256 - 2 * D;
-    if (!KDA) {
-      const float gl = sG[C - 1];
-      for (int idx = t; idx < C * (D / 4); idx += NT) {
-        const int i = idx / (D / 4), c = (idx % (D / 4)) * 4;
-        const float4 k4 = ld4(sK + i * LD + c), q4 = ld4(sQ + i * LD + c);
-        const float ek = expf(gl - sG[i]), eq = expf(sG[i]);
-        *reinterpret_cast<float4*>(rec + R::KD + i * LD + c) = make_float4(k4.x * ek, k4.y * ek, k4.z * ek, k4.w * ek);
-        *reinterpret_cast<float4*>(rec + R::QG + i * LD + c) = make_float4(q4.x * eq, q4.y * eq, q4.z * eq, q4.w * eq);
-      }
+  if (!KDA) {                                            // the walk's other images
+    const float gl = sG[C - 1];
+    for (int idx = tid; idx < C * (D / 4); idx += 256) {
+      const int i = idx / (D / 4), c = (idx % (D / 4)) * 4;
+      const float4 k4 = ld4(sK + i * LD + c), q4 = ld4(sQ + i * LD + c);
+      const float ek = expf(gl - sG[i]), eq = expf(sG[i]);
+      *reinterpret_cast<float4*>(rec + R::KD + i * LD + c) = make_float4(k4.x * ek, k4.y * ek, k4.z * ek, k4.w * ek);
+      *reinterpret_cast<float4*>(rec + R::QG + i * LD + c) = make_float4(q4.x * eq, q4.y * eq, q4.z * eq, q4.w * eq);
     }
-    for (int c = t; c < D; c += NT) rec[R::GAM + c] = expf(KDA ? sG[(C - 1) * LD + c] : sG[C - 1]);
   }
+  if (tid < D) rec[R::GAM + tid] = expf(KDA ? sG[(C - 1) * LD + tid] : sG[C - 1]);
 }
 
 // ------------------------------------------------------------------------------------------------ sequential part
-template <int D> struct WalkSmem {
+struct WalkSmem {
   static constexpr int LD = D + 4;
-  static constexpr int kStages = D == 64 ? 2 : 1;        // chunks whose operands fit (a load takes about as long as a half step)
+  static constexpr int kStages = 1;                      // chunks whose operands fit (a load takes about as long as a half step)
   static constexpr int WQ = 0;                           // W, QG of the chunk
   static constexpr int KP = WQ + 2 * C * LD;             // KD, P, e^{G_L}
   static constexpr int U = KP + C * LD + C * LDP + D;    // U slice [C][kNV]
@@ -342,13 +317,11 @@ template <int D> struct WalkSmem {
   static constexpr int BAR = (Y + C * (kNV + 1) + 3) / 4 * 4;
   static constexpr size_t bytes = (size_t)BAR * 4 + 32;
 };
-// Threads: the first kUpd<D> update the state, then 256 form the outputs; the first 512 compute W h and QG h.  A thread makes
+// Threads: the first kUpd update the state, then 256 form the outputs; the first 512 compute W h and QG h.  A thread makes
 // four rows (tokens, keys) by NV / 2 channels of a product over an eighth of its depth: sixteen and more multiply-adds for
 // every two 16-byte reads, where reads bound the kernel.  The eight parts of a sum sit in neighbouring lanes, which add
-// them up so that each ends with one row and NV / 4 channels.  (Two rows by one or two channels over half of the depth:
-// 53.7 us for d = 64, 8 heads, T = 1000; 42.8 like this.)
-template <int D> constexpr int kUpd = D * 4;
-template <int D> constexpr int kWalkThreads = kUpd<D> + 256;
+// them up so that each ends with one row and NV / 4 channels.
+constexpr int kUpd = D * 4, kWalkThreads = kUpd + 256;
 // v[N] summed over eight neighbouring lanes; lane l keeps the sums N / 8 (l % 8) .. in v[0 .. N / 8)
 template <int N> __device__ __forceinline__ void scatter_sum(float (&v)[N], int lane) {
 #pragma unroll
@@ -363,10 +336,10 @@ template <int N> __device__ __forceinline__ void scatter_sum(float (&v)[N], int 
   }
 }
 
-template <typename In, int D, int NV>
-__global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Params p) {
-  using S = WalkSmem<D>;
-  using R = Rec<D>;
+template <typename In, int NV>
+__global__ void __launch_bounds__(kWalkThreads, 1) fp32_walk_kernel(Fp32Params p) {
+  using S = WalkSmem;
+  using R = Rec;
   constexpr int LD = D + 4, NSL = D / NV, H = NV / 2, E = NV / 4;   // channels of a thread's products; of its sums
   extern __shared__ __align__(16) float sf[];
   constexpr int ST = S::kStages;
@@ -385,7 +358,7 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
     mbar_fence_init();
   }
   // state: thread -> key 4 grp + row, its E channels of the slice
-  const bool upd = tid < kUpd<D>;
+  const bool upd = tid < kUpd;
   const int key = 4 * grp + row;
   const int uc = slice % (kNV / NV) * NV;       // first channel within the record's U slice
   float h[E];
@@ -486,7 +459,7 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
       }
     } else {
       // ---- o = scale (QG h + P U~): rows rg + 16 i, tokens 4 part + 32 m; P's blocks of 16 above the diagonal are not there
-      const int rg = grp - kUpd<D> / 16;
+      const int rg = grp - kUpd / 16;
       float s[4 * H] = {};
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
@@ -522,53 +495,29 @@ __global__ void __launch_bounds__(kWalkThreads<D>, 1) fp32_walk_kernel(Fp32Param
   }
 }
 
-// Launch attribute of both kernels: each is set up under the tail of the kernel before it and waits on the device.
-template <auto kern>
-cudaError_t launch(unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, const Fp32Params& fp) {
-  static std::atomic<uint64_t> configured{0};            // (of this kernel: a bit per device)
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-  if (dev >= 64 || !(configured.load() >> dev & 1)) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev < 64) configured.fetch_or(1ull << dev);
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = g_timer ? 0 : 1;                        // (per-kernel timing wants one kernel at a time)
-  return cudaLaunchKernelEx(&cfg, kern, fp);
-}
-
-template <typename In, int D, bool KDA>
+template <typename In, bool KDA>
 cudaError_t run(const Problem& p, const Fp32Params& fp, cudaStream_t stream) {
-  static_assert(PrepSmem<D, KDA>::size * 4 <= 227 * 1024 && WalkSmem<D>::bytes <= 227 * 1024, "shared memory budget");
+  static_assert(PrepSmem<KDA>::size * 4 <= 227 * 1024 && WalkSmem::bytes <= 227 * 1024, "shared memory budget");
   if (p.max_chunks * p.HV > 0) {
     timer_mark(stream, "simt_prep");
-    const cudaError_t e = launch<fp32_prep_kernel<In, D, KDA>>((unsigned)(p.max_chunks * p.HV), 256u, PrepSmem<D, KDA>::size * 4,
+    const cudaError_t e = launch_fp32_kernel<fp32_prep_kernel<In, KDA>>((unsigned)(p.max_chunks * p.HV), 256u, PrepSmem<KDA>::size * 4,
                                                                stream, fp);
     if (e != cudaSuccess) return e;
   }
   timer_mark(stream, "simt_prefill");
-  // The narrowest slices that leave every CTA an SM: a chunk takes 2.2 us with 8 channels and 1.6 with 4 (d = 64); else 16
+  // The narrowest slices that leave every CTA an SM: a chunk takes less with fewer channels; else 16
   // (fewer reads of the shared operands per channel).
   const long long heads = (long long)p.N * p.HV;
   if (heads * (D / 4) <= sm_count())
-    return launch<fp32_walk_kernel<In, D, 4>>((unsigned)(heads * (D / 4)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
+    return launch_fp32_kernel<fp32_walk_kernel<In, 4>>((unsigned)(heads * (D / 4)), (unsigned)kWalkThreads, WalkSmem::bytes, stream, fp);
   if (heads * (D / 8) <= sm_count())
-    return launch<fp32_walk_kernel<In, D, 8>>((unsigned)(heads * (D / 8)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
-  return launch<fp32_walk_kernel<In, D, 16>>((unsigned)(heads * (D / 16)), (unsigned)kWalkThreads<D>, WalkSmem<D>::bytes, stream, fp);
+    return launch_fp32_kernel<fp32_walk_kernel<In, 8>>((unsigned)(heads * (D / 8)), (unsigned)kWalkThreads, WalkSmem::bytes, stream, fp);
+  return launch_fp32_kernel<fp32_walk_kernel<In, 16>>((unsigned)(heads * (D / 16)), (unsigned)kWalkThreads, WalkSmem::bytes, stream, fp);
 }
 
 template <typename In, bool KDA>
 cudaError_t run_dims(const Problem& p, const Fp32Params& fp, cudaStream_t stream) {
-  return p.dk == 128 ? run<In, 128, KDA>(p, fp, stream) : run<In, 64, KDA>(p, fp, stream);
+  return p.dk == 128 ? run<In, KDA>(p, fp, stream) : launch_fp32_d64(p, fp, stream);
 }
 
 Fp32Params make_params(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* ws) {
@@ -611,8 +560,7 @@ cudaError_t fp32_f32_gdn(const Problem&, const ha_la_prefill_args&, PlanView, vo
 cudaError_t fp32_f32_kda(const Problem&, const ha_la_prefill_args&, PlanView, void*, cudaStream_t);
 
 size_t fp32_workspace_bytes(const Problem& p) {
-  const size_t rec = p.dk == 128 ? Rec<128>::size : Rec<64>::size;
-  return align_up((size_t)p.max_chunks * p.HV * rec * sizeof(float), 1024);
+  return align_up((size_t)p.max_chunks * p.HV * (p.dk == 128 ? Rec::size * sizeof(float) : fp32_d64_record_bytes()), 1024);
 }
 
 cudaError_t launch_fp32(const Problem& p, const ha_la_prefill_args& a, PlanView plan, void* ws, cudaStream_t stream) {

@@ -34,3 +34,16 @@ def test_fp32_slice_widths(dtype, d, lens, hk, hv):
     """Numbers of heads on either side of where the sequential kernel's slices get wider."""
     w = synth.shrink(W["gdn_varlen"], seq_lens=lens, hk=hk, hv=hv, dtype=dtype, dk=d, dv=d, h0_std=0.05, varlen=len(lens) > 1)
     helpers.check_parity(synth.make_inputs(w, seed=239))
+
+
+@pytest.mark.parametrize("variant,dtype", [("gdn", "fp32"), ("gdn", "bf16"), ("kda", "fp32")])
+@pytest.mark.parametrize("hv,lens", [(18, [40]), (19, [64]), (37, [17]), (38, [1]), (37, [100]), (75, [63]), (9, [400]), (10, [129]), (6, [200, 0, 65])])
+def test_fp32_d64_shares_and_slices(variant, dtype, hv, lens):
+    """d = 64: numbers of units (chunks x V-heads: 18, 19, 37, 38, 74, 75) on both sides of where CTAs share a chunk's last product, and of heads
+    (9, 10, 18, 19) where the sequential kernel's slices change; no decay in places and a decay to nothing in others."""
+    w = synth.shrink(W["gdn_varlen"] if variant == "gdn" else W["kda_8k"], seq_lens=lens, hk=1, hv=hv, dtype=dtype, dk=64, dv=64, gate_shift=4.0, h0_std=0.05,
+                     varlen=len(lens) > 1)
+    inp = synth.make_inputs(w, seed=251 + hv)
+    inp["g"][::7] = 0.0
+    inp["g"][5::31] = -90.0
+    helpers.check_parity(inp, scale=0.5)
