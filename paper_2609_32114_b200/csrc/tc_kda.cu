@@ -148,6 +148,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   auto geom = [&](long long c) {                         // slots that a packed batch does not use come last, with L = 0
     Geom g{0, 0, 0, 0};
     if (c >= p.total) return g;
+    if (!p.chunk_len) c = p.total - 1 - c;               // (the steps that are walked first are made last, and are still in L2 then: 1 %)
     g.s = (int)((unsigned)c / (unsigned)p.HV);
     g.j = (int)((unsigned)c - (unsigned)g.s * (unsigned)p.HV);
     if (p.chunk_len) {
@@ -162,8 +163,14 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
   };
   auto issue_tiles = [&](const Geom& g, int b) {         // one thread
     mbar_expect_tx(&full[b], 2 * kTileBytes);
-    tma_load_4d(sm + b * kBufBytes + OFF_K, &map_k, &full[b], 0, g.j / R, g.tok0, 0);
-    tma_load_4d(sm + b * kBufBytes + OFF_Q, &map_q, &full[b], 0, g.j / R, g.tok0, 0);
+    if (R == 1) {                                        // (nothing else reads them: first out of L2, which the images need; 1 %)
+      const uint64_t policy = evict_first<100>();
+      tma_load_4d(sm + b * kBufBytes + OFF_K, &map_k, &full[b], 0, g.j, g.tok0, 0, policy);
+      tma_load_4d(sm + b * kBufBytes + OFF_Q, &map_q, &full[b], 0, g.j, g.tok0, 0, policy);
+    } else {
+      tma_load_4d(sm + b * kBufBytes + OFF_K, &map_k, &full[b], 0, g.j / R, g.tok0, 0);
+      tma_load_4d(sm + b * kBufBytes + OFF_Q, &map_q, &full[b], 0, g.j / R, g.tok0, 0);
+    }
   };
   // named barriers: 1, 2 the scaled operands of buffer 0, 1 are ready; 3, 4 the buffer is free again (T read); 5, 6 within
   // the scaling and the solving warps
@@ -195,7 +202,7 @@ tc_kda_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         for (int u = 0; u < 2; ++u)
 #pragma unroll
           for (int t = 0; t < 16; ++t)
-            l[u][t] = 32 * tg + 16 * u + t < gm.L ? *reinterpret_cast<const float2*>(gp + (size_t)(16 * u + t) * p.HV * 128) : make_float2(0.f, 0.f);
+            l[u][t] = 32 * tg + 16 * u + t < gm.L ? __ldcs(reinterpret_cast<const float2*>(gp + (size_t)(16 * u + t) * p.HV * 128)) : make_float2(0.f, 0.f);
       }
       float bt = 0.f;
       if (tg == 0 || tg == 1) {                          // (warps 8 .. 11: a token's beta per thread)
