@@ -13,7 +13,8 @@
 // and the walk does    U~ = U - W h;   o = scale (QG h + P U~);   h <- e^{G_L} h + KD^T U~.
 //
 // What bounds it: shared-memory reads (a 16-byte read costs four cycles of the SM's 128 bytes, 2.2 where neighbouring lanes share
-// addresses), the walk's two barriers per chunk, and for short sequences its chain of chunks: 2.2 us each.  4 heads, T = 400: 34 us.
+// addresses), the walk's two barriers per chunk, and for short sequences its chain of chunks: 2.2 us each.  4 heads, T = 400: 31.7 us (32.2 with lanes that share rows
+// apart and the gates summed behind a barrier of their own), KDA, T = 300 42.7 (44.2).
 #include "fp32_common.cuh"
 
 namespace ha_la {
@@ -106,34 +107,32 @@ __global__ void __launch_bounds__(256) fp32_prep_kernel(Fp32Params p) {
     if (!kLateV) *reinterpret_cast<float4*>(sf + S::RHS + i * 2 * D + D + c) = v_row(i, c);
     if (KDA) *reinterpret_cast<float4*>(sG + i * LD + c) = g4;
   }
-  if (tid < C) {
-    sB[tid] = tid < L ? p.beta[(size_t)(t0 + tid) * p.HV + j] : 0.f;
-    if (!KDA) sG[tid] = tid < L ? p.g[(size_t)(t0 + tid) * p.HV + j] : 0.f;
+  const int warp = tid >> 5, lane = tid & 31;
+  if (warp < 2) sB[tid] = tid < L ? p.beta[(size_t)(t0 + tid) * p.HV + j] : 0.f;
+  // ---- op #1 Gate: chunk-local inclusive cumulative sum of the log-gate (GDN: by a warp while the tiles are on their way)
+  if (!KDA && warp == 2) {
+    float x0 = lane < L ? p.g[(size_t)(t0 + lane) * p.HV + j] : 0.f, x1 = lane + 32 < L ? p.g[(size_t)(t0 + lane + 32) * p.HV + j] : 0.f;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
+      if (lane >= o) { x0 += y0; x1 += y1; }
+    }
+    x1 += __shfl_sync(0xffffffffu, x0, 31);
+    sG[lane] = x0;
+    sG[lane + 32] = x1;
   }
   __syncthreads();
-
-  // ---- op #1 Gate: chunk-local inclusive cumulative sum of the log-gate
   if (KDA) {
     if (tid < D) {
       float acc = 0.f;
       for (int i = 0; i < C; ++i) { acc += sG[i * LD + tid]; sG[i * LD + tid] = acc; }
     }
-  } else if (tid < 32) {
-    float x0 = sG[tid], x1 = sG[tid + 32];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
-      if (tid >= o) { x0 += y0; x1 += y1; }
-    }
-    x1 += __shfl_sync(0xffffffffu, x0, 31);
-    sG[tid] = x0;
-    sG[tid + 32] = x1;
+    __syncthreads();
   }
-  __syncthreads();
 
   // ---- op #2: A (strictly lower, beta-scaled, negated: what the substitution adds) and P (lower incl. diagonal), in
-  // 16 x 16 blocks; thread (tr, tc) owns one entry of every block.
-  const int tr = tid >> 4, tc = tid & 15;
+  // 16 x 16 blocks; thread (tr, tc) owns one entry of every block.  Neighbouring lanes share columns: their reads are then one.
+  const int tr = (warp << 1) | (lane & 1), tc = lane >> 1;
   float kk[4][4], qk[4][4];                              // [block row][block column <= block row]
 #pragma unroll
   for (int a = 0; a < 4; ++a)
