@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(TURNS ? 512 : 256, 1) span_fix_kernel(SpanBuff
   };
   if (threadIdx.x == 0)
     for (int s = 1; s <= BUFS; ++s) fetch(s);
+  __syncwarp();                                          // (what comes is for converged warps: barriers, matrix instructions)
   struct Tile { float2 x[NT][2]; };                      // [n-tile][sigma(g8), sigma(g8 + 8)]
   auto load_tile = [&](int s) {
     Tile d;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(TURNS ? 512 : 256, 1) span_fix_kernel(SpanBuff
   auto take = [&](int s) {
     const int f = s % BUFS, ph = (s - 1) / BUFS & 1;
     if (!mbar_test_wait(&full[f], ph)) mbar_wait(&full[f], ph, abort_flag);
+    __syncwarp();                                        // (threads leave the wait one by one)
     const uint32_t sp = smem_u32(sm) + f * kPhiBytes + warp * 8192 + lane * 16;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -115,6 +117,7 @@ __global__ void __launch_bounds__(TURNS ? 512 : 256, 1) span_fix_kernel(SpanBuff
     else if (grp == 0) asm volatile("bar.sync 1, 512;" ::: "memory");
     else asm volatile("bar.sync 2, 512;" ::: "memory");
     if ((threadIdx.x & 255) == 0) fetch(s + BUFS);        // (Phi_s is in registers)
+    __syncwarp();
     if (s > first) save(h, TURNS ? s - 1 : s);
     float c[NT][3][4] = {};
 #pragma unroll

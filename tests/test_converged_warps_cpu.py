@@ -82,3 +82,41 @@ def test_planted_in_the_kernel(behind, find):
     src = open(os.path.join(CSRC, "tc_walk.cu")).read()
     first = src.index(behind)
     assert find(src[:first] + src[first:].replace("__syncwarp();", "", 1))
+
+
+# The start states' kernel issues its copies behind a test of the thread index, polls in every thread, and has its barriers and warp-wide
+# instructions in the code itself.
+ALIGNED = re.compile(r"__syncwarp|__syncthreads|\"bar\.|\b(?:ldsm4t?|stsm\w+|mma_\w+|transpose8x8|put|sync4)\(")
+
+
+def split_warps(src):
+    """Where threads of a warp may part, behind a polling wait or a block for one thread, and what aligned instruction comes next in the source
+    if not a __syncwarp or a __syncthreads."""
+    src = re.sub(r"//[^\n]*", "", src)
+    ends = [src.index(";", m.end()) + 1 for m in re.finditer(r"\bmbar_wait\(", src)]
+    ends += [_statement_end(src, m.end()) for m in re.finditer(r"\bif \((?:\(?threadIdx\.x(?: & \d+\))?|tid|lane) (?:==|<) \d+\)", src)]
+    bad = []
+    for end in ends:
+        nxt = ALIGNED.search(src, end)
+        if nxt and nxt.group() not in ("__syncwarp", "__syncthreads"):
+            bad.append((src.count("\n", 0, end) + 1, nxt.group()))
+    return bad
+
+
+def test_the_start_states_warps_stay_together():
+    src = open(os.path.join(CSRC, "tc_span.cu")).read()
+    assert src.count("mbar_wait(") == 1 and src.count("fetch(s") == 2   # (what there is to be found)
+    assert split_warps(src) == []
+
+
+@pytest.mark.parametrize("src", ["mbar_wait(a, 0, f);\n}; asm volatile(\"bar.sync 1, 512;\");", "if (lane == 0) x(); asm volatile(\"bar.arrive 2, 512;\");",
+                                 "if ((threadIdx.x & 255) == 0) fetch(s);\n ldsm4(w, a);", "if (threadIdx.x == 0)\n for (;;) fetch(s);\n put(h, 1); __syncwarp();",
+                                 "if (lane < 16) {\n y();\n } sync4();"])
+def test_planted_split(src):
+    assert len(split_warps(src)) == 1
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_planted_in_the_start_states(which):
+    src = open(os.path.join(CSRC, "tc_span.cu")).read().split("__syncwarp();")
+    assert len(src) == 4 and len(split_warps("__syncwarp();".join(src[:which + 1]) + "__syncwarp();".join(src[which + 1:]))) == 1
