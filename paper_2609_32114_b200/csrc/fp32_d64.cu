@@ -309,7 +309,10 @@ __global__ void __launch_bounds__(kPrepThreads, 1) fp32_prep64_kernel(Fp32Params
   // ---- op #3 Solve: T = (I + A)^-1 by four warps, blocks of 16 and two levels of joining, T_lo = T_hi (-A_lo T_lo').  Meanwhile the others make the
   // right-hand sides diag(beta) [K e^G | V] and (GDN) KD.
   if (warp < 4) {
-    auto sync4 = [&]() { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+    auto sync4 = [&]() {                                 // (lanes come out of stores and loops of their own)
+      __syncwarp();
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+    };
     {                                                    // diagonal block `warp`, a column per lane (the upper lanes repeat the lower)
       const int c = lane & 15, o = 16 * warp;
       float y[16];

@@ -120,3 +120,11 @@ def test_planted_split(src):
 def test_planted_in_the_start_states(which):
     src = open(os.path.join(CSRC, "tc_span.cu")).read().split("__syncwarp();")
     assert len(src) == 4 and len(split_warps("__syncwarp();".join(src[:which + 1]) + "__syncwarp();".join(src[which + 1:]))) == 1
+
+
+def test_barriers_behind_unequal_work():
+    """d = 64: half of a warp stores its columns and lanes run through loops of different length ahead of the barrier of the solving warps."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "fp32_d64.cu")).read())
+    assert "if (lane < 16)" in src and "for (int m = c & 16;" in src
+    barriers = re.findall(r"(__syncwarp\(\);\s*)?asm volatile\(\"bar\.", src)
+    assert barriers and all(barriers)
