@@ -195,7 +195,9 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
 
   // KDA's images, records and V do not fit L2 with what comes after them: what this launch is the last to read goes first, and of what the launch with outputs
   // reads again two thirds, so that the rest is still there then.  (T = 8192, 32 heads 241.6 -> 236 us with the images and records, 233 with V too; 16 heads on 8 q/k heads
-  // 127.1 -> 125.2 by the two thirds.  GDN's tiles the same way: 803 -> 836 us for 136 k tokens.)
+  // 127.1 -> 125.2 by the two thirds.  GDN's tiles the same way: 803 -> 836 us for 136 k tokens.)  The outputs are the caller's, who reads them next: streamed
+  // as well, a call takes up to 0.9 % less (T = 8192, 32 heads 234 -> 232) and a kernel that reads them 2 - 4 more (22.5 -> 26.6; call and reader, 32 heads, T = 4096 140.8 -> 143.4;
+  // 8 x 500 tokens 62.3 -> 63.7; only outputs larger than L2 gain, T = 16000 483 -> 481).
   uint64_t policy = 0;
   if (KDA) policy = OUT ? evict_first<100>() : evict_first<65>();
   auto copy = [&](void* dst, const void* src, uint32_t bytes, uint64_t* b) {
@@ -420,7 +422,7 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
             const int t = it * 8 + (lane >> 2);
             uint32_t w[4];
             lds4(w, tile + sw64_offset(t, lane & 3));
-            if (64 * half + t < left) __stcs(reinterpret_cast<uint4*>(orow + (size_t)(64 * half + t) * p.HV * 128), make_uint4(w[0], w[1], w[2], w[3]));
+            if (64 * half + t < left) *reinterpret_cast<uint4*>(orow + (size_t)(64 * half + t) * p.HV * 128) = make_uint4(w[0], w[1], w[2], w[3]);
           }
           __syncwarp();
         };

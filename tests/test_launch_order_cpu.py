@@ -77,3 +77,9 @@ def test_that_pause_is_by_the_clock():
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "tc_ptx.cuh")).read())
     body = src[src.index("void settle_copies()"):].split("\n}")[0]
     assert "%globaltimer" in src and re.search(r"for \(int i = 0; i < \d+ && global_ns\(\) - t0 < \d+;", body)
+
+
+def test_outputs_are_not_sent_past_l2():
+    """They are what the caller's next kernel reads."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "tc_walk.cu")).read())
+    assert "orow + " in src and not re.search(r"__st(?:cs|cg|wt)\(|st\.global\.(?:cs|L1::no_allocate)|L2::cache_hint", src)
