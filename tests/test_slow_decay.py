@@ -107,3 +107,35 @@ def test_start_states_are_seen(variant, hv, lens, runs, least, monkeypatch):
     assert got >= least
     off = list(_without(inp, _runs(inp, got)))
     assert len(off) >= (least if runs is None else 2 * runs // 3) - 2 and min(x.min() for x in off) > 10
+
+
+# ---- d = 64: a chunk's affine map h' = M h + b, o = N h + c.  Slices of 4, 8 and 16 channels in the sequential kernel (up to 9, 18 and more
+# (sequence, V-head) pairs), with chunks enough that every stage is used three times.
+CHUNKS = [(3, [700]), (12, [600]), (20, [450]), (10, [230, 400]), (7, [64, 0, 500])]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("keys", ["unit", "repeated"])
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("hv,lens", CHUNKS)
+def test_chunks_d64(variant, dtype, hv, lens, keys):
+    helpers.check_parity(_inputs(variant, lens, hv, 64, dtype, 419, keys))
+
+
+@pytest.mark.parametrize("keys", ["unit", "repeated"])
+@pytest.mark.parametrize("variant", ["gdn", "kda"])
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("hv,lens", CHUNKS)
+def test_chunks_d64_are_seen(variant, dtype, hv, lens, keys):
+    """... without M h, and with the decay alone for M."""
+    inp = _inputs(variant, lens, hv, 64, dtype, 419, keys)
+    seqs = _pieces(inp, CHUNK, lambda units: 1)
+
+    def decay(inp, r, h):
+        g = np.exp(inp["g"][r[0]:r[1]].astype(np.float64).sum(axis=0))
+        return h * (g[:, None, None] if variant == "gdn" else g[:, :, None])
+
+    for keep in (None, decay):
+        off = list(_without(inp, seqs, keep))
+        assert len(off) >= 5 and min(x.min() for x in off) > 1.5, keep
