@@ -83,3 +83,30 @@ def test_outputs_are_not_sent_past_l2():
     """They are what the caller's next kernel reads."""
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "tc_walk.cu")).read())
     assert "orow + " in src and not re.search(r"__st(?:cs|cg|wt)\(|st\.global\.(?:cs|L1::no_allocate)|L2::cache_hint", src)
+
+
+def _copying_kernels():
+    """Every kernel that copies in bulk, its body."""
+    for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        src = re.sub(r"//[^\n]*", "", open(f).read())
+        for part in src.split("__global__")[1:]:
+            name, body = re.search(r"(\w+_kernel)\s*\(", part), part[part.index("{"):part.index("\n}")]
+            if re.search(r"\b(?:bulk_load|tma_load_4d)\(", body):
+                yield name.group(1), body
+
+
+def unreported(kernels, header):
+    """Kernels that copy in bulk and neither report a wait that ran out, themselves or by the header's helper, nor let their copies land then."""
+    pause = r"report_status\([^;]*HA_LA_ERR_TIMEOUT\);\s*(?:ptx::)?settle_copies\(\);"
+    helper = re.search(r"void report_timeout\([^)]*\) \{\s*" + pause, re.sub(r"//[^\n]*", "", header))
+    return [k for k, body in kernels if not re.search(pause, body) and not (helper and "report_timeout(" in body)]
+
+
+def test_kernels_that_copy_report_a_wait_that_ran_out():
+    header = open(os.path.join(CSRC, "fp32_common.cuh")).read()
+    kernels = list(_copying_kernels())
+    assert {k for k, _ in kernels} == {"tc_tp_kernel", "tc_kda_kernel", "tc_walk_kernel", "span_fix_kernel", "fp32_walk_kernel", "fp32_walk64_kernel"}
+    assert unreported(kernels, header) == []
+    assert unreported(kernels, header.replace("ptx::settle_copies();", "")) == ["fp32_walk64_kernel"]
+    for k, body in kernels:                                # (planted: nobody reports)
+        assert unreported([(k, re.sub(r"report_\w+\(", "x(", body))], header) == [k]
