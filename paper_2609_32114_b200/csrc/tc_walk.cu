@@ -194,12 +194,15 @@ tc_walk_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant_
   };
 
   // KDA's images, records and V do not fit L2 with what comes after them: what this launch is the last to read goes first, and of what the launch with outputs
-  // reads again two thirds, so that the rest is still there then.  (T = 8192, 32 heads 241.6 -> 236 us with the images and records, 233 with V too; 16 heads on 8 q/k heads
-  // 127.1 -> 125.2 by the two thirds.  GDN's tiles the same way: 803 -> 836 us for 136 k tokens.)  The outputs are the caller's, who reads them next: streamed
-  // as well, a call takes up to 0.9 % less (T = 8192, 32 heads 234 -> 232) and a kernel that reads them 2 - 4 more (22.5 -> 26.6; call and reader, 32 heads, T = 4096 140.8 -> 143.4;
-  // 8 x 500 tokens 62.3 -> 63.7; only outputs larger than L2 gain, T = 16000 483 -> 481).
+  // reads again a third, so that the rest is still there then.  HBM bytes of a call without these policies -> with them (and those of tc_kda.cu): 16 heads, T = 4096 235 -> 201 MB,
+  // T = 8192 572 -> 502; 32 heads, T = 8192 1123 -> 1093.  Why a third: it loses nowhere.  None, 35, 50, 65, 100 % of what the states-only launch reads, us for a call: 16 heads,
+  // T = 8192 130.4 128.5 127.8 128.1 129.3; 8 heads, T = 16000 135.7 133.6 132.8 132.7 134.0; 32 heads on 16 q/k heads, T = 6000 177.4 175.6 175.5 177.6 179.8;
+  // 32 heads, T = 4096 126.4 126.0 126.7 127.7 128.3; two rows of 3000, 16 heads on 8 102.3 102.6 102.9 103.3 103.7; T = 8192 with 4 or 32 heads within 0.4 %.
+  // GDN's tiles the same way: 803 -> 836 us for 136 k tokens.  The outputs are the caller's, who reads them next: streamed as well, a call takes up to 0.9 % less (32 heads, T = 8192
+  // 234 -> 232) and a kernel that reads them 2 - 4 us more (22.5 -> 26.6; call and reader, 32 heads, T = 4096 140.8 -> 143.4; 8 x 500 tokens 62.3 -> 63.7; only outputs
+  // larger than L2 gain, T = 16000 483 -> 481).
   uint64_t policy = 0;
-  if (KDA) policy = OUT ? evict_first<100>() : evict_first<65>();
+  if (KDA) policy = OUT ? evict_first<100>() : evict_first<35>();
   auto copy = [&](void* dst, const void* src, uint32_t bytes, uint64_t* b) {
     if constexpr (KDA) bulk_load(dst, src, bytes, b, policy);
     else bulk_load(dst, src, bytes, b);
