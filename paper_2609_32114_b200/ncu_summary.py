@@ -63,12 +63,12 @@ def report(rep: str, workload: str, title: str, cmd: str) -> str:
 _UNIT = {"byte": 1.0, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9}
 
 
-KERNELS = (("tc_tp", "tc_prep"), ("tc_kda", "tc_prep"), ("span_fix", "tc_span_fix"), ("decode", "decode"),
+KERNELS = (("tc_tp", "tc_prep"), ("tc_kda", "tc_prep"), ("span_fix", "tc_span_fix"), ("decode", "decode"), ("fp32_prep", "simt_prep"), ("fp32_walk", "simt_prefill"),
            ("simt_prefill", "simt_prefill"), ("plan", "plan"))
 
 
 def kernel_key(name: str) -> str:
-    """Short kernel name used by bench.py: tc_prep, tc_span (states only), tc_span_fix, tc_chain, decode, simt_prefill, plan."""
+    """Short kernel name used by bench.py: tc_prep, tc_span (states only), tc_span_fix, tc_chain, decode, simt_prep, simt_prefill, plan."""
     if "tc_walk" in name:                                  # <KDA, OUT>
         return "tc_span" if re.search(r"tc_walk_kernel<[^,]*, *(0|false)>", name) else "tc_chain"
     for part, key in KERNELS:
