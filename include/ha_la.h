@@ -130,7 +130,7 @@ typedef struct {
 /* Host only: bytes of scratch ha_la_prefill needs for these shapes (pointers are ignored).
  * Returns HA_LA_OK and writes *out_bytes, or an error for invalid / unsupported shapes.
  * What takes the room: on the tensor-core path 37 KiB (GDN) or 133 KiB (KDA) per 128 tokens and V-head, and
- * 128 KiB per run, sequence and V-head where sequences are cut into runs; on the fp32 path 68 KB (d = 64) or
+ * 128 KiB per run, sequence and V-head where sequences are cut into runs; on the fp32 path 66 KB (d = 64) or
  * 152 KB (d = 128) per 64 tokens and V-head, 1.25 GB for 16,384 tokens and 32 heads at d = 128.  A caller who
  * cannot spare that has ha_la_prefill_noalloc, which keeps nothing per chunk and takes many times as long.  */
 int ha_la_prefill_workspace_bytes(const ha_la_prefill_args* args, size_t* out_bytes);

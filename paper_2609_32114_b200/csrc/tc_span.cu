@@ -7,7 +7,7 @@
 // So few columns to a CTA while every CTA has an SM, and everything else kept out of the chain: Phi_s comes split and in fragment
 // order from the walk (phi_word), two groups of warps take the products in turn, one reading Phi_{s+1} into its registers under the other's product, and
 // b_s is fetched two products ahead (its latency alone was half of a product's time).  Per product, on B200: 8 columns 0.72 us, 16 columns 1.1; 16 columns by one group that
-// split Phi_s itself 1.2.  Calls: 2 heads, T = 16384, 22 runs 65.5 -> 55.6 us; 16 heads, T = 4096, 6 runs 55.9 -> 55.5.
+// split Phi_s itself 1.2.  Calls: 2 heads, T = 16384 65.5 us in 22 runs -> 55.1 in 26; 16 heads, T = 4096, 6 runs 55.2 either way.
 #include "tc_common.cuh"
 #include "tc_mma.cuh"
 
