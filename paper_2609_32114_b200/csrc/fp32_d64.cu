@@ -13,7 +13,7 @@
 // product is exact there, their sums of 64 are the matrix unit's fp32), the inverse 2, L = [KD^T; P] T 1.9, L [K e^G | V] 4.4 of which fp32 multiply-adds are 3.4.
 // Measured on B200, calls, against one phase more per chunk and a substitution in the chunk-local kernel (us): 1 head, T = 256, fp32 16.8 -> 14.3; 8 heads, T = 1000,
 // bf16 34.5 -> 23.8, KDA 41.9 -> 30.7; two rows of 1000, 16 heads 88.2 -> 77.9; eight sequences of 100 to 512, 16 heads, fp32 144.3 -> 139.3; one chunk 12.7 -> 12.4.
-// Errors against 64 bits (rms of hT and of o) are 0.69 to 1.00 of what they were with gates of -0.13 per token and less on average.  With hardly any decay the new state is the sum of two large terms, M h and b,
+// Errors against 64 bits (rms of hT and of o) are 0.69 to 1.00 of what they were with gates of -0.18 per token and less on average.  With hardly any decay the new state is the sum of two large terms, M h and b,
 // where it was e^{G_L} h and a small one, and errors are 0.67 to 1.12 of what they were at -0.004 per token and 0.70 to 1.28 without any decay: 2.5e-7 instead of 2.1e-7 for independent keys,
 // 8.4e-7 instead of 6.7e-7 for eight keys over and over, less for keys that lean one way (T = 1000, 8 heads, GDN and KDA).
 #include "common.cuh"
